@@ -461,6 +461,27 @@ hm_status radix_sort_rows_cols(int32_t *rows, int32_t *tmp, int64_t nrows, int w
                                const int *key_cols, const int *key_bits, const uint32_t *key_xor,
                                int nkey, cudaStream_t stream, int *launches = nullptr);
 
+// Sorts of at most this many rows place each row by counting the rows before
+// it (n^2 compares over the whole GPU) instead of by a radix sort.  The two
+// cost the same at about 16,000 rows (155 us, hm_sort.cu); at 12,288 counting
+// takes about 95 us.
+constexpr int64_t kRankMaxRows = 12288;
+
+// 64 rows, from row0 on, of a list of n rows of `width` words: the list starts
+// at word `src` of the caller's rows, at word `dst` of the temporary and at
+// key `key0` of the packed keys.
+struct RankTile {
+  int64_t src, dst;
+  int32_t key0, n, width, row0;
+};
+constexpr int kRankTileRows = 64;
+
+// Sorts many lists (nrows rows in all, at most `longest` in one), each
+// lexicographically by all its columns (values below 2^bits), through `tmp`;
+// `tiles` (device) lists every list's tiles.
+hm_status rank_sort_tiles(int32_t *rows, int32_t *tmp, const RankTile *tiles, int ntiles, int64_t nrows,
+                          int64_t longest, int width_max, int bits, cudaStream_t stream);
+
 // out[i] = in[0] + ... + in[i-1] for i in [0, n); values and total below 2^32.
 hm_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, cudaStream_t stream);
 
