@@ -164,21 +164,19 @@ __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__rest
   }
 }
 
-__device__ __forceinline__ void filter_insert(uint64_t h, uint32_t nblk, uint32_t *__restrict__ words) {
-  const FilterSlot f = filter_slot_of(h, nblk);
-  uint32_t *w = words + 8 * (size_t)f.blk;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) atomicOr(w + i, 1u << filter_bit(f.bits, i));
+__device__ __forceinline__ void filter_insert(ArcKey k, uint32_t nword, unsigned long long *__restrict__ words) {
+  const uint2 m = filter_bits(k);
+  atomicOr(words + filter_word(k, nword), ((unsigned long long)m.y << 32) | m.x);
 }
 
 __global__ void k_filter(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
-                         const int32_t *__restrict__ elab, int64_t m, uint32_t nblk,
-                         uint32_t *__restrict__ words) {
+                         const int32_t *__restrict__ elab, int64_t m, uint32_t nword,
+                         unsigned long long *__restrict__ words) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t h = pair_key(src[e], dst[e]);
-    filter_insert(h, nblk, words);
-    filter_insert(labelled_key(h, elab[e]), nblk, words);
+    const ArcKey h = pair_key(src[e], dst[e]);
+    filter_insert(h, nword, words);
+    filter_insert(labelled_key(h, elab[e]), nword, words);
   }
 }
 
@@ -350,9 +348,9 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   HM_CUDA_TRY(dmalloc(&g->vi, n));
   HM_CUDA_TRY(dmalloc(&g->off, n));
   HM_CUDA_TRY(dmalloc(&g->vdir, n));
-  g->afilt_nblk = (uint32_t)std::max<int64_t>(1, (m + 7) / 8);
-  HM_CUDA_TRY(dmalloc(&g->afilt, 2 * (int64_t)g->afilt_nblk));
-  HM_CUDA_TRY(cudaMemsetAsync(g->afilt, 0, 32 * (size_t)g->afilt_nblk, s));
+  g->afilt_nword = (uint32_t)(4 * std::max<int64_t>(1, (m + 7) / 8));
+  HM_CUDA_TRY(dmalloc(&g->afilt, (int64_t)g->afilt_nword));
+  HM_CUDA_TRY(cudaMemsetAsync(g->afilt, 0, 8 * (size_t)g->afilt_nword, s));
   g->ahash_nbkt = (uint32_t)std::max<int64_t>(1, m);
   HM_CUDA_TRY(dmalloc(&g->ahash, 2 * (int64_t)g->ahash_nbkt));
   HM_CUDA_TRY(cudaMemsetAsync(g->ahash, 0xff, 32 * (size_t)g->ahash_nbkt, s));
@@ -370,8 +368,8 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     if (st != HM_OK) return st;
     k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 0, 1, g->src, g->out_adj, g->out_elab,
                                              out_off, err);
-    k_filter<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->afilt_nblk,
-                                              reinterpret_cast<uint32_t *>(g->afilt));
+    k_filter<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->afilt_nword,
+                                              reinterpret_cast<unsigned long long *>(g->afilt));
     k_hash<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->ahash_nbkt,
                                             g->ahash, err);
     st = build_groups(rows, tmp, m, n, 0, 1, d_vlab, out_off, nbits, be, xe, bv, xv, s, T,
@@ -401,7 +399,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   if (h_err & kErrDup) return HM_ERR_DUP_EDGE;
   if (h_err & kErrHash) return HM_ERR_CUDA;  // cannot happen (twice as many slots as arcs)
   g->bytes = sizeof(int32_t) * 7 * (size_t)m + (sizeof(int4) * 2 + sizeof(int2)) * (size_t)n +
-             sizeof(int4) * (size_t)(g->ndir_out + g->ndir_in) + 32 * (size_t)g->afilt_nblk +
+             sizeof(int4) * (size_t)(g->ndir_out + g->ndir_in) + 8 * (size_t)g->afilt_nword +
              32 * (size_t)g->ahash_nbkt;
   return HM_OK;
 }

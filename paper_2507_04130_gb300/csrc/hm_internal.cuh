@@ -9,7 +9,7 @@
 //   in_elab  int32[m]  label of each in-arc, parallel to in_adj
 //   vi       int4[n]   {vertex label, out-degree, in-degree, 0}
 //   off      int2[n]   {first out-arc, first in-arc}   (m < 2^31, so 32-bit offsets)
-//   afilt    uint4[2*B] arc filter: B = ceil(m/8) blocks of 256 bits holding two
+//   afilt    uint2[W]  arc filter: W = 4 * ceil(m/8) words of 64 bits holding two
 //                      keys per arc, (u, v) and (u, v, label), 16 bits per key
 //                      (64 MB for 16M arcs, within the 129 MB L2)
 //   ahash    int4[2*H] arc hash table: H = m buckets of two 16-byte slots
@@ -53,8 +53,8 @@ struct DevGraph {
   // split-block Bloom filter over the arcs, keyed by (u, v) and by (u, v,
   // label): a "no" is exact, a "maybe" needs the search.  Searches over more
   // than filt_min entries probe it first (filt_min < 0: never).
-  const uint4 *afilt;
-  uint32_t afilt_nblk;
+  const uint2 *afilt;
+  uint32_t afilt_nword;
   int32_t filt_min;
   // exact arc lookup in one or two 32-byte reads, for what the filter lets through
   const int4 *ahash;
@@ -70,7 +70,7 @@ enum CheckSite : int {
   kChkDirOut = 2,   // gdir_out entry
   kChkDirIn = 3,    // gdir_in entry
   kChkList = 4,     // src, out/in adjacency and labels, grouped lists (position < m)
-  kChkFilter = 5,   // arc filter block
+  kChkFilter = 5,   // arc filter word
   kChkHash = 6,     // arc hash bucket
 };
 
@@ -217,46 +217,49 @@ __device__ __forceinline__ int32_t search_c(const int32_t *__restrict__ a, int32
 // Every arc (u, v) with label l enters the filter under two keys: the pair
 // (u, v) -- "is there an arc at all", for induced non-arcs and the opposite-arc
 // test -- and the triple (u, v, l) -- "is there an arc with this label", for
-// the pattern's arcs.  A key owns one 256-bit block (eight 32-bit words)
-// chosen by the high half of its 64-bit hash and sets one bit in each word;
-// bit i sits at the top five bits of the low half times the i-th of eight odd
-// constants (a split-block Bloom filter).  The pair hash is the splitmix64
-// finalizer (Steele, Lea and Flood, "Fast splittable pseudorandom number
-// generators", OOPSLA 2014); the triple's hash is the pair's xor a
-// label-dependent constant.  The eight constants are splitmix64 outputs from
-// seed 0x243F6A8885A308D3, made odd.  At 16 bits per key a key that was never
-// inserted passes all eight bits with probability about 0.1 %; an inserted key
-// always passes.
-__host__ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-  return z ^ (z >> 31);
-}
+// the pattern's arcs.  A key's two 64-bit hashes are sums A u + B v (+ C (l + 1))
+// with fixed odd constants (multilinear hashing: the upper halves of such sums
+// are pairwise independent over the choice of the constants; Dietzfelbinger,
+// "Universal hashing and k-wise independent random variables via integer
+// arithmetic without primes", STACS 1996).  The constants are the first six
+// splitmix64 outputs from seed 0x243F6A8885A308D3, made odd.  The first sum's
+// upper half chooses a 64-bit word, the second's four bits in it, two in each
+// half.  At 16 bits per key a key that was never inserted passes with
+// probability about 0.5 % (measured on R-MAT arcs); an inserted key always
+// passes.  The sums are linear, so the part of an endpoint that stays the same
+// over many probes is computed once; a probe is about 20 instructions and one
+// 8-byte load.  (A 256-bit block with one bit in each of eight words and a
+// 64-bit finalizer as the hash passed 0.1 % but took about 60 instructions,
+// two loads, and eight atomics per key to build; with this one the R-MAT scale
+// 20 bi-fan takes 7.78 instead of 8.37 ms.)
+constexpr uint64_t kHashU1 = 0x2cb0f69f4abea221ull, kHashV1 = 0x9417034723148989ull,
+                   kHashL1 = 0xdd555950609dfe03ull, kHashU2 = 0xdbafb150deb12801ull,
+                   kHashV2 = 0x7e789b2e6c442cb7ull, kHashL2 = 0xf41e5636c7e4f8c5ull;
 
-struct FilterSlot {
-  uint32_t blk;   // block index
-  uint32_t bits;  // low half of the key's hash; bit i is at filter_bit(bits, i)
+struct ArcKey {
+  uint64_t a, b;
 };
 
-__host__ __device__ __forceinline__ FilterSlot filter_slot_of(uint64_t h, uint32_t nblk) {
-  FilterSlot f;
-  f.blk = (uint32_t)(((h >> 32) * (uint64_t)nblk) >> 32);
-  f.bits = (uint32_t)h;
-  return f;
+__host__ __device__ __forceinline__ ArcKey pair_key(int32_t u, int32_t v) {
+  return ArcKey{kHashU1 * (uint32_t)u + kHashV1 * (uint32_t)v, kHashU2 * (uint32_t)u + kHashV2 * (uint32_t)v};
 }
 
-__host__ __device__ __forceinline__ uint32_t filter_bit(uint32_t bits, int i) {
-  const uint32_t salt[8] = {0x2cb0f69fu, 0x94170347u, 0xdd555951u, 0xdbafb151u,
-                            0x7e789b2fu, 0xf41e5637u, 0x0959d151u, 0xa97316f1u};
-  return (bits * salt[i]) >> 27;
+__host__ __device__ __forceinline__ ArcKey labelled_key(ArcKey k, int32_t lab) {
+  const uint64_t l = (uint64_t)(uint32_t)lab + 1;
+  return ArcKey{k.a + kHashL1 * l, k.b + kHashL2 * l};
 }
 
-__host__ __device__ __forceinline__ uint64_t pair_key(int32_t u, int32_t v) {
-  return mix64(((uint64_t)(uint32_t)u << 32) | (uint32_t)v);
+__host__ __device__ __forceinline__ uint32_t filter_word(ArcKey k, uint32_t nword) {
+  return (uint32_t)(((k.a >> 32) * (uint64_t)nword) >> 32);
 }
 
-__host__ __device__ __forceinline__ uint64_t labelled_key(uint64_t pair, int32_t lab) {
-  return pair ^ (0x632be59bd9b4e019ull * ((uint64_t)(uint32_t)lab + 1));
+// The key's bits in its word: two in each 32-bit half.
+__host__ __device__ __forceinline__ uint2 filter_bits(ArcKey k) {
+  const uint32_t h = (uint32_t)(k.b >> 32);
+  uint2 m;
+  m.x = (1u << (h >> 27)) | (1u << ((h >> 22) & 31u));
+  m.y = (1u << ((h >> 17) & 31u)) | (1u << ((h >> 12) & 31u));
+  return m;
 }
 
 // ---- bounds checks -------------------------------------------------------------
@@ -298,22 +301,11 @@ __device__ __forceinline__ int32_t search_g(const DevGraph &G, const int32_t *__
 }
 
 template <bool kCount>
-__device__ __forceinline__ bool filter_has(const DevGraph &G, uint64_t h, Bytes &bytes) {
-  const FilterSlot f = filter_slot_of(h, G.afilt_nblk);
-  const size_t blk = (size_t)HM_AT(G, f.blk, G.afilt_nblk, kChkFilter);
-  // the block is one 32-byte sector; its first four words already reject
-  // about 98 % of the keys that were never inserted, so the other four are
-  // read (from the same sector, now in L1) and tested only when those pass
-  const uint4 a = __ldg(G.afilt + 2 * blk);
-  if (kCount) bytes += 32;
-  const uint32_t x = f.bits;
-  const uint32_t t = (a.x >> filter_bit(x, 0)) & (a.y >> filter_bit(x, 1)) & (a.z >> filter_bit(x, 2)) &
-                     (a.w >> filter_bit(x, 3));
-  if (!(t & 1u)) return false;
-  const uint4 b = __ldg(G.afilt + 2 * blk + 1);
-  const uint32_t u = (b.x >> filter_bit(x, 4)) & (b.y >> filter_bit(x, 5)) & (b.z >> filter_bit(x, 6)) &
-                     (b.w >> filter_bit(x, 7));
-  return u & 1u;
+__device__ __forceinline__ bool filter_has(const DevGraph &G, ArcKey k, Bytes &bytes) {
+  const uint2 w = __ldg(G.afilt + HM_AT(G, filter_word(k, G.afilt_nword), G.afilt_nword, kChkFilter));
+  if (kCount) bytes += 8;
+  const uint2 m = filter_bits(k);
+  return ((m.x & ~w.x) | (m.y & ~w.y)) == 0;
 }
 
 // false: there is certainly no arc u -> v.  true: there may be.
@@ -328,8 +320,8 @@ __device__ __forceinline__ bool arc_maybe(const DevGraph &G, int32_t u, int32_t 
 // pair's hash selects.  Slots fill in order and are never removed, so an empty
 // slot (u = -1) ends a probe sequence.  There are as many buckets as arcs
 // (half the slots used), so a lookup nearly always reads one sector.
-__host__ __device__ __forceinline__ uint32_t hash_bucket(uint64_t pair, uint32_t nbkt) {
-  return (uint32_t)(((pair & 0xffffffffull) * (uint64_t)nbkt) >> 32);
+__host__ __device__ __forceinline__ uint32_t hash_bucket(ArcKey pair, uint32_t nbkt) {
+  return (uint32_t)(((pair.b >> 32) * (uint64_t)nbkt) >> 32);
 }
 
 // Is u -> v an arc?  If so, *lab is its label.
@@ -405,8 +397,8 @@ struct hm_graph {
   int2 *off;
   int32_t *gout_adj, *gin_adj;
   int4 *gdir_out, *gdir_in, *vdir;
-  uint4 *afilt;
-  uint32_t afilt_nblk;
+  uint2 *afilt;
+  uint32_t afilt_nword;
   int4 *ahash;
   uint32_t ahash_nbkt;
   int64_t ndir_out, ndir_in;
@@ -420,7 +412,7 @@ struct hm_graph {
   hm::DevGraph dev() const {
     return hm::DevGraph{n,        m,        src,     out_adj,  out_elab, in_adj,     in_elab,
                         vi,       off,      gout_adj, gin_adj, gdir_out, gdir_in,    vdir,
-                        afilt,    afilt_nblk, hm::filter_min(), ahash, ahash_nbkt, ndir_out, ndir_in, check};
+                        afilt,    afilt_nword, hm::filter_min(), ahash, ahash_nbkt, ndir_out, ndir_in, check};
   }
 };
 
