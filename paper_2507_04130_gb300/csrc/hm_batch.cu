@@ -206,7 +206,7 @@ constexpr uint64_t kRankMaxCompares = 1ull << 29;  // run_batch: below, rows are
 // patterns that fit and flag them (fit[i] = 1); the others' rows are not valid.
 hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int32_t *modes,
                     int32_t npat, int32_t *rows, const uint64_t *row_offsets, uint64_t *counts,
-                    cudaStream_t s, uint8_t *fit = nullptr) {
+                    cudaStream_t s, uint8_t *fit = nullptr, uint64_t workspace = kLevelWorkspace) {
   if (!g || npat < 0 || (npat > 0 && (!pats || !modes || !counts))) return HM_ERR_ARG;
   if (npat == 0) return HM_OK;
   const bool want_rows = rows != nullptr || row_offsets != nullptr;
@@ -359,6 +359,36 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
   t_ov.stop();
 
   // ---- one persistent extension launch for every pattern
+  const hm_tuning tu = tuning();
+  const bool counters = counters_enabled();
+  NvtxRange r_ext("hm.batch_extend");
+  Timer t_ext(s, timing);
+  bool ran_levels = false;
+  if (default_search(tu) && !counters && budget_chunks() == 0 && nraw) {
+    LvLaunch L{};
+    L.g = g;
+    L.ctl = &ctl->lv;
+    L.seeds = seeds;
+    L.nseeds = nseeds;
+    L.max_seeds = (int64_t)nraw;
+    L.rows = rows;
+    L.npat = npat;
+    L.plans = plans.data();
+    L.seed_pid = seed_pid;
+    L.counts = d_counts;
+    L.row_off = d_off;
+    L.row_cap = d_cap;
+    L.row_cursor = d_cursor;
+    L.want_rows = want_rows;
+    L.workspace = workspace;
+    int grid = 0, threads = 0;
+    const hm_status r = levels_run(L, s, &ran_levels, &grid, &threads);
+    if (r != HM_OK) return r;
+    st.extend_grid = grid;
+    st.extend_block = threads;
+    if (ran_levels) ++launches;
+  }
+  if (!ran_levels) {
   Task *qbuf;
   unsigned long long *qseq;
   HM_CUDA_TRY(sc.get((void **)&qbuf, sizeof(Task) * kQueueCap));
@@ -366,7 +396,6 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
   k_qinit<<<64, 256, 0, s>>>(qseq);
   launches += 1;
   ExtArgs A{};
-  const hm_tuning tu = tuning();
   A.split_min = tu.split_min;
   A.pair_mode = tu.pair_mode;
   A.seeds_per_fetch = tu.seeds_per_fetch;
@@ -393,17 +422,15 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
   A.grp_slots = grp_slots;
   const int slot = min_blocks_slot(tu.extend_min_blocks);
   const size_t smem = warp_smem_bytes(grp_slots) * kExtWarps;
-  const bool counters = counters_enabled();
   bool sym = false;
   for (const Plan &pl : plans) sym |= pl.naut > 1;
   const int grid = extend_grid<true>(want_rows, counters, smem, slot, false, sym);
   if (grid <= 0) return HM_ERR_CUDA;
   st.extend_grid = grid;
   st.extend_block = kExtThreads;
-  NvtxRange r_ext("hm.batch_extend");
-  Timer t_ext(s, timing);
   extend_kernel<true>(want_rows, counters, slot, false, sym)<<<grid, kExtThreads, smem, s>>>(G, plans[0], A);
   launches += 1;
+  }
   t_ext.stop();
   HM_CUDA_TRY(cudaGetLastError());
   Ctl h;
@@ -417,6 +444,10 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
   st.ms_extend = t_ext.ms();
   st.seeds_scanned = (uint64_t)m;
   st.states_injected = any_ov ? h.nseeds : h.nseeds_raw;
+  if (ran_levels) {
+    h.status = h.lv.status;
+    h.chunks = h.lv.chunks;
+  }
   st.tasks_donated = h.donated;
   st.chunks = h.chunks;
   st.bytes_extend = h.bytes_extend;
@@ -513,11 +544,10 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
 }  // namespace hm
 
 namespace hm {
-hm_status enumerate_batch_fit(const hm_graph *g, const hm_pattern *const *patterns, const int32_t *modes,
-                              int32_t npat, int32_t *rows_dev, const uint64_t *row_offsets, uint64_t *counts,
-                              uint8_t *fit, cudaStream_t stream) {
-  if (npat > 0 && (!rows_dev || !row_offsets || !fit)) return HM_ERR_ARG;
-  return run_batch(g, patterns, modes, npat, rows_dev, row_offsets, counts, stream, fit);
+hm_status batch_run(const hm_graph *g, const hm_pattern *const *patterns, const int32_t *modes, int32_t npat,
+                    int32_t *rows_dev, const uint64_t *row_offsets, uint64_t *counts, uint8_t *fit,
+                    uint64_t workspace, cudaStream_t stream) {
+  return run_batch(g, patterns, modes, npat, rows_dev, row_offsets, counts, stream, fit, workspace);
 }
 }  // namespace hm
 

@@ -29,6 +29,7 @@ namespace hm {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int64_t kMaxDense = 64;  // classes with dense group offsets (k_dense holds them in one 64-bit mask)
 constexpr int kW = 4;  // row width: src, dst, arc label, aux
 
 enum : uint32_t { kErrRange = 1, kErrSelf = 2, kErrDup = 4, kErrHash = 8 };
@@ -161,6 +162,45 @@ __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__rest
     uint32_t os = oidx ? oidx[o0] : 0, oe = oidx ? oidx[o1] : 0;
     uint32_t is = iidx ? iidx[i0] : 0, ie = iidx ? iidx[i1] : 0;
     vdir[v] = make_int4((int32_t)os, (int32_t)(oe - os), (int32_t)is, (int32_t)(ie - is));
+  }
+}
+
+// Dense group offsets of one direction (see DevGraph): one warp per vertex, the
+// vertex's directory entries on its lanes, two rounds of 32 classes.  A class
+// without a group starts where the next one does.
+__global__ void k_dense(const int4 *__restrict__ vdir, const int2 *__restrict__ off, const int4 *__restrict__ vi,
+                        const int4 *__restrict__ dir, int32_t n, int64_t m, int in, int32_t ncls, int32_t nvl,
+                        int32_t al0, int32_t vl0, int32_t *__restrict__ gofs) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
+    const int4 vd = vdir[v];
+    const int2 o = off[v];
+    const int4 info = vi[v];
+    const int32_t first = in ? vd.z : vd.x, cnt = in ? vd.w : vd.y, base = in ? o.y : o.x;
+    const int32_t len = in ? info.z : info.y;
+    // which classes have a group, and where the lane's entries (lane, lane + 32) start
+    unsigned long long have = 0;
+    int32_t s0 = len, s1 = len;
+    if (lane < cnt) {
+      const int4 e = dir[(int64_t)first + lane];
+      have |= 1ull << ((e.x - al0) * nvl + (e.y - vl0));
+      s0 = e.z;
+    }
+    if (lane + 32 < cnt) {
+      const int4 e = dir[(int64_t)first + lane + 32];
+      have |= 1ull << ((e.x - al0) * nvl + (e.y - vl0));
+      s1 = e.z;
+    }
+    const unsigned long long all = (unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)have) |
+                                   (unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)(have >> 32)) << 32;
+    for (int c0 = 0; c0 < ncls; c0 += 32) {
+      const int c = c0 + lane;
+      const int at = __popcll(all & ((1ull << (c & 63)) - 1));  // groups of earlier classes
+      const int32_t a = __shfl_sync(0xffffffffu, s0, at & 31), b = __shfl_sync(0xffffffffu, s1, at & 31);
+      if (c < ncls) gofs[v * ncls + c] = base + (at >= cnt ? len : at < 32 ? a : b);
+    }
+    if (v == n - 1 && lane == 0) gofs[(int64_t)n * ncls] = (int32_t)m;
   }
 }
 
@@ -393,6 +433,23 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   if (n)
     k_vertex<<<grid_for(n), kThreads, 0, s>>>(d_vlab, out_off, in_off, oidx, iidx, n, g->vi, g->off,
                                               g->vdir);
+  // dense group offsets while there are few classes and the tables are no larger than the arcs' own data
+  const int64_t nal = m ? (int64_t)hb.emax - hb.emin + 1 : 0, nvl = m ? (int64_t)hb.vmax - hb.vmin + 1 : 0;
+  if (m && nal <= kMaxDense && nvl <= kMaxDense && nal * nvl <= kMaxDense &&
+      (int64_t)n * nal * nvl <= 8 * std::max<int64_t>(m, 1 << 16)) {
+    g->nal = (int32_t)nal;
+    g->nvl = (int32_t)nvl;
+    g->al0 = hb.emin;
+    g->vl0 = hb.vmin;
+    g->ncls = (int32_t)(nal * nvl);
+    const int64_t len = (int64_t)n * g->ncls + 1;
+    HM_CUDA_TRY(dmalloc(&g->gofs_out, len));
+    HM_CUDA_TRY(dmalloc(&g->gofs_in, len));
+    for (int in = 0; in < 2; ++in)
+      k_dense<<<grid_for(32 * (int64_t)n), kThreads, 0, s>>>(g->vdir, g->off, g->vi, in ? g->gdir_in : g->gdir_out, n,
+                                                             m, in, g->ncls, g->nvl, g->al0, g->vl0,
+                                                             in ? g->gofs_in : g->gofs_out);
+  }
   HM_CUDA_TRY(cudaMemcpyAsync(&h_err, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaStreamSynchronize(s));
   HM_CUDA_TRY(cudaGetLastError());
@@ -400,14 +457,14 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   if (h_err & kErrHash) return HM_ERR_CUDA;  // cannot happen (twice as many slots as arcs)
   g->bytes = sizeof(int32_t) * 7 * (size_t)m + (sizeof(int4) * 2 + sizeof(int2)) * (size_t)n +
              sizeof(int4) * (size_t)(g->ndir_out + g->ndir_in) + 8 * (size_t)g->afilt_nword +
-             32 * (size_t)g->ahash_nbkt;
+             32 * (size_t)g->ahash_nbkt + (g->ncls ? sizeof(int32_t) * 2 * ((size_t)n * g->ncls + 1) : 0);
   return HM_OK;
 }
 
 void free_graph_arrays(hm_graph *g) {
   void *ptrs[] = {g->src,     g->out_adj,  g->out_elab, g->in_adj,   g->in_elab, g->vi,
                   g->off,     g->gout_adj, g->gin_adj,  g->gdir_out, g->gdir_in, g->vdir,
-                  g->afilt,   g->ahash,    g->check};
+                  g->afilt,   g->ahash,    g->check,    g->gofs_out, g->gofs_in};
   for (void *p : ptrs)
     if (p) cudaFree(p);
 }

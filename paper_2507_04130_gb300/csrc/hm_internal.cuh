@@ -59,6 +59,12 @@ struct DevGraph {
   // exact arc lookup in one or two 32-byte reads, for what the filter lets through
   const int4 *ahash;
   uint32_t ahash_nbkt;
+  // dense group offsets: the group of class c = (arc label - first arc label) *
+  // vertex labels + (neighbour label - first vertex label) of vertex v is
+  // [gofs[v * ncls + c], gofs[v * ncls + c + 1]) of the grouped lists; ncls = 0:
+  // too many classes, only the directory
+  const int32_t *gofs_out, *gofs_in;
+  int32_t ncls;
   // directory lengths, and the violation word of bounds-checked builds (null otherwise)
   int64_t ndir_out, ndir_in;
   unsigned long long *check;
@@ -72,6 +78,7 @@ enum CheckSite : int {
   kChkList = 4,     // src, out/in adjacency and labels, grouped lists (position < m)
   kChkFilter = 5,   // arc filter word
   kChkHash = 6,     // arc hash bucket
+  kChkGroup = 7,    // dense group offset
 };
 
 // One pairwise condition between the position being extended (p) and an
@@ -402,6 +409,8 @@ struct hm_graph {
   int4 *ahash;
   uint32_t ahash_nbkt;
   int64_t ndir_out, ndir_in;
+  int32_t *gofs_out, *gofs_in;  // dense group offsets (null: ncls = 0)
+  int32_t ncls, al0, vl0, nal, nvl;  // classes; first labels and label counts
   unsigned long long *check;  // bounds-checked builds: the violation word (device)
   size_t bytes;
   // multi-property graphs (hm_load_graph_props): the sorted distinct property
@@ -412,7 +421,7 @@ struct hm_graph {
   hm::DevGraph dev() const {
     return hm::DevGraph{n,        m,        src,     out_adj,  out_elab, in_adj,     in_elab,
                         vi,       off,      gout_adj, gin_adj, gdir_out, gdir_in,    vdir,
-                        afilt,    afilt_nword, hm::filter_min(), ahash, ahash_nbkt, ndir_out, ndir_in, check};
+                        afilt,    afilt_nword, hm::filter_min(), ahash, ahash_nbkt, gofs_out, gofs_in, ncls, ndir_out, ndir_in, check};
   }
 };
 
@@ -434,6 +443,11 @@ hm_tuning tuning();  // current process-wide extension knobs (validated)
 inline int32_t wps_shift(const hm_tuning &t, bool shared = false) {
   if (t.warps_per_state == 0) return shared ? 2 : 0;
   return t.warps_per_state >= 4 ? 2 : t.warps_per_state >= 2 ? 1 : 0;
+}
+// All knobs at their defaults: the extension runs level by level (hm_levels.cu).
+inline bool default_search(const hm_tuning &t) {
+  return t.extend_min_blocks == 4 && t.split_min == 64 && t.pair_mode == 0 && t.seeds_per_fetch == 1 &&
+         t.poll_every == 128 && t.leaf_flatten > 0 && t.arc_filter == 1 && t.warps_per_state == 0 && t.lookahead <= 0;
 }
 uint64_t budget_ms();
 uint64_t budget_chunks();
@@ -477,12 +491,14 @@ hm_status rank_sort_tiles(int32_t *rows, int32_t *tmp, const RankTile *tiles, in
 // out[i] = in[0] + ... + in[i-1] for i in [0, n); values and total below 2^32.
 hm_status exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t n, cudaStream_t stream);
 
-// Batched enumeration that keeps what fits (the query server's single pass):
-// every count, and for each pattern whose count fits its region [row_offsets[i],
-// row_offsets[i+1]) its sorted rows there and fit[i] = 1; fit[i] = 0 otherwise.
-hm_status enumerate_batch_fit(const hm_graph *g, const hm_pattern *const *patterns, const int32_t *modes,
-                              int32_t npat, int32_t *rows_dev, const uint64_t *row_offsets, uint64_t *counts,
-                              uint8_t *fit, cudaStream_t stream);
+// A batched call (hm_count_batch, hm_enumerate_batch) with a limit on the
+// memory its extension takes for the levels' states.  With `fit` (the query
+// server's single pass) it keeps what fits: every count, and for each pattern
+// whose count fits its region [row_offsets[i], row_offsets[i+1]) its sorted
+// rows there and fit[i] = 1; fit[i] = 0 otherwise.
+hm_status batch_run(const hm_graph *g, const hm_pattern *const *patterns, const int32_t *modes, int32_t npat,
+                    int32_t *rows_dev, const uint64_t *row_offsets, uint64_t *counts, uint8_t *fit,
+                    uint64_t workspace, cudaStream_t stream);
 
 int bits_for(int64_t n);  // bits needed for values in [0, n)
 int num_sms();

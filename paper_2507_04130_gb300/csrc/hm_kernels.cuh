@@ -51,6 +51,7 @@
 #include <vector>
 
 #include "hm_internal.cuh"
+#include "hm_levels.cuh"
 
 namespace hm {
 
@@ -100,6 +101,7 @@ struct Ctl {
   unsigned long long lanes;                   // candidates examined (instrumented launches only)
   unsigned long long level_chunks[kMaxK];     // per depth (instrumented launches only)
   unsigned long long level_lanes[kMaxK];
+  LvCtl lv;                                   // extension level by level
 };
 
 struct ExtArgs {

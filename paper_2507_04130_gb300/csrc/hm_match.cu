@@ -163,6 +163,8 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   // (induced calls: at most kInducedGroupCap seeds per group).
   const hm_tuning tu = tuning();
   const bool share = p->k > 2 && plan.defer1 && tu.share_seeds > 0;
+  // default knobs: level by level; the instrumented kernels and a chunk budget belong to the depth-first search
+  const bool by_level = p->k > 2 && default_search(tu) && !counters && budget_chunks() == 0;
   const int4 *groups = nullptr;
   Timer t_grp(s, timing && share);
   if (share) {
@@ -187,7 +189,8 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
       if (r != HM_OK) return r;
       launches += nl;
       const int gb = (int)std::min<unsigned long long>((ns + 256) / 256, (unsigned long long)sms * 8);
-      k_seed_group_flags<<<gb, 256, 0, s>>>(seeds, (int64_t)ns, plan.induced ? kInducedGroupCap : 0, flag);
+      k_seed_group_flags<<<gb, 256, 0, s>>>(seeds, (int64_t)ns, plan.induced && !by_level ? kInducedGroupCap : 0,
+                                           flag);
       r = exclusive_scan_u32(flag, idx, (int64_t)ns + 1, s);
       if (r != HM_OK) return r;
       k_seed_groups<<<gb, 256, 0, s>>>(seeds, (int64_t)ns, flag, idx, gr, &ctl->ngroups);
@@ -202,9 +205,36 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   // a4 + a5: state injection and extension
   const bool rows = want == Want::kRows;
   Timer t_ext(s, timing && p->k > 2);
+  bool ran_levels = false;
   {  // the extension's launches
   NvtxRange r_ext("hm.extend");
-  if (p->k == 2) {
+  if (by_level) {
+    LvLaunch L{};
+    L.g = g;
+    L.ctl = &ctl->lv;
+    L.seeds = seeds;
+    L.nseeds = share ? &ctl->ngroups : nseeds;
+    L.max_seeds = m;
+    L.groups = groups;
+    L.sorted_seeds = share ? seeds : nullptr;
+    L.root_mask = root_mask;
+    L.plan = &plan;
+    L.rows = rows ? out : nullptr;
+    L.cap = rows ? cap : 0;
+    L.want_rows = rows;
+    L.workspace = kLevelWorkspace;
+    int grid = 0, threads = 0;
+    const hm_status r = levels_run(L, s, &ran_levels, &grid, &threads);
+    if (r != HM_OK) return r;
+    if (ran_levels) {
+      ++launches;
+      st.extend_grid = grid;
+      st.extend_block = threads;
+      t_ext.stop();
+    }
+  }
+  if (ran_levels) {
+  } else if (p->k == 2) {
     k_seed_rows<<<sms * 4, 256, 0, s>>>(plan, seeds, nseeds, rows ? out : nullptr, cap, ctl);
     ++launches;
     HM_CUDA_TRY(cudaGetLastError());
@@ -259,6 +289,11 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   st.ms_extend = t_ext.ms();
   st.seeds_scanned = (uint64_t)(e_end - e_begin);
   st.states_injected = plan.ov_need > 0 ? h.nseeds : h.nseeds_raw;
+  if (ran_levels) {
+    h.status = h.lv.status;
+    h.count = h.lv.count;
+    h.chunks = h.lv.chunks;
+  }
   st.tasks_donated = h.donated;
   st.chunks = h.chunks;
   st.matches = h.count;

@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "hm_internal.cuh"
+#include "hm_levels.cuh"
 
 namespace {
 
@@ -70,6 +71,7 @@ struct hm_server {
   int32_t nslots = 1;
   int32_t max_batch = 64;
   uint64_t mem_budget = 0;
+  uint64_t workspace = 0;         // bytes a slot's extension may take for its levels
   uint64_t row_guess = 1u << 18;  // rows a query's region holds on the first pass
   // arcs per (source label, arc label, target label)
   std::map<std::tuple<int32_t, int32_t, int32_t>, uint64_t> triples;
@@ -92,8 +94,10 @@ struct hm_server {
 namespace {
 
 // Device memory a batch takes besides its queries' seed queues and rows: the
-// donation queue, its sequence words and the control block.
+// states of the extension's levels (or the depth-first search's donation
+// queue) and the control block.
 constexpr uint64_t kBatchFixed = (12ull << 20);
+constexpr uint64_t kSlotWorkspace = (8ull << 20);
 
 void serve_slot(hm_server *S, int slot) {
   cudaSetDevice(S->device);
@@ -140,7 +144,8 @@ void serve_slot(hm_server *S, int slot) {
     }
     hm_status st = HM_OK;
     if (!any_rows) {
-      st = hm_count_batch(S->g, pats.data(), modes.data(), nb, counts.data(), stream);
+      st = hm::batch_run(S->g, pats.data(), modes.data(), nb, nullptr, nullptr, counts.data(), nullptr, S->workspace,
+                         stream);
       for (int32_t i = 0; i < nb && st == HM_OK; ++i) batch[i]->count = counts[i];
     } else {
       // one pass: rows into regions of row_guess rows (as many as the budget holds)
@@ -166,8 +171,8 @@ void serve_slot(hm_server *S, int slot) {
         (void)cudaGetLastError();
         st = HM_ERR_OOM;
       } else {
-        st = hm::enumerate_batch_fit(S->g, pats.data(), modes.data(), nb, d_rows, off.data(), counts.data(),
-                                     fit.data(), stream);
+        st = hm::batch_run(S->g, pats.data(), modes.data(), nb, d_rows, off.data(), counts.data(), fit.data(),
+                           S->workspace, stream);
         if (st == HM_OK) {
           for (int32_t i = 0; i < nb; ++i) {
             auto &q = batch[i];
@@ -224,7 +229,8 @@ void serve_slot(hm_server *S, int slot) {
             (void)cudaGetLastError();
             st = HM_ERR_OOM;
           } else {
-            st = hm_enumerate_batch(S->g, rp.data(), rm.data(), nr, d2, off2.data(), rc.data(), stream);
+            st = hm::batch_run(S->g, rp.data(), rm.data(), nr, d2, off2.data(), rc.data(), nullptr, S->workspace,
+                               stream);
             if (st == HM_OK) {
               for (int32_t j = 0; j < nr; ++j) {
                 auto &q = batch[take[j]];
@@ -315,6 +321,10 @@ extern "C" hm_status hm_server_create(const hm_graph *g, int32_t nslots, int32_t
     delete S;
     return HM_ERR_ARG;  // the budget cannot admit even one batch
   }
+  // what a slot's extension may take for its levels: what kBatchFixed leaves beside the control block, more
+  // under a budget that hardly notices it (then taken off the budget)
+  S->workspace = std::min<uint64_t>(hm::kLevelWorkspace, std::max<uint64_t>(kSlotWorkspace, S->mem_budget / (64u * (uint64_t)nslots)));
+  S->mem_budget -= (S->workspace - kSlotWorkspace) * (uint64_t)nslots;
   for (int32_t i = 0; i < nslots; ++i) S->threads.emplace_back(serve_slot, S, i);
   *out = S;
   return HM_OK;
