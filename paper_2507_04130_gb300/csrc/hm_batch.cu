@@ -330,8 +330,12 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
   t_edge.stop();
   HM_CUDA_TRY(cudaGetLastError());
   // ---- overlap test (patterns without one pass their seeds through)
+  const hm_tuning tu = tuning();
+  const bool counters = counters_enabled();
+  const bool by_level = g->ncls > 0 && default_search(tu) && !counters && budget_chunks() == 0;
   bool any_ov = false;
   for (const Plan &P : plans) any_ov |= P.ov_need > 0;
+  any_ov = any_ov && !by_level;  // level by level the test costs more than the states it removes (see run_match)
   const int2 *seeds = seeds_a;
   const int32_t *seed_pid = pid_a;
   const unsigned long long *nseeds = &ctl->nseeds_raw;
@@ -359,12 +363,10 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
   t_ov.stop();
 
   // ---- one persistent extension launch for every pattern
-  const hm_tuning tu = tuning();
-  const bool counters = counters_enabled();
   NvtxRange r_ext("hm.batch_extend");
   Timer t_ext(s, timing);
   bool ran_levels = false;
-  if (default_search(tu) && !counters && budget_chunks() == 0 && nraw) {
+  if (by_level && nraw) {
     LvLaunch L{};
     L.g = g;
     L.ctl = &ctl->lv;

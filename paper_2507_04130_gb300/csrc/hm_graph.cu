@@ -35,7 +35,7 @@ constexpr int kW = 4;  // row width: src, dst, arc label, aux
 enum : uint32_t { kErrRange = 1, kErrSelf = 2, kErrDup = 4, kErrHash = 8 };
 
 struct Bounds {
-  int32_t emin, emax, vmin, vmax;
+  int32_t emin, emax, vmin, vmax, maxdeg;
 };
 
 __global__ void k_pack(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
@@ -153,7 +153,8 @@ __global__ void k_zero_off(int64_t *__restrict__ off, int32_t n) {
 __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__restrict__ out_off,
                          const int64_t *__restrict__ in_off, const uint32_t *__restrict__ oidx,
                          const uint32_t *__restrict__ iidx, int32_t n, int4 *__restrict__ vi,
-                         int2 *__restrict__ voff, int4 *__restrict__ vdir) {
+                         int2 *__restrict__ voff, int4 *__restrict__ vdir, Bounds *__restrict__ bnd) {
+  int32_t most = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
     int64_t o0 = out_off[v], o1 = out_off[v + 1], i0 = in_off[v], i1 = in_off[v + 1];
@@ -162,7 +163,10 @@ __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__rest
     uint32_t os = oidx ? oidx[o0] : 0, oe = oidx ? oidx[o1] : 0;
     uint32_t is = iidx ? iidx[i0] : 0, ie = iidx ? iidx[i1] : 0;
     vdir[v] = make_int4((int32_t)os, (int32_t)(oe - os), (int32_t)is, (int32_t)(ie - is));
+    most = max(most, (int32_t)max(o1 - o0, i1 - i0));
   }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((threadIdx.x & 31) == 0 && most) atomicMax(&bnd->maxdeg, most);
 }
 
 // Dense group offsets of one direction (see DevGraph): one warp per vertex, the
@@ -366,7 +370,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   HM_CUDA_TRY(T.get((void **)&err, sizeof(uint32_t)));
   HM_CUDA_TRY(T.get((void **)&bnd, sizeof(Bounds)));
   HM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-  const Bounds init{INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN};
+  const Bounds init{INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN, 0};
   HM_CUDA_TRY(cudaMemcpyAsync(bnd, &init, sizeof(Bounds), cudaMemcpyHostToDevice, s));
 
   if (m) k_pack<<<grid_for(m), kThreads, 0, s>>>(d_src, d_dst, d_elab, m, n, rows, err, bnd);
@@ -432,7 +436,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   }
   if (n)
     k_vertex<<<grid_for(n), kThreads, 0, s>>>(d_vlab, out_off, in_off, oidx, iidx, n, g->vi, g->off,
-                                              g->vdir);
+                                              g->vdir, bnd);
   // dense group offsets while there are few classes and the tables are no larger than the arcs' own data
   const int64_t nal = m ? (int64_t)hb.emax - hb.emin + 1 : 0, nvl = m ? (int64_t)hb.vmax - hb.vmin + 1 : 0;
   if (m && nal <= kMaxDense && nvl <= kMaxDense && nal * nvl <= kMaxDense &&
@@ -451,8 +455,10 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
                                                              in ? g->gofs_in : g->gofs_out);
   }
   HM_CUDA_TRY(cudaMemcpyAsync(&h_err, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  HM_CUDA_TRY(cudaMemcpyAsync(&hb, bnd, sizeof(Bounds), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaStreamSynchronize(s));
   HM_CUDA_TRY(cudaGetLastError());
+  g->maxdeg = hb.maxdeg;
   if (h_err & kErrDup) return HM_ERR_DUP_EDGE;
   if (h_err & kErrHash) return HM_ERR_CUDA;  // cannot happen (twice as many slots as arcs)
   g->bytes = sizeof(int32_t) * 7 * (size_t)m + (sizeof(int4) * 2 + sizeof(int2)) * (size_t)n +

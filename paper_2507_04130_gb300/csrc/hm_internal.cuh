@@ -65,6 +65,7 @@ struct DevGraph {
   // too many classes, only the directory
   const int32_t *gofs_out, *gofs_in;
   int32_t ncls;
+  int32_t maxdeg;  // largest out- or in-degree
   // directory lengths, and the violation word of bounds-checked builds (null otherwise)
   int64_t ndir_out, ndir_in;
   unsigned long long *check;
@@ -411,6 +412,7 @@ struct hm_graph {
   int64_t ndir_out, ndir_in;
   int32_t *gofs_out, *gofs_in;  // dense group offsets (null: ncls = 0)
   int32_t ncls, al0, vl0, nal, nvl;  // classes; first labels and label counts
+  int32_t maxdeg;                    // largest out- or in-degree
   unsigned long long *check;  // bounds-checked builds: the violation word (device)
   size_t bytes;
   // multi-property graphs (hm_load_graph_props): the sorted distinct property
@@ -421,7 +423,7 @@ struct hm_graph {
   hm::DevGraph dev() const {
     return hm::DevGraph{n,        m,        src,     out_adj,  out_elab, in_adj,     in_elab,
                         vi,       off,      gout_adj, gin_adj, gdir_out, gdir_in,    vdir,
-                        afilt,    afilt_nword, hm::filter_min(), ahash, ahash_nbkt, gofs_out, gofs_in, ncls, ndir_out, ndir_in, check};
+                        afilt,    afilt_nword, hm::filter_min(), ahash, ahash_nbkt, gofs_out, gofs_in, ncls, maxdeg, ndir_out, ndir_in, check};
   }
 };
 

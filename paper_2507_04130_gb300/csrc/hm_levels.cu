@@ -14,10 +14,10 @@
 //            group dies here.  States are taken in groups of up to 32, and a
 //            prefix sum over the groups' chunks of 32 candidates numbers all
 //            chunks of the level.
-//   expand   each warp takes an equal run of consecutive chunks, finds the
-//            group its run starts in, and reads 32 candidates at a time: one
-//            of the other positive conditions' filter probes rejects most;
-//            survivors wait in the warp's buffer until 128 are there, then
+//   expand   each warp takes runs of consecutive chunks, finds the group a
+//            run starts in, and reads 32 candidates at a time: the filter
+//            probes of the other positive conditions reject most; survivors
+//            wait in the warp's buffer until 128 are there, then
 //            the exact checks run on full warps and the survivors of those
 //            become states of the next level, or matches.
 // Memory is bounded: an expansion takes no more chunks than the next level's
@@ -84,10 +84,15 @@ struct LvShared {
   unsigned long long wsum[kLvWarps];
   int4 rec[kLvWarps][32];                    // the group's states with candidates, in order
   int2 buf[kLvWarps][kLvBuf];                // {state, candidate}
+  // values all warps share, and each warp's matches, kept out of the registers of the expansion
+  unsigned long long made, deadline, begin, take;
+  unsigned long long count[kLvWarps];
+  uint32_t run_len, nrun;
+  unsigned int *claim;
   int ok;
 };
 
-__device__ __forceinline__ bool lv_barrier(const LvArgs &A, LvShared &sm, unsigned int target, uint64_t deadline) {
+__device__ __forceinline__ bool lv_barrier(const LvArgs &A, LvShared &sm, unsigned int target) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -96,7 +101,7 @@ __device__ __forceinline__ bool lv_barrier(const LvArgs &A, LvShared &sm, unsign
     for (;;) {
       if (*(volatile unsigned int *)&A.ctl->bar >= target) break;
       if (*(volatile int32_t *)&A.ctl->status != 0) break;
-      if (globaltimer_ns() > deadline + kLvBarrierNs) {
+      if (globaltimer_ns() > sm.deadline + kLvBarrierNs) {
         atomicCAS(&A.ctl->status, 0, kStatQueue);
         break;
       }
@@ -136,14 +141,39 @@ __device__ __forceinline__ unsigned long long lv_block_scan(unsigned long long v
 
 // States per group: all 32 lanes' worth when there are enough states for every
 // warp, else fewer, so that a small level still spreads over the warps.
-__device__ __forceinline__ int lv_group_size(unsigned long long cnt, unsigned long long warps) {
+// Positions inside a group are 32-bit: g lists of at most maxdeg entries.
+__device__ __forceinline__ int lv_group_size(unsigned long long cnt, unsigned long long warps, int32_t maxdeg) {
   int g = 32;
+  while (g > 1 && (unsigned long long)maxdeg * g > 0xffffffffull) g >>= 1;
   while (g > 1 && cnt < (unsigned long long)g * warps) g >>= 1;
   return g;
 }
 
 __device__ __forceinline__ const int32_t *lv_state(const LvArgs &A, int p, int64_t s) {
   return A.base[p] + s * A.stride[p];
+}
+
+// A state's first four images, in registers: most patterns' checks read no
+// more of it.  What is not a vertex (unmapped positions, the group in the
+// place of a deferred position 1, a pattern number) is -1.
+template <bool kShared>
+__device__ __forceinline__ int4 lv_images(const int32_t *mp, int p) {
+  int4 m;
+  if (p == 2) {
+    const int2 v = *reinterpret_cast<const int2 *>(mp);
+    m = make_int4(v.x, v.y, -1, -1);
+  } else {
+    m = *reinterpret_cast<const int4 *>(mp);
+    if (p == 3) m.w = -1;
+  }
+  if (kShared) m.y = -1;
+  return m;
+}
+
+__device__ __forceinline__ int32_t lv_image(const int4 &m, const int32_t *mp, int q) {
+  if (q >= 4) return mp[q];
+  const int32_t a = q & 1 ? m.y : m.x, b = q & 1 ? m.w : m.z;
+  return q & 2 ? b : a;
 }
 
 // The candidates of state `s` of level p: {first, number, driving condition | list << 8, pattern}.
@@ -258,8 +288,10 @@ __device__ __forceinline__ bool lv_group_has(const int2 *__restrict__ sv, int32_
 template <bool kShared, bool kSym>
 __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan &L, const int32_t *mp, int p,
                                                 int drive, int32_t c, Bytes &none) {
-  for (int i = 0; i < p; ++i)
-    if (!(kShared && i == 1) && mp[i] == c) return false;  // injective
+  const int4 m = lv_images<kShared>(mp, p);
+  if (m.x == c || m.y == c || m.z == c || m.w == c) return false;  // injective
+  for (int i = 4; i < p; ++i)
+    if (mp[i] == c) return false;
   if (L.root && !A.root_mask[c]) return false;
   if (kSym) {
     uint32_t g = L.sym_gt, l = L.sym_lt;
@@ -277,15 +309,20 @@ __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan
   for (int j = 0; j < L.npos; ++j) {
     if (j == drive) continue;
     const LvCons cs = L.cons[j];
-    const int32_t f = mp[cs.q];
-    if (!arc_maybe_l<false>(A.G, cs.kind == kOut ? f : c, cs.kind == kOut ? c : f, cs.lab, none)) return false;
+    const int32_t f = lv_image(m, mp, cs.q);
+    ArcKey k = pair_key(cs.kind == kOut ? f : c, cs.kind == kOut ? c : f);
+    k.a += cs.la;
+    k.b += cs.lb;
+    if (!filter_has<false>(A.G, k, none)) return false;
   }
   return true;
 }
 
 // The exact checks of a candidate that passed the cheap ones.
-__device__ __forceinline__ bool lv_exact_checks(const LvArgs &A, const LevelPlan &L, const int32_t *mp, int drive,
+template <bool kShared>
+__device__ __forceinline__ bool lv_exact_checks(const LvArgs &A, const LevelPlan &L, const int32_t *mp, int p, int drive,
                                                 int32_t c, Bytes &none) {
+  const int4 m = lv_images<kShared>(mp, p);
   if (L.need_deg) {
     const int4 vi = __ldg(&A.G.vi[HM_AT(A.G, c, A.G.n, kChkVertex)]);
     if (vi.y < L.dout || vi.z < L.din) return false;
@@ -293,7 +330,7 @@ __device__ __forceinline__ bool lv_exact_checks(const LvArgs &A, const LevelPlan
   for (int j = 0; j < L.ncons; ++j) {
     if (j == drive) continue;
     const LvCons cs = L.cons[j];
-    const int32_t f = mp[cs.q];
+    const int32_t f = lv_image(m, mp, cs.q);
     const bool fwd = cs.kind == kOut || cs.kind == kNotOut;
     const int32_t x = fwd ? f : c, y = fwd ? c : f;
     int32_t lab;
@@ -344,12 +381,11 @@ __device__ __forceinline__ void lv_write_images(const EmitPlan &E, const int8_t 
 }
 
 // Exact checks on the nbuf waiting survivors; those that pass become states of
-// the next level (whose counter stood at `made` when its buffer was empty) or
+// the next level (whose counter stood at sm.made when its buffer was empty) or
 // matches.
 template <bool kRows, bool kBatch, bool kShared, bool kSym>
 __device__ __forceinline__ void lv_drain(const LvArgs &A, LvShared &sm, int p, unsigned long long slice_first,
-                                         unsigned long long made, int2 *buf, int nbuf, int lane,
-                                         unsigned long long &count) {
+                                         int2 *buf, int nbuf, int lane) {
   Bytes none;
   const uint32_t lt = lanemask_lt();
   const bool deferred = kShared && p == A.kmax;
@@ -366,7 +402,7 @@ __device__ __forceinline__ void lv_drain(const LvArgs &A, LvShared &sm, int p, u
       } else {
         const int4 r = A.rng[p][(uint32_t)sc.x];
         const LevelPlan &L = kBatch ? A.levels[(int64_t)r.w * A.kmax + p] : A.level1[p];
-        ok = lv_exact_checks(A, L, mp, r.z & 0xff, sc.y, none);
+        ok = lv_exact_checks<kShared>(A, L, mp, p, r.z & 0xff, sc.y, none);
       }
     }
     const uint32_t bal = __ballot_sync(kFull, ok);
@@ -406,7 +442,7 @@ __device__ __forceinline__ void lv_drain(const LvArgs &A, LvShared &sm, int p, u
       if (bal) {
         unsigned long long at = 0;
         if (lane == 0) at = atomicAdd(&A.ctl->next_n[p + 1], (unsigned long long)__popc(bal));
-        at = __shfl_sync(kFull, at, 0) - made + __popc(bal & lt);
+        at = __shfl_sync(kFull, at, 0) - sm.made + __popc(bal & lt);
         if (inner) {
           int32_t *dst = const_cast<int32_t *>(lv_state(A, p + 1, (int64_t)at));
           for (int i = 0; i < p; ++i) dst[i] = mp[i];
@@ -432,10 +468,10 @@ __device__ __forceinline__ void lv_drain(const LvArgs &A, LvShared &sm, int p, u
       add += (unsigned long long)(gr.z - gr.y - used);
     }
     for (int o = 16; o; o >>= 1) add += __shfl_xor_sync(kFull, add, o);
-    count += add;
+    if (lane == 0) sm.count[threadIdx.x >> 5] += add;
   } else if (last && (!kShared || deferred)) {
     const int naut = kSym ? A.emit1.naut : 1;
-    count += (unsigned long long)nok * naut;
+    if (lane == 0) sm.count[threadIdx.x >> 5] += (unsigned long long)nok * naut;
     if (kRows) {
       unsigned long long at = 0;
       if (lane == 0) at = atomicAdd(&A.ctl->rows, (unsigned long long)nok * naut);
@@ -451,7 +487,7 @@ __device__ __forceinline__ void lv_drain(const LvArgs &A, LvShared &sm, int p, u
   } else {
     unsigned long long at = 0;
     if (lane == 0) at = atomicAdd(&A.ctl->next_n[p + 1], (unsigned long long)nok);
-    at = __shfl_sync(kFull, at, 0) - made;
+    at = __shfl_sync(kFull, at, 0) - sm.made;
     for (int e = lane; e < nok; e += 32) {
       const int2 sc = buf[e];
       const int64_t s = (int64_t)(slice_first + (uint32_t)sc.x);
@@ -473,132 +509,164 @@ __device__ __forceinline__ void lv_drain(const LvArgs &A, LvShared &sm, int p, u
 }
 
 // The group that chunk x of the level lies in: the last one whose first chunk
-// is at or before x.  Returns its number in the slice; *start is that first chunk.
-__device__ __forceinline__ int64_t lv_locate(const LvArgs &A, const LvShared &sm, int p, unsigned long long x,
-                                             int64_t ngroups, int64_t per_groups, int lane,
-                                             unsigned long long *start) {
+// is at or before x.  Returns its number in the slice; *start is that first
+// chunk.  `gi` is the group of the chunk before x, in the block's groups that
+// begin at chunk `b0` and end at group `b1` (b1 = 0: none): mostly x lies
+// in one of the 32 groups after it, which takes one load; otherwise the block
+// is searched for in shared memory and the group in two loads.
+__device__ __forceinline__ uint32_t lv_locate(const LvArgs &A, const LvShared &sm, int p, unsigned long long x,
+                                              uint32_t ngroups, uint32_t per_groups, int lane, uint32_t gi,
+                                              unsigned long long &b0, uint32_t &b1, unsigned long long *start) {
+  const unsigned long long *up = A.upre[p];
+  if (b1) {
+    const uint32_t i = gi + 1 + lane;
+    const unsigned long long u = i < b1 ? up[i] : ~0ull;
+    const uint32_t le = __ballot_sync(kFull, u <= x - b0);
+    // the last of them starts at or before x: it is the group unless all 32 do or the block ends there
+    if (le && le != kFull && gi + 1 + __popc(le) < b1) {
+      const int at = 31 - __clz(le);
+      *start = b0 + __shfl_sync(kFull, u, at);
+      return gi + 1 + at;
+    }
+  }
   int lo = 0, hi = (int)gridDim.x - 1;  // the last block whose first chunk is <= x
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (sm.first[mid] <= x) lo = mid; else hi = mid - 1;
   }
-  const unsigned long long rel = x - sm.first[lo];
-  const unsigned long long *up = A.upre[p];
-  int64_t a = (int64_t)lo * per_groups, n = min(per_groups, ngroups - a);  // groups [a, a + n)
+  b0 = sm.first[lo];
+  uint32_t a = (uint32_t)lo * per_groups, n = min(per_groups, ngroups - a);  // groups [a, a + n)
+  b1 = a + n;
   while (n > 1) {
-    const int64_t step = (n + 31) >> 5;
-    const int64_t i = (int64_t)lane * step;
-    const bool le = i < n && up[a + i] <= rel;
-    const int64_t at = (31 - __clz(__ballot_sync(kFull, le))) * step;  // lane 0 always holds
+    const uint32_t step = (n + 31) >> 5;
+    const uint32_t i = (uint32_t)lane * step;
+    const bool le = i < n && up[a + i] <= x - b0;
+    const uint32_t at = (31 - __clz(__ballot_sync(kFull, le))) * step;  // lane 0 always holds
     a += at;
     n = min(step, n - at);
   }
-  *start = sm.first[lo] + up[a];
+  *start = b0 + up[a];
   return a;
 }
 
+// The expansion of the level's chunks [sm.begin, sm.begin + sm.take) by this
+// warp: run `run` of sm.nrun, then runs claimed from the level's counter.
+// Returns the number of chunks it took.
 template <bool kRows, bool kBatch, bool kShared, bool kSym>
-__device__ __forceinline__ void lv_expand(const LvArgs &A, LvShared &sm, int p, unsigned long long first,
-                                          unsigned long long cnt, int g, unsigned long long x0,
-                                          unsigned long long x1, unsigned long long made, uint64_t deadline,
-                                          unsigned long long &count) {
+__device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int p, unsigned long long first,
+                                              unsigned long long cnt, int g, uint32_t run) {
   Bytes none;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = lanemask_lt();
   int4 *rec = sm.rec[warp];
   int2 *buf = sm.buf[warp];
   const int64_t chunks = (int64_t)((cnt + 31) >> 5), per = (chunks + gridDim.x - 1) / gridDim.x;
-  const int64_t per_groups = per * (32 / g), ngroups = chunks * (32 / g);
+  const uint32_t per_groups = (uint32_t)(per * (32 / g)), ngroups = (uint32_t)(chunks * (32 / g));
+  uint32_t gi = 0, b1 = 0;
+  unsigned long long b0 = 0;
   const bool deferred = kShared && p == A.kmax;
+  const int32_t *states = A.base[p] + first * A.stride[p];
   int nbuf = 0;
-  unsigned long long x = x0;
   uint32_t look = 0;
-  while (x < x1) {
-    unsigned long long start;
-    const int64_t gi = lv_locate(A, sm, p, x, ngroups, per_groups, lane, &start);
-    // the group's states that have candidates, in order, to shared memory
-    const unsigned long long i = (unsigned long long)gi * g + lane;
-    int4 r = make_int4(0, 0, 0, 0);
-    if (lane < g && i < cnt) r = A.rng[p][i];
-    const uint32_t have = __ballot_sync(kFull, r.y > 0);
-    unsigned long long incl = (unsigned long long)(uint32_t)r.y;
+  while (run < sm.nrun) {
+    unsigned long long x = sm.begin + (unsigned long long)run * sm.run_len;
+    uint32_t left = (uint32_t)min((unsigned long long)sm.run_len, sm.take - (unsigned long long)run * sm.run_len);
+    // the next run, claimed early so that its number is there when this one is done
+    if (lane == 0) run = atomicAdd(sm.claim, 1u);
+    b1 = 0;
+    while (left) {
+      unsigned long long start;
+      gi = lv_locate(A, sm, p, x, ngroups, per_groups, lane, gi, b0, b1, &start);
+      // the group's states that have candidates, in order, to shared memory
+      const unsigned long long i = (unsigned long long)gi * g + lane;
+      int4 r = make_int4(0, 0, 0, 0);
+      if (lane < g && i < cnt) r = A.rng[p][i];
+      const uint32_t have = __ballot_sync(kFull, r.y > 0);
+      uint32_t incl = (uint32_t)r.y;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const unsigned long long total = __shfl_sync(kFull, incl, 31);
-    const unsigned long long excl = incl - (uint32_t)r.y;
-    if (r.y > 0) rec[__popc(have & lt)] = make_int4((int32_t)((uint32_t)r.x - (uint32_t)excl), r.z, (int32_t)i, r.w);
-    __syncwarp();
-    const unsigned long long end = start + ((total + 31) >> 5);
-    if (end <= x) {  // cannot happen (the ranges phase counted the same chunks); never spin
-      if (lane == 0) atomicCAS(&A.ctl->status, 0, kStatQueue);
-      return;
-    }
-    for (; x < x1 && x < end; ++x) {
-      if ((++look & 31u) == 0) {
-        int stop = 0;
-        if (lane == 0) {
-          if (*(volatile int32_t *)&A.ctl->status != 0) stop = 1;
-          else if (globaltimer_ns() > deadline) {
-            atomicCAS(&A.ctl->status, 0, kStatBudget);
-            stop = 1;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const uint32_t total = __shfl_sync(kFull, incl, 31);
+      const uint32_t excl = r.y > 0 ? incl - (uint32_t)r.y : 0xffffffffu;
+      if (r.y > 0) rec[__popc(have & lt)] = make_int4((int32_t)((uint32_t)r.x - excl), r.z, (int32_t)i, r.w);
+      __syncwarp();
+      uint32_t pos0 = (uint32_t)(x - start) << 5;
+      if (x - start >= ((unsigned long long)total + 31) >> 5) {
+        // cannot happen (the ranges phase counted the same chunks); never spin
+        if (lane == 0) atomicCAS(&A.ctl->status, 0, kStatQueue);
+        return look;
+      }
+      const uint32_t n = min(left, ((total - 1) >> 5) + 1 - (pos0 >> 5));  // chunks of this group
+      left -= n;
+      x += n;
+      for (uint32_t c0 = 0; c0 < n; ++c0, pos0 += 32) {
+        if ((++look & 31u) == 0) {
+          int stop = 0;
+          if (lane == 0) {
+            if (*(volatile int32_t *)&A.ctl->status != 0) stop = 1;
+            else if (globaltimer_ns() > sm.deadline) {
+              atomicCAS(&A.ctl->status, 0, kStatBudget);
+              stop = 1;
+            }
+          }
+          if (__shfl_sync(kFull, stop, 0)) return look;
+        }
+        // the owner of position pos0 + lane: states that start at or before pos0, then the starts inside the chunk
+        const uint32_t rel = excl - pos0;
+        const uint32_t starts = __reduce_or_sync(kFull, r.y > 0 && excl > pos0 && rel < 32 ? 1u << rel : 0u);
+        const int before = __popc(__ballot_sync(kFull, excl <= pos0 && r.y > 0)) - 1;
+        const int ow = before + __popc(starts & (lt | (1u << lane)));
+        bool ok = false;
+        int32_t c = 0, s = 0;
+        if (total - pos0 > (uint32_t)lane) {
+          const int4 o = rec[ow];
+          s = o.z;
+          const uint32_t at = (uint32_t)o.x + pos0 + lane;
+          const int list = o.y >> 8;
+          if (kShared && list == 2)
+            c = __ldg(&A.sorted_seeds[at].y);
+          else
+            c = __ldg((list ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
+          if (deferred) {
+            ok = true;
+          } else {
+            const LevelPlan &L = kBatch ? A.levels[(int64_t)o.w * A.kmax + p] : A.level1[p];
+            ok = lv_first_checks<kShared, kSym>(A, L, states + (uint64_t)(uint32_t)s * (uint32_t)A.stride[p], p,
+                                                o.y & 0xff, c, none);
           }
         }
-        if (__shfl_sync(kFull, stop, 0)) return;
-      }
-      const unsigned long long pos0 = (x - start) << 5;
-      // the owner of position pos0 + lane: states that start at or before pos0, then the starts inside the chunk
-      const long long rel = (long long)(excl - pos0);
-      const uint32_t bit = r.y > 0 && rel > 0 && rel < 32 ? 1u << (int)rel : 0u;
-      const uint32_t starts = __reduce_or_sync(kFull, bit);
-      const int before = __popc(__ballot_sync(kFull, r.y > 0 && rel <= 0)) - 1;
-      const int ow = before + __popc(starts & (lt | (1u << lane)));
-      bool ok = false;
-      int32_t c = 0, s = 0;
-      if (pos0 + lane < total) {
-        const int4 o = rec[ow];
-        s = o.z;
-        const uint32_t at = (uint32_t)o.x + (uint32_t)pos0 + lane;
-        const int list = o.y >> 8;
-        if (kShared && list == 2)
-          c = __ldg(&A.sorted_seeds[at].y);
-        else
-          c = __ldg((list ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
-        if (deferred) {
-          ok = true;
-        } else {
-          const LevelPlan &L = kBatch ? A.levels[(int64_t)o.w * A.kmax + p] : A.level1[p];
-          ok = lv_first_checks<kShared, kSym>(A, L, lv_state(A, p, (int64_t)(first + (uint32_t)s)), p, o.y & 0xff, c,
-                                              none);
+        const uint32_t bal = __ballot_sync(kFull, ok);
+        if (ok) buf[nbuf + __popc(bal & lt)] = make_int2(s, c);
+        nbuf += __popc(bal);
+        __syncwarp();
+        if (nbuf >= kLvDrain) {
+          lv_drain<kRows, kBatch, kShared, kSym>(A, sm, p, first, buf, nbuf, lane);
+          nbuf = 0;
         }
       }
-      const uint32_t bal = __ballot_sync(kFull, ok);
-      if (ok) buf[nbuf + __popc(bal & lt)] = make_int2(s, c);
-      nbuf += __popc(bal);
-      __syncwarp();
-      if (nbuf >= kLvDrain) {
-        lv_drain<kRows, kBatch, kShared, kSym>(A, sm, p, first, made, buf, nbuf, lane, count);
-        nbuf = 0;
-      }
+      __syncwarp();  // every lane is done with rec
     }
-    __syncwarp();  // every lane is done with rec
+    run = gridDim.x * kLvWarps + __shfl_sync(kFull, run, 0);
   }
-  if (nbuf) lv_drain<kRows, kBatch, kShared, kSym>(A, sm, p, first, made, buf, nbuf, lane, count);
+  if (nbuf) lv_drain<kRows, kBatch, kShared, kSym>(A, sm, p, first, buf, nbuf, lane);
+  return look;
 }
 
 template <bool kRows, bool kBatch, bool kShared, bool kSym>
 __global__ void __launch_bounds__(kLvThreads, kLvMinBlocks) k_levels(const __grid_constant__ LvArgs A) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   LvShared &sm = *reinterpret_cast<LvShared *>(s_raw);
-  const uint64_t deadline = globaltimer_ns() + A.budget_ns;
   const unsigned long long warps = (unsigned long long)gridDim.x * kLvWarps;
-  const unsigned long long me = (unsigned long long)blockIdx.x * kLvWarps + (threadIdx.x >> 5);
+  const uint32_t me = blockIdx.x * kLvWarps + (threadIdx.x >> 5);
   const int last = kShared && (kRows || A.ndefer) ? A.kmax : A.kmax - 1;  // the deepest level
   const unsigned long long nseeds = *A.nseeds;
-  unsigned long long count = 0, my_chunks = 0, cursor = 0;
-  unsigned int target = 0;
+  if ((threadIdx.x & 31) == 0) sm.count[threadIdx.x >> 5] = 0;
+  if (threadIdx.x == 0) sm.deadline = globaltimer_ns() + A.budget_ns;
+  __syncthreads();
+  unsigned long long my_chunks = 0, cursor = 0;
+  unsigned int target = 0, turn = 0;
   // the levels being worked on: states [first, first + n) and chunks [done, total)
   unsigned long long first = 0;
   unsigned long long n[kMaxK + 2], done[kMaxK + 2], total[kMaxK + 2];
@@ -617,24 +685,34 @@ __global__ void __launch_bounds__(kLvThreads, kLvMinBlocks) k_levels(const __gri
       // expand as many chunks as the next level can hold survivors of
       const unsigned long long left = total[p] - done[p];
       const unsigned long long take = p < last ? min(left, (unsigned long long)(A.fcap >> 5)) : left;
-      const unsigned long long x0 = done[p] + (unsigned long long)((unsigned __int128)take * me / warps);
-      const unsigned long long x1 = done[p] + (unsigned long long)((unsigned __int128)take * (me + 1) / warps);
-      if (x0 < x1)
-        lv_expand<kRows, kBatch, kShared, kSym>(A, sm, p, p == 2 ? first : 0, n[p], lv_group_size(n[p], warps), x0, x1,
-                                                made[p + 1], deadline, count);
-      my_chunks += x1 - x0;
+      // runs of chunks: the first is the warp's own, the rest are claimed, so that
+      // warps with cheap chunks (lists in cache) take more of them
+      if (threadIdx.x == 0) {
+        const unsigned long long run = max(take / (warps * 8), 1ull);
+        sm.begin = done[p];
+        sm.take = take;
+        sm.run_len = (uint32_t)min(run, 1ull << 31);
+        sm.nrun = (uint32_t)((take + sm.run_len - 1) / sm.run_len);
+        sm.made = made[p + 1];
+        sm.claim = &A.ctl->claim[turn % 3];
+        if (blockIdx.x == 0) A.ctl->claim[(turn + 1) % 3] = 0;  // read two expansions ago
+      }
+      ++turn;
+      __syncthreads();
+      my_chunks += lv_expand<kRows, kBatch, kShared, kSym>(A, sm, p, p == 2 ? first : 0, n[p],
+                                                           lv_group_size(n[p], warps, A.G.maxdeg), me);
       done[p] += take;
       if (p == last && done[p] == total[p]) {  // nothing below: up again, past levels that are done too
         while (p > 1 && done[p] == total[p]) --p;
         if (p == 1 && cursor >= nseeds) break;
         // the next step overwrites buffers that other warps may still read
         target += gridDim.x;
-        ok = lv_barrier(A, sm, target, deadline);
+        ok = lv_barrier(A, sm, target);
         if (p > 1) goto reload;
         continue;
       }
       target += gridDim.x;
-      if (!(ok = lv_barrier(A, sm, target, deadline))) break;
+      if (!(ok = lv_barrier(A, sm, target))) break;
       if (p == last) continue;
       const unsigned long long now = *(volatile unsigned long long *)&A.ctl->next_n[p + 1];
       const unsigned long long fresh = now - made[p + 1];
@@ -642,7 +720,7 @@ __global__ void __launch_bounds__(kLvThreads, kLvMinBlocks) k_levels(const __gri
       if (fresh == 0) {
         // another block may not have read the counter yet that the next expansion adds to
         target += gridDim.x;
-        if (!(ok = lv_barrier(A, sm, target, deadline))) break;
+        if (!(ok = lv_barrier(A, sm, target))) break;
         if (done[p] < total[p]) continue;
         while (p > 1 && done[p] == total[p]) --p;
         if (p > 1) goto reload;
@@ -656,9 +734,9 @@ __global__ void __launch_bounds__(kLvThreads, kLvMinBlocks) k_levels(const __gri
       continue;
     }
     // the ranges of the new states
-    lv_ranges<kBatch, kShared, kRows, kSym>(A, sm, p, p == 2 ? first : 0, n[p], lv_group_size(n[p], warps));
+    lv_ranges<kBatch, kShared, kRows, kSym>(A, sm, p, p == 2 ? first : 0, n[p], lv_group_size(n[p], warps, A.G.maxdeg));
     target += gridDim.x;
-    if (!(ok = lv_barrier(A, sm, target, deadline))) break;
+    if (!(ok = lv_barrier(A, sm, target))) break;
     done[p] = 0;
   reload: {
       // the first chunk of each block's groups at this level
@@ -675,6 +753,7 @@ __global__ void __launch_bounds__(kLvThreads, kLvMinBlocks) k_levels(const __gri
     }
   }
   if ((threadIdx.x & 31) == 0) {
+    const unsigned long long count = sm.count[threadIdx.x >> 5];
     if (count) atomicAdd(&A.ctl->count, count);
     if (my_chunks) atomicAdd(&A.ctl->chunks, my_chunks);
   }
@@ -729,7 +808,8 @@ void lv_level(const hm_graph *g, const Plan &P, int p, LevelPlan &L) {
   L.sym_lt = P.sym_lt[p];
   for (int j = 0; j < P.ncons[p]; ++j) {
     const Cons cs = P.cons[p][j];
-    L.cons[j] = LvCons{cs.q, cs.kind, j < P.npos[p] ? lv_class(g, cs.lab, P.vlab[p]) : (int16_t)0, cs.lab};
+    const ArcKey l = j < P.npos[p] ? labelled_key(ArcKey{0, 0}, cs.lab) : ArcKey{0, 0};
+    L.cons[j] = LvCons{cs.q, cs.kind, j < P.npos[p] ? lv_class(g, cs.lab, P.vlab[p]) : (int16_t)0, cs.lab, l.a, l.b};
   }
   // arcs to later positions: one or two are found missing by the next ranges phase anyway
   L.need_deg = !L.last && P.dout[p] + P.din[p] - P.npos[p] >= 2;

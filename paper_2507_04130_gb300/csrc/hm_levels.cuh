@@ -12,6 +12,7 @@ struct LvCons {
   int8_t q, kind;
   int16_t cls;
   int32_t lab;
+  uint64_t la, lb;  // the label's part of the two hashes of the arc filter
 };
 
 // What a candidate for one position must satisfy.
@@ -37,6 +38,7 @@ struct EmitPlan {
 struct LvCtl {
   alignas(128) unsigned int bar;  // arrivals at the grid barrier
   alignas(128) int32_t status;
+  alignas(128) unsigned int claim[3];                 // runs of chunks taken, one word per expansion in turn
   alignas(128) unsigned long long next_n[kMaxK + 2];  // states appended for each level
   alignas(128) unsigned long long count;              // matches
   unsigned long long rows;                            // row cursor

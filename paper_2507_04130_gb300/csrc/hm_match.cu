@@ -97,13 +97,23 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   if (tuning().symmetry < 0) strip_symmetry(plan);
   const DevGraph G = g->dev();
   const int64_t m = g->m;
+  const hm_tuning tu = tuning();
+  // default knobs: level by level; the instrumented kernels and a chunk budget belong to the depth-first search
+  const bool by_level = p->k > 2 && g->ncls > 0 && want != Want::kStates && default_search(tu) && !counters &&
+                        budget_chunks() == 0;
+  // The overlap test only prunes: a common neighbour that a match needs is a
+  // candidate of a later position, checked there with its labels.  Level by
+  // level that costs a few lookups per state; the test merges whole lists, one
+  // warp per state (five connectome counts: 5.5 of 14.5 ms, and 1.26 of 5.0 ms
+  // for 256 patterns), so only the depth-first search and the injected states take it.
+  const bool overlap = plan.ov_need > 0 && !by_level;
   Scratch sc(s);
   Ctl *ctl;
   int2 *seeds_a, *seeds_b = nullptr;
   HM_CUDA_TRY(sc.get((void **)&ctl, sizeof(Ctl)));
   HM_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Ctl), s));
   HM_CUDA_TRY(sc.get((void **)&seeds_a, sizeof(int2) * (size_t)std::max<int64_t>(m, 1)));
-  if (plan.ov_need > 0)
+  if (overlap)
     HM_CUDA_TRY(sc.get((void **)&seeds_b, sizeof(int2) * (size_t)std::max<int64_t>(m, 1)));
   const int sms = num_sms();
 
@@ -129,8 +139,8 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   }
   const int2 *seeds = seeds_a;
   const unsigned long long *nseeds = &ctl->nseeds_raw;
-  Timer t_ov(s, timing && plan.ov_need > 0);
-  if (plan.ov_need > 0) {
+  Timer t_ov(s, timing && overlap);
+  if (overlap) {
     NvtxRange r_ov("hm.overlap_test");
     if (counters)
       k_seed_overlap<true><<<sms * 8, kSeedThreads, 0, s>>>(G, plan.ov_need, seeds_a, &ctl->nseeds_raw,
@@ -151,7 +161,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
     Ctl h;
     HM_CUDA_TRY(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     HM_CUDA_TRY(cudaStreamSynchronize(s));
-    unsigned long long n = plan.ov_need > 0 ? h.nseeds : h.nseeds_raw;
+    unsigned long long n = overlap ? h.nseeds : h.nseeds_raw;
     *count = n;
     if (n > cap) return HM_ERR_CAPACITY;
     if (n)
@@ -161,10 +171,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
 
   // Shared position-0 states: group the seeds by their position-0 image
   // (induced calls: at most kInducedGroupCap seeds per group).
-  const hm_tuning tu = tuning();
   const bool share = p->k > 2 && plan.defer1 && tu.share_seeds > 0;
-  // default knobs: level by level; the instrumented kernels and a chunk budget belong to the depth-first search
-  const bool by_level = p->k > 2 && default_search(tu) && !counters && budget_chunks() == 0;
   const int4 *groups = nullptr;
   Timer t_grp(s, timing && share);
   if (share) {
@@ -288,7 +295,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   st.ms_overlap = t_ov.ms() + t_grp.ms();
   st.ms_extend = t_ext.ms();
   st.seeds_scanned = (uint64_t)(e_end - e_begin);
-  st.states_injected = plan.ov_need > 0 ? h.nseeds : h.nseeds_raw;
+  st.states_injected = overlap ? h.nseeds : h.nseeds_raw;
   if (ran_levels) {
     h.status = h.lv.status;
     h.count = h.lv.count;

@@ -69,7 +69,7 @@ def test_label_sets(nv, ne, shift):
 def test_every_depth_agrees_with_the_depth_first_search():
     import paper_2507_04130_gb300 as hm
 
-    g = synth.er_graph(3000, 24000, 2, 1, seed=31)
+    g = synth.er_graph(1500, 6000, 2, 1, seed=31)
     G = hm.Graph.from_synth(g)
     rng = np.random.default_rng(8)
     pats = []
