@@ -201,262 +201,11 @@ __global__ void k_unpack_rows(const int32_t *__restrict__ packed, const unsigned
 
 constexpr uint64_t kRankMaxCompares = 1ull << 29;  // run_batch: below, rows are sorted by counting
 
-// fit (may be NULL): instead of failing with HM_ERR_CAPACITY when some
-// pattern's rows exceed its region, return every count, sort the rows of the
-// patterns that fit and flag them (fit[i] = 1); the others' rows are not valid.
-hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int32_t *modes,
-                    int32_t npat, int32_t *rows, const uint64_t *row_offsets, uint64_t *counts,
-                    cudaStream_t s, uint8_t *fit = nullptr, uint64_t workspace = kLevelWorkspace) {
-  if (!g || npat < 0 || (npat > 0 && (!pats || !modes || !counts))) return HM_ERR_ARG;
-  if (npat == 0) return HM_OK;
-  const bool want_rows = rows != nullptr || row_offsets != nullptr;
-  if (want_rows && (!rows || !row_offsets)) return HM_ERR_ARG;
-  ensure_pool();
-  hm_stats &st = tls_stats();
-  std::memset(&st, 0, sizeof(st));
-  const bool timing = timing_enabled();
-
-  // ---- host tables: plans, signatures, row regions
-  std::vector<Plan> plans(npat);
-  std::vector<int32_t> ks(npat);
-  int32_t grp_slots = 0, kmax = 0;
-  for (int32_t i = 0; i < npat; ++i) {
-    if (!pats[i] || (modes[i] != HM_MONO && modes[i] != HM_INDUCED)) return HM_ERR_ARG;
-    plans[i] = pats[i]->plan[modes[i]];
-    if (tuning().symmetry < 0) strip_symmetry(plans[i]);
-    ks[i] = pats[i]->k;
-    grp_slots = std::max(grp_slots, plans[i].ngrp);
-    kmax = std::max(kmax, ks[i]);
-  }
-  std::vector<unsigned long long> off(npat + 1, 0), cap(npat, 0);
-  if (want_rows) {
-    for (int32_t i = 0; i < npat; ++i) {
-      if (row_offsets[i + 1] < row_offsets[i]) return HM_ERR_ARG;
-      off[i] = row_offsets[i];
-      cap[i] = (row_offsets[i + 1] - row_offsets[i]) / (uint64_t)ks[i];
-    }
-  }
-  // signature (arc label, label of the arc's source, label of its target) -> patterns
-  struct Sig {
-    int32_t lab, vs, vd, pid;
-  };
-  std::vector<Sig> sigs(npat);
-  for (int32_t i = 0; i < npat; ++i) {
-    const Plan &P = plans[i];
-    // normal seeding: arc (f(0), f(1)); reversed: arc (f(1), f(0))
-    sigs[i] = P.seed_rev ? Sig{P.seed_lab, P.vlab[1], P.vlab[0], i} : Sig{P.seed_lab, P.vlab[0], P.vlab[1], i};
-  }
-  std::sort(sigs.begin(), sigs.end(), [](const Sig &x, const Sig &y) {
-    if (x.lab != y.lab) return x.lab < y.lab;
-    if (x.vs != y.vs) return x.vs < y.vs;
-    if (x.vd != y.vd) return x.vd < y.vd;
-    return x.pid < y.pid;
-  });
-  uint32_t tsize = 16;
-  while (tsize < 2u * (uint32_t)npat) tsize <<= 1;
-  std::vector<SigKey> keys(tsize, SigKey{0, 0, 0, 0});
-  std::vector<int2> vals(tsize, make_int2(0, 0));
-  std::vector<int32_t> pid_list(npat);
-  for (int32_t i = 0; i < npat;) {
-    int32_t j = i;
-    while (j < npat && sigs[j].lab == sigs[i].lab && sigs[j].vs == sigs[i].vs && sigs[j].vd == sigs[i].vd) {
-      pid_list[j] = sigs[j].pid;
-      ++j;
-    }
-    uint32_t h = sig_hash(sigs[i].lab, sigs[i].vs, sigs[i].vd) & (tsize - 1);
-    while (keys[h].used) h = (h + 1) & (tsize - 1);
-    keys[h] = SigKey{sigs[i].lab, sigs[i].vs, sigs[i].vd, 1};
-    vals[h] = make_int2(i, j - i);
-    i = j;
-  }
-
-  // ---- device copies
-  Scratch sc(s);
-  Plan *d_plans;
-  SigKey *d_keys;
-  int2 *d_vals;
-  int32_t *d_pids, *d_ks;
-  unsigned long long *d_ull;  // counts, off, cap, cursor, start, nseeds x2
-  Ctl *ctl;
-  HM_CUDA_TRY(sc.get((void **)&d_plans, sizeof(Plan) * npat));
-  HM_CUDA_TRY(sc.get((void **)&d_keys, sizeof(SigKey) * tsize));
-  HM_CUDA_TRY(sc.get((void **)&d_vals, sizeof(int2) * tsize));
-  HM_CUDA_TRY(sc.get((void **)&d_pids, sizeof(int32_t) * npat));
-  HM_CUDA_TRY(sc.get((void **)&d_ks, sizeof(int32_t) * npat));
-  HM_CUDA_TRY(sc.get((void **)&d_ull, sizeof(unsigned long long) * (size_t)(5 * npat + 2)));
-  HM_CUDA_TRY(sc.get((void **)&ctl, sizeof(Ctl)));
-  unsigned long long *d_counts = d_ull, *d_off = d_ull + npat, *d_cap = d_ull + 2 * npat,
-                     *d_cursor = d_ull + 3 * npat, *d_start = d_ull + 4 * npat;
-  HM_CUDA_TRY(cudaMemcpyAsync(d_plans, plans.data(), sizeof(Plan) * npat, cudaMemcpyHostToDevice, s));
-  HM_CUDA_TRY(cudaMemcpyAsync(d_keys, keys.data(), sizeof(SigKey) * tsize, cudaMemcpyHostToDevice, s));
-  HM_CUDA_TRY(cudaMemcpyAsync(d_vals, vals.data(), sizeof(int2) * tsize, cudaMemcpyHostToDevice, s));
-  HM_CUDA_TRY(cudaMemcpyAsync(d_pids, pid_list.data(), sizeof(int32_t) * npat, cudaMemcpyHostToDevice, s));
-  HM_CUDA_TRY(cudaMemcpyAsync(d_ks, ks.data(), sizeof(int32_t) * npat, cudaMemcpyHostToDevice, s));
-  HM_CUDA_TRY(cudaMemsetAsync(d_ull, 0, sizeof(unsigned long long) * (size_t)(5 * npat + 2), s));
-  HM_CUDA_TRY(cudaMemcpyAsync(d_off, off.data(), sizeof(unsigned long long) * npat, cudaMemcpyHostToDevice, s));
-  HM_CUDA_TRY(cudaMemcpyAsync(d_cap, cap.data(), sizeof(unsigned long long) * npat, cudaMemcpyHostToDevice, s));
-  HM_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Ctl), s));
-  const SigTable T{d_keys, d_vals, d_pids, tsize - 1};
-  const DevGraph G = g->dev();
-  const int64_t m = g->m;
-  const int sms = num_sms();
-  uint32_t launches = 0;
-
-  // ---- edge scan: count, size, write
-  NvtxRange r_edge("hm.batch_edge_scan");
-  Timer t_edge(s, timing);
-  const int grid_e = (int)std::max<int64_t>(1, std::min<int64_t>((m + kSeedThreads - 1) / kSeedThreads,
-                                                                   (int64_t)sms * 8));
-  unsigned long long nraw = 0;
-  if (m) {
-    k_edge_seed_batch<false><<<grid_e, kSeedThreads, 0, s>>>(G, d_plans, T, nullptr, nullptr, 0,
-                                                             &ctl->nseeds_raw);
-    HM_CUDA_TRY(cudaMemcpyAsync(&nraw, &ctl->nseeds_raw, sizeof(nraw), cudaMemcpyDeviceToHost, s));
-    HM_CUDA_TRY(cudaStreamSynchronize(s));
-    launches += 1;
-  }
-  int2 *seeds_a, *seeds_b;
-  int32_t *pid_a, *pid_b;
-  HM_CUDA_TRY(sc.get((void **)&seeds_a, sizeof(int2) * (size_t)std::max<unsigned long long>(nraw, 1)));
-  HM_CUDA_TRY(sc.get((void **)&pid_a, sizeof(int32_t) * (size_t)std::max<unsigned long long>(nraw, 1)));
-  HM_CUDA_TRY(sc.get((void **)&seeds_b, sizeof(int2) * (size_t)std::max<unsigned long long>(nraw, 1)));
-  HM_CUDA_TRY(sc.get((void **)&pid_b, sizeof(int32_t) * (size_t)std::max<unsigned long long>(nraw, 1)));
-  if (nraw) {
-    HM_CUDA_TRY(cudaMemsetAsync(&ctl->nseeds_raw, 0, sizeof(unsigned long long), s));
-    k_edge_seed_batch<true><<<grid_e, kSeedThreads, 0, s>>>(G, d_plans, T, seeds_a, pid_a, nraw,
-                                                            &ctl->nseeds_raw);
-    launches += 1;
-  }
-  t_edge.stop();
-  HM_CUDA_TRY(cudaGetLastError());
-  // ---- overlap test (patterns without one pass their seeds through)
-  const hm_tuning tu = tuning();
-  const bool counters = counters_enabled();
-  const bool by_level = g->ncls > 0 && default_search(tu) && !counters && budget_chunks() == 0;
-  bool any_ov = false;
-  for (const Plan &P : plans) any_ov |= P.ov_need > 0;
-  any_ov = any_ov && !by_level;  // level by level the test costs more than the states it removes (see run_match)
-  const int2 *seeds = seeds_a;
-  const int32_t *seed_pid = pid_a;
-  const unsigned long long *nseeds = &ctl->nseeds_raw;
-  Timer t_ov(s, timing && any_ov);
-  if (any_ov && nraw) {
-    int2 *seeds_c;
-    int32_t *pid_c;
-    unsigned long long *ntest;
-    HM_CUDA_TRY(sc.get((void **)&seeds_c, sizeof(int2) * (size_t)nraw));
-    HM_CUDA_TRY(sc.get((void **)&pid_c, sizeof(int32_t) * (size_t)nraw));
-    HM_CUDA_TRY(sc.get((void **)&ntest, sizeof(unsigned long long)));
-    HM_CUDA_TRY(cudaMemsetAsync(ntest, 0, sizeof(unsigned long long), s));
-    const int grid_s = (int)std::max<unsigned long long>(
-        1, std::min<unsigned long long>((nraw + kSeedThreads - 1) / kSeedThreads, (unsigned long long)sms * 8));
-    k_overlap_split<<<grid_s, kSeedThreads, 0, s>>>(d_plans, seeds_a, pid_a, &ctl->nseeds_raw, seeds_b, pid_b,
-                                                     &ctl->nseeds, seeds_c, pid_c, ntest);
-    k_seed_overlap<false, true><<<sms * 8, kSeedThreads, 0, s>>>(G, 0, seeds_c, ntest, seeds_b, nraw,
-                                                                  &ctl->nseeds, &ctl->bytes_overlap, d_plans,
-                                                                  pid_c, pid_b);
-    launches += 2;
-    seeds = seeds_b;
-    seed_pid = pid_b;
-    nseeds = &ctl->nseeds;
-  }
-  t_ov.stop();
-
-  // ---- one persistent extension launch for every pattern
-  NvtxRange r_ext("hm.batch_extend");
-  Timer t_ext(s, timing);
-  bool ran_levels = false;
-  if (by_level && nraw) {
-    LvLaunch L{};
-    L.g = g;
-    L.ctl = &ctl->lv;
-    L.seeds = seeds;
-    L.nseeds = nseeds;
-    L.max_seeds = (int64_t)nraw;
-    L.rows = rows;
-    L.npat = npat;
-    L.plans = plans.data();
-    L.seed_pid = seed_pid;
-    L.counts = d_counts;
-    L.row_off = d_off;
-    L.row_cap = d_cap;
-    L.row_cursor = d_cursor;
-    L.want_rows = want_rows;
-    L.workspace = workspace;
-    int grid = 0, threads = 0;
-    const hm_status r = levels_run(L, s, &ran_levels, &grid, &threads);
-    if (r != HM_OK) return r;
-    st.extend_grid = grid;
-    st.extend_block = threads;
-    if (ran_levels) ++launches;
-  }
-  if (!ran_levels) {
-  Task *qbuf;
-  unsigned long long *qseq;
-  HM_CUDA_TRY(sc.get((void **)&qbuf, sizeof(Task) * kQueueCap));
-  HM_CUDA_TRY(sc.get((void **)&qseq, sizeof(unsigned long long) * kQueueCap));
-  k_qinit<<<64, 256, 0, s>>>(qseq);
-  launches += 1;
-  ExtArgs A{};
-  A.split_min = tu.split_min;
-  A.pair_mode = tu.pair_mode;
-  A.seeds_per_fetch = tu.seeds_per_fetch;
-  A.poll_mask = (uint32_t)tu.poll_every - 1u;
-  A.leaf_flatten = tu.leaf_flatten > 0 ? 1 : 0;
-  A.wps_shift = wps_shift(tu);
-  A.lookahead = tu.lookahead > 0 ? 1 : 0;
-  A.seeds = seeds;
-  A.nseeds = nseeds;
-  A.qbuf = qbuf;
-  A.qseq = qseq;
-  A.ctl = ctl;
-  A.rows = rows;
-  A.cap = 0;
-  A.root_mask = nullptr;
-  A.budget_ns = budget_ms() * 1000000ull;
-  A.max_chunks = budget_chunks();
-  A.plans = d_plans;
-  A.seed_pid = seed_pid;
-  A.counts = d_counts;
-  A.row_off = d_off;
-  A.row_cap = d_cap;
-  A.row_cursor = d_cursor;
-  A.grp_slots = grp_slots;
-  const int slot = min_blocks_slot(tu.extend_min_blocks);
-  const size_t smem = warp_smem_bytes(grp_slots) * kExtWarps;
-  bool sym = false;
-  for (const Plan &pl : plans) sym |= pl.naut > 1;
-  const int grid = extend_grid<true>(want_rows, counters, smem, slot, false, sym);
-  if (grid <= 0) return HM_ERR_CUDA;
-  st.extend_grid = grid;
-  st.extend_block = kExtThreads;
-  extend_kernel<true>(want_rows, counters, slot, false, sym)<<<grid, kExtThreads, smem, s>>>(G, plans[0], A);
-  launches += 1;
-  }
-  t_ext.stop();
-  HM_CUDA_TRY(cudaGetLastError());
-  Ctl h;
-  std::vector<unsigned long long> hc(npat);
-  HM_CUDA_TRY(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
-  HM_CUDA_TRY(cudaMemcpyAsync(hc.data(), d_counts, sizeof(unsigned long long) * npat,
-                              cudaMemcpyDeviceToHost, s));
-  HM_CUDA_TRY(cudaStreamSynchronize(s));
-  st.ms_edge_scan = t_edge.ms();
-  st.ms_overlap = t_ov.ms();
-  st.ms_extend = t_ext.ms();
-  st.seeds_scanned = (uint64_t)m;
-  st.states_injected = any_ov ? h.nseeds : h.nseeds_raw;
-  if (ran_levels) {
-    h.status = h.lv.status;
-    h.chunks = h.lv.chunks;
-  }
-  st.tasks_donated = h.donated;
-  st.chunks = h.chunks;
-  st.bytes_extend = h.bytes_extend;
-  st.model_bytes_extend = h.bytes_extend_model;
-  st.candidates = h.lanes;
-  if (h.status == kStatBudget) return HM_ERR_BUDGET;
-  if (h.status != kStatOk) return HM_ERR_CUDA;
+// Counts to the caller and, of the patterns whose rows fit their regions, the rows in order.
+hm_status finish_batch(const hm_graph *g, int32_t npat, const std::vector<int32_t> &ks, int32_t kmax, int32_t *rows,
+                       bool want_rows, const unsigned long long *off, const unsigned long long *cap,
+                       const unsigned long long *d_off, const std::vector<unsigned long long> &hc, uint64_t *counts,
+                       uint8_t *fit, Scratch &sc, cudaStream_t s, bool timing, hm_stats &st) {
   uint64_t total = 0;
   bool over = false;
   for (int32_t i = 0; i < npat; ++i) {
@@ -465,7 +214,6 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
     if (want_rows && hc[i] > cap[i]) over = true;
   }
   st.matches = total;
-  st.kernel_launches = launches;
   if (!want_rows) return HM_OK;
   if (over && !fit) return HM_ERR_CAPACITY;
   // ---- one sort for all patterns whose rows fit: key (pattern id, row), then back to each region
@@ -513,13 +261,18 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
     }
     return HM_OK;
   }
+  unsigned long long *d_start;
+  int32_t *d_ks;
+  HM_CUDA_TRY(sc.get((void **)&d_start, sizeof(unsigned long long) * npat));
+  HM_CUDA_TRY(sc.get((void **)&d_ks, sizeof(int32_t) * npat));
   HM_CUDA_TRY(cudaMemcpyAsync(d_start, start.data(), sizeof(unsigned long long) * npat,
                               cudaMemcpyHostToDevice, s));
+  HM_CUDA_TRY(cudaMemcpyAsync(d_ks, ks.data(), sizeof(int32_t) * npat, cudaMemcpyHostToDevice, s));
   const int width = kmax + 1;
   int32_t *packed, *tmp;
   HM_CUDA_TRY(sc.get((void **)&packed, sizeof(int32_t) * (size_t)total * width));
   HM_CUDA_TRY(sc.get((void **)&tmp, sizeof(int32_t) * (size_t)total * width));
-  const int grid_r = (int)std::max<uint64_t>(1, std::min<uint64_t>((total + 255) / 256, (uint64_t)sms * 16));
+  const int grid_r = (int)std::max<uint64_t>(1, std::min<uint64_t>((total + 255) / 256, (uint64_t)num_sms() * 16));
   k_pack_rows<<<grid_r, 256, 0, s>>>(rows, d_off, d_start, d_ks, npat, total, width, packed);
   int cols[kMaxK + 1], bits[kMaxK + 1];
   uint32_t xr[kMaxK + 1];
@@ -540,6 +293,277 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
     st.ms_sort = t_sort.ms();
   }
   return HM_OK;
+}
+
+// fit (may be NULL): instead of failing with HM_ERR_CAPACITY when some
+// pattern's rows exceed its region, return every count, sort the rows of the
+// patterns that fit and flag them (fit[i] = 1); the others' rows are not valid.
+hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int32_t *modes,
+                    int32_t npat, int32_t *rows, const uint64_t *row_offsets, uint64_t *counts,
+                    cudaStream_t s, uint8_t *fit = nullptr, uint64_t workspace = 0) {
+  if (!g || npat < 0 || (npat > 0 && (!pats || !modes || !counts))) return HM_ERR_ARG;
+  if (npat == 0) return HM_OK;
+  const bool want_rows = rows != nullptr || row_offsets != nullptr;
+  if (want_rows && (!rows || !row_offsets)) return HM_ERR_ARG;
+  ensure_pool();
+  hm_stats &st = tls_stats();
+  std::memset(&st, 0, sizeof(st));
+  const bool timing = timing_enabled();
+
+  // ---- patterns and row regions
+  const hm_tuning tu = tuning();
+  const bool counters = counters_enabled();
+  std::vector<int32_t> ks(npat);
+  int32_t kmax = 0;
+  for (int32_t i = 0; i < npat; ++i) {
+    if (!pats[i] || (modes[i] != HM_MONO && modes[i] != HM_INDUCED)) return HM_ERR_ARG;
+    ks[i] = pats[i]->k;
+    kmax = std::max(kmax, ks[i]);
+  }
+  std::vector<Plan> plans;  // copies: for the depth-first search, and without symmetry breaking
+  auto copy_plans = [&] {
+    plans.resize(npat);
+    for (int32_t i = 0; i < npat; ++i) {
+      plans[i] = pats[i]->plan[modes[i]];
+      if (tu.symmetry < 0) strip_symmetry(plans[i]);
+    }
+  };
+  // counts, row cursors (zero), first words and capacities of the row regions, in one block
+  std::vector<unsigned long long> regions((size_t)4 * npat, 0);
+  unsigned long long *off = regions.data() + 2 * npat, *cap = regions.data() + 3 * npat;
+  if (want_rows) {
+    for (int32_t i = 0; i < npat; ++i) {
+      if (row_offsets[i + 1] < row_offsets[i]) return HM_ERR_ARG;
+      off[i] = row_offsets[i];
+      cap[i] = (row_offsets[i + 1] - row_offsets[i]) / (uint64_t)ks[i];
+    }
+  }
+  Scratch sc(s);
+  unsigned long long *d_counts;
+  HM_CUDA_TRY(sc.get((void **)&d_counts, sizeof(unsigned long long) * regions.size()));
+  HM_CUDA_TRY(cudaMemcpyAsync(d_counts, regions.data(), sizeof(unsigned long long) * regions.size(),
+                              cudaMemcpyHostToDevice, s));
+  unsigned long long *d_cursor = d_counts + npat, *d_off = d_counts + 2 * npat, *d_cap = d_counts + 3 * npat;
+  const int64_t m = g->m;
+  const int sms = num_sms();
+  uint32_t launches = 0;
+  std::vector<unsigned long long> hc(npat);
+
+  // ---- level by level
+  if (g->ncls > 0 && default_search(tu) && !counters && budget_chunks() == 0) {
+    NvtxRange r_lv("hm.batch_extend");
+    std::vector<const Plan *> pp(npat);
+    if (tu.symmetry < 0) copy_plans();
+    for (int32_t i = 0; i < npat; ++i) pp[i] = tu.symmetry < 0 ? &plans[i] : &pats[i]->plan[modes[i]];
+    LvLaunch L{};
+    L.g = g;
+    L.want_rows = want_rows;
+    L.rows = rows;
+    L.workspace = workspace ? workspace : level_workspace(g);
+    L.defer = tu.share_seeds > 0;
+    L.npat = npat;
+    L.plans = pp.data();
+    L.counts = d_counts;
+    L.counts_host = hc.data();
+    L.row_off = d_off;
+    L.row_cap = d_cap;
+    L.row_cursor = d_cursor;
+    LvCtl h;
+    bool ran = false;
+    int grid = 0, threads = 0;
+    const hm_status r = levels_run(L, s, &ran, &h, &grid, &threads, timing ? &st.ms_extend : nullptr);
+    if (r != HM_OK) return r;
+    if (ran) {
+      st.extend_grid = grid;
+      st.extend_block = threads;
+      st.seeds_scanned = (uint64_t)m;
+      st.states_injected = h.injected;
+      st.chunks = h.chunks;
+      st.kernel_launches = 1;
+      if (h.status == kStatBudget) return HM_ERR_BUDGET;
+      if (h.status != kStatOk) return HM_ERR_CUDA;
+      return finish_batch(g, npat, ks, kmax, rows, want_rows, off, cap, d_off, hc, counts, fit, sc, s, timing, st);
+    }
+  }
+
+  // ---- depth first
+  copy_plans();
+  int32_t grp_slots = 0;
+  for (const Plan &P : plans) grp_slots = std::max(grp_slots, P.ngrp);
+  // signature (arc label, label of the arc's source, label of its target) -> patterns
+  struct Sig {
+    int32_t lab, vs, vd, pid;
+  };
+  std::vector<Sig> sigs(npat);
+  for (int32_t i = 0; i < npat; ++i) {
+    const Plan &P = plans[i];
+    // normal seeding: arc (f(0), f(1)); reversed: arc (f(1), f(0))
+    sigs[i] = P.seed_rev ? Sig{P.seed_lab, P.vlab[1], P.vlab[0], i} : Sig{P.seed_lab, P.vlab[0], P.vlab[1], i};
+  }
+  std::sort(sigs.begin(), sigs.end(), [](const Sig &x, const Sig &y) {
+    if (x.lab != y.lab) return x.lab < y.lab;
+    if (x.vs != y.vs) return x.vs < y.vs;
+    if (x.vd != y.vd) return x.vd < y.vd;
+    return x.pid < y.pid;
+  });
+  uint32_t tsize = 16;
+  while (tsize < 2u * (uint32_t)npat) tsize <<= 1;
+  std::vector<SigKey> keys(tsize, SigKey{0, 0, 0, 0});
+  std::vector<int2> vals(tsize, make_int2(0, 0));
+  std::vector<int32_t> pid_list(npat);
+  for (int32_t i = 0; i < npat;) {
+    int32_t j = i;
+    while (j < npat && sigs[j].lab == sigs[i].lab && sigs[j].vs == sigs[i].vs && sigs[j].vd == sigs[i].vd) {
+      pid_list[j] = sigs[j].pid;
+      ++j;
+    }
+    uint32_t h = sig_hash(sigs[i].lab, sigs[i].vs, sigs[i].vd) & (tsize - 1);
+    while (keys[h].used) h = (h + 1) & (tsize - 1);
+    keys[h] = SigKey{sigs[i].lab, sigs[i].vs, sigs[i].vd, 1};
+    vals[h] = make_int2(i, j - i);
+    i = j;
+  }
+
+  // ---- device copies
+  Plan *d_plans;
+  SigKey *d_keys;
+  int2 *d_vals;
+  int32_t *d_pids;
+  Ctl *ctl;
+  HM_CUDA_TRY(sc.get((void **)&d_plans, sizeof(Plan) * npat));
+  HM_CUDA_TRY(sc.get((void **)&d_keys, sizeof(SigKey) * tsize));
+  HM_CUDA_TRY(sc.get((void **)&d_vals, sizeof(int2) * tsize));
+  HM_CUDA_TRY(sc.get((void **)&d_pids, sizeof(int32_t) * npat));
+  HM_CUDA_TRY(sc.get((void **)&ctl, sizeof(Ctl)));
+  HM_CUDA_TRY(cudaMemcpyAsync(d_plans, plans.data(), sizeof(Plan) * npat, cudaMemcpyHostToDevice, s));
+  HM_CUDA_TRY(cudaMemcpyAsync(d_keys, keys.data(), sizeof(SigKey) * tsize, cudaMemcpyHostToDevice, s));
+  HM_CUDA_TRY(cudaMemcpyAsync(d_vals, vals.data(), sizeof(int2) * tsize, cudaMemcpyHostToDevice, s));
+  HM_CUDA_TRY(cudaMemcpyAsync(d_pids, pid_list.data(), sizeof(int32_t) * npat, cudaMemcpyHostToDevice, s));
+  HM_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Ctl), s));
+  const SigTable T{d_keys, d_vals, d_pids, tsize - 1};
+  const DevGraph G = g->dev();
+
+  // ---- edge scan: count, size, write
+  NvtxRange r_edge("hm.batch_edge_scan");
+  Timer t_edge(s, timing);
+  const int grid_e = (int)std::max<int64_t>(1, std::min<int64_t>((m + kSeedThreads - 1) / kSeedThreads,
+                                                                   (int64_t)sms * 8));
+  unsigned long long nraw = 0;
+  if (m) {
+    k_edge_seed_batch<false><<<grid_e, kSeedThreads, 0, s>>>(G, d_plans, T, nullptr, nullptr, 0,
+                                                             &ctl->nseeds_raw);
+    HM_CUDA_TRY(cudaMemcpyAsync(&nraw, &ctl->nseeds_raw, sizeof(nraw), cudaMemcpyDeviceToHost, s));
+    HM_CUDA_TRY(cudaStreamSynchronize(s));
+    launches += 1;
+  }
+  int2 *seeds_a, *seeds_b;
+  int32_t *pid_a, *pid_b;
+  HM_CUDA_TRY(sc.get((void **)&seeds_a, sizeof(int2) * (size_t)std::max<unsigned long long>(nraw, 1)));
+  HM_CUDA_TRY(sc.get((void **)&pid_a, sizeof(int32_t) * (size_t)std::max<unsigned long long>(nraw, 1)));
+  HM_CUDA_TRY(sc.get((void **)&seeds_b, sizeof(int2) * (size_t)std::max<unsigned long long>(nraw, 1)));
+  HM_CUDA_TRY(sc.get((void **)&pid_b, sizeof(int32_t) * (size_t)std::max<unsigned long long>(nraw, 1)));
+  if (nraw) {
+    HM_CUDA_TRY(cudaMemsetAsync(&ctl->nseeds_raw, 0, sizeof(unsigned long long), s));
+    k_edge_seed_batch<true><<<grid_e, kSeedThreads, 0, s>>>(G, d_plans, T, seeds_a, pid_a, nraw,
+                                                            &ctl->nseeds_raw);
+    launches += 1;
+  }
+  t_edge.stop();
+  HM_CUDA_TRY(cudaGetLastError());
+  // ---- overlap test (patterns without one pass their seeds through)
+  bool any_ov = false;
+  for (const Plan &P : plans) any_ov |= P.ov_need > 0;
+  const int2 *seeds = seeds_a;
+  const int32_t *seed_pid = pid_a;
+  const unsigned long long *nseeds = &ctl->nseeds_raw;
+  Timer t_ov(s, timing && any_ov);
+  if (any_ov && nraw) {
+    int2 *seeds_c;
+    int32_t *pid_c;
+    unsigned long long *ntest;
+    HM_CUDA_TRY(sc.get((void **)&seeds_c, sizeof(int2) * (size_t)nraw));
+    HM_CUDA_TRY(sc.get((void **)&pid_c, sizeof(int32_t) * (size_t)nraw));
+    HM_CUDA_TRY(sc.get((void **)&ntest, sizeof(unsigned long long)));
+    HM_CUDA_TRY(cudaMemsetAsync(ntest, 0, sizeof(unsigned long long), s));
+    const int grid_s = (int)std::max<unsigned long long>(
+        1, std::min<unsigned long long>((nraw + kSeedThreads - 1) / kSeedThreads, (unsigned long long)sms * 8));
+    k_overlap_split<<<grid_s, kSeedThreads, 0, s>>>(d_plans, seeds_a, pid_a, &ctl->nseeds_raw, seeds_b, pid_b,
+                                                     &ctl->nseeds, seeds_c, pid_c, ntest);
+    k_seed_overlap<false, true><<<sms * 8, kSeedThreads, 0, s>>>(G, 0, seeds_c, ntest, seeds_b, nraw,
+                                                                  &ctl->nseeds, &ctl->bytes_overlap, d_plans,
+                                                                  pid_c, pid_b);
+    launches += 2;
+    seeds = seeds_b;
+    seed_pid = pid_b;
+    nseeds = &ctl->nseeds;
+  }
+  t_ov.stop();
+
+  // ---- one persistent extension launch for every pattern
+  NvtxRange r_ext("hm.batch_extend");
+  Timer t_ext(s, timing);
+  Task *qbuf;
+  unsigned long long *qseq;
+  HM_CUDA_TRY(sc.get((void **)&qbuf, sizeof(Task) * kQueueCap));
+  HM_CUDA_TRY(sc.get((void **)&qseq, sizeof(unsigned long long) * kQueueCap));
+  k_qinit<<<64, 256, 0, s>>>(qseq);
+  launches += 1;
+  ExtArgs A{};
+  A.split_min = tu.split_min;
+  A.pair_mode = tu.pair_mode;
+  A.seeds_per_fetch = tu.seeds_per_fetch;
+  A.poll_mask = (uint32_t)tu.poll_every - 1u;
+  A.leaf_flatten = tu.leaf_flatten > 0 ? 1 : 0;
+  A.wps_shift = wps_shift(tu);
+  A.lookahead = tu.lookahead > 0 ? 1 : 0;
+  A.seeds = seeds;
+  A.nseeds = nseeds;
+  A.qbuf = qbuf;
+  A.qseq = qseq;
+  A.ctl = ctl;
+  A.rows = rows;
+  A.cap = 0;
+  A.root_mask = nullptr;
+  A.budget_ns = budget_ms() * 1000000ull;
+  A.max_chunks = budget_chunks();
+  A.plans = d_plans;
+  A.seed_pid = seed_pid;
+  A.counts = d_counts;
+  A.row_off = d_off;
+  A.row_cap = d_cap;
+  A.row_cursor = d_cursor;
+  A.grp_slots = grp_slots;
+  const int slot = min_blocks_slot(tu.extend_min_blocks);
+  const size_t smem = warp_smem_bytes(grp_slots) * kExtWarps;
+  bool sym = false;
+  for (const Plan &pl : plans) sym |= pl.naut > 1;
+  const int grid = extend_grid<true>(want_rows, counters, smem, slot, false, sym);
+  if (grid <= 0) return HM_ERR_CUDA;
+  st.extend_grid = grid;
+  st.extend_block = kExtThreads;
+  extend_kernel<true>(want_rows, counters, slot, false, sym)<<<grid, kExtThreads, smem, s>>>(G, plans[0], A);
+  launches += 1;
+  t_ext.stop();
+  HM_CUDA_TRY(cudaGetLastError());
+  Ctl h;
+  HM_CUDA_TRY(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
+  HM_CUDA_TRY(cudaMemcpyAsync(hc.data(), d_counts, sizeof(unsigned long long) * npat,
+                              cudaMemcpyDeviceToHost, s));
+  HM_CUDA_TRY(cudaStreamSynchronize(s));
+  st.ms_edge_scan = t_edge.ms();
+  st.ms_overlap = t_ov.ms();
+  st.ms_extend = t_ext.ms();
+  st.seeds_scanned = (uint64_t)m;
+  st.states_injected = any_ov ? h.nseeds : h.nseeds_raw;
+  st.tasks_donated = h.donated;
+  st.chunks = h.chunks;
+  st.bytes_extend = h.bytes_extend;
+  st.model_bytes_extend = h.bytes_extend_model;
+  st.candidates = h.lanes;
+  st.kernel_launches = launches;
+  if (h.status == kStatBudget) return HM_ERR_BUDGET;
+  if (h.status != kStatOk) return HM_ERR_CUDA;
+  return finish_batch(g, npat, ks, kmax, rows, want_rows, off, cap, d_off, hc, counts, fit, sc, s, timing, st);
 }
 
 }  // namespace

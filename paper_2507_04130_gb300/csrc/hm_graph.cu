@@ -171,10 +171,15 @@ __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__rest
 
 // Dense group offsets of one direction (see DevGraph): one warp per vertex, the
 // vertex's directory entries on its lanes, two rounds of 32 classes.  A class
-// without a group starts where the next one does.
+// without a group starts where the next one does.  Counts the groups of each
+// (vertex label, class) for k_class_place.
 __global__ void k_dense(const int4 *__restrict__ vdir, const int2 *__restrict__ off, const int4 *__restrict__ vi,
                         const int4 *__restrict__ dir, int32_t n, int64_t m, int in, int32_t ncls, int32_t nvl,
-                        int32_t al0, int32_t vl0, int32_t *__restrict__ gofs) {
+                        int32_t al0, int32_t vl0, int32_t *__restrict__ gofs, uint32_t *__restrict__ cnt_of) {
+  __shared__ uint32_t h[kMaxDense * kMaxDense];
+  const int nbin = ncls * nvl;
+  for (int b = threadIdx.x; b < nbin; b += blockDim.x) h[b] = 0;
+  __syncthreads();
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
@@ -188,13 +193,17 @@ __global__ void k_dense(const int4 *__restrict__ vdir, const int2 *__restrict__ 
     int32_t s0 = len, s1 = len;
     if (lane < cnt) {
       const int4 e = dir[(int64_t)first + lane];
-      have |= 1ull << ((e.x - al0) * nvl + (e.y - vl0));
+      const int c = (e.x - al0) * nvl + (e.y - vl0);
+      have |= 1ull << c;
       s0 = e.z;
+      atomicAdd(&h[(info.x - vl0) * ncls + c], 1u);
     }
     if (lane + 32 < cnt) {
       const int4 e = dir[(int64_t)first + lane + 32];
-      have |= 1ull << ((e.x - al0) * nvl + (e.y - vl0));
+      const int c = (e.x - al0) * nvl + (e.y - vl0);
+      have |= 1ull << c;
       s1 = e.z;
+      atomicAdd(&h[(info.x - vl0) * ncls + c], 1u);
     }
     const unsigned long long all = (unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)have) |
                                    (unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)(have >> 32)) << 32;
@@ -205,6 +214,45 @@ __global__ void k_dense(const int4 *__restrict__ vdir, const int2 *__restrict__ 
       if (c < ncls) gofs[v * ncls + c] = base + (at >= cnt ? len : at < 32 ? a : b);
     }
     if (v == n - 1 && lane == 0) gofs[(int64_t)n * ncls] = (int32_t)m;
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < nbin; b += blockDim.x)
+    if (h[b]) atomicAdd(cnt_of + b, h[b]);
+}
+
+// The vertices of each (vertex label, class) that have such a group, one
+// direction: tiles of vertices, each reserving its part of every list, so that
+// neighbours in a list stay neighbours in the graph.
+constexpr int kClassTile = 256;
+
+__global__ void k_class_place(const int4 *__restrict__ vdir, const int4 *__restrict__ vi, const int4 *__restrict__ dir,
+                              int32_t n, int in, int32_t ncls, int32_t nvl, int32_t al0, int32_t vl0,
+                              const uint32_t *__restrict__ start, uint32_t *__restrict__ cur,
+                              int32_t *__restrict__ vby) {
+  __shared__ uint32_t h[kMaxDense * kMaxDense];
+  const int nbin = ncls * nvl, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (int64_t t0 = (int64_t)blockIdx.x * kClassTile; t0 < n; t0 += (int64_t)gridDim.x * kClassTile) {
+    const int64_t t1 = min((int64_t)n, t0 + kClassTile);
+    for (int b = threadIdx.x; b < nbin; b += blockDim.x) h[b] = 0;
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int64_t v = t0 + warp; v < t1; v += warps) {
+        const int4 vd = vdir[v];
+        const int l = (vi[v].x - vl0) * ncls;
+        const int32_t first = in ? vd.z : vd.x, cnt = in ? vd.w : vd.y;
+        for (int e = lane; e < cnt; e += 32) {
+          const int4 d = dir[(int64_t)first + e];
+          const uint32_t at = atomicAdd(&h[l + (d.x - al0) * nvl + (d.y - vl0)], 1u);
+          if (pass) vby[at] = (int32_t)v;
+        }
+      }
+      __syncthreads();
+      if (!pass) {
+        for (int b = threadIdx.x; b < nbin; b += blockDim.x)
+          if (h[b]) h[b] = start[b] + atomicAdd(cur + b, h[b]);
+        __syncthreads();
+      }
+    }
   }
 }
 
@@ -437,6 +485,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   if (n)
     k_vertex<<<grid_for(n), kThreads, 0, s>>>(d_vlab, out_off, in_off, oidx, iidx, n, g->vi, g->off,
                                               g->vdir, bnd);
+  std::vector<uint32_t> h_bins;
   // dense group offsets while there are few classes and the tables are no larger than the arcs' own data
   const int64_t nal = m ? (int64_t)hb.emax - hb.emin + 1 : 0, nvl = m ? (int64_t)hb.vmax - hb.vmin + 1 : 0;
   if (m && nal <= kMaxDense && nvl <= kMaxDense && nal * nvl <= kMaxDense &&
@@ -449,28 +498,49 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     const int64_t len = (int64_t)n * g->ncls + 1;
     HM_CUDA_TRY(dmalloc(&g->gofs_out, len));
     HM_CUDA_TRY(dmalloc(&g->gofs_in, len));
-    for (int in = 0; in < 2; ++in)
-      k_dense<<<grid_for(32 * (int64_t)n), kThreads, 0, s>>>(g->vdir, g->off, g->vi, in ? g->gdir_in : g->gdir_out, n,
-                                                             m, in, g->ncls, g->nvl, g->al0, g->vl0,
-                                                             in ? g->gofs_in : g->gofs_out);
+    const int nbin = g->ncls * g->nvl;
+    uint32_t *bins;  // counts and cursors of both directions, then the list starts
+    HM_CUDA_TRY(T.get((void **)&bins, sizeof(uint32_t) * 6 * (size_t)(nbin + 1)));
+    HM_CUDA_TRY(cudaMemsetAsync(bins, 0, sizeof(uint32_t) * 4 * (size_t)(nbin + 1), s));
+    h_bins.resize(2 * (size_t)(nbin + 1));
+    for (int in = 0; in < 2; ++in) {
+      const int4 *dir = in ? g->gdir_in : g->gdir_out;
+      int32_t *&vby = in ? g->vby_in : g->vby_out;
+      uint32_t *cnt = bins + in * (nbin + 1), *cur = cnt + 2 * (nbin + 1), *start = cnt + 4 * (nbin + 1);
+      HM_CUDA_TRY(dmalloc(&vby, in ? g->ndir_in : g->ndir_out));
+      k_dense<<<grid_for(32 * (int64_t)n), kThreads, 0, s>>>(g->vdir, g->off, g->vi, dir, n, m, in, g->ncls, g->nvl,
+                                                             g->al0, g->vl0, in ? g->gofs_in : g->gofs_out, cnt);
+      const hm_status st = exclusive_scan_u32(cnt, start, nbin + 1, s);
+      if (st != HM_OK) return st;
+      k_class_place<<<grid_for((int64_t)n), kThreads, 0, s>>>(g->vdir, g->vi, dir, n, in, g->ncls, g->nvl, g->al0,
+                                                             g->vl0, start, cur, vby);
+      HM_CUDA_TRY(cudaMemcpyAsync(h_bins.data() + (size_t)in * (nbin + 1), start, sizeof(uint32_t) * (nbin + 1),
+                                  cudaMemcpyDeviceToHost, s));
+    }
   }
   HM_CUDA_TRY(cudaMemcpyAsync(&h_err, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaMemcpyAsync(&hb, bnd, sizeof(Bounds), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaStreamSynchronize(s));
   HM_CUDA_TRY(cudaGetLastError());
   g->maxdeg = hb.maxdeg;
+  if (!h_bins.empty()) {
+    g->vstart = (uint32_t *)malloc(sizeof(uint32_t) * h_bins.size());
+    if (!g->vstart) return HM_ERR_OOM;
+    std::memcpy(g->vstart, h_bins.data(), sizeof(uint32_t) * h_bins.size());
+  }
   if (h_err & kErrDup) return HM_ERR_DUP_EDGE;
   if (h_err & kErrHash) return HM_ERR_CUDA;  // cannot happen (twice as many slots as arcs)
   g->bytes = sizeof(int32_t) * 7 * (size_t)m + (sizeof(int4) * 2 + sizeof(int2)) * (size_t)n +
              sizeof(int4) * (size_t)(g->ndir_out + g->ndir_in) + 8 * (size_t)g->afilt_nword +
-             32 * (size_t)g->ahash_nbkt + (g->ncls ? sizeof(int32_t) * 2 * ((size_t)n * g->ncls + 1) : 0);
+             32 * (size_t)g->ahash_nbkt + (g->ncls ? sizeof(int32_t) * (2 * ((size_t)n * g->ncls + 1) + (size_t)(g->ndir_out + g->ndir_in)) : 0);
   return HM_OK;
 }
 
 void free_graph_arrays(hm_graph *g) {
   void *ptrs[] = {g->src,     g->out_adj,  g->out_elab, g->in_adj,   g->in_elab, g->vi,
                   g->off,     g->gout_adj, g->gin_adj,  g->gdir_out, g->gdir_in, g->vdir,
-                  g->afilt,   g->ahash,    g->check,    g->gofs_out, g->gofs_in};
+                  g->afilt,   g->ahash,    g->check,    g->gofs_out, g->gofs_in, g->vby_out,
+                  g->vby_in};
   for (void *p : ptrs)
     if (p) cudaFree(p);
 }
@@ -502,6 +572,7 @@ extern "C" hm_status hm_load_graph(int32_t n, int64_t m, const int32_t *src, con
     cudaStreamSynchronize(s);
     (void)cudaGetLastError();
     free_graph_arrays(g);
+    free(g->vstart);
     delete g;
     return st;
   }
@@ -514,6 +585,7 @@ extern "C" void hm_free_graph(hm_graph *g) {
   free_graph_arrays(g);
   free(g->vtab);
   free(g->etab);
+  free(g->vstart);
   delete g;
 }
 

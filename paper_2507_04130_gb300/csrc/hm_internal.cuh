@@ -413,6 +413,11 @@ struct hm_graph {
   int32_t *gofs_out, *gofs_in;  // dense group offsets (null: ncls = 0)
   int32_t ncls, al0, vl0, nal, nvl;  // classes; first labels and label counts
   int32_t maxdeg;                    // largest out- or in-degree
+  // with ncls: the vertices of label vl0 + l that have an out- (in-) group of
+  // class c are vby_out (vby_in) [vstart[b], vstart[b + 1]), b = l * ncls + c
+  // (in: b = ncls * nvl + 1 + l * ncls + c); vstart is host memory
+  int32_t *vby_out, *vby_in;
+  uint32_t *vstart;
   unsigned long long *check;  // bounds-checked builds: the violation word (device)
   size_t bytes;
   // multi-property graphs (hm_load_graph_props): the sorted distinct property

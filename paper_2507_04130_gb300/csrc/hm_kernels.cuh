@@ -101,7 +101,6 @@ struct Ctl {
   unsigned long long lanes;                   // candidates examined (instrumented launches only)
   unsigned long long level_chunks[kMaxK];     // per depth (instrumented launches only)
   unsigned long long level_lanes[kMaxK];
-  LvCtl lv;                                   // extension level by level
 };
 
 struct ExtArgs {

@@ -1,4 +1,4 @@
-// hm_levels.cu -- state extension, level by level, in one persistent launch.
+// hm_levels.cu -- a whole match, level by level, in one persistent launch.
 //
 // The states of a level (p mapped positions each) are extended together: every
 // candidate of every state is one lane's work, so the lanes are full and all
@@ -7,22 +7,33 @@
 // the warps busy wherever a few hubs own the work: a connectome query of 121 M
 // leaf candidates took 17.4 ms, of which 90 % was waiting for the last warps.)
 //
-// A level has two phases, each ended by a grid barrier:
-//   ranges   one thread per state: the anchors' label groups (dense group
-//            offsets: one lookup of two neighbouring words each), the shortest
-//            of which holds the candidates; a state whose anchor has an empty
-//            group dies here.  States are taken in groups of up to 32, and a
-//            prefix sum over the groups' chunks of 32 candidates numbers all
-//            chunks of the level.
-//   expand   each warp takes runs of consecutive chunks, finds the group a
-//            run starts in, and reads 32 candidates at a time: the filter
-//            probes of the other positive conditions reject most; survivors
-//            wait in the warp's buffer until 128 are there, then
-//            the exact checks run on full warps and the survivors of those
-//            become states of the next level, or matches.
-// Memory is bounded: an expansion takes no more chunks than the next level's
-// buffer can hold survivors of, then the deeper levels are worked off before
-// the rest (depth first over slices of levels).
+// The first level is the vertices with position 0's label and a neighbour that
+// position 1 could take (listed per class when the graph is loaded); position 1
+// is extended like every other, along the seeding arc's label group.  That takes
+// the place of the scan over all arcs (the loop over E2 of the HiPerMotif
+// algorithm): only arcs with the seeding arc's three labels are read, 4 bytes
+// each and in source order, instead of 12 bytes of every arc and two vertex
+// records per candidate.
+//
+// Expanding a level: its states stand in groups of up to 32, and the groups'
+// chunks of 32 candidates are numbered through.  Each warp takes runs of
+// consecutive chunks, finds the group a run starts in, and reads 32 candidates
+// at a time: the filter probes of the other positive conditions reject most;
+// survivors wait in the warp's buffer until 64 are there, then the exact checks
+// run on full warps.  What passes becomes a match, or a state of the next
+// level: its anchors' label groups (dense group offsets: one lookup of two
+// neighbouring words each), the shortest of which holds its candidates.  A
+// state whose anchor has an empty group is dropped, and so is one whose last
+// position has no other condition, if only its number is asked for: it is the
+// group's length.  Up to 64 states go to the next level with one addition,
+// which reserves their groups and numbers their chunks.  A grid barrier ends
+// the expansion.
+// Memory is bounded: when the states of some warp do not fit the next level any
+// more, all remember where they stand; the deeper levels are worked off, and
+// then they go on (depth first over parts of levels).
+//
+// A pendant position 1 (Plan::defer1: no later position has an arc to it) is
+// matched last, so the search over the others is shared by all its images.
 //
 // Bound by the latency of its lookups in L2 and HBM (list entry, then filter
 // word, per candidate), which many independent warps hide.
@@ -40,55 +51,104 @@ constexpr int kLvThreads = 512;
 constexpr int kLvWarps = kLvThreads / 32;
 constexpr int kLvMinBlocks = 2;
 constexpr uint32_t kFull = 0xffffffffu;
-constexpr int kLvBuf = 160;       // survivors of a warp waiting for the exact checks
-constexpr int kLvDrain = 128;     // checked when this many wait (a chunk adds at most 32)
-constexpr int kLvMaxGrid = 1024;
-constexpr int kLvMaxGroups = 1024;  // groups of one block in the ranges phase
-constexpr int64_t kLvSeedSlice = 1 << 21;  // depth-2 states taken at a time
+constexpr int kLvBuf = 96;        // survivors of a warp waiting for the exact checks
+constexpr int kLvDrain = 64;      // checked when this many wait (a chunk adds at most 32)
+constexpr int kLvChunkBits = 40;  // of a level's counter; the groups are above
+constexpr unsigned long long kLvChunkMask = (1ull << kLvChunkBits) - 1;
+constexpr int64_t kLvMaxGroups = 1 << 20;  // of a level (2^24 would fit the counter)
 constexpr uint64_t kLvBarrierNs = 10ull * 1000 * 1000 * 1000;
+
+// A condition of a level: Cons with the class (arc label, vertex label) whose
+// group of f(q) holds the candidates, -1 if the graph has no such label.
+struct LvCons {
+  int8_t q, kind;
+  int16_t cls;
+  int32_t lab;
+  uint64_t la, lb;  // the label's part of the two hashes of the arc filter
+};
+
+// What a candidate for one position must satisfy.
+struct LevelPlan {
+  int16_t npos, ncons;    // positive conditions first
+  int8_t last;            // the position completes a match
+  int8_t need_deg;        // test the degrees: at least two pattern arcs lead to positions after the next
+  int8_t root;            // the root mask applies to this position
+  int8_t closed;          // the last position has one condition, and only the number of its images is wanted
+  int8_t final;           // level 1 of a plan with a deferred position 1: the level that matches it, else 0
+  int32_t dout, din;
+  uint32_t sym_gt, sym_lt;
+  LvCons cons[kMaxCons];
+};
+
+// How a pattern's matches are written.
+struct EmitPlan {
+  int32_t k, naut;
+  int32_t aut;            // first byte of its automorphisms in the table, kMaxK each
+  int32_t orig[kMaxK];
+};
+
+// A group of states: its first chunk and its number of states.  Its states are
+// those numbered from 32 times the group's number on.
+struct LvGroup {
+  unsigned long long start;
+  uint32_t n, pad;
+};
+
+// Where a warp goes on whose states did not fit the next level.
+struct LvPause {
+  unsigned long long x;     // next chunk
+  uint32_t left, run;       // chunks left of the run; the claimed run after it
+  int32_t on, nwait, nbuf, pad;  // paused at all; states waiting for room, survivors waiting for their checks
+  int2 buf[kLvBuf];         // both, {parent, candidate}
+};
 
 struct LvArgs {
   DevGraph G;
   LvCtl *ctl;
-  const int32_t *base[kMaxK + 2];  // states of each level; stride[p] words each
-  int4 *rng[kMaxK + 2];            // {first candidate, number, driving condition, pattern}
-  unsigned long long *upre[kMaxK + 2];  // chunks of the earlier groups of the same block
-  unsigned long long *bsum[kMaxK + 2];  // chunks of each block's groups
-  int32_t stride[kMaxK + 2];
-  int64_t fcap;                    // states a level's buffer holds
-  int64_t slice;                   // depth-2 states of a slice
-  const unsigned long long *nseeds;
-  const int4 *groups;
-  const int2 *sorted_seeds;
+  // each level: states (stride[p] words each, with the pattern's number after the images in a
+  // batch), their candidates {first, number, driving condition | list << 6 | pattern << 7, 0}, groups
+  int32_t *base[kMaxK + 1];
+  int4 *rng[kMaxK + 1];
+  LvGroup *grp[kMaxK + 1];
+  LvPause *pause[kMaxK + 1];
+  int32_t stride[kMaxK + 1];
+  uint32_t gcap[kMaxK + 1];        // groups each level holds
+  uint32_t fill_warps;             // warps that fill the first level
+  unsigned long long slice;        // vertices of a slice of the first level
+  unsigned long long nvert;        // vertices the first level starts from
+  const int32_t *vert;
+  // batch: vertices are numbered pattern after pattern (vert_n), vertex s of pattern pid is vert_at[pid][s]
+  const unsigned long long *vert_n;
+  const int32_t *const *vert_at;
+  int32_t npat;
+  int32_t dout0, din0, root0;      // position 0 of a single pattern: degrees, root mask
+  const int2 *deg0;                // batch: {out, in}
   const uint8_t *root_mask;
   unsigned long long budget_ns;
   int32_t *rows;
   unsigned long long cap;
-  const int32_t *seed_pid;
   const LevelPlan *levels;         // batch: [pattern][kmax]
   const EmitPlan *emit;
   const int8_t *aut;
   unsigned long long *counts;
   const unsigned long long *row_off, *row_cap;
   unsigned long long *row_cursor;
-  int32_t kmax;                    // levels 2 .. kmax - 1 (kmax: the deferred position 1)
-  int32_t ndefer;
-  Cons defer[kMaxCons];
+  int32_t kmax;                    // levels 1 .. kmax - 1
   EmitPlan emit1;
   LevelPlan level1[kMaxK];
 };
 
 struct LvShared {
-  unsigned long long sum[kLvMaxGroups];      // ranges: chunks of this block's groups
-  unsigned long long first[kLvMaxGrid];      // expand: first chunk of each block's groups
-  unsigned long long wsum[kLvWarps];
-  int4 rec[kLvWarps][32];                    // the group's states with candidates, in order
-  int2 buf[kLvWarps][kLvBuf];                // {state, candidate}
+  int4 rec[kLvWarps][32];          // the group's states
+  int2 buf[kLvWarps][kLvBuf];      // {state, candidate}
+  int4 fresh[kLvWarps][kLvDrain];  // states of the next level: {first candidate, number, what, parent}
   // values all warps share, and each warp's matches, kept out of the registers of the expansion
-  unsigned long long made, deadline, begin, take;
+  unsigned long long deadline, total;
   unsigned long long count[kLvWarps];
-  uint32_t run_len, nrun;
-  unsigned int *claim;
+  uint32_t injected[kLvWarps];
+  unsigned long long *made;        // the next level's counter
+  uint32_t run_len, nrun, ngroup;
+  unsigned int *claim, *paused;
   int ok;
 };
 
@@ -115,58 +175,16 @@ __device__ __forceinline__ bool lv_barrier(const LvArgs &A, LvShared &sm, unsign
   return sm.ok != 0;
 }
 
-// Exclusive prefix sum over the block of one value per thread; *total is the sum.
-__device__ __forceinline__ unsigned long long lv_block_scan(unsigned long long v, LvShared &sm,
-                                                            unsigned long long *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(kFull, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) sm.wsum[warp] = x;
-  __syncthreads();
-  unsigned long long before = 0, all = 0;
-#pragma unroll
-  for (int w = 0; w < kLvWarps; ++w) {
-    const unsigned long long s = sm.wsum[w];
-    if (w < warp) before += s;
-    all += s;
-  }
-  __syncthreads();
-  *total = all;
-  return before + x - v;
-}
-
-// States per group: all 32 lanes' worth when there are enough states for every
-// warp, else fewer, so that a small level still spreads over the warps.
-// Positions inside a group are 32-bit: g lists of at most maxdeg entries.
-__device__ __forceinline__ int lv_group_size(unsigned long long cnt, unsigned long long warps, int32_t maxdeg) {
-  int g = 32;
-  while (g > 1 && (unsigned long long)maxdeg * g > 0xffffffffull) g >>= 1;
-  while (g > 1 && cnt < (unsigned long long)g * warps) g >>= 1;
-  return g;
-}
-
-__device__ __forceinline__ const int32_t *lv_state(const LvArgs &A, int p, int64_t s) {
-  return A.base[p] + s * A.stride[p];
-}
-
 // A state's first four images, in registers: most patterns' checks read no
-// more of it.  What is not a vertex (unmapped positions, the group in the
-// place of a deferred position 1, a pattern number) is -1.
-template <bool kShared>
+// more of it.  What is not a vertex (unmapped positions, a pattern number) is -1.
 __device__ __forceinline__ int4 lv_images(const int32_t *mp, int p) {
-  int4 m;
+  if (p == 1) return make_int4(mp[0], -1, -1, -1);
   if (p == 2) {
     const int2 v = *reinterpret_cast<const int2 *>(mp);
-    m = make_int4(v.x, v.y, -1, -1);
-  } else {
-    m = *reinterpret_cast<const int4 *>(mp);
-    if (p == 3) m.w = -1;
+    return make_int4(v.x, v.y, -1, -1);
   }
-  if (kShared) m.y = -1;
+  int4 m = *reinterpret_cast<const int4 *>(mp);
+  if (p == 3) m.w = -1;
   return m;
 }
 
@@ -176,119 +194,89 @@ __device__ __forceinline__ int32_t lv_image(const int4 &m, const int32_t *mp, in
   return q & 2 ? b : a;
 }
 
-// The candidates of state `s` of level p: {first, number, driving condition | list << 8, pattern}.
-// list: 0 out-groups, 1 in-groups, 2 the seeds of a shared group.
-template <bool kBatch, bool kShared, bool kSym>
-__device__ __forceinline__ int4 lv_range(const LvArgs &A, int p, int64_t s, int32_t pid) {
-  const int32_t *mp = lv_state(A, p, s);
-  if (kShared && p == A.kmax) {
-    const int4 gr = __ldg(A.groups + mp[1]);
-    return make_int4(gr.y, gr.z - gr.y, 2 << 8, 0);
-  }
-  const LevelPlan &L = kBatch ? A.levels[(int64_t)pid * A.kmax + p] : A.level1[p];
-  if (kSym && p == 2) {
-    // the order constraint between positions 0 and 1 (the injected states stay the validators' output)
-    const LevelPlan &L1 = kBatch ? A.levels[(int64_t)pid * A.kmax + 1] : A.level1[1];
-    if ((L1.sym_gt && mp[1] <= mp[0]) || (L1.sym_lt && mp[1] >= mp[0])) return make_int4(0, 0, 0, pid);
-  }
-  int32_t best = INT32_MAX, lo = 0, what = 0;
-  for (int j = 0; j < L.npos; ++j) {
-    const LvCons cs = L.cons[j];
-    if (cs.cls < 0) return make_int4(0, 0, 0, pid);
-    const int32_t *ofs = cs.kind == kOut ? A.G.gofs_out : A.G.gofs_in;
-    const int64_t at = (int64_t)mp[cs.q] * A.G.ncls + cs.cls;
-    const int32_t a = __ldg(ofs + HM_AT(A.G, at, (int64_t)A.G.n * A.G.ncls, kChkGroup));
-    const int32_t b = __ldg(ofs + at + 1);
-    if (b - a < best) {
-      best = b - a;
-      lo = a;
-      what = j | (cs.kind == kOut ? 0 : 1 << 8);
-    }
-  }
-  return make_int4(lo, best, what, pid);
+// What is packed into a range's third word.
+__device__ __forceinline__ int lv_drive(int32_t what) { return what & 63; }
+__device__ __forceinline__ int lv_list(int32_t what) { return what >> 6 & 1; }
+__device__ __forceinline__ int32_t lv_pid(int32_t what) { return what >> 7; }
+
+// The group of f(q) = v that condition cs names.
+__device__ __forceinline__ int2 lv_group(const LvArgs &A, const LvCons &cs, int32_t v) {
+  const int32_t *ofs = cs.kind == kOut ? A.G.gofs_out : A.G.gofs_in;
+  const int64_t at = (int64_t)v * A.G.ncls + cs.cls;
+  const int32_t a = __ldg(ofs + HM_AT(A.G, at, (int64_t)A.G.n * A.G.ncls, kChkGroup));
+  return make_int2(a, __ldg(ofs + at + 1) - a);
 }
 
-template <bool kBatch, bool kShared, bool kRows, bool kSym>
-__device__ __forceinline__ void lv_ranges(const LvArgs &A, LvShared &sm, int p, unsigned long long first,
-                                          unsigned long long cnt, int g) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t chunks = (int64_t)((cnt + 31) >> 5), per = (chunks + gridDim.x - 1) / gridDim.x;
-  const int64_t c0 = min(chunks, (int64_t)blockIdx.x * per), c1 = min(chunks, c0 + per);
-  const int gpc = 32 / g, ngl = (int)(c1 - c0) * gpc;
-  for (int64_t c = c0 + warp; c < c1; c += kLvWarps) {
-    const unsigned long long i = (unsigned long long)c * 32 + lane;
-    int4 r = make_int4(0, 0, 0, 0);
-    bool matched = false;
-    if (i < cnt) {
-      const int64_t s = (int64_t)(first + i);
-      int32_t pid = 0;
-      if (kBatch) pid = p == 2 ? __ldg(A.seed_pid + s) : lv_state(A, p, s)[p];
-      matched = kBatch && A.levels[(int64_t)pid * A.kmax + p].done;
-      if (!matched) r = lv_range<kBatch, kShared, kSym>(A, p, s, pid);
-      else r.w = pid;
-      A.rng[p][i] = r;
-    }
-    if (kBatch && __any_sync(kFull, matched)) {
-      // two-vertex patterns: the validated seed is the match
-      const uint32_t peers = __match_any_sync(kFull, matched ? r.w : -1 - lane);
-      const int leader = __ffs(peers) - 1;
-      unsigned long long at = 0;
-      if (matched && lane == leader) {
-        atomicAdd(A.counts + r.w, (unsigned long long)__popc(peers));
-        if (kRows) at = atomicAdd(A.row_cursor + r.w, (unsigned long long)__popc(peers));
-      }
-      if (kRows) {
-        at = __shfl_sync(kFull, at, leader) + __popc(peers & lanemask_lt());
-        if (matched && at < A.row_cap[r.w]) {
-          const int32_t *mp = lv_state(A, p, (int64_t)(first + i));
-          int32_t *row = A.rows + A.row_off[r.w] + at * 2;
-          const EmitPlan &E = A.emit[r.w];
-          row[E.orig[0]] = mp[0];
-          row[E.orig[1]] = mp[1];
-        }
-      }
-    }
-    unsigned long long t = (unsigned long long)(uint32_t)r.y;
-    for (int o = 1; o < g; o <<= 1) t += __shfl_xor_sync(kFull, t, o);
-    if ((lane & (g - 1)) == 0) sm.sum[(c - c0) * gpc + lane / g] = (t + 31) >> 5;
-  }
-  __syncthreads();
-  // prefix sum over the block's groups
-  constexpr int kPer = kLvMaxGroups / kLvThreads;
-  unsigned long long v[kPer], sum = 0, all;
-#pragma unroll
-  for (int t = 0; t < kPer; ++t) {
-    const int i = threadIdx.x * kPer + t;
-    v[t] = i < ngl ? sm.sum[i] : 0;
-    sum += v[t];
-  }
-  unsigned long long run = lv_block_scan(sum, sm, &all);
-#pragma unroll
-  for (int t = 0; t < kPer; ++t) {
-    const int i = threadIdx.x * kPer + t;
-    if (i < ngl) A.upre[p][c0 * gpc + i] = run;
-    run += v[t];
-  }
-  if (threadIdx.x == 0) A.bsum[p][blockIdx.x] = all;
-}
-
-// Is x among the group's images sorted_seeds[lo, hi).y (ascending)?
-__device__ __forceinline__ bool lv_group_has(const int2 *__restrict__ sv, int32_t lo, int32_t hi, int32_t x) {
-  while (lo < hi) {
-    const int32_t mid = lo + ((hi - lo) >> 1);
-    const int32_t y = __ldg(&sv[mid].y);
-    if (y < x) lo = mid + 1;
-    else if (y > x) hi = mid;
-    else return true;
+// Has u a neighbour that the deferred position 1 (level plan Z) may take?  The
+// search over the other positions would be for nothing.  With arcs in both
+// directions, the filter is asked if the shorter list has at most 8 entries.
+__device__ __forceinline__ bool lv_has_final(const LvArgs &A, const LevelPlan &Z, int32_t u) {
+  if (Z.cons[0].cls < 0) return false;
+  const int2 r = lv_group(A, Z.cons[0], u);
+  if (Z.npos < 2 || r.y == 0) return r.y > 0;
+  if (Z.cons[1].cls < 0) return false;
+  const int2 r1 = lv_group(A, Z.cons[1], u);
+  const bool second = r1.y < r.y;
+  const int2 w = second ? r1 : r;
+  if (w.y > 8) return true;
+  const LvCons &cs = Z.cons[second ? 1 : 0], &other = Z.cons[second ? 0 : 1];
+  const int32_t *list = cs.kind == kOut ? A.G.gout_adj : A.G.gin_adj;
+  Bytes none;
+#pragma unroll 1
+  for (int i = 0; i < w.y; ++i) {
+    const int32_t c = __ldg(list + HM_AT(A.G, (int64_t)w.x + i, A.G.m, kChkList));
+    if (arc_maybe_l<false>(A.G, other.kind == kOut ? u : c, other.kind == kOut ? c : u, other.lab, none)) return true;
   }
   return false;
 }
 
+// The candidates of a state of level p: of the parent at mp (images m) with
+// candidate c at position p - 1.  kClosed: this call only counts, and where the
+// level is closed the matches are added to `found` instead.  The fourth word is
+// not set.
+template <bool kBatch, bool kClosed>
+__device__ __forceinline__ int4 lv_range(const LvArgs &A, int p, const int4 &m, const int32_t *mp, int32_t c,
+                                         int32_t pid, unsigned long long &found) {
+  const LevelPlan &L = kBatch ? A.levels[(int64_t)pid * A.kmax + p] : A.level1[p];
+  const int4 dead = make_int4(0, 0, 0, 0);
+  if (p == 1) {
+    // the vertex validator (Alg. 2; the label is the list's) and a root mask on position 0
+    if (A.root0 && !A.root_mask[c]) return dead;
+    const int2 need = kBatch ? A.deg0[pid] : make_int2(A.dout0, A.din0);
+    const int4 vi = __ldg(&A.G.vi[HM_AT(A.G, c, A.G.n, kChkVertex)]);
+    if (vi.y < need.x || vi.z < need.y) return dead;
+    if (L.final && !lv_has_final(A, kBatch ? A.levels[(int64_t)pid * A.kmax + L.final] : A.level1[L.final], c))
+      return dead;
+  }
+  int32_t best = INT32_MAX, lo = 0, what = 0;
+  for (int j = 0; j < L.npos; ++j) {
+    const LvCons cs = L.cons[j];
+    if (cs.cls < 0) return dead;
+    const int2 r = lv_group(A, cs, cs.q == p - 1 ? c : lv_image(m, mp, cs.q));
+    if (r.y < best) {
+      best = r.y;
+      lo = r.x;
+      what = j | (cs.kind == kOut ? 0 : 1 << 6);
+    }
+  }
+  if (kClosed && L.closed && best > 0) {
+    // every entry of the group that the state does not use already
+    const int32_t *list = lv_list(what) ? A.G.gin_adj : A.G.gout_adj;
+    Bytes none;
+    int used = 0;
+    for (int i = 0; i < p; ++i)
+      if (search_g<false>(A.G, list, lo, best, i == p - 1 ? c : lv_image(m, mp, i), none) >= 0) ++used;
+    found = (unsigned long long)(best - used);
+    best = 0;
+  }
+  return make_int4(lo, best, what | pid << 7, 0);
+}
+
 // The cheap checks: candidate c of the state at mp for position p.
-template <bool kShared, bool kSym>
+template <bool kSym>
 __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan &L, const int32_t *mp, int p,
                                                 int drive, int32_t c, Bytes &none) {
-  const int4 m = lv_images<kShared>(mp, p);
+  const int4 m = lv_images(mp, p);
   if (m.x == c || m.y == c || m.z == c || m.w == c) return false;  // injective
   for (int i = 4; i < p; ++i)
     if (mp[i] == c) return false;
@@ -319,10 +307,9 @@ __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan
 }
 
 // The exact checks of a candidate that passed the cheap ones.
-template <bool kShared>
 __device__ __forceinline__ bool lv_exact_checks(const LvArgs &A, const LevelPlan &L, const int32_t *mp, int p, int drive,
                                                 int32_t c, Bytes &none) {
-  const int4 m = lv_images<kShared>(mp, p);
+  const int4 m = lv_images(mp, p);
   if (L.need_deg) {
     const int4 vi = __ldg(&A.G.vi[HM_AT(A.G, c, A.G.n, kChkVertex)]);
     if (vi.y < L.dout || vi.z < L.din) return false;
@@ -343,28 +330,7 @@ __device__ __forceinline__ bool lv_exact_checks(const LvArgs &A, const LevelPlan
   return true;
 }
 
-// Position 1 chosen from a shared group: v must differ from the match's other
-// images and keep the induced non-arcs.
-__device__ __forceinline__ bool lv_defer_checks(const LvArgs &A, const int32_t *mp, int k, int32_t v, Bytes &none) {
-  for (int i = 0; i < k; ++i)
-    if (i != 1 && mp[i] == v) return false;
-  for (int j = 0; j < A.ndefer; ++j) {
-    const Cons cs = A.defer[j];
-    const int32_t f = mp[cs.q];
-    const bool fwd = cs.kind == kNotOut;  // the forbidden arc is f(q) -> v
-    int32_t lab;
-    if (arc_maybe<false>(A.G, fwd ? f : v, fwd ? v : f, none) && arc_find<false>(A.G, fwd ? f : v, fwd ? v : f, &lab, none))
-      return false;
-  }
-  return true;
-}
-
-__device__ __forceinline__ void lv_write_row(const EmitPlan &E, int32_t *row, const int32_t *mp, int p, int32_t c,
-                                             bool deferred) {
-  if (deferred) {
-    for (int i = 0; i < E.k; ++i) row[E.orig[i]] = i == 1 ? c : mp[i];
-    return;
-  }
+__device__ __forceinline__ void lv_write_row(const EmitPlan &E, int32_t *row, const int32_t *mp, int p, int32_t c) {
   for (int i = 0; i < p; ++i) row[E.orig[i]] = mp[i];
   row[E.orig[p]] = c;
 }
@@ -380,400 +346,497 @@ __device__ __forceinline__ void lv_write_images(const EmitPlan &E, const int8_t 
     }
 }
 
-// Exact checks on the nbuf waiting survivors; those that pass become states of
-// the next level (whose counter stood at sm.made when its buffer was empty) or
-// matches.
-template <bool kRows, bool kBatch, bool kShared, bool kSym>
-__device__ __forceinline__ void lv_drain(const LvArgs &A, LvShared &sm, int p, unsigned long long slice_first,
-                                         int2 *buf, int nbuf, int lane) {
-  Bytes none;
-  const uint32_t lt = lanemask_lt();
-  const bool deferred = kShared && p == A.kmax;
-  int nok = 0;
-  for (int b = 0; b < nbuf; b += 32) {
-    const int e = b + lane;
-    bool ok = false;
-    int2 sc = make_int2(0, 0);
-    if (e < nbuf) {
-      sc = buf[e];
-      const int32_t *mp = lv_state(A, p, (int64_t)(slice_first + (uint32_t)sc.x));
-      if (deferred) {
-        ok = lv_defer_checks(A, mp, p, sc.y, none);
-      } else {
-        const int4 r = A.rng[p][(uint32_t)sc.x];
-        const LevelPlan &L = kBatch ? A.levels[(int64_t)r.w * A.kmax + p] : A.level1[p];
-        ok = lv_exact_checks<kShared>(A, L, mp, p, r.z & 0xff, sc.y, none);
-      }
-    }
-    const uint32_t bal = __ballot_sync(kFull, ok);
-    if (ok) buf[nok + __popc(bal & lt)] = sc;  // at or before the entry just read
-    nok += __popc(bal);
-    __syncwarp();
-  }
-  if (!nok) return;
+// Adds what a warp's lanes found in closed levels to the counts.
+template <bool kBatch, bool kSym>
+__device__ __forceinline__ void lv_add_found(const LvArgs &A, LvShared &sm, unsigned long long found, int32_t pid,
+                                             int lane) {
+  if (!__any_sync(kFull, found != 0)) return;
   if (kBatch) {
-    for (int b = 0; b < nok; b += 32) {
-      const int e = b + lane;
-      const bool valid = e < nok;
-      const int2 sc = valid ? buf[e] : make_int2(0, 0);
-      const int64_t s = (int64_t)(slice_first + (uint32_t)sc.x);
-      const int32_t *mp = lv_state(A, p, s);
-      const int32_t pid = valid ? A.rng[p][(uint32_t)sc.x].w : -1;
-      const bool last = valid && A.levels[(int64_t)pid * A.kmax + p].last;
-      const uint32_t peers = __match_any_sync(kFull, last ? pid : -1 - lane);
-      const int leader = __ffs(peers) - 1;
-      if (last) {
-        const int naut = kSym ? A.emit[pid].naut : 1;
-        unsigned long long at = 0;
-        if (lane == leader) {
-          atomicAdd(A.counts + pid, (unsigned long long)__popc(peers) * naut);
-          if (kRows) at = atomicAdd(A.row_cursor + pid, (unsigned long long)__popc(peers) * naut);
-        }
-        if (kRows) {
-          at = __shfl_sync(peers, at, leader) + (unsigned long long)__popc(peers & lt) * naut;
-          const EmitPlan &E = A.emit[pid];
-          int32_t *rows = A.rows + A.row_off[pid];
-          if (naut > 1) lv_write_images(E, A.aut + E.aut, rows, at, A.row_cap[pid], mp, p, sc.y);
-          else if (at < A.row_cap[pid]) lv_write_row(E, rows + at * E.k, mp, p, sc.y, false);
-        }
-      }
-      const bool inner = valid && !last;
-      const uint32_t bal = __ballot_sync(kFull, inner);
-      if (bal) {
-        unsigned long long at = 0;
-        if (lane == 0) at = atomicAdd(&A.ctl->next_n[p + 1], (unsigned long long)__popc(bal));
-        at = __shfl_sync(kFull, at, 0) - sm.made + __popc(bal & lt);
-        if (inner) {
-          int32_t *dst = const_cast<int32_t *>(lv_state(A, p + 1, (int64_t)at));
-          for (int i = 0; i < p; ++i) dst[i] = mp[i];
-          dst[p] = sc.y;
-          dst[p + 1] = pid;
-        }
-      }
-    }
-    __syncwarp();
-    return;
-  }
-  const bool last = deferred || A.level1[p].last;
-  if (kShared && !deferred && last && !kRows && A.ndefer == 0) {
-    // a count without induced non-arcs: every image of the group that the match does not use
-    unsigned long long add = 0;
-    for (int e = lane; e < nok; e += 32) {
-      const int2 sc = buf[e];
-      const int32_t *mp = lv_state(A, p, (int64_t)(slice_first + (uint32_t)sc.x));
-      const int4 gr = __ldg(A.groups + (p == 2 ? (int64_t)(slice_first + (uint32_t)sc.x) : (int64_t)mp[1]));
-      int used = lv_group_has(A.sorted_seeds, gr.y, gr.z, sc.y) ? 1 : 0;
-      for (int i = 0; i < p; ++i)
-        if (i != 1 && lv_group_has(A.sorted_seeds, gr.y, gr.z, mp[i])) ++used;
-      add += (unsigned long long)(gr.z - gr.y - used);
-    }
-    for (int o = 16; o; o >>= 1) add += __shfl_xor_sync(kFull, add, o);
-    if (lane == 0) sm.count[threadIdx.x >> 5] += add;
-  } else if (last && (!kShared || deferred)) {
-    const int naut = kSym ? A.emit1.naut : 1;
-    if (lane == 0) sm.count[threadIdx.x >> 5] += (unsigned long long)nok * naut;
-    if (kRows) {
-      unsigned long long at = 0;
-      if (lane == 0) at = atomicAdd(&A.ctl->rows, (unsigned long long)nok * naut);
-      at = __shfl_sync(kFull, at, 0);
-      for (int e = lane; e < nok; e += 32) {
-        const int2 sc = buf[e];
-        const int32_t *mp = lv_state(A, p, (int64_t)(slice_first + (uint32_t)sc.x));
-        const unsigned long long r = at + (unsigned long long)e * naut;
-        if (kSym && naut > 1) lv_write_images(A.emit1, A.aut, A.rows, r, A.cap, mp, p, sc.y);
-        else if (r < A.cap) lv_write_row(A.emit1, A.rows + r * A.emit1.k, mp, p, sc.y, deferred);
-      }
-    }
+    if (kSym && found) found *= A.emit[pid].naut;
+    // neighbouring states mostly belong to one pattern: one addition per warp then
+    const int32_t p0 = __shfl_sync(kFull, pid, __ffs(__ballot_sync(kFull, found != 0)) - 1);
+    const bool same = __all_sync(kFull, pid == p0 || !found);
+    unsigned long long all = found;
+    for (int o = 16; o; o >>= 1) all += __shfl_xor_sync(kFull, all, o);
+    if (same ? lane == 0 : found != 0) atomicAdd(A.counts + (same ? p0 : pid), same ? all : found);
   } else {
-    unsigned long long at = 0;
-    if (lane == 0) at = atomicAdd(&A.ctl->next_n[p + 1], (unsigned long long)nok);
-    at = __shfl_sync(kFull, at, 0) - sm.made;
-    for (int e = lane; e < nok; e += 32) {
-      const int2 sc = buf[e];
-      const int64_t s = (int64_t)(slice_first + (uint32_t)sc.x);
-      const int32_t *mp = lv_state(A, p, s);
-      int32_t *dst = const_cast<int32_t *>(lv_state(A, p + 1, (int64_t)(at + e)));
-      if (p <= 3) {
-        int4 v = make_int4(mp[0], mp[1], 0, 0);
-        if (kShared && p == 2) v.y = (int32_t)s;  // the group, in the place of position 1's image
-        if (p == 3) v.z = mp[2];
-        if (p == 2) v.z = sc.y; else v.w = sc.y;
+    for (int o = 16; o; o >>= 1) found += __shfl_xor_sync(kFull, found, o);
+    if (lane == 0) sm.count[threadIdx.x >> 5] += kSym ? found * A.emit1.naut : found;
+  }
+}
+
+// The warp's n (at most 64) new states to level p: fresh[] holds their ranges and
+// parents, buf[].y the candidates at position p - 1.  False: no room.
+__device__ __noinline__ bool lv_append(const LvArgs &A, LvShared &sm, int p, const int4 *fresh, const int2 *buf,
+                                          int n, int lane) {
+  // chunks of the first and of the second group
+  unsigned long long t0 = lane < n ? (uint32_t)fresh[lane].y : 0, t1 = lane + 32 < n ? (uint32_t)fresh[lane + 32].y : 0;
+  for (int o = 16; o; o >>= 1) {
+    t0 += __shfl_xor_sync(kFull, t0, o);
+    t1 += __shfl_xor_sync(kFull, t1, o);
+  }
+  t0 = (t0 + 31) >> 5;
+  t1 = (t1 + 31) >> 5;
+  const int ng = n > 32 ? 2 : 1;
+  const unsigned long long add = ((unsigned long long)ng << kLvChunkBits) + t0 + t1;
+  unsigned long long at = 0;
+  int fits = 0;
+  if (lane == 0) {
+    at = atomicAdd(sm.made, add);
+    fits = (at >> kLvChunkBits) + ng <= A.gcap[p];
+    // taken back, so the groups that were given stay without gaps: whoever adds
+    // in between sees an even fuller level and takes back too
+    if (!fits) atomicAdd(sm.made, 0ull - add);
+  }
+  if (!__shfl_sync(kFull, fits, 0)) return false;
+  at = __shfl_sync(kFull, at, 0);
+  const uint32_t g0 = (uint32_t)(at >> kLvChunkBits);
+  const unsigned long long chunk = at & kLvChunkMask;
+  if (lane < ng) {
+    LvGroup g;
+    g.start = lane ? chunk + t0 : chunk;
+    g.n = lane ? n - 32 : min(n, 32);
+    g.pad = 0;
+    A.grp[p][g0 + lane] = g;
+  }
+  for (int e = lane; e < n; e += 32) {
+    const uint64_t slot = (uint64_t)g0 * 32 + e;
+    const int4 f = fresh[e];
+    const int32_t c = buf[e].y;
+    A.rng[p][slot] = make_int4(f.x, f.y, f.z, 0);
+    int32_t *dst = A.base[p] + slot * (uint32_t)A.stride[p];
+    if (p == 1) {
+      dst[0] = c;
+    } else {
+      const int32_t *mp = A.base[p - 1] + (uint64_t)(uint32_t)f.w * (uint32_t)A.stride[p - 1];
+      if (p == 2) {
+        *reinterpret_cast<int2 *>(dst) = make_int2(mp[0], c);
+      } else if (p <= 4) {
+        int4 v = lv_images(mp, p - 1);
+        if (p == 3) v.z = c; else v.w = c;
         *reinterpret_cast<int4 *>(dst) = v;
       } else {
-        for (int i = 0; i < p; ++i) dst[i] = mp[i];
-        dst[p] = sc.y;
+        for (int i = 0; i < p - 1; ++i) dst[i] = mp[i];
+        dst[p - 1] = c;
       }
     }
   }
   __syncwarp();
+  return true;
+}
+
+// Exact checks on the nbuf waiting survivors of level p (verified: they passed
+// them before); those that pass become matches, or states of the next level.
+// Returns how many states wait in buf because the next level is full (0: none).
+template <bool kRows, bool kBatch, bool kSym>
+__device__ __forceinline__ int lv_drain(const LvArgs &A, LvShared &sm, int p, int2 *buf, int nbuf, bool verified,
+                                        int lane) {
+  Bytes none;
+  const uint32_t lt = lanemask_lt();
+  const int warp = threadIdx.x >> 5;
+  int4 *fresh = sm.fresh[warp];
+  int done = 0;  // entries [0, done) of buf: states of the next level, their ranges in fresh
+  const bool all_last = !kBatch && A.level1[p].last;
+  for (int b = 0; b < nbuf; b += 32) {
+    const int e = b + lane;
+    bool ok = false;
+    int2 sc = make_int2(0, 0);
+    int32_t pid = 0;
+    const int32_t *mp = nullptr;
+    if (e < nbuf) {
+      sc = buf[e];
+      const int4 r = A.rng[p][(uint32_t)sc.x];
+      pid = lv_pid(r.z);
+      mp = A.base[p] + (uint64_t)(uint32_t)sc.x * (uint32_t)A.stride[p];
+      ok = verified ||
+           lv_exact_checks(A, kBatch ? A.levels[(int64_t)pid * A.kmax + p] : A.level1[p], mp, p, lv_drive(r.z), sc.y,
+                           none);
+    }
+    if (kBatch ? true : all_last) {
+      const bool last = kBatch ? ok && A.levels[(int64_t)pid * A.kmax + p].last : ok;
+      const uint32_t bal = __ballot_sync(kFull, last);
+      if (bal) {
+        if (kBatch) {
+          const uint32_t peers = __match_any_sync(kFull, last ? pid : -1 - lane);
+          const int leader = __ffs(peers) - 1;
+          if (last) {
+            const int naut = kSym ? A.emit[pid].naut : 1;
+            unsigned long long at = 0;
+            if (lane == leader) {
+              atomicAdd(A.counts + pid, (unsigned long long)__popc(peers) * naut);
+              if (kRows) at = atomicAdd(A.row_cursor + pid, (unsigned long long)__popc(peers) * naut);
+            }
+            if (kRows) {
+              at = __shfl_sync(peers, at, leader) + (unsigned long long)__popc(peers & lt) * naut;
+              const EmitPlan &E = A.emit[pid];
+              int32_t *rows = A.rows + A.row_off[pid];
+              if (naut > 1) lv_write_images(E, A.aut + E.aut, rows, at, A.row_cap[pid], mp, p, sc.y);
+              else if (at < A.row_cap[pid]) lv_write_row(E, rows + at * E.k, mp, p, sc.y);
+            }
+          }
+        } else {
+          const int naut = kSym ? A.emit1.naut : 1;
+          if (lane == 0) sm.count[warp] += (unsigned long long)__popc(bal) * naut;
+          if (kRows) {
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(&A.ctl->rows, (unsigned long long)__popc(bal) * naut);
+            at = __shfl_sync(kFull, at, 0) + (unsigned long long)__popc(bal & lt) * naut;
+            if (last) {
+              if (kSym && naut > 1) lv_write_images(A.emit1, A.aut, A.rows, at, A.cap, mp, p, sc.y);
+              else if (at < A.cap) lv_write_row(A.emit1, A.rows + at * A.emit1.k, mp, p, sc.y);
+            }
+          }
+        }
+      }
+      ok = ok && !last;
+    }
+    if (all_last) continue;
+    // the range of the new state
+    int4 r = make_int4(0, 0, 0, 0);
+    unsigned long long found = 0;
+    if (ok) r = lv_range<kBatch, !kRows>(A, p + 1, lv_images(mp, p), mp, sc.y, pid, found);
+    if (p == 1 && !verified) {
+      const uint32_t made = __popc(__ballot_sync(kFull, ok));
+      if (lane == 0) sm.injected[warp] += made;
+    }
+    if (!kRows) lv_add_found<kBatch, kSym>(A, sm, found, pid, lane);
+    const uint32_t bal = __ballot_sync(kFull, r.y > 0);
+    if (r.y > 0) {
+      const int at = done + __popc(bal & lt);  // at or before the entry just read
+      r.w = sc.x;
+      buf[at] = sc;
+      fresh[at] = r;
+    }
+    done += __popc(bal);
+    __syncwarp();
+  }
+  if (!done) return 0;
+  if (lv_append(A, sm, p + 1, fresh, buf, done, lane)) return 0;
+  return done;
+}
+
+// The vertices [v0, v0 + cnt) of the first level's list, those with candidates, to level 1.
+template <bool kRows, bool kBatch, bool kSym>
+__device__ __forceinline__ void lv_fill(const LvArgs &A, LvShared &sm, unsigned long long v0, unsigned long long cnt,
+                                        uint32_t me) {
+  if (me >= A.fill_warps) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t lt = lanemask_lt();
+  int4 *fresh = sm.fresh[warp];
+  int2 *buf = sm.buf[warp];
+  // each warp an equal piece of the list, so that its groups hold neighbours
+  const unsigned long long chunks = (cnt + 31) >> 5;
+  const unsigned long long a = chunks * me / A.fill_warps, b = chunks * (me + 1) / A.fill_warps;
+  int n = 0;
+  for (unsigned long long ch = a; ch < b; ++ch) {
+    const unsigned long long i = ch * 32 + lane;
+    int4 r = make_int4(0, 0, 0, 0);
+    unsigned long long found = 0;
+    int32_t pid = 0, u = 0;
+    if (i < cnt) {
+      const unsigned long long s = v0 + i;
+      if (kBatch) {
+        int32_t lo = 0, hi = A.npat - 1;  // the last pattern whose first vertex is at or before the chunk's
+        while (lo < hi) {
+          const int32_t mid = (lo + hi + 1) >> 1;
+          if (__ldg(A.vert_n + mid) <= v0 + ch * 32) lo = mid; else hi = mid - 1;
+        }
+        pid = lo;
+        while (__ldg(A.vert_n + pid + 1) <= s) ++pid;
+        u = __ldg(A.vert_at[pid] + s);
+      } else {
+        u = __ldg(A.vert + s);
+      }
+      r = lv_range<kBatch, !kRows>(A, 1, make_int4(0, 0, 0, 0), nullptr, u, pid, found);
+    }
+    if (!kRows) lv_add_found<kBatch, kSym>(A, sm, found, pid, lane);
+    const uint32_t bal = __ballot_sync(kFull, r.y > 0);
+    if (r.y > 0) {
+      const int at = n + __popc(bal & lt);
+      fresh[at] = r;
+      buf[at] = make_int2(0, u);
+    }
+    n += __popc(bal);
+    __syncwarp();
+    if (n >= 32) {  // one full group; the rest moves down
+      if (!lv_append(A, sm, 1, fresh, buf, 32, lane)) break;
+      const int4 f = fresh[32 + lane];
+      const int2 v = buf[32 + lane];
+      __syncwarp();
+      n -= 32;
+      if (lane < n) {
+        fresh[lane] = f;
+        buf[lane] = v;
+      }
+      __syncwarp();
+    }
+  }
+  // the slice is so small that its groups fit
+  if (n && !lv_append(A, sm, 1, fresh, buf, n, lane) && lane == 0) atomicCAS(&A.ctl->status, 0, kStatQueue);
 }
 
 // The group that chunk x of the level lies in: the last one whose first chunk
-// is at or before x.  Returns its number in the slice; *start is that first
-// chunk.  `gi` is the group of the chunk before x, in the block's groups that
-// begin at chunk `b0` and end at group `b1` (b1 = 0: none): mostly x lies
-// in one of the 32 groups after it, which takes one load; otherwise the block
-// is searched for in shared memory and the group in two loads.
-__device__ __forceinline__ uint32_t lv_locate(const LvArgs &A, const LvShared &sm, int p, unsigned long long x,
-                                              uint32_t ngroups, uint32_t per_groups, int lane, uint32_t gi,
-                                              unsigned long long &b0, uint32_t &b1, unsigned long long *start) {
-  const unsigned long long *up = A.upre[p];
-  if (b1) {
+// is at or before x.  `gi` is the group of the chunk before x (or none, ~0u):
+// mostly x lies in one of the 32 groups after it, which takes one load.
+__device__ __forceinline__ uint32_t lv_locate(const LvGroup *grp, uint32_t ngroup, unsigned long long x, int lane,
+                                              uint32_t gi) {
+  if (gi != ~0u) {
     const uint32_t i = gi + 1 + lane;
-    const unsigned long long u = i < b1 ? up[i] : ~0ull;
-    const uint32_t le = __ballot_sync(kFull, u <= x - b0);
-    // the last of them starts at or before x: it is the group unless all 32 do or the block ends there
-    if (le && le != kFull && gi + 1 + __popc(le) < b1) {
-      const int at = 31 - __clz(le);
-      *start = b0 + __shfl_sync(kFull, u, at);
-      return gi + 1 + at;
-    }
+    const uint32_t le = __ballot_sync(kFull, i < ngroup && grp[i].start <= x);
+    if (le && le != kFull) return gi + 32 - __clz(le);
   }
-  int lo = 0, hi = (int)gridDim.x - 1;  // the last block whose first chunk is <= x
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (sm.first[mid] <= x) lo = mid; else hi = mid - 1;
-  }
-  b0 = sm.first[lo];
-  uint32_t a = (uint32_t)lo * per_groups, n = min(per_groups, ngroups - a);  // groups [a, a + n)
-  b1 = a + n;
+  uint32_t a = 0, n = ngroup;  // groups [a, a + n); the first starts at or before x
   while (n > 1) {
     const uint32_t step = (n + 31) >> 5;
     const uint32_t i = (uint32_t)lane * step;
-    const bool le = i < n && up[a + i] <= x - b0;
-    const uint32_t at = (31 - __clz(__ballot_sync(kFull, le))) * step;  // lane 0 always holds
+    const uint32_t at = (31 - __clz(__ballot_sync(kFull, i < n && grp[a + i].start <= x))) * step;
     a += at;
     n = min(step, n - at);
   }
-  *start = b0 + up[a];
   return a;
 }
 
-// The expansion of the level's chunks [sm.begin, sm.begin + sm.take) by this
-// warp: run `run` of sm.nrun, then runs claimed from the level's counter.
-// Returns the number of chunks it took.
-template <bool kRows, bool kBatch, bool kShared, bool kSym>
-__device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int p, unsigned long long first,
-                                              unsigned long long cnt, int g, uint32_t run) {
+// The expansion of a level by this warp: its own first run of chunks and then
+// runs claimed from the level's counter, or (resume) what it left when the next
+// level was full.  Returns the number of chunks it took.
+template <bool kRows, bool kBatch, bool kSym>
+__device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int p, bool resume, uint32_t me) {
   Bytes none;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = lanemask_lt();
   int4 *rec = sm.rec[warp];
   int2 *buf = sm.buf[warp];
-  const int64_t chunks = (int64_t)((cnt + 31) >> 5), per = (chunks + gridDim.x - 1) / gridDim.x;
-  const uint32_t per_groups = (uint32_t)(per * (32 / g)), ngroups = (uint32_t)(chunks * (32 / g));
-  uint32_t gi = 0, b1 = 0;
-  unsigned long long b0 = 0;
-  const bool deferred = kShared && p == A.kmax;
-  const int32_t *states = A.base[p] + first * A.stride[p];
-  int nbuf = 0;
-  uint32_t look = 0;
-  while (run < sm.nrun) {
-    unsigned long long x = sm.begin + (unsigned long long)run * sm.run_len;
-    uint32_t left = (uint32_t)min((unsigned long long)sm.run_len, sm.take - (unsigned long long)run * sm.run_len);
-    // the next run, claimed early so that its number is there when this one is done
-    if (lane == 0) run = atomicAdd(sm.claim, 1u);
-    b1 = 0;
-    while (left) {
-      unsigned long long start;
-      gi = lv_locate(A, sm, p, x, ngroups, per_groups, lane, gi, b0, b1, &start);
-      // the group's states that have candidates, in order, to shared memory
-      const unsigned long long i = (unsigned long long)gi * g + lane;
-      int4 r = make_int4(0, 0, 0, 0);
-      if (lane < g && i < cnt) r = A.rng[p][i];
-      const uint32_t have = __ballot_sync(kFull, r.y > 0);
-      uint32_t incl = (uint32_t)r.y;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const uint32_t total = __shfl_sync(kFull, incl, 31);
-      const uint32_t excl = r.y > 0 ? incl - (uint32_t)r.y : 0xffffffffu;
-      if (r.y > 0) rec[__popc(have & lt)] = make_int4((int32_t)((uint32_t)r.x - excl), r.z, (int32_t)i, r.w);
+  const LvGroup *grp = A.grp[p];
+  uint32_t run = me, look = 0, left = 0;
+  unsigned long long x = 0;
+  int nbuf = 0, wait = 0;
+  const bool inner = p + 1 < A.kmax;
+  bool stop_here = false;  // another warp found the next level full
+  unsigned int full = 0;
+  if (resume) {
+    LvPause &P = A.pause[p][me];
+    if (!P.on) return 0;
+    x = P.x;
+    left = P.left;
+    run = P.run;
+    wait = P.nwait;
+    nbuf = P.nbuf;
+    for (int e = lane; e < wait + nbuf; e += 32) buf[e] = P.buf[e];
+    __syncwarp();
+    const int first = wait;
+    wait = lv_drain<kRows, kBatch, kSym>(A, sm, p, buf, wait, true, lane);
+    if (!wait) {
+      int2 v = make_int2(0, 0);
+      if (lane < nbuf) v = buf[first + lane];
       __syncwarp();
-      uint32_t pos0 = (uint32_t)(x - start) << 5;
-      if (x - start >= ((unsigned long long)total + 31) >> 5) {
-        // cannot happen (the ranges phase counted the same chunks); never spin
-        if (lane == 0) atomicCAS(&A.ctl->status, 0, kStatQueue);
-        return look;
-      }
-      const uint32_t n = min(left, ((total - 1) >> 5) + 1 - (pos0 >> 5));  // chunks of this group
-      left -= n;
-      x += n;
-      for (uint32_t c0 = 0; c0 < n; ++c0, pos0 += 32) {
-        if ((++look & 31u) == 0) {
-          int stop = 0;
-          if (lane == 0) {
-            if (*(volatile int32_t *)&A.ctl->status != 0) stop = 1;
-            else if (globaltimer_ns() > sm.deadline) {
-              atomicCAS(&A.ctl->status, 0, kStatBudget);
-              stop = 1;
-            }
-          }
-          if (__shfl_sync(kFull, stop, 0)) return look;
-        }
-        // the owner of position pos0 + lane: states that start at or before pos0, then the starts inside the chunk
-        const uint32_t rel = excl - pos0;
-        const uint32_t starts = __reduce_or_sync(kFull, r.y > 0 && excl > pos0 && rel < 32 ? 1u << rel : 0u);
-        const int before = __popc(__ballot_sync(kFull, excl <= pos0 && r.y > 0)) - 1;
-        const int ow = before + __popc(starts & (lt | (1u << lane)));
-        bool ok = false;
-        int32_t c = 0, s = 0;
-        if (total - pos0 > (uint32_t)lane) {
-          const int4 o = rec[ow];
-          s = o.z;
-          const uint32_t at = (uint32_t)o.x + pos0 + lane;
-          const int list = o.y >> 8;
-          if (kShared && list == 2)
-            c = __ldg(&A.sorted_seeds[at].y);
-          else
-            c = __ldg((list ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
-          if (deferred) {
-            ok = true;
-          } else {
-            const LevelPlan &L = kBatch ? A.levels[(int64_t)o.w * A.kmax + p] : A.level1[p];
-            ok = lv_first_checks<kShared, kSym>(A, L, states + (uint64_t)(uint32_t)s * (uint32_t)A.stride[p], p,
-                                                o.y & 0xff, c, none);
-          }
-        }
-        const uint32_t bal = __ballot_sync(kFull, ok);
-        if (ok) buf[nbuf + __popc(bal & lt)] = make_int2(s, c);
-        nbuf += __popc(bal);
-        __syncwarp();
-        if (nbuf >= kLvDrain) {
-          lv_drain<kRows, kBatch, kShared, kSym>(A, sm, p, first, buf, nbuf, lane);
-          nbuf = 0;
-        }
-      }
-      __syncwarp();  // every lane is done with rec
+      if (lane < nbuf) buf[lane] = v;
+      __syncwarp();
     }
-    run = gridDim.x * kLvWarps + __shfl_sync(kFull, run, 0);
+  } else {
+    if (run < sm.nrun) {
+      x = (unsigned long long)run * sm.run_len;
+      left = (uint32_t)min((unsigned long long)sm.run_len, sm.total - x);
+      // the next run, claimed early so that its number is there when this one is done
+      if (lane == 0) run = gridDim.x * kLvWarps + atomicAdd(sm.claim, 1u);
+    }
   }
-  if (nbuf) lv_drain<kRows, kBatch, kShared, kSym>(A, sm, p, first, buf, nbuf, lane);
+  uint32_t gi = ~0u;
+  while (!wait && !stop_here) {
+    if (!left) {
+      run = __shfl_sync(kFull, run, 0);
+      if (run >= sm.nrun) break;
+      x = (unsigned long long)run * sm.run_len;
+      left = (uint32_t)min((unsigned long long)sm.run_len, sm.total - x);
+      if (lane == 0) run = gridDim.x * kLvWarps + atomicAdd(sm.claim, 1u);
+      gi = ~0u;
+    }
+    gi = lv_locate(grp, sm.ngroup, x, lane, gi);
+    // the group's states to shared memory
+    const LvGroup G = grp[gi];
+    int4 r = make_int4(0, 0, 0, 0);
+    if (lane < (int)G.n) r = A.rng[p][(uint64_t)gi * 32 + lane];
+    uint32_t incl = (uint32_t)r.y;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const uint32_t total = __shfl_sync(kFull, incl, 31);
+    const uint32_t excl = r.y > 0 ? incl - (uint32_t)r.y : 0xffffffffu;
+    rec[lane] = make_int4((int32_t)((uint32_t)r.x - excl), r.z, 0, 0);
+    __syncwarp();
+    if (x < G.start || x - G.start >= ((unsigned long long)total + 31) >> 5) {
+      // cannot happen (the group's chunks were counted from the same numbers); never spin
+      if (lane == 0) atomicCAS(&A.ctl->status, 0, kStatQueue);
+      return look;
+    }
+    uint32_t pos0 = (uint32_t)(x - G.start) << 5;
+    uint32_t n = min(left, ((total - 1) >> 5) + 1 - (pos0 >> 5));  // chunks of this group
+    for (; n && !wait && !stop_here; --n, --left, ++x, pos0 += 32) {
+      // (read four chunks before it is asked, so that nothing waits for it)
+      if (inner && (look & 7u) == 0 && lane == 0) full = *(volatile unsigned int *)sm.paused;
+      if (inner && (look & 7u) == 4u) stop_here = __shfl_sync(kFull, full, 0) != 0;
+      if ((++look & 31u) == 0) {
+        int stop = 0;
+        if (lane == 0) {
+          if (*(volatile int32_t *)&A.ctl->status != 0) stop = 1;
+          else if (globaltimer_ns() > sm.deadline) {
+            atomicCAS(&A.ctl->status, 0, kStatBudget);
+            stop = 1;
+          }
+        }
+        if (__shfl_sync(kFull, stop, 0)) return look;
+      }
+      // the owner of position pos0 + lane: states that start at or before pos0, then the starts inside the chunk
+      const uint32_t rel = excl - pos0;
+      const uint32_t starts = __reduce_or_sync(kFull, r.y > 0 && excl > pos0 && rel < 32 ? 1u << rel : 0u);
+      const int before = __popc(__ballot_sync(kFull, excl <= pos0 && r.y > 0)) - 1;
+      const int ow = before + __popc(starts & (lt | (1u << lane)));
+      bool ok = false;
+      int32_t c = 0;
+      if (total - pos0 > (uint32_t)lane) {
+        const int4 o = rec[ow];
+        const uint32_t at = (uint32_t)o.x + pos0 + lane;
+        c = __ldg((lv_list(o.y) ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
+        const LevelPlan &L = kBatch ? A.levels[(int64_t)lv_pid(o.y) * A.kmax + p] : A.level1[p];
+        const int32_t *mp = A.base[p] + ((uint64_t)gi * 32 + ow) * (uint32_t)A.stride[p];
+        ok = lv_first_checks<kSym>(A, L, mp, p, lv_drive(o.y), c, none);
+      }
+      const uint32_t bal = __ballot_sync(kFull, ok);
+      if (ok) buf[nbuf + __popc(bal & lt)] = make_int2((int32_t)(gi * 32 + ow), c);
+      nbuf += __popc(bal);
+      __syncwarp();
+      if (nbuf >= kLvDrain) {
+        // the first 64; the rest moves down
+        wait = lv_drain<kRows, kBatch, kSym>(A, sm, p, buf, kLvDrain, false, lane);
+        const int more = nbuf - kLvDrain;
+        int2 v = make_int2(0, 0);
+        if (lane < more) v = buf[kLvDrain + lane];
+        __syncwarp();
+        if (lane < more) buf[wait + lane] = v;  // behind the states that wait for room, if any
+        nbuf = more;
+        __syncwarp();
+      }
+    }
+    __syncwarp();  // every lane is done with rec
+  }
+  if (!wait && !stop_here && nbuf) {
+    wait = lv_drain<kRows, kBatch, kSym>(A, sm, p, buf, nbuf, false, lane);
+    nbuf = 0;
+  }
+  if (inner) {
+    LvPause &P = A.pause[p][me];
+    if (wait || stop_here) {
+      for (int e = lane; e < wait + nbuf; e += 32) P.buf[e] = buf[e];
+      if (lane == 0) {
+        P.x = x;
+        P.left = left;
+        P.run = run;
+        P.nwait = wait;
+        P.nbuf = nbuf;
+        atomicAdd(sm.paused, 1u);
+      }
+    }
+    if (lane == 0) P.on = wait || stop_here ? 1 : 0;
+  }
   return look;
 }
 
-template <bool kRows, bool kBatch, bool kShared, bool kSym>
+template <bool kRows, bool kBatch, bool kSym>
 __global__ void __launch_bounds__(kLvThreads, kLvMinBlocks) k_levels(const __grid_constant__ LvArgs A) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   LvShared &sm = *reinterpret_cast<LvShared *>(s_raw);
-  const unsigned long long warps = (unsigned long long)gridDim.x * kLvWarps;
-  const uint32_t me = blockIdx.x * kLvWarps + (threadIdx.x >> 5);
-  const int last = kShared && (kRows || A.ndefer) ? A.kmax : A.kmax - 1;  // the deepest level
-  const unsigned long long nseeds = *A.nseeds;
-  if ((threadIdx.x & 31) == 0) sm.count[threadIdx.x >> 5] = 0;
+  const uint32_t warps = gridDim.x * kLvWarps, me = blockIdx.x * kLvWarps + (threadIdx.x >> 5);
+  const int last = A.kmax - 1;  // the deepest level
+  if ((threadIdx.x & 31) == 0) sm.count[threadIdx.x >> 5] = sm.injected[threadIdx.x >> 5] = 0;
   if (threadIdx.x == 0) sm.deadline = globaltimer_ns() + A.budget_ns;
-  __syncthreads();
   unsigned long long my_chunks = 0, cursor = 0;
-  unsigned int target = 0, turn = 0;
-  // the levels being worked on: states [first, first + n) and chunks [done, total)
-  unsigned long long first = 0;
-  unsigned long long n[kMaxK + 2], done[kMaxK + 2], total[kMaxK + 2];
-  unsigned long long made[kMaxK + 2];  // states each level's counter had counted when last read
-  for (int i = 0; i < kMaxK + 2; ++i) made[i] = 0;
-  int p = 1;
-  bool ok = true;
-  while (ok) {
-    if (p == 1) {  // the next slice of depth-2 states
-      if (cursor >= nseeds) break;
-      p = 2;
-      first = cursor;
-      n[2] = min((unsigned long long)A.slice, nseeds - cursor);
-      cursor += n[2];
-    } else if (done[p] < total[p]) {
-      // expand as many chunks as the next level can hold survivors of
-      const unsigned long long left = total[p] - done[p];
-      const unsigned long long take = p < last ? min(left, (unsigned long long)(A.fcap >> 5)) : left;
-      // runs of chunks: the first is the warp's own, the rest are claimed, so that
-      // warps with cheap chunks (lists in cache) take more of them
-      if (threadIdx.x == 0) {
-        const unsigned long long run = max(take / (warps * 8), 1ull);
-        sm.begin = done[p];
-        sm.take = take;
-        sm.run_len = (uint32_t)min(run, 1ull << 31);
-        sm.nrun = (uint32_t)((take + sm.run_len - 1) / sm.run_len);
-        sm.made = made[p + 1];
-        sm.claim = &A.ctl->claim[turn % 3];
-        if (blockIdx.x == 0) A.ctl->claim[(turn + 1) % 3] = 0;  // read two expansions ago
+  unsigned int target = 0, phase = 0;
+  // each level: which filling of it this is, its groups and chunks, whether warps paused in it
+  uint32_t fill[kMaxK + 1];
+  unsigned long long made[kMaxK + 1];
+  bool open[kMaxK + 1], begun[kMaxK + 1];
+  for (int i = 0; i <= kMaxK; ++i) {
+    fill[i] = 0;
+    open[i] = false;
+  }
+  int p = 0;
+  for (;;) {
+    // what this phase fills is level p + 1
+    if (p == 0 && cursor >= A.nvert) break;
+    if (p < last) ++fill[p + 1];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (p < last) {
+        sm.made = &A.ctl->made[p + 1][fill[p + 1] % 3];
+        if (blockIdx.x == 0) {
+          A.ctl->made[p + 1][(fill[p + 1] + 1) % 3] = 0;
+          A.ctl->claim[p + 1][(fill[p + 1] + 1) % 3] = 0;
+        }
       }
-      ++turn;
-      __syncthreads();
-      my_chunks += lv_expand<kRows, kBatch, kShared, kSym>(A, sm, p, p == 2 ? first : 0, n[p],
-                                                           lv_group_size(n[p], warps, A.G.maxdeg), me);
-      done[p] += take;
-      if (p == last && done[p] == total[p]) {  // nothing below: up again, past levels that are done too
-        while (p > 1 && done[p] == total[p]) --p;
-        if (p == 1 && cursor >= nseeds) break;
-        // the next step overwrites buffers that other warps may still read
-        target += gridDim.x;
-        ok = lv_barrier(A, sm, target);
-        if (p > 1) goto reload;
-        continue;
+      if (p > 0) {
+        sm.total = made[p] & kLvChunkMask;
+        sm.ngroup = (uint32_t)(made[p] >> kLvChunkBits);
+        sm.run_len = (uint32_t)min(max(sm.total / (warps * 8ull), 1ull), 1ull << 30);
+        sm.nrun = (uint32_t)((sm.total + sm.run_len - 1) / sm.run_len);
+        sm.claim = &A.ctl->claim[p][fill[p] % 3];
+        sm.paused = &A.ctl->paused[phase % 3];
+        if (blockIdx.x == 0) A.ctl->paused[(phase + 1) % 3] = 0;
       }
-      target += gridDim.x;
-      if (!(ok = lv_barrier(A, sm, target))) break;
-      if (p == last) continue;
-      const unsigned long long now = *(volatile unsigned long long *)&A.ctl->next_n[p + 1];
-      const unsigned long long fresh = now - made[p + 1];
-      made[p + 1] = now;
-      if (fresh == 0) {
-        // another block may not have read the counter yet that the next expansion adds to
-        target += gridDim.x;
-        if (!(ok = lv_barrier(A, sm, target))) break;
-        if (done[p] < total[p]) continue;
-        while (p > 1 && done[p] == total[p]) --p;
-        if (p > 1) goto reload;
-        continue;
-      }
-      ++p;
-      n[p] = fresh;
+    }
+    __syncthreads();
+    if (p == 0) {
+      const unsigned long long n = min(A.slice, A.nvert - cursor);
+      lv_fill<kRows, kBatch, kSym>(A, sm, cursor, n, me);
+      cursor += n;
     } else {
-      while (p > 1 && done[p] == total[p]) --p;
-      if (p > 1) goto reload;
-      continue;
+      my_chunks += lv_expand<kRows, kBatch, kSym>(A, sm, p, begun[p], me);
+      begun[p] = true;
     }
-    // the ranges of the new states
-    lv_ranges<kBatch, kShared, kRows, kSym>(A, sm, p, p == 2 ? first : 0, n[p], lv_group_size(n[p], warps, A.G.maxdeg));
+    if (p == last) {  // does anything follow?
+      bool more = cursor < A.nvert;
+      for (int q = 1; q < last; ++q) more |= open[q];
+      if (!more) break;
+    }
     target += gridDim.x;
-    if (!(ok = lv_barrier(A, sm, target))) break;
-    done[p] = 0;
-  reload: {
-      // the first chunk of each block's groups at this level
-      unsigned long long all = 0, run = 0;
-      for (int b = 0; b < (int)gridDim.x; b += kLvThreads) {
-        const int i = b + threadIdx.x;
-        const unsigned long long v = i < (int)gridDim.x ? __ldcg(A.bsum[p] + i) : 0;
-        const unsigned long long at = lv_block_scan(v, sm, &all);
-        if (i < (int)gridDim.x) sm.first[i] = run + at;
-        run += all;
-      }
-      total[p] = run;
-      __syncthreads();
+    if (!lv_barrier(A, sm, target)) break;
+    if (p > 0) {
+      open[p] = p < last && *(volatile unsigned int *)&A.ctl->paused[phase % 3] != 0;
+      ++phase;
     }
+    if (p < last) {
+      const unsigned long long m = *(volatile unsigned long long *)&A.ctl->made[p + 1][fill[p + 1] % 3];
+      if (m & kLvChunkMask) {
+        ++p;
+        made[p] = m;
+        begun[p] = false;
+        continue;
+      }
+    }
+    while (p > 0 && !open[p]) --p;
   }
   if ((threadIdx.x & 31) == 0) {
     const unsigned long long count = sm.count[threadIdx.x >> 5];
     if (count) atomicAdd(&A.ctl->count, count);
     if (my_chunks) atomicAdd(&A.ctl->chunks, my_chunks);
+    if (sm.injected[threadIdx.x >> 5]) atomicAdd(&A.ctl->injected, (unsigned long long)sm.injected[threadIdx.x >> 5]);
   }
 }
 
 using LvKernel = void (*)(LvArgs);
 
-LvKernel lv_kernel(bool rows, bool batch, bool shared, bool sym) {
+LvKernel lv_kernel(bool rows, bool batch, bool sym) {
   if (batch) {
-    if (sym) return rows ? k_levels<true, true, false, true> : k_levels<false, true, false, true>;
-    return rows ? k_levels<true, true, false, false> : k_levels<false, true, false, false>;
+    if (sym) return rows ? k_levels<true, true, true> : k_levels<false, true, true>;
+    return rows ? k_levels<true, true, false> : k_levels<false, true, false>;
   }
-  if (shared) return rows ? k_levels<true, false, true, false> : k_levels<false, false, true, false>;
-  if (sym) return rows ? k_levels<true, false, false, true> : k_levels<false, false, false, true>;
-  return rows ? k_levels<true, false, false, false> : k_levels<false, false, false, false>;
+  if (sym) return rows ? k_levels<true, false, true> : k_levels<false, false, true>;
+  return rows ? k_levels<true, false, false> : k_levels<false, false, false>;
 }
 
 // Resident blocks of a variant (0: the device cannot run it).
 int lv_grid(LvKernel f, int slot) {
-  static std::atomic<int> cache[16];
+  static std::atomic<int> cache[8];
   int v = cache[slot].load(std::memory_order_relaxed);
   if (!v) {
     int per_sm = 0, coop = 0, dev = 0;
@@ -783,7 +846,7 @@ int lv_grid(LvKernel f, int slot) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kLvThreads, sizeof(LvShared)) != cudaSuccess)
       per_sm = 0;
     (void)cudaGetLastError();
-    v = per_sm > 0 ? std::min(per_sm * num_sms(), kLvMaxGrid) : -1;
+    v = per_sm > 0 ? per_sm * num_sms() : -1;
     cache[slot].store(v, std::memory_order_relaxed);
   }
   return std::max(v, 0);
@@ -795,24 +858,103 @@ int16_t lv_class(const hm_graph *g, int32_t alab, int32_t vlab) {
   return (int16_t)(a * g->nvl + v);
 }
 
-void lv_level(const hm_graph *g, const Plan &P, int p, LevelPlan &L) {
+// The conditions of position p towards earlier positions, position 1 included
+// (there the seeding arc and, if asked for, its opposite).
+int lv_conditions(const Plan &P, int p, Cons *out, int *npos) {
+  if (p > 1) {
+    *npos = P.npos[p];
+    for (int j = 0; j < P.ncons[p]; ++j) out[j] = P.cons[p][j];
+    return P.ncons[p];
+  }
+  int n = 0;
+  out[n++] = Cons{0, P.seed_rev ? kIn : kOut, 0, P.seed_lab};
+  if (P.back_req) out[n++] = Cons{0, P.seed_rev ? kOut : kIn, 0, P.back_lab};
+  *npos = n;
+  if (P.back_forbid) out[n++] = Cons{0, P.seed_rev ? kNotOut : kNotIn, 0, 0};
+  return n;
+}
+
+// The plan with position 1 matched last: position i > 1 becomes i - 1.  Only
+// induced non-arcs and order constraints can name position 1 in a later
+// position; they are read from the other side.
+void lv_defer(Plan &P) {
+  const Plan O = P;
+  const int k = O.k, z = k - 1;
+  auto pos = [&](int i) { return i == 0 ? 0 : i == 1 ? z : i - 1; };
+  Cons tail[kMaxCons];
+  int tpos = 0, tn = lv_conditions(O, 1, tail, &tpos);
+  P.sym_gt[z] = O.sym_gt[1] & 1u;
+  P.sym_lt[z] = O.sym_lt[1] & 1u;
+  for (int p = 2; p < k; ++p) {
+    const int q = p - 1;
+    int c = 0;
+    for (int j = 0; j < O.ncons[p]; ++j) {
+      Cons cs = O.cons[p][j];
+      if (cs.q == 1) {
+        tail[tn++] = Cons{(int8_t)q, cs.kind == kNotOut ? kNotIn : kNotOut, 0, 0};
+        continue;
+      }
+      cs.q = (int8_t)pos(cs.q);
+      P.cons[q][c++] = cs;
+    }
+    P.ncons[q] = c;
+    P.npos[q] = O.npos[p];
+    uint32_t gt = 0, lt = 0;
+    for (int i = 0; i < p; ++i) {
+      if (i == 1) continue;
+      gt |= (O.sym_gt[p] >> i & 1u) << pos(i);
+      lt |= (O.sym_lt[p] >> i & 1u) << pos(i);
+    }
+    P.sym_gt[z] |= (O.sym_lt[p] >> 1 & 1u) << q;  // f(p) < f(1)
+    P.sym_lt[z] |= (O.sym_gt[p] >> 1 & 1u) << q;  // f(p) > f(1)
+    P.sym_gt[q] = gt;
+    P.sym_lt[q] = lt;
+    P.vlab[q] = O.vlab[p];
+    P.orig[q] = O.orig[p];
+    P.din[q] = O.din[p];
+    P.dout[q] = O.dout[p];
+  }
+  for (int j = 0; j < tn; ++j) P.cons[z][j] = tail[j];
+  P.ncons[z] = tn;
+  P.npos[z] = tpos;
+  P.vlab[z] = O.vlab[1];
+  P.orig[z] = O.orig[1];
+  P.din[z] = O.din[1];
+  P.dout[z] = O.dout[1];
+  for (int s = 0; s < O.naut && O.naut > 1; ++s)
+    for (int v = 0; v < k; ++v) P.aut[s][v] = (int8_t)pos(O.aut[s][v]);
+  if (O.root_pos >= 0) P.root_pos = pos(O.root_pos);
+}
+
+// `deferred`: lv_defer has been applied, position 1 is like any other.
+void lv_level(const hm_graph *g, const Plan &P, bool deferred, int p, bool want_rows, LevelPlan &L) {
   std::memset(&L, 0, sizeof(L));
   if (p >= P.k) return;
-  L.npos = (int16_t)P.npos[p];
-  L.ncons = (int16_t)P.ncons[p];
+  Cons cons[kMaxCons];
+  int npos = 0, n = 0;
+  if (p == 1 && deferred) {
+    npos = P.npos[1];
+    n = P.ncons[1];
+    for (int j = 0; j < n; ++j) cons[j] = P.cons[1][j];
+  } else {
+    n = lv_conditions(P, p, cons, &npos);
+  }
+  L.npos = (int16_t)npos;
+  L.ncons = (int16_t)n;
   L.last = p == P.k - 1;
   L.root = P.root_pos == p;
   L.dout = P.dout[p];
   L.din = P.din[p];
   L.sym_gt = P.sym_gt[p];
   L.sym_lt = P.sym_lt[p];
-  for (int j = 0; j < P.ncons[p]; ++j) {
-    const Cons cs = P.cons[p][j];
-    const ArcKey l = j < P.npos[p] ? labelled_key(ArcKey{0, 0}, cs.lab) : ArcKey{0, 0};
-    L.cons[j] = LvCons{cs.q, cs.kind, j < P.npos[p] ? lv_class(g, cs.lab, P.vlab[p]) : (int16_t)0, cs.lab, l.a, l.b};
+  for (int j = 0; j < n; ++j) {
+    const ArcKey l = j < npos ? labelled_key(ArcKey{0, 0}, cons[j].lab) : ArcKey{0, 0};
+    L.cons[j] = LvCons{cons[j].q, cons[j].kind, j < npos ? lv_class(g, cons[j].lab, P.vlab[p]) : (int16_t)0,
+                       cons[j].lab, l.a, l.b};
   }
-  // arcs to later positions: one or two are found missing by the next ranges phase anyway
-  L.need_deg = !L.last && P.dout[p] + P.din[p] - P.npos[p] >= 2;
+  // arcs to later positions: one is found missing by the next ranges phase anyway
+  L.need_deg = !L.last && P.dout[p] + P.din[p] - npos >= 2;
+  L.closed = L.last && !want_rows && npos == 1 && n == 1 && !L.root && !(L.sym_gt | L.sym_lt);
 }
 
 void lv_emit(const Plan &P, EmitPlan &E, std::vector<int8_t> &aut) {
@@ -825,130 +967,212 @@ void lv_emit(const Plan &P, EmitPlan &E, std::vector<int8_t> &aut) {
     for (int s = 0; s < P.naut; ++s) aut.insert(aut.end(), P.aut[s], P.aut[s] + kMaxK);
 }
 
-}  // namespace
-
-hm_status levels_run(const LvLaunch &L, cudaStream_t s, bool *ran, int *grid_out, int *threads_out) {
+hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result, int *grid_out, int *threads_out,
+                     float *ms) {
   *ran = false;
   const hm_graph *g = L.g;
-  if (!g->ncls || filter_min() != 1) return HM_OK;
-  const bool batch = L.npat > 0, shared = L.groups != nullptr;
+  const bool batch = L.npat > 0;
   bool sym = false;
   int kmax = 0;
-  if (batch) {
-    for (int32_t i = 0; i < L.npat; ++i) {
-      sym |= L.plans[i].naut > 1;
-      kmax = std::max({kmax, (int)L.plans[i].k, 3});
-    }
-  } else {
-    sym = L.plan->naut > 1;
-    kmax = L.plan->k;
+  const int32_t np = batch ? L.npat : 1;
+  for (int32_t i = 0; i < np; ++i) {
+    const Plan &P = batch ? *L.plans[i] : *L.plan;
+    sym |= P.naut > 1;
+    kmax = std::max(kmax, (int)P.k);
   }
-  const LvKernel f = lv_kernel(L.want_rows, batch, shared, sym);
-  int grid = lv_grid(f, (L.want_rows ? 8 : 0) + (batch ? 4 : 0) + (shared ? 2 : 0) + (sym ? 1 : 0));
-  if (grid <= 0) return HM_OK;
+  const LvKernel f = lv_kernel(L.want_rows, batch, sym);
+  int grid = lv_grid(f, (L.want_rows ? 4 : 0) + (batch ? 2 : 0) + (sym ? 1 : 0));
+  if (grid <= 0 || np >= 1 << 24) return HM_OK;
   // a small graph's levels do not need every block, and barriers cost less with fewer
   grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, (g->m + 255) / 256));
 
-  const int64_t warps = (int64_t)grid * kLvWarps;
-  const int top = shared ? kmax : kmax - 1;  // deepest level with states
   LvArgs A{};
-  // a quarter of the workspace for the depth-2 states' ranges, the rest for the deeper levels
-  A.slice = std::max<int64_t>(1, std::min<int64_t>({L.max_seeds, kLvSeedSlice, (int64_t)kLvMaxGroups * 32 * grid,
-                                                    (int64_t)(L.workspace / 4 / 32)}));
-  // bytes per state of all levels; the buffers are sized by the workspace and the graph
-  int64_t per_state = 0;
-  for (int p = 3; p <= top; ++p) per_state += 16 + 4 * ((p + (batch ? 1 : 0) + 3) / 4 * 4) + 1;
-  int64_t fcap = per_state ? (int64_t)(L.workspace / 4 * 3 / (uint64_t)per_state) : 0;
-  fcap = std::min<int64_t>({fcap, std::max<int64_t>(8 * g->m, 1 << 16), (int64_t)kLvMaxGroups * 32 * grid,
-                            (int64_t)1 << 24});
-  fcap = std::max<int64_t>(fcap & ~int64_t(31), 4096);
-  A.fcap = fcap;
-  auto round = [](size_t b) { return (b + 255) / 256 * 256; };
-  auto groups_of = [&](int64_t states) { return (size_t)(states / 32 + 2 * warps + 64); };
-  size_t bytes = 0, at_rng[kMaxK + 2] = {}, at_up[kMaxK + 2] = {}, at_bs[kMaxK + 2] = {}, at_st[kMaxK + 2] = {};
-  for (int p = 2; p <= top; ++p) {
-    const int64_t states = p == 2 ? A.slice : fcap;
-    A.stride[p] = p == 2 ? (shared ? 4 : 2) : (p + (batch ? 1 : 0) + 3) / 4 * 4;
-    at_rng[p] = bytes;
-    bytes += round(sizeof(int4) * (size_t)states);
-    at_up[p] = bytes;
-    bytes += round(8 * groups_of(states));
-    at_bs[p] = bytes;
-    bytes += round(8 * (size_t)grid);
-    at_st[p] = bytes;
-    if (p > 2) bytes += round(4 * (size_t)A.stride[p] * (size_t)states);
-  }
-  // batch: level and emission plans; symmetric patterns: automorphisms
   std::vector<int8_t> aut;
-  std::vector<LevelPlan> levels;
-  std::vector<EmitPlan> emit;
-  if (batch) {
-    levels.resize((size_t)L.npat * kmax);
-    emit.resize(L.npat);
-    for (int32_t i = 0; i < L.npat; ++i) {
-      for (int p = 1; p < kmax; ++p) lv_level(g, L.plans[i], p, levels[(size_t)i * kmax + p]);
-      levels[(size_t)i * kmax + 2].done = L.plans[i].k == 2;
-      lv_emit(L.plans[i], emit[i], aut);
+  std::vector<LevelPlan> levels(batch ? (size_t)np * kmax : 0);
+  std::vector<EmitPlan> emit(batch ? np : 0);
+  std::vector<unsigned long long> vert_n(batch ? np + 1 : 0);
+  std::vector<const int32_t *> vert_at(batch ? np : 0);
+  std::vector<int2> deg0(batch ? np : 0);
+  const int32_t *first_vertex = g->vby_out;
+  for (int32_t i = 0; i < np; ++i) {
+    const Plan &P0 = batch ? *L.plans[i] : *L.plan;
+    const bool defer = P0.k > 2 && P0.defer1 && L.defer;
+    Plan moved;
+    if (defer) {
+      moved = P0;
+      lv_defer(moved);
     }
-  } else {
-    for (int p = 1; p < kmax; ++p) lv_level(g, *L.plan, p, A.level1[p]);
-    lv_emit(*L.plan, A.emit1, aut);
-    A.ndefer = shared ? L.plan->ndefer : 0;
-    for (int j = 0; j < A.ndefer; ++j) A.defer[j] = L.plan->defer[j];
+    const Plan &P = defer ? moved : P0;
+    LevelPlan *lv = batch ? &levels[(size_t)i * kmax] : A.level1;
+    for (int p = 1; p < kmax; ++p) lv_level(g, P, defer, p, L.want_rows, lv[p]);
+    lv[1].final = defer ? (int8_t)(P.k - 1) : 0;
+    lv_emit(P, batch ? emit[i] : A.emit1, aut);
+    // the vertices with position 0's label and a group for one of position 1's conditions: the shortest list
+    const int64_t lab = (int64_t)P.vlab[0] - g->vl0;
+    const int32_t *list = g->vby_out;
+    int64_t cnt = 0;
+    if (lab >= 0 && lab < g->nvl) {
+      cnt = INT64_MAX;
+      for (int j = 0; j < lv[1].npos; ++j) {
+        const LvCons &cs = lv[1].cons[j];
+        const bool in = cs.kind == kIn;
+        const uint32_t *b = g->vstart + (in ? g->ncls * g->nvl + 1 : 0) + lab * g->ncls + std::max<int>(cs.cls, 0);
+        const int64_t here = cs.cls < 0 ? 0 : (int64_t)b[1] - b[0];
+        if (here < cnt) {
+          cnt = here;
+          list = (in ? g->vby_in : g->vby_out) + b[0];
+        }
+      }
+    }
+    if (batch) {
+      vert_n[i] = A.nvert;
+      vert_at[i] = list - (int64_t)A.nvert;
+      deg0[i] = make_int2(P.dout[0], P.din[0]);
+    } else {
+      first_vertex = list;
+      A.dout0 = P.dout[0];
+      A.din0 = P.din[0];
+      A.root0 = L.root_mask && P.root_pos == 0;
+    }
+    A.nvert += (unsigned long long)cnt;
   }
-  const size_t at_tab = bytes;
-  const size_t tab_levels = round(sizeof(LevelPlan) * levels.size()), tab_emit = round(sizeof(EmitPlan) * emit.size());
-  bytes += tab_levels + tab_emit + round(aut.size());
+  if (batch) vert_n[np] = A.nvert;
 
-  unsigned char *ws = nullptr;
-  HM_CUDA_TRY(cudaMallocAsync((void **)&ws, std::max<size_t>(bytes, 256), s));
-  for (int p = 2; p <= top; ++p) {
-    A.rng[p] = reinterpret_cast<int4 *>(ws + at_rng[p]);
-    A.upre[p] = reinterpret_cast<unsigned long long *>(ws + at_up[p]);
-    A.bsum[p] = reinterpret_cast<unsigned long long *>(ws + at_bs[p]);
-    A.base[p] = reinterpret_cast<const int32_t *>(ws + at_st[p]);
-  }
-  A.base[2] = shared ? reinterpret_cast<const int32_t *>(L.groups) : reinterpret_cast<const int32_t *>(L.seeds);
-  cudaError_t e = cudaSuccess;
-  auto up = [&](size_t at, const void *src, size_t n) {
-    if (n && e == cudaSuccess) e = cudaMemcpyAsync(ws + at, src, n, cudaMemcpyHostToDevice, s);
+  // The workspace: a quarter for the warps' resume points (fewer blocks if they
+  // do not fit), the rest for the levels' states, equal numbers of groups each.
+  const int top = kmax - 1;  // deepest level
+  if (top > 1)
+    grid = (int)std::min<uint64_t>((uint64_t)grid, std::max<uint64_t>(1, L.workspace / 4 / ((uint64_t)(top - 1) * kLvWarps *
+                                                                                           sizeof(LvPause))));
+  const int64_t warps = (int64_t)grid * kLvWarps;
+  auto stride_of = [&](int p) { return p <= 2 ? p : (p + 3) / 4 * 4; };
+  auto group_bytes = [&](int p) { return sizeof(LvGroup) + 32 * (sizeof(int4) + 4 * (uint64_t)stride_of(p)); };
+  uint64_t per_group = 0;
+  for (int p = 2; p <= top; ++p) per_group += group_bytes(p);
+  const uint64_t most = std::min<uint64_t>({(uint64_t)kLvMaxGroups, std::max<uint64_t>((uint64_t)g->m, 8192),
+                                            (kLvChunkMask >> 1) / (uint64_t)std::max(g->maxdeg, 1)});
+  // the first level holds all its vertices if they fit an eighth of the workspace
+  const uint64_t first = std::min<uint64_t>({most, (A.nvert + 31) / 32 + (uint64_t)warps,
+                                             L.workspace / 8 / group_bytes(1)});
+  A.gcap[1] = (uint32_t)std::max<uint64_t>(first, 64);
+  for (int p = 2; p <= top; ++p)
+    A.gcap[p] = (uint32_t)std::max<uint64_t>(std::min(most, L.workspace / 8 * 5 / per_group), 64);
+  A.fill_warps = std::min((uint32_t)warps, A.gcap[1] / 2);  // each may leave a group that is not full
+  A.slice = (uint64_t)(A.gcap[1] - A.fill_warps) * 32;
+  auto round = [](size_t b) { return (b + 255) / 256 * 256; };
+  size_t bytes = round(sizeof(LvCtl));
+  size_t at_rng[kMaxK + 1] = {}, at_grp[kMaxK + 1] = {}, at_ps[kMaxK + 1] = {}, at_st[kMaxK + 1] = {};
+  auto reserve = [&](size_t n) {
+    const size_t a = bytes;
+    bytes += round(n);
+    return a;
   };
-  up(at_tab, levels.data(), sizeof(LevelPlan) * levels.size());
-  up(at_tab + tab_levels, emit.data(), sizeof(EmitPlan) * emit.size());
-  up(at_tab + tab_levels + tab_emit, aut.data(), aut.size());
-  A.levels = reinterpret_cast<const LevelPlan *>(ws + at_tab);
-  A.emit = reinterpret_cast<const EmitPlan *>(ws + at_tab + tab_levels);
-  A.aut = reinterpret_cast<const int8_t *>(ws + at_tab + tab_levels + tab_emit);
+  for (int p = 1; p <= top; ++p) {
+    A.stride[p] = stride_of(p);
+    at_rng[p] = reserve(sizeof(int4) * 32 * A.gcap[p]);
+    at_grp[p] = reserve(sizeof(LvGroup) * A.gcap[p]);
+    at_st[p] = reserve(4 * (size_t)A.stride[p] * 32 * A.gcap[p]);
+    if (p < top) at_ps[p] = reserve(sizeof(LvPause) * (size_t)warps);
+  }
+  // a batch's tables, and the automorphisms of symmetric patterns, in one host block and one copy
+  size_t at_tab = bytes, tab = 0;
+  auto place = [&](size_t n) {
+    const size_t a = tab;
+    tab += round(n);
+    return a;
+  };
+  const size_t t_levels = place(sizeof(LevelPlan) * levels.size()), t_emit = place(sizeof(EmitPlan) * emit.size()),
+               t_vn = place(8 * vert_n.size()), t_va = place(8 * vert_at.size()), t_deg = place(8 * deg0.size()),
+               t_aut = place(aut.size());
+  std::vector<unsigned char> host(tab);
+  auto put = [&](size_t a, const void *src, size_t n) {
+    if (n) std::memcpy(host.data() + a, src, n);
+  };
+  put(t_levels, levels.data(), sizeof(LevelPlan) * levels.size());
+  put(t_emit, emit.data(), sizeof(EmitPlan) * emit.size());
+  put(t_vn, vert_n.data(), 8 * vert_n.size());
+  put(t_va, vert_at.data(), 8 * vert_at.size());
+  put(t_deg, deg0.data(), 8 * deg0.size());
+  put(t_aut, aut.data(), aut.size());
+  bytes += tab;
+
+  struct Space {
+    unsigned char *p = nullptr;
+    cudaStream_t s;
+    ~Space() {
+      if (p) cudaFreeAsync(p, s);
+    }
+  } ws{nullptr, s};
+  HM_CUDA_TRY(cudaMallocAsync((void **)&ws.p, bytes, s));
+  for (int p = 1; p <= top; ++p) {
+    A.rng[p] = reinterpret_cast<int4 *>(ws.p + at_rng[p]);
+    A.grp[p] = reinterpret_cast<LvGroup *>(ws.p + at_grp[p]);
+    A.base[p] = reinterpret_cast<int32_t *>(ws.p + at_st[p]);
+    if (p < top) A.pause[p] = reinterpret_cast<LvPause *>(ws.p + at_ps[p]);
+  }
+  A.vert = first_vertex;
+  A.ctl = reinterpret_cast<LvCtl *>(ws.p);
+  unsigned char *t = ws.p + at_tab;
+  A.levels = reinterpret_cast<const LevelPlan *>(t + t_levels);
+  A.emit = reinterpret_cast<const EmitPlan *>(t + t_emit);
+  A.vert_n = reinterpret_cast<const unsigned long long *>(t + t_vn);
+  A.vert_at = reinterpret_cast<const int32_t *const *>(t + t_va);
+  A.deg0 = reinterpret_cast<const int2 *>(t + t_deg);
+  A.aut = reinterpret_cast<const int8_t *>(t + t_aut);
   A.G = g->dev();
-  A.ctl = L.ctl;
-  A.nseeds = L.nseeds;
-  A.groups = L.groups;
-  A.sorted_seeds = L.sorted_seeds;
+  A.npat = L.npat;
   A.root_mask = L.root_mask;
   A.budget_ns = budget_ms() * 1000000ull;
   A.rows = L.rows;
   A.cap = L.cap;
-  A.seed_pid = L.seed_pid;
   A.counts = L.counts;
   A.row_off = L.row_off;
   A.row_cap = L.row_cap;
   A.row_cursor = L.row_cursor;
   A.kmax = kmax;
-  if (e == cudaSuccess) {
-    void *args[] = {&A};
-    const cudaError_t le = cudaLaunchCooperativeKernel((const void *)f, dim3(grid), dim3(kLvThreads), args,
-                                                       sizeof(LvShared), s);
-    if (le == cudaSuccess) *ran = true;
-    else (void)cudaGetLastError();  // not launched: the caller searches depth first
+  HM_CUDA_TRY(cudaMemsetAsync(A.ctl, 0, sizeof(LvCtl), s));
+  if (tab) HM_CUDA_TRY(cudaMemcpyAsync(t, host.data(), tab, cudaMemcpyHostToDevice, s));
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  if (ms) {
+    cudaEventCreate(&ev[0]);
+    cudaEventCreate(&ev[1]);
+    cudaEventRecord(ev[0], s);
   }
-  cudaFreeAsync(ws, s);
-  if (e != cudaSuccess) {
-    (void)cudaGetLastError();
-    return HM_ERR_CUDA;
+  void *args[] = {&A};
+  const cudaError_t le = cudaLaunchCooperativeKernel((const void *)f, dim3(grid), dim3(kLvThreads), args,
+                                                     sizeof(LvShared), s);
+  hm_status st = HM_OK;
+  if (le == cudaSuccess) {
+    *ran = true;
+    if (ms) cudaEventRecord(ev[1], s);
+    if (cudaMemcpyAsync(result, A.ctl, sizeof(LvCtl), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        (L.counts_host && cudaMemcpyAsync(L.counts_host, L.counts, sizeof(unsigned long long) * L.npat,
+                                          cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+      st = HM_ERR_CUDA;
+    if (ms && st == HM_OK) cudaEventElapsedTime(ms, ev[0], ev[1]);
   }
-  if (grid_out) *grid_out = grid;
-  if (threads_out) *threads_out = kLvThreads;
-  return HM_OK;
+  (void)cudaGetLastError();  // a launch that was refused: the caller searches depth first
+  if (ms) {
+    cudaEventDestroy(ev[0]);
+    cudaEventDestroy(ev[1]);
+  }
+  *grid_out = grid;
+  *threads_out = kLvThreads;
+  return st;
+}
+
+}  // namespace
+
+hm_status levels_run(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result, int *grid, int *threads,
+                     float *ms) {
+  LvLaunch M = L;
+  for (;;) {
+    const hm_status st = levels_try(M, s, ran, result, grid, threads, ms);
+    // a device that is nearly full: the levels in smaller parts
+    if (st != HM_ERR_OOM || M.workspace <= kLevelWorkspaceMin) return st;
+    M.workspace = std::max(M.workspace / 4, kLevelWorkspaceMin);
+  }
 }
 
 }  // namespace hm

@@ -75,6 +75,28 @@ int64_t part_start(int64_t m, int32_t part, int32_t nparts) {
   return (int64_t)((__int128)m * part / nparts) & ~int64_t(3);
 }
 
+// The rows of a call in lexicographic order of the original pattern ids.
+hm_status sort_rows(const hm_graph *g, int k, int32_t *rows, uint64_t count, Scratch &sc, cudaStream_t s, bool timing,
+                    hm_stats &st) {
+  if (count <= 1) return HM_OK;
+  NvtxRange r_sort("hm.sort_rows");
+  Timer t(s, timing);
+  int32_t *tmp;
+  HM_CUDA_TRY(sc.get((void **)&tmp, sizeof(int32_t) * (size_t)count * k));
+  int cols[kMaxK];
+  for (int i = 0; i < k; ++i) cols[i] = i;
+  int nl = 0;
+  const hm_status r = radix_sort_rows(rows, tmp, (int64_t)count, k, cols, k, bits_for(g->n), s, &nl);
+  st.kernel_launches += nl;
+  t.stop();
+  if (r != HM_OK) return r;
+  if (timing) {
+    HM_CUDA_TRY(cudaStreamSynchronize(s));
+    st.ms_sort = t.ms();
+  }
+  return HM_OK;
+}
+
 hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_t root,
                     const uint8_t *root_mask, int32_t *out, uint64_t cap, uint64_t *count,
                     cudaStream_t s, Want want, int32_t part = 0, int32_t nparts = 1) {
@@ -98,22 +120,49 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   const DevGraph G = g->dev();
   const int64_t m = g->m;
   const hm_tuning tu = tuning();
-  // default knobs: level by level; the instrumented kernels and a chunk budget belong to the depth-first search
-  const bool by_level = p->k > 2 && g->ncls > 0 && want != Want::kStates && default_search(tu) && !counters &&
-                        budget_chunks() == 0;
-  // The overlap test only prunes: a common neighbour that a match needs is a
-  // candidate of a later position, checked there with its labels.  Level by
-  // level that costs a few lookups per state; the test merges whole lists, one
-  // warp per state (five connectome counts: 5.5 of 14.5 ms, and 1.26 of 5.0 ms
-  // for 256 patterns), so only the depth-first search and the injected states take it.
-  const bool overlap = plan.ov_need > 0 && !by_level;
+  const bool rows = want == Want::kRows;
   Scratch sc(s);
+  // Default knobs: the whole match level by level (hm_levels.cu).  The
+  // depth-first search below keeps the other knobs, the instrumented kernels,
+  // chunk budgets, arc-range parts, graphs with too many label classes, and
+  // the injected states.
+  if (g->ncls > 0 && want != Want::kStates && nparts == 1 && default_search(tu) && !counters && budget_chunks() == 0) {
+    NvtxRange r_lv("hm.extend");
+    LvLaunch L{};
+    L.g = g;
+    L.root_mask = root_mask;
+    L.want_rows = rows;
+    L.rows = out;
+    L.workspace = level_workspace(g);
+    L.plan = &plan;
+    L.cap = cap;
+    L.defer = tu.share_seeds > 0;
+    LvCtl h;
+    bool ran = false;
+    int grid = 0, threads = 0;
+    const hm_status r = levels_run(L, s, &ran, &h, &grid, &threads, timing ? &st.ms_extend : nullptr);
+    if (r != HM_OK) return r;
+    if (ran) {
+      st.extend_grid = grid;
+      st.extend_block = threads;
+      st.seeds_scanned = (uint64_t)m;
+      st.states_injected = p->k > 2 ? h.injected : h.count;
+      st.chunks = h.chunks;
+      st.matches = h.count;
+      st.kernel_launches = 1;
+      if (h.status == kStatBudget) return HM_ERR_BUDGET;
+      if (h.status != kStatOk) return HM_ERR_CUDA;
+      *count = h.count;
+      if (!rows) return HM_OK;
+      return h.count > cap ? HM_ERR_CAPACITY : sort_rows(g, p->k, out, h.count, sc, s, timing, st);
+    }
+  }
   Ctl *ctl;
   int2 *seeds_a, *seeds_b = nullptr;
   HM_CUDA_TRY(sc.get((void **)&ctl, sizeof(Ctl)));
   HM_CUDA_TRY(cudaMemsetAsync(ctl, 0, sizeof(Ctl), s));
   HM_CUDA_TRY(sc.get((void **)&seeds_a, sizeof(int2) * (size_t)std::max<int64_t>(m, 1)));
-  if (overlap)
+  if (plan.ov_need > 0)
     HM_CUDA_TRY(sc.get((void **)&seeds_b, sizeof(int2) * (size_t)std::max<int64_t>(m, 1)));
   const int sms = num_sms();
 
@@ -139,8 +188,8 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   }
   const int2 *seeds = seeds_a;
   const unsigned long long *nseeds = &ctl->nseeds_raw;
-  Timer t_ov(s, timing && overlap);
-  if (overlap) {
+  Timer t_ov(s, timing && plan.ov_need > 0);
+  if (plan.ov_need > 0) {
     NvtxRange r_ov("hm.overlap_test");
     if (counters)
       k_seed_overlap<true><<<sms * 8, kSeedThreads, 0, s>>>(G, plan.ov_need, seeds_a, &ctl->nseeds_raw,
@@ -161,7 +210,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
     Ctl h;
     HM_CUDA_TRY(cudaMemcpyAsync(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     HM_CUDA_TRY(cudaStreamSynchronize(s));
-    unsigned long long n = overlap ? h.nseeds : h.nseeds_raw;
+    unsigned long long n = plan.ov_need > 0 ? h.nseeds : h.nseeds_raw;
     *count = n;
     if (n > cap) return HM_ERR_CAPACITY;
     if (n)
@@ -196,8 +245,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
       if (r != HM_OK) return r;
       launches += nl;
       const int gb = (int)std::min<unsigned long long>((ns + 256) / 256, (unsigned long long)sms * 8);
-      k_seed_group_flags<<<gb, 256, 0, s>>>(seeds, (int64_t)ns, plan.induced && !by_level ? kInducedGroupCap : 0,
-                                           flag);
+      k_seed_group_flags<<<gb, 256, 0, s>>>(seeds, (int64_t)ns, plan.induced ? kInducedGroupCap : 0, flag);
       r = exclusive_scan_u32(flag, idx, (int64_t)ns + 1, s);
       if (r != HM_OK) return r;
       k_seed_groups<<<gb, 256, 0, s>>>(seeds, (int64_t)ns, flag, idx, gr, &ctl->ngroups);
@@ -210,38 +258,10 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   t_grp.stop();
 
   // a4 + a5: state injection and extension
-  const bool rows = want == Want::kRows;
   Timer t_ext(s, timing && p->k > 2);
-  bool ran_levels = false;
   {  // the extension's launches
   NvtxRange r_ext("hm.extend");
-  if (by_level) {
-    LvLaunch L{};
-    L.g = g;
-    L.ctl = &ctl->lv;
-    L.seeds = seeds;
-    L.nseeds = share ? &ctl->ngroups : nseeds;
-    L.max_seeds = m;
-    L.groups = groups;
-    L.sorted_seeds = share ? seeds : nullptr;
-    L.root_mask = root_mask;
-    L.plan = &plan;
-    L.rows = rows ? out : nullptr;
-    L.cap = rows ? cap : 0;
-    L.want_rows = rows;
-    L.workspace = kLevelWorkspace;
-    int grid = 0, threads = 0;
-    const hm_status r = levels_run(L, s, &ran_levels, &grid, &threads);
-    if (r != HM_OK) return r;
-    if (ran_levels) {
-      ++launches;
-      st.extend_grid = grid;
-      st.extend_block = threads;
-      t_ext.stop();
-    }
-  }
-  if (ran_levels) {
-  } else if (p->k == 2) {
+  if (p->k == 2) {
     k_seed_rows<<<sms * 4, 256, 0, s>>>(plan, seeds, nseeds, rows ? out : nullptr, cap, ctl);
     ++launches;
     HM_CUDA_TRY(cudaGetLastError());
@@ -295,12 +315,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   st.ms_overlap = t_ov.ms() + t_grp.ms();
   st.ms_extend = t_ext.ms();
   st.seeds_scanned = (uint64_t)(e_end - e_begin);
-  st.states_injected = overlap ? h.nseeds : h.nseeds_raw;
-  if (ran_levels) {
-    h.status = h.lv.status;
-    h.count = h.lv.count;
-    h.chunks = h.lv.chunks;
-  }
+  st.states_injected = plan.ov_need > 0 ? h.nseeds : h.nseeds_raw;
   st.tasks_donated = h.donated;
   st.chunks = h.chunks;
   st.matches = h.count;
@@ -321,25 +336,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   *count = h.count;
   if (!rows) return HM_OK;
   if (h.count > cap) return HM_ERR_CAPACITY;
-  if (h.count > 1) {
-    NvtxRange r_sort("hm.sort_rows");
-    Timer t(s, timing);
-    int32_t *tmp;
-    HM_CUDA_TRY(sc.get((void **)&tmp, sizeof(int32_t) * (size_t)h.count * p->k));
-    int cols[kMaxK];
-    for (int i = 0; i < p->k; ++i) cols[i] = i;
-    const int sort_cols = p->k;
-    int nl = 0;
-    hm_status r = radix_sort_rows(out, tmp, (int64_t)h.count, p->k, cols, sort_cols, bits_for(g->n), s, &nl);
-    st.kernel_launches += nl;
-    t.stop();
-    if (r != HM_OK) return r;
-    if (timing) {
-      HM_CUDA_TRY(cudaStreamSynchronize(s));
-      st.ms_sort = t.ms();
-    }
-  }
-  return HM_OK;
+  return sort_rows(g, p->k, out, h.count, sc, s, timing, st);
 }
 
 }  // namespace
