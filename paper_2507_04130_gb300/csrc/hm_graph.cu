@@ -8,14 +8,18 @@
 //   1. pack rows (src, dst, label, aux), check ids / self-loops, and find
 //      the label ranges                                         (k_pack, k_bounds)
 //   2. stable radix sort by (src, dst); split into src / out_adj / out_elab,
-//      check repeated pairs, fill out-offsets                    (k_split_out)
-//   3. aux = label of dst; stable sort by (src, arc label, dst label): the
-//      label-grouped out-lists, and a directory with one entry per
-//      (vertex, arc label, neighbour label) group                (k_group_*)
-//   4. the same for in-lists, keyed on dst (steps 2-3 mirrored)
-//   5. per-vertex records {label, degrees}, {offsets}, {directory spans}
-//   6. the arc filter: every arc sets its bits under two keys       (k_filter)
-//   7. the arc hash table: every arc claims a slot                  (k_hash)
+//      check repeated pairs, fill out-offsets                        (k_split)
+//   3. the label-grouped out-lists: each list counted and placed by class
+//      (arc label, neighbour label) on its own      (k_group_lists, k_group_hubs)
+//   4. stable sort by dst alone (the rows are in source order), and steps 2-3
+//      for the in-lists
+//   5. a directory with one entry per (vertex, class) group, and the vertices
+//      of each (vertex label, class)            (k_group_dirs, k_class_place)
+//   6. per-vertex records {label, degrees}, {offsets}, {directory spans}
+//   7. the arc filter: every arc sets its bits under two keys       (k_filter)
+//   8. the arc hash table: every arc claims a slot                  (k_hash)
+// With more than 64 classes steps 3-5 sort the rows by (key, arc label,
+// neighbour label) instead and read groups off the sorted rows (build_groups).
 // The grouped lists let the extension kernel jump straight to the candidates
 // whose arc label and vertex label already match (checkAttributes of Alg. 2
 // and Alg. 3 applied as a range lookup instead of per candidate).
@@ -29,7 +33,7 @@ namespace hm {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int64_t kMaxDense = 64;  // classes with dense group offsets (k_dense holds them in one 64-bit mask)
+constexpr int64_t kMaxDense = 64;  // classes with dense group offsets (two per lane of a warp)
 constexpr int kW = 4;  // row width: src, dst, arc label, aux
 
 enum : uint32_t { kErrRange = 1, kErrSelf = 2, kErrDup = 4, kErrHash = 8 };
@@ -38,25 +42,50 @@ struct Bounds {
   int32_t emin, emax, vmin, vmax, maxdeg;
 };
 
+// Smallest and largest value of the block's threads: one atomic each (with one
+// per thread, packing 3.9M arcs took 37 instead of 21 us).
+__device__ __forceinline__ void block_bounds(int32_t lo, int32_t hi, int32_t *glo, int32_t *ghi) {
+  __shared__ int32_t s_lo[kThreads / 32], s_hi[kThreads / 32];
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0) {
+    s_lo[threadIdx.x >> 5] = lo;
+    s_hi[threadIdx.x >> 5] = hi;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kThreads / 32; ++w) {
+      lo = min(lo, s_lo[w]);
+      hi = max(hi, s_hi[w]);
+    }
+    atomicMin(glo, lo);
+    atomicMax(ghi, hi);
+  }
+}
+
+__global__ void k_begin(uint32_t *err, Bounds *bnd) {
+  err[0] = err[1] = 0;
+  *bnd = Bounds{INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN, 0};
+}
+
 __global__ void k_pack(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
                        const int32_t *__restrict__ elab, int64_t m, int32_t n,
                        int32_t *__restrict__ rows, uint32_t *__restrict__ err,
                        Bounds *__restrict__ bnd) {
   int32_t lo = INT32_MAX, hi = INT32_MIN;
+  uint32_t bad = 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
     int32_t a = src[e], b = dst[e], l = elab[e];
-    uint32_t f = 0;
-    if (a < 0 || a >= n || b < 0 || b >= n) f |= kErrRange;
-    else if (a == b) f |= kErrSelf;
-    if (f) atomicOr(err, f);
+    if (a < 0 || a >= n || b < 0 || b >= n) bad |= kErrRange;
+    else if (a == b) bad |= kErrSelf;
     int4 r = make_int4(min(max(a, 0), max(n - 1, 0)), min(max(b, 0), max(n - 1, 0)), l, 0);
     reinterpret_cast<int4 *>(rows)[e] = r;
     lo = min(lo, l);
     hi = max(hi, l);
   }
-  atomicMin(&bnd->emin, lo);
-  atomicMax(&bnd->emax, hi);
+  if (bad) atomicOr(err, bad);
+  block_bounds(lo, hi, &bnd->emin, &bnd->emax);
 }
 
 __global__ void k_vbounds(const int32_t *__restrict__ vlab, int32_t n, Bounds *__restrict__ bnd) {
@@ -66,8 +95,7 @@ __global__ void k_vbounds(const int32_t *__restrict__ vlab, int32_t n, Bounds *_
     lo = min(lo, vlab[v]);
     hi = max(hi, vlab[v]);
   }
-  atomicMin(&bnd->vmin, lo);
-  atomicMax(&bnd->vmax, hi);
+  block_bounds(lo, hi, &bnd->vmin, &bnd->vmax);
 }
 
 // off[v] = first row whose key column is >= v, for v in [0, n]; rows sorted by that column.
@@ -150,9 +178,11 @@ __global__ void k_zero_off(int64_t *__restrict__ off, int32_t n) {
     off[v] = 0;
 }
 
+// Per-vertex records.  The directory indexes are per row (rows sorted by key:
+// index of the group the row starts or continues) or, by_vertex, per vertex.
 __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__restrict__ out_off,
                          const int64_t *__restrict__ in_off, const uint32_t *__restrict__ oidx,
-                         const uint32_t *__restrict__ iidx, int32_t n, int4 *__restrict__ vi,
+                         const uint32_t *__restrict__ iidx, bool by_vertex, int32_t n, int4 *__restrict__ vi,
                          int2 *__restrict__ voff, int4 *__restrict__ vdir, Bounds *__restrict__ bnd) {
   int32_t most = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
@@ -160,8 +190,12 @@ __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__rest
     int64_t o0 = out_off[v], o1 = out_off[v + 1], i0 = in_off[v], i1 = in_off[v + 1];
     vi[v] = make_int4(vlab[v], (int32_t)(o1 - o0), (int32_t)(i1 - i0), 0);
     voff[v] = make_int2((int32_t)o0, (int32_t)i0);
-    uint32_t os = oidx ? oidx[o0] : 0, oe = oidx ? oidx[o1] : 0;
-    uint32_t is = iidx ? iidx[i0] : 0, ie = iidx ? iidx[i1] : 0;
+    uint32_t os = oidx ? oidx[by_vertex ? v : o0] : 0, oe = oidx ? oidx[by_vertex ? v + 1 : o1] : 0;
+    uint32_t is = iidx ? iidx[by_vertex ? v : i0] : 0, ie = iidx ? iidx[by_vertex ? v + 1 : i1] : 0;
+    if (by_vertex) {  // one prefix sum runs over both directions
+      is -= iidx[0];
+      ie -= iidx[0];
+    }
     vdir[v] = make_int4((int32_t)os, (int32_t)(oe - os), (int32_t)is, (int32_t)(ie - is));
     most = max(most, (int32_t)max(o1 - o0, i1 - i0));
   }
@@ -169,87 +203,265 @@ __global__ void k_vertex(const int32_t *__restrict__ vlab, const int64_t *__rest
   if ((threadIdx.x & 31) == 0 && most) atomicMax(&bnd->maxdeg, most);
 }
 
-// Dense group offsets of one direction (see DevGraph): one warp per vertex, the
-// vertex's directory entries on its lanes, two rounds of 32 classes.  A class
-// without a group starts where the next one does.  Counts the groups of each
-// (vertex label, class) for k_class_place.
-__global__ void k_dense(const int4 *__restrict__ vdir, const int2 *__restrict__ off, const int4 *__restrict__ vi,
-                        const int4 *__restrict__ dir, int32_t n, int64_t m, int in, int32_t ncls, int32_t nvl,
-                        int32_t al0, int32_t vl0, int32_t *__restrict__ gofs, uint32_t *__restrict__ cnt_of) {
-  __shared__ uint32_t h[kMaxDense * kMaxDense];
-  const int nbin = ncls * nvl;
-  for (int b = threadIdx.x; b < nbin; b += blockDim.x) h[b] = 0;
-  __syncthreads();
+// ---- label-grouped lists, few classes ------------------------------------------
+//
+// One direction's lists (sorted by neighbour) regrouped by class, stably: each
+// list is counted and placed on its own, one warp per vertex, and the dense
+// group offsets are the counts' prefix sums.  (A radix sort of all rows by
+// (key, arc label, neighbour label), flags, a scan and a walk to each group's
+// end took 394 us per direction for 3.9M arcs, R-MAT scale 18; this takes 150
+// with the directory.  Bound by the latency of the list and label loads: a
+// warp has one list at a time, and most lists are short.)
+struct Classes {
+  int32_t ncls, nvl, al0, vl0;
+};
+
+constexpr int kHub = 1024;  // longer lists get a block of 32 warps
+
+__device__ __forceinline__ int class_of(const Classes &C, int32_t alab, int32_t vlab) {
+  return (alab - C.al0) * C.nvl + (vlab - C.vl0);
+}
+
+// Group starts from the counts of classes lane and lane + 32; the starts replace
+// the counts in shared memory, relative to the list, and go to gofs.  Returns
+// the number of groups.
+__device__ __forceinline__ int class_starts(const Classes &C, uint32_t *cnt, int lane, int64_t base,
+                                            int32_t *__restrict__ gofs) {
+  const uint32_t c0 = cnt[lane], c1 = cnt[lane + 32];
+  uint32_t x = c0, y = c1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t a = __shfl_up_sync(0xffffffffu, x, o), b = __shfl_up_sync(0xffffffffu, y, o);
+    if (lane >= o) {
+      x += a;
+      y += b;
+    }
+  }
+  const uint32_t s0 = x - c0, s1 = __shfl_sync(0xffffffffu, x, 31) + y - c1;
+  cnt[lane] = s0;
+  cnt[lane + 32] = s1;
+  if (lane < C.ncls) gofs[lane] = (int32_t)(base + s0);
+  if (lane + 32 < C.ncls) gofs[lane + 32] = (int32_t)(base + s1);
+  __syncwarp();
+  return __popc(__ballot_sync(0xffffffffu, c0 > 0)) + __popc(__ballot_sync(0xffffffffu, c1 > 0));
+}
+
+__global__ void __launch_bounds__(kThreads)
+k_group_lists(const int64_t *__restrict__ off, const int32_t *__restrict__ adj, const int32_t *__restrict__ elab,
+              const int32_t *__restrict__ vlab, int32_t n, int64_t m, Classes C, int32_t *__restrict__ gadj,
+              int32_t *__restrict__ gofs, uint32_t *__restrict__ ngroup, int32_t *__restrict__ hubs,
+              uint32_t *__restrict__ nhub) {
+  __shared__ uint32_t s_cnt[kThreads / 32][64];
   const int lane = threadIdx.x & 31;
+  uint32_t *cnt = s_cnt[threadIdx.x >> 5];
+  uint32_t lt;
+  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
-    const int4 vd = vdir[v];
-    const int2 o = off[v];
-    const int4 info = vi[v];
-    const int32_t first = in ? vd.z : vd.x, cnt = in ? vd.w : vd.y, base = in ? o.y : o.x;
-    const int32_t len = in ? info.z : info.y;
-    // which classes have a group, and where the lane's entries (lane, lane + 32) start
-    unsigned long long have = 0;
-    int32_t s0 = len, s1 = len;
-    if (lane < cnt) {
-      const int4 e = dir[(int64_t)first + lane];
-      const int c = (e.x - al0) * nvl + (e.y - vl0);
-      have |= 1ull << c;
-      s0 = e.z;
-      atomicAdd(&h[(info.x - vl0) * ncls + c], 1u);
+    const int64_t base = off[v], len = off[v + 1] - base;
+    if (len > kHub) {
+      if (lane == 0) hubs[atomicAdd(nhub, 1u)] = (int32_t)v;
+      continue;
     }
-    if (lane + 32 < cnt) {
-      const int4 e = dir[(int64_t)first + lane + 32];
-      const int c = (e.x - al0) * nvl + (e.y - vl0);
-      have |= 1ull << c;
-      s1 = e.z;
-      atomicAdd(&h[(info.x - vl0) * ncls + c], 1u);
+    cnt[lane] = cnt[lane + 32] = 0;
+    __syncwarp();
+    int32_t id = 0;
+    int c = 64;
+    for (int64_t i = lane; i < len; i += 32) {
+      id = adj[base + i];
+      c = class_of(C, elab[base + i], vlab[id]);
+      atomicAdd(&cnt[c], 1u);
     }
-    const unsigned long long all = (unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)have) |
-                                   (unsigned long long)__reduce_or_sync(0xffffffffu, (uint32_t)(have >> 32)) << 32;
-    for (int c0 = 0; c0 < ncls; c0 += 32) {
+    __syncwarp();
+    const int g = class_starts(C, cnt, lane, base, gofs + v * C.ncls);
+    if (lane == 0) ngroup[v] = g;
+    for (int64_t b = 0; b < len; b += 32) {
+      const bool valid = b + lane < len;
+      if (len > 32 && valid) {  // a list of one chunk is in registers
+        id = adj[base + b + lane];
+        c = class_of(C, elab[base + b + lane], vlab[id]);
+      }
+      const uint32_t peers = __match_any_sync(0xffffffffu, valid ? c : 64 + lane);
+      const uint32_t at = valid ? cnt[c] : 0;
+      __syncwarp();
+      if (valid) {
+        gadj[base + at + __popc(peers & lt)] = id;
+        if ((peers & lt) == 0) cnt[c] = at + __popc(peers);
+      }
+      __syncwarp();
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    gofs[(int64_t)n * C.ncls] = (int32_t)m;
+    ngroup[n] = 0;
+  }
+}
+
+// The lists left out above: 32 warps each count and place an equal piece.
+__global__ void __launch_bounds__(1024)
+k_group_hubs(const int64_t *__restrict__ off, const int32_t *__restrict__ adj, const int32_t *__restrict__ elab,
+             const int32_t *__restrict__ vlab, Classes C, int32_t *__restrict__ gadj, int32_t *__restrict__ gofs,
+             uint32_t *__restrict__ ngroup, const int32_t *__restrict__ hubs, const uint32_t *__restrict__ nhub) {
+  __shared__ uint32_t s_cnt[32][64], s_all[64];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t *cnt = s_cnt[warp];
+  uint32_t lt;
+  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
+  for (uint32_t h = blockIdx.x; h < *nhub; h += gridDim.x) {
+    const int32_t v = hubs[h];
+    const int64_t base = off[v], len = off[v + 1] - base;
+    const int64_t piece = ((len + 31) / 32 + 31) / 32 * 32;
+    const int64_t a = base + min(len, warp * piece), z = base + min(len, (warp + 1) * piece);
+    cnt[lane] = cnt[lane + 32] = 0;
+    __syncwarp();
+    for (int64_t i = a + lane; i < z; i += 32) atomicAdd(&cnt[class_of(C, elab[i], vlab[adj[i]])], 1u);
+    __syncthreads();
+    if (threadIdx.x < 64) {  // each warp's part of every class, and the classes' sizes
+      uint32_t run = 0;
+      for (int w = 0; w < 32; ++w) {
+        const uint32_t t = s_cnt[w][threadIdx.x];
+        s_cnt[w][threadIdx.x] = run;
+        run += t;
+      }
+      s_all[threadIdx.x] = run;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const int g = class_starts(C, s_all, lane, base, gofs + (int64_t)v * C.ncls);
+      if (lane == 0) ngroup[v] = g;
+    }
+    __syncthreads();
+    cnt[lane] += s_all[lane];
+    cnt[lane + 32] += s_all[lane + 32];
+    __syncwarp();
+    for (int64_t b = a; b < z; b += 32) {
+      const bool valid = b + lane < z;
+      int32_t id = 0;
+      int c = 64 + lane;
+      if (valid) {
+        id = adj[b + lane];
+        c = class_of(C, elab[b + lane], vlab[id]);
+      }
+      const uint32_t peers = __match_any_sync(0xffffffffu, c);
+      const uint32_t at = valid ? cnt[c] : 0;
+      __syncwarp();
+      if (valid) {
+        gadj[base + at + __popc(peers & lt)] = id;
+        if ((peers & lt) == 0) cnt[c] = at + __popc(peers);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+  }
+}
+
+// Both directions of the steps below run in one launch (blockIdx.y).
+struct Direction {
+  const int32_t *gofs;
+  const uint32_t *didx;  // first directory entry of each vertex, counted from didx[0] on
+  int4 *dir;
+  uint32_t *cnt, *cur, *start;  // per (vertex label, class): groups, cursors, list starts
+  int32_t *vby;
+};
+
+// The directory from the dense group offsets, one warp per vertex, classes on
+// the lanes; counts the groups of each (vertex label, class) for k_class_place.
+__global__ void __launch_bounds__(kThreads)
+k_group_dirs(const __grid_constant__ Direction D0, const __grid_constant__ Direction D1,
+             const int32_t *__restrict__ vlab, int32_t n, Classes C) {
+  __shared__ uint32_t h[kMaxDense * kMaxDense];
+  const Direction &D = blockIdx.y ? D1 : D0;
+  const int32_t *gofs = D.gofs;
+  const uint32_t *didx = D.didx, first = D.didx[0];
+  int4 *dir = D.dir;
+  uint32_t *cnt_of = D.cnt;
+  const int nbin = C.ncls * C.nvl, lane = threadIdx.x & 31;
+  for (int b = threadIdx.x; b < nbin; b += blockDim.x) h[b] = 0;
+  __syncthreads();
+  uint32_t lt;
+  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
+    const int32_t *o = gofs + v * C.ncls;
+    const int32_t base = o[0];
+    uint32_t at = didx[v];
+    if (at == didx[v + 1]) continue;
+    const int l = (vlab[v] - C.vl0) * C.ncls;
+    for (int c0 = 0; c0 < C.ncls; c0 += 32) {
       const int c = c0 + lane;
-      const int at = __popcll(all & ((1ull << (c & 63)) - 1));  // groups of earlier classes
-      const int32_t a = __shfl_sync(0xffffffffu, s0, at & 31), b = __shfl_sync(0xffffffffu, s1, at & 31);
-      if (c < ncls) gofs[v * ncls + c] = base + (at >= cnt ? len : at < 32 ? a : b);
+      const int32_t a = c < C.ncls ? o[c] : 0, b = c < C.ncls ? o[c + 1] : 0;
+      const uint32_t have = __ballot_sync(0xffffffffu, b > a);
+      if (b > a) {
+        dir[at - first + __popc(have & lt)] = make_int4(C.al0 + c / C.nvl, C.vl0 + c % C.nvl, a - base, b - base);
+        atomicAdd(&h[l + c], 1u);
+      }
+      at += __popc(have);
     }
-    if (v == n - 1 && lane == 0) gofs[(int64_t)n * ncls] = (int32_t)m;
   }
   __syncthreads();
   for (int b = threadIdx.x; b < nbin; b += blockDim.x)
     if (h[b]) atomicAdd(cnt_of + b, h[b]);
 }
 
-// The vertices of each (vertex label, class) that have such a group, one
-// direction: tiles of vertices, each reserving its part of every list, so that
-// neighbours in a list stay neighbours in the graph.
+// Exclusive prefix sums of the counts, one block per direction.
+__global__ void __launch_bounds__(1024)
+k_class_starts(const __grid_constant__ Direction D0, const __grid_constant__ Direction D1, int nbin) {
+  const Direction &D = blockIdx.x ? D1 : D0;
+  __shared__ uint32_t s_sum[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t run = 0;
+  for (int b0 = 0; b0 <= nbin; b0 += 1024) {
+    const int b = b0 + threadIdx.x;
+    const uint32_t v = b < nbin ? D.cnt[b] : 0;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_sum[warp] = x;
+    __syncthreads();
+    uint32_t before = run, all = 0;
+    for (int w = 0; w < 32; ++w) {
+      if (w < warp) before += s_sum[w];
+      all += s_sum[w];
+    }
+    if (b <= nbin) D.start[b] = before + x - v;
+    run += all;
+    __syncthreads();
+  }
+}
+
+// The vertices of each (vertex label, class) that have such a group: tiles of
+// vertices, each reserving its part of every list, so that neighbours in a list
+// stay neighbours in the graph.
 constexpr int kClassTile = 256;
 
-__global__ void k_class_place(const int4 *__restrict__ vdir, const int4 *__restrict__ vi, const int4 *__restrict__ dir,
-                              int32_t n, int in, int32_t ncls, int32_t nvl, int32_t al0, int32_t vl0,
-                              const uint32_t *__restrict__ start, uint32_t *__restrict__ cur,
-                              int32_t *__restrict__ vby) {
+__global__ void __launch_bounds__(kThreads)
+k_class_place(const __grid_constant__ Direction D0, const __grid_constant__ Direction D1,
+              const int32_t *__restrict__ vlab, int32_t n, Classes C) {
   __shared__ uint32_t h[kMaxDense * kMaxDense];
-  const int nbin = ncls * nvl, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const Direction &D = blockIdx.y ? D1 : D0;
+  const uint32_t first = D.didx[0];
+  const int nbin = C.ncls * C.nvl, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = kThreads / 32;
   for (int64_t t0 = (int64_t)blockIdx.x * kClassTile; t0 < n; t0 += (int64_t)gridDim.x * kClassTile) {
     const int64_t t1 = min((int64_t)n, t0 + kClassTile);
-    for (int b = threadIdx.x; b < nbin; b += blockDim.x) h[b] = 0;
+    for (int b = threadIdx.x; b < nbin; b += kThreads) h[b] = 0;
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
       for (int64_t v = t0 + warp; v < t1; v += warps) {
-        const int4 vd = vdir[v];
-        const int l = (vi[v].x - vl0) * ncls;
-        const int32_t first = in ? vd.z : vd.x, cnt = in ? vd.w : vd.y;
-        for (int e = lane; e < cnt; e += 32) {
-          const int4 d = dir[(int64_t)first + e];
-          const uint32_t at = atomicAdd(&h[l + (d.x - al0) * nvl + (d.y - vl0)], 1u);
-          if (pass) vby[at] = (int32_t)v;
+        const int l = (vlab[v] - C.vl0) * C.ncls;
+        const uint32_t end = D.didx[v + 1] - first;
+        for (uint32_t e = D.didx[v] - first + lane; e < end; e += 32) {
+          const int4 d = D.dir[e];
+          const uint32_t at = atomicAdd(&h[l + class_of(C, d.x, d.y)], 1u);
+          if (pass) D.vby[at] = (int32_t)v;
         }
       }
       __syncthreads();
       if (!pass) {
-        for (int b = threadIdx.x; b < nbin; b += blockDim.x)
-          if (h[b]) h[b] = start[b] + atomicAdd(cur + b, h[b]);
+        for (int b = threadIdx.x; b < nbin; b += kThreads)
+          if (h[b]) h[b] = D.start[b] + atomicAdd(D.cur + b, h[b]);
         __syncthreads();
       }
     }
@@ -303,10 +515,36 @@ int grid_for(int64_t work) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, (int64_t)num_sms() * 16));
 }
 
+// An array of the graph's own (freed with it).
 template <typename T>
-cudaError_t dmalloc(T **p, int64_t count) {
-  return cudaMalloc((void **)p, sizeof(T) * (size_t)std::max<int64_t>(count, 1));
+cudaError_t own(hm_graph *g, T **p, int64_t count) {
+  const cudaError_t e = cudaMalloc((void **)p, sizeof(T) * (size_t)std::max<int64_t>(count, 1));
+  if (e == cudaSuccess) g->owned[g->nowned++] = *p;
+  return e;
 }
+
+// Several arrays in one allocation, each on a 256-byte boundary: cudaMalloc and
+// cudaFree cost 20 to 100 us each, and a graph has 19 arrays.
+struct Arena {
+  size_t bytes = 0;
+  struct Part {
+    void **p;
+    size_t at;
+  };
+  std::vector<Part> parts;
+  template <typename T>
+  void add(T **p, int64_t count) {
+    parts.push_back(Part{(void **)p, bytes});
+    bytes += (sizeof(T) * (size_t)std::max<int64_t>(count, 1) + 255) / 256 * 256;
+  }
+  cudaError_t allocate(hm_graph *g) {
+    unsigned char *base = nullptr;
+    const cudaError_t e = own(g, &base, (int64_t)bytes);
+    if (e == cudaSuccess)
+      for (const Part &q : parts) *q.p = base + q.at;
+    return e;
+  }
+};
 
 void label_key(int32_t lo, int32_t hi, int *bits, uint32_t *xr) {
   if (lo >= 0 && hi < (1 << 24)) {
@@ -358,9 +596,8 @@ namespace {
 // then write the grouped list and its directory.
 hm_status build_groups(int32_t *rows, int32_t *tmp, int64_t m, int32_t n, int key, int other,
                        const int32_t *vlab, const int64_t *off, int nbits, int be, uint32_t xe,
-                       int bv, uint32_t xv, cudaStream_t s, Temps &T, int32_t **gadj, int4 **dir,
+                       int bv, uint32_t xv, cudaStream_t s, Temps &T, int32_t *gadj, hm_graph *g, int4 **dir,
                        int64_t *ndir, uint32_t **idx_out) {
-  HM_CUDA_TRY(dmalloc(gadj, m));
   k_set_aux<<<grid_for(m), kThreads, 0, s>>>(rows, m, other, vlab);
   const int cols[3] = {key, 2, 3};
   const int bits[3] = {nbits, be, bv};
@@ -370,14 +607,14 @@ hm_status build_groups(int32_t *rows, int32_t *tmp, int64_t m, int32_t n, int ke
   uint32_t *flags, *idx;
   HM_CUDA_TRY(T.get((void **)&flags, sizeof(uint32_t) * (size_t)(m + 1)));
   HM_CUDA_TRY(T.get((void **)&idx, sizeof(uint32_t) * (size_t)(m + 1)));
-  k_group_flags<<<grid_for(m + 1), kThreads, 0, s>>>(rows, m, key, other, *gadj, flags);
+  k_group_flags<<<grid_for(m + 1), kThreads, 0, s>>>(rows, m, key, other, gadj, flags);
   st = exclusive_scan_u32(flags, idx, m + 1, s);
   if (st != HM_OK) return st;
   uint32_t total = 0;
   HM_CUDA_TRY(cudaMemcpyAsync(&total, idx + m, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaStreamSynchronize(s));
   *ndir = total;
-  HM_CUDA_TRY(dmalloc(dir, (int64_t)total));
+  HM_CUDA_TRY(own(g, dir, (int64_t)total));
   k_group_entries<<<grid_for(m), kThreads, 0, s>>>(rows, m, key, flags, idx, off, *dir);
   *idx_out = idx;
   return HM_OK;
@@ -388,7 +625,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
                           cudaStream_t s, hm_graph *g) {
   Temps T(s);
 #if HM_CHECK
-  HM_CUDA_TRY(dmalloc(&g->check, 1));  // the bounds checks' violation word
+  HM_CUDA_TRY(own(g, &g->check, 1));  // the bounds checks' violation word
   HM_CUDA_TRY(cudaMemsetAsync(g->check, 0, sizeof(unsigned long long), s));
 #endif
   const int32_t *d_src = src, *d_dst = dst, *d_vlab = vlab, *d_elab = elab;
@@ -407,19 +644,38 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     d_elab = t + 2 * m;
     d_vlab = t + 3 * m;
   }
-  int32_t *rows, *tmp;
+  // working memory: rows and their copy, offsets, groups per vertex and their
+  // prefix sums (both directions one after the other), long lists, class counts
+  int32_t *rows, *tmp, *hubs;
   int64_t *out_off, *in_off;
-  uint32_t *err;
+  uint32_t *err, *ngroup, *didx, *bins;
   Bounds *bnd;
-  HM_CUDA_TRY(T.get((void **)&rows, sizeof(int32_t) * (size_t)(kW * m + kW)));
-  HM_CUDA_TRY(T.get((void **)&tmp, sizeof(int32_t) * (size_t)(kW * m + kW)));
-  HM_CUDA_TRY(T.get((void **)&out_off, sizeof(int64_t) * (size_t)(2 * (n + 1)) + 64));
-  in_off = out_off + (n + 1);
-  HM_CUDA_TRY(T.get((void **)&err, sizeof(uint32_t)));
-  HM_CUDA_TRY(T.get((void **)&bnd, sizeof(Bounds)));
-  HM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
-  const Bounds init{INT32_MAX, INT32_MIN, INT32_MAX, INT32_MIN, 0};
-  HM_CUDA_TRY(cudaMemcpyAsync(bnd, &init, sizeof(Bounds), cudaMemcpyHostToDevice, s));
+  {
+    size_t at = 0;
+    auto part = [&](size_t b) {
+      const size_t a = at;
+      at += (b + 255) / 256 * 256;
+      return a;
+    };
+    const size_t bin_words = 6 * (size_t)(kMaxDense * kMaxDense + 1);
+    const size_t a_rows = part(sizeof(int32_t) * (size_t)(kW * m + kW)), a_tmp = part(sizeof(int32_t) * (size_t)(kW * m + kW)),
+                 a_off = part(sizeof(int64_t) * 2 * (size_t)(n + 1)), a_grp = part(sizeof(uint32_t) * 4 * (size_t)(n + 1)),
+                 a_hub = part(sizeof(int32_t) * 2 * (size_t)(m / kHub + 1)),
+                 a_zero = part(sizeof(uint32_t) * (bin_words + 4)), a_bnd = part(sizeof(Bounds));
+    unsigned char *w;
+    HM_CUDA_TRY(T.get((void **)&w, at));
+    rows = reinterpret_cast<int32_t *>(w + a_rows);
+    tmp = reinterpret_cast<int32_t *>(w + a_tmp);
+    out_off = reinterpret_cast<int64_t *>(w + a_off);
+    in_off = out_off + (n + 1);
+    ngroup = reinterpret_cast<uint32_t *>(w + a_grp);
+    didx = ngroup + 2 * (size_t)(n + 1);
+    hubs = reinterpret_cast<int32_t *>(w + a_hub);
+    err = reinterpret_cast<uint32_t *>(w + a_zero);  // {input errors, sort error}, then two list lengths, then the bins
+    bins = err + 4;
+    bnd = reinterpret_cast<Bounds *>(w + a_bnd);
+  }
+  k_begin<<<1, 1, 0, s>>>(err, bnd);
 
   if (m) k_pack<<<grid_for(m), kThreads, 0, s>>>(d_src, d_dst, d_elab, m, n, rows, err, bnd);
   if (n) k_vbounds<<<grid_for(n), kThreads, 0, s>>>(d_vlab, n, bnd);
@@ -432,60 +688,6 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   if (h_err & kErrRange) return HM_ERR_ARG;
   if (h_err & kErrSelf) return HM_ERR_SELF_LOOP;
 
-  HM_CUDA_TRY(dmalloc(&g->src, m));
-  HM_CUDA_TRY(dmalloc(&g->out_adj, m));
-  HM_CUDA_TRY(dmalloc(&g->out_elab, m));
-  HM_CUDA_TRY(dmalloc(&g->in_adj, m));
-  HM_CUDA_TRY(dmalloc(&g->in_elab, m));
-  HM_CUDA_TRY(dmalloc(&g->vi, n));
-  HM_CUDA_TRY(dmalloc(&g->off, n));
-  HM_CUDA_TRY(dmalloc(&g->vdir, n));
-  g->afilt_nword = (uint32_t)(4 * std::max<int64_t>(1, (m + 7) / 8));
-  HM_CUDA_TRY(dmalloc(&g->afilt, (int64_t)g->afilt_nword));
-  HM_CUDA_TRY(cudaMemsetAsync(g->afilt, 0, 8 * (size_t)g->afilt_nword, s));
-  g->ahash_nbkt = (uint32_t)std::max<int64_t>(1, m);
-  HM_CUDA_TRY(dmalloc(&g->ahash, 2 * (int64_t)g->ahash_nbkt));
-  HM_CUDA_TRY(cudaMemsetAsync(g->ahash, 0xff, 32 * (size_t)g->ahash_nbkt, s));
-
-  const int nbits = bits_for(n);
-  int be = 1, bv = 1;
-  uint32_t xe = 0, xv = 0;
-  if (m) label_key(hb.emin, hb.emax, &be, &xe);
-  if (n) label_key(hb.vmin, hb.vmax, &bv, &xv);
-  uint32_t *oidx = nullptr, *iidx = nullptr;
-  if (m) {
-    const int by_src[2] = {0, 1};
-    const int by_dst[2] = {1, 0};
-    hm_status st = radix_sort_rows(rows, tmp, m, kW, by_src, 2, nbits, s);
-    if (st != HM_OK) return st;
-    k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 0, 1, g->src, g->out_adj, g->out_elab,
-                                             out_off, err);
-    k_filter<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->afilt_nword,
-                                              reinterpret_cast<unsigned long long *>(g->afilt));
-    k_hash<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->ahash_nbkt,
-                                            g->ahash, err);
-    st = build_groups(rows, tmp, m, n, 0, 1, d_vlab, out_off, nbits, be, xe, bv, xv, s, T,
-                      &g->gout_adj, &g->gdir_out, &g->ndir_out, &oidx);
-    if (st != HM_OK) return st;
-    st = radix_sort_rows(rows, tmp, m, kW, by_dst, 2, nbits, s);
-    if (st != HM_OK) return st;
-    k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 1, 0, nullptr, g->in_adj, g->in_elab,
-                                             in_off, nullptr);
-    st = build_groups(rows, tmp, m, n, 1, 0, d_vlab, in_off, nbits, be, xe, bv, xv, s, T,
-                      &g->gin_adj, &g->gdir_in, &g->ndir_in, &iidx);
-    if (st != HM_OK) return st;
-  } else {
-    k_zero_off<<<grid_for(n + 1), kThreads, 0, s>>>(out_off, n);
-    k_zero_off<<<grid_for(n + 1), kThreads, 0, s>>>(in_off, n);
-    HM_CUDA_TRY(dmalloc(&g->gout_adj, 1));
-    HM_CUDA_TRY(dmalloc(&g->gin_adj, 1));
-    HM_CUDA_TRY(dmalloc(&g->gdir_out, 1));
-    HM_CUDA_TRY(dmalloc(&g->gdir_in, 1));
-  }
-  if (n)
-    k_vertex<<<grid_for(n), kThreads, 0, s>>>(d_vlab, out_off, in_off, oidx, iidx, n, g->vi, g->off,
-                                              g->vdir, bnd);
-  std::vector<uint32_t> h_bins;
   // dense group offsets while there are few classes and the tables are no larger than the arcs' own data
   const int64_t nal = m ? (int64_t)hb.emax - hb.emin + 1 : 0, nvl = m ? (int64_t)hb.vmax - hb.vmin + 1 : 0;
   if (m && nal <= kMaxDense && nvl <= kMaxDense && nal * nvl <= kMaxDense &&
@@ -495,33 +697,131 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     g->al0 = hb.emin;
     g->vl0 = hb.vmin;
     g->ncls = (int32_t)(nal * nvl);
-    const int64_t len = (int64_t)n * g->ncls + 1;
-    HM_CUDA_TRY(dmalloc(&g->gofs_out, len));
-    HM_CUDA_TRY(dmalloc(&g->gofs_in, len));
-    const int nbin = g->ncls * g->nvl;
-    uint32_t *bins;  // counts and cursors of both directions, then the list starts
-    HM_CUDA_TRY(T.get((void **)&bins, sizeof(uint32_t) * 6 * (size_t)(nbin + 1)));
-    HM_CUDA_TRY(cudaMemsetAsync(bins, 0, sizeof(uint32_t) * 4 * (size_t)(nbin + 1), s));
-    h_bins.resize(2 * (size_t)(nbin + 1));
-    for (int in = 0; in < 2; ++in) {
-      const int4 *dir = in ? g->gdir_in : g->gdir_out;
-      int32_t *&vby = in ? g->vby_in : g->vby_out;
-      uint32_t *cnt = bins + in * (nbin + 1), *cur = cnt + 2 * (nbin + 1), *start = cnt + 4 * (nbin + 1);
-      HM_CUDA_TRY(dmalloc(&vby, in ? g->ndir_in : g->ndir_out));
-      k_dense<<<grid_for(32 * (int64_t)n), kThreads, 0, s>>>(g->vdir, g->off, g->vi, dir, n, m, in, g->ncls, g->nvl,
-                                                             g->al0, g->vl0, in ? g->gofs_in : g->gofs_out, cnt);
-      const hm_status st = exclusive_scan_u32(cnt, start, nbin + 1, s);
-      if (st != HM_OK) return st;
-      k_class_place<<<grid_for((int64_t)n), kThreads, 0, s>>>(g->vdir, g->vi, dir, n, in, g->ncls, g->nvl, g->al0,
-                                                             g->vl0, start, cur, vby);
-      HM_CUDA_TRY(cudaMemcpyAsync(h_bins.data() + (size_t)in * (nbin + 1), start, sizeof(uint32_t) * (nbin + 1),
-                                  cudaMemcpyDeviceToHost, s));
-    }
   }
-  HM_CUDA_TRY(cudaMemcpyAsync(&h_err, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  const Classes C{g->ncls, g->nvl, g->al0, g->vl0};
+  g->afilt_nword = (uint32_t)(4 * std::max<int64_t>(1, (m + 7) / 8));
+  g->ahash_nbkt = (uint32_t)std::max<int64_t>(1, m);
+  Arena A;
+  A.add(&g->src, m);
+  A.add(&g->out_adj, m);
+  A.add(&g->out_elab, m);
+  A.add(&g->in_adj, m);
+  A.add(&g->in_elab, m);
+  A.add(&g->gout_adj, m);
+  A.add(&g->gin_adj, m);
+  A.add(&g->vi, n);
+  A.add(&g->off, n);
+  A.add(&g->vdir, n);
+  A.add(&g->afilt, (int64_t)g->afilt_nword);
+  A.add(&g->ahash, 2 * (int64_t)g->ahash_nbkt);
+  if (g->ncls) {
+    A.add(&g->gofs_out, (int64_t)n * g->ncls + 1);
+    A.add(&g->gofs_in, (int64_t)n * g->ncls + 1);
+  }
+  HM_CUDA_TRY(A.allocate(g));
+  HM_CUDA_TRY(cudaMemsetAsync(g->afilt, 0, 8 * (size_t)g->afilt_nword, s));
+  HM_CUDA_TRY(cudaMemsetAsync(g->ahash, 0xff, 32 * (size_t)g->ahash_nbkt, s));
+
+  const int nbits = bits_for(n);
+  int be = 1, bv = 1;
+  uint32_t xe = 0, xv = 0;
+  if (m) label_key(hb.emin, hb.emax, &be, &xe);
+  if (n) label_key(hb.vmin, hb.vmax, &bv, &xv);
+  uint32_t *oidx = nullptr, *iidx = nullptr;
+  std::vector<uint32_t> h_bins;
+  const int nbin = g->ncls * g->nvl;
+  int *sort_err = reinterpret_cast<int *>(err + 1);  // looked at when the load is done
+  if (m) {
+    const int by_src[2] = {0, 1}, by_dst[2] = {1, 0}, bits[2] = {nbits, nbits};
+    const uint32_t xr[2] = {0u, 0u};
+    hm_status st = radix_sort_rows_cols(rows, tmp, m, kW, by_src, bits, xr, 2, s, nullptr, sort_err);
+    if (st != HM_OK) return st;
+    k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 0, 1, g->src, g->out_adj, g->out_elab,
+                                             out_off, err);
+    k_filter<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->afilt_nword,
+                                              reinterpret_cast<unsigned long long *>(g->afilt));
+    k_hash<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->ahash_nbkt,
+                                            g->ahash, err);
+    if (g->ncls) {
+      // counts and cursors of both directions are zero; the starts follow them
+      HM_CUDA_TRY(cudaMemsetAsync(err + 2, 0, sizeof(uint32_t) * (2 + 4 * (size_t)(nbin + 1)), s));
+      uint32_t *nhub = err + 2;
+      uint32_t total[2] = {0, 0};
+      for (int in = 0; in < 2; ++in) {
+        if (in) {
+          // the rows are in (src, dst) order: sorted by dst alone they are in (dst, src) order
+          st = radix_sort_rows_cols(rows, tmp, m, kW, by_dst, bits, xr, 1, s, nullptr, sort_err);
+          if (st != HM_OK) return st;
+          k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 1, 0, nullptr, g->in_adj, g->in_elab, in_off, nullptr);
+        }
+        const int64_t *off = in ? in_off : out_off;
+        const int32_t *adj = in ? g->in_adj : g->out_adj, *elab = in ? g->in_elab : g->out_elab;
+        int32_t *gadj = in ? g->gin_adj : g->gout_adj, *gofs = in ? g->gofs_in : g->gofs_out;
+        int32_t *list = hubs + (size_t)in * (m / kHub + 1);
+        uint32_t *ng = ngroup + (size_t)in * (n + 1);
+        k_group_lists<<<grid_for(32 * (int64_t)n), kThreads, 0, s>>>(off, adj, elab, d_vlab, n, m, C, gadj, gofs,
+                                                                     ng, list, nhub + in);
+        k_group_hubs<<<(unsigned)std::min<int64_t>(m / kHub + 1, num_sms()), 1024, 0, s>>>(
+            off, adj, elab, d_vlab, C, gadj, gofs, ng, list, nhub + in);
+      }
+      st = exclusive_scan_u32(ngroup, didx, 2 * ((int64_t)n + 1), s);
+      if (st != HM_OK) return st;
+      oidx = didx;
+      iidx = didx + (n + 1);
+      HM_CUDA_TRY(cudaMemcpyAsync(&total[0], oidx + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+      HM_CUDA_TRY(cudaMemcpyAsync(&total[1], iidx + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+      HM_CUDA_TRY(cudaStreamSynchronize(s));
+      total[1] -= total[0];
+      g->ndir_out = total[0];
+      g->ndir_in = total[1];
+      Arena D;
+      D.add(&g->gdir_out, g->ndir_out);
+      D.add(&g->gdir_in, g->ndir_in);
+      D.add(&g->vby_out, g->ndir_out);
+      D.add(&g->vby_in, g->ndir_in);
+      HM_CUDA_TRY(D.allocate(g));
+    } else {
+      st = build_groups(rows, tmp, m, n, 0, 1, d_vlab, out_off, nbits, be, xe, bv, xv, s, T,
+                        g->gout_adj, g, &g->gdir_out, &g->ndir_out, &oidx);
+      if (st != HM_OK) return st;
+      st = radix_sort_rows(rows, tmp, m, kW, by_dst, 2, nbits, s);
+      if (st != HM_OK) return st;
+      k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 1, 0, nullptr, g->in_adj, g->in_elab,
+                                               in_off, nullptr);
+      st = build_groups(rows, tmp, m, n, 1, 0, d_vlab, in_off, nbits, be, xe, bv, xv, s, T,
+                        g->gin_adj, g, &g->gdir_in, &g->ndir_in, &iidx);
+      if (st != HM_OK) return st;
+    }
+  } else {
+    k_zero_off<<<grid_for(n + 1), kThreads, 0, s>>>(out_off, n);
+    k_zero_off<<<grid_for(n + 1), kThreads, 0, s>>>(in_off, n);
+    HM_CUDA_TRY(own(g, &g->gdir_out, 1));
+    HM_CUDA_TRY(own(g, &g->gdir_in, 1));
+  }
+  if (n)
+    k_vertex<<<grid_for(n), kThreads, 0, s>>>(d_vlab, out_off, in_off, oidx, iidx, g->ncls > 0, n, g->vi, g->off,
+                                              g->vdir, bnd);
+  if (g->ncls) {
+    h_bins.resize(2 * (size_t)(nbin + 1));
+    Direction D[2];
+    for (int in = 0; in < 2; ++in) {
+      uint32_t *cnt = bins + in * (nbin + 1);
+      D[in] = Direction{in ? g->gofs_in : g->gofs_out, in ? iidx : oidx, in ? g->gdir_in : g->gdir_out, cnt,
+                        cnt + 2 * (nbin + 1), cnt + 4 * (nbin + 1), in ? g->vby_in : g->vby_out};
+    }
+    k_group_dirs<<<dim3(grid_for(16 * (int64_t)n), 2), kThreads, 0, s>>>(D[0], D[1], d_vlab, n, C);
+    k_class_starts<<<2, 1024, 0, s>>>(D[0], D[1], nbin);
+    k_class_place<<<dim3(grid_for((int64_t)n), 2), kThreads, 0, s>>>(D[0], D[1], d_vlab, n, C);
+    HM_CUDA_TRY(cudaMemcpyAsync(h_bins.data(), bins + 4 * (nbin + 1), sizeof(uint32_t) * h_bins.size(),
+                                cudaMemcpyDeviceToHost, s));
+  }
+  uint32_t h_errs[2] = {0, 0};
+  HM_CUDA_TRY(cudaMemcpyAsync(h_errs, err, sizeof(h_errs), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaMemcpyAsync(&hb, bnd, sizeof(Bounds), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaStreamSynchronize(s));
   HM_CUDA_TRY(cudaGetLastError());
+  h_err = h_errs[0];
+  if (h_errs[1]) return HM_ERR_CUDA;
   g->maxdeg = hb.maxdeg;
   if (!h_bins.empty()) {
     g->vstart = (uint32_t *)malloc(sizeof(uint32_t) * h_bins.size());
@@ -537,12 +837,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
 }
 
 void free_graph_arrays(hm_graph *g) {
-  void *ptrs[] = {g->src,     g->out_adj,  g->out_elab, g->in_adj,   g->in_elab, g->vi,
-                  g->off,     g->gout_adj, g->gin_adj,  g->gdir_out, g->gdir_in, g->vdir,
-                  g->afilt,   g->ahash,    g->check,    g->gofs_out, g->gofs_in, g->vby_out,
-                  g->vby_in};
-  for (void *p : ptrs)
-    if (p) cudaFree(p);
+  for (int i = 0; i < g->nowned; ++i) cudaFree(g->owned[i]);
 }
 
 }  // namespace

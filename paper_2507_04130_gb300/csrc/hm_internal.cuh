@@ -237,9 +237,8 @@ __device__ __forceinline__ int32_t search_c(const int32_t *__restrict__ a, int32
 // passes.  The sums are linear, so the part of an endpoint that stays the same
 // over many probes is computed once; a probe is about 20 instructions and one
 // 8-byte load.  (A 256-bit block with one bit in each of eight words and a
-// 64-bit finalizer as the hash passed 0.1 % but took about 60 instructions,
-// two loads, and eight atomics per key to build; with this one the R-MAT scale
-// 20 bi-fan takes 7.78 instead of 8.37 ms.)
+// 64-bit finalizer as the hash passed 0.1 % but took about 60 instructions and
+// two loads, and eight atomics per key to build: 286 us for 3.9M arcs, now 43.)
 constexpr uint64_t kHashU1 = 0x2cb0f69f4abea221ull, kHashV1 = 0x9417034723148989ull,
                    kHashL1 = 0xdd555950609dfe03ull, kHashU2 = 0xdbafb150deb12801ull,
                    kHashV2 = 0x7e789b2e6c442cb7ull, kHashL2 = 0xf41e5636c7e4f8c5ull;
@@ -420,6 +419,8 @@ struct hm_graph {
   uint32_t *vstart;
   unsigned long long *check;  // bounds-checked builds: the violation word (device)
   size_t bytes;
+  void *owned[8];  // the device allocations behind the arrays
+  int nowned;
   // multi-property graphs (hm_load_graph_props): the sorted distinct property
   // tuples of vertices and arcs (host, malloc'ed); a label is a tuple's rank
   int32_t nvp, nep;
@@ -468,11 +469,12 @@ hm_status radix_sort_rows(int32_t *rows, int32_t *tmp, int64_t nrows, int width,
                           const int *key_cols, int nkey, int bits, cudaStream_t stream,
                           int *launches = nullptr);
 
+// With `err` (device, zero) a failure sets *err instead of being waited for.
 // As radix_sort_rows, with a bit width (1..32) and an xor mask per key column
 // (the xor maps signed values to an unsigned order, e.g. 0x80000000).
 hm_status radix_sort_rows_cols(int32_t *rows, int32_t *tmp, int64_t nrows, int width,
                                const int *key_cols, const int *key_bits, const uint32_t *key_xor,
-                               int nkey, cudaStream_t stream, int *launches = nullptr);
+                               int nkey, cudaStream_t stream, int *launches = nullptr, int *err = nullptr);
 
 // Sorts of at most this many rows place each row by counting the rows before
 // it (n^2 compares over the whole GPU) instead of by a radix sort.  The two

@@ -965,7 +965,7 @@ hm_status radix_sort_rows(int32_t *rows, int32_t *tmp, int64_t nrows, int width,
 // hold a grid of resident blocks for it; the caller then runs the passes as
 // separate kernels.
 static hm_status sort4_fused(int32_t *rows, int32_t *tmp, int64_t nrows, KeySpec ks, int passes,
-                             cudaStream_t stream, bool *ran) {
+                             cudaStream_t stream, bool *ran, int *err_out) {
   *ran = false;
   static std::atomic<int> per_sm{-1};
   int nb = per_sm.load(std::memory_order_relaxed);
@@ -997,7 +997,7 @@ static hm_status sort4_fused(int32_t *rows, int32_t *tmp, int64_t nrows, KeySpec
   F.part = buf + nhist;
   F.tot = buf + 2 * nhist;
   F.bar = reinterpret_cast<unsigned int *>(buf + 2 * nhist + kRadix);
-  F.err = reinterpret_cast<int *>(buf + 2 * nhist + kRadix + 1);
+  F.err = err_out ? err_out : reinterpret_cast<int *>(buf + 2 * nhist + kRadix + 1);
   for (int p = 0; p < passes; ++p) {
     set_pass(ks, p * kDigitBits);
     Digit4 &d = F.ks[p];
@@ -1022,6 +1022,10 @@ static hm_status sort4_fused(int32_t *rows, int32_t *tmp, int64_t nrows, KeySpec
   *ran = true;
   if (passes & 1)
     HM_CUDA_TRY(cudaMemcpyAsync(rows, tmp, sizeof(int4) * (size_t)nrows, cudaMemcpyDeviceToDevice, stream));
+  if (err_out) {
+    HM_CUDA_TRY(cudaFreeAsync(buf, stream));
+    return HM_OK;
+  }
   int err = 0;
   HM_CUDA_TRY(cudaMemcpyAsync(&err, F.err, sizeof(int), cudaMemcpyDeviceToHost, stream));
   HM_CUDA_TRY(cudaFreeAsync(buf, stream));
@@ -1044,7 +1048,7 @@ hm_status rank_sort_tiles(int32_t *rows, int32_t *tmp, const RankTile *tiles, in
 
 hm_status radix_sort_rows_cols(int32_t *rows, int32_t *tmp, int64_t nrows, int width,
                                const int *key_cols, const int *key_bits, const uint32_t *key_xor,
-                               int nkey, cudaStream_t stream, int *launches) {
+                               int nkey, cudaStream_t stream, int *launches, int *err) {
   if (nrows <= 1) return HM_OK;
   ScatterFn scatter = scatter_for(width);
   if (!scatter || nkey < 1 || nkey > kMaxKeyCols) return HM_ERR_ARG;
@@ -1079,7 +1083,7 @@ hm_status radix_sort_rows_cols(int32_t *rows, int32_t *tmp, int64_t nrows, int w
   if (width == 4 && nrows >= kFusedMinRows &&
       (((reinterpret_cast<uintptr_t>(rows) | reinterpret_cast<uintptr_t>(tmp)) & 15u) == 0)) {
     bool ran = false;
-    const hm_status fs = sort4_fused(rows, tmp, nrows, ks, passes, stream, &ran);
+    const hm_status fs = sort4_fused(rows, tmp, nrows, ks, passes, stream, &ran, err);
     if (fs != HM_OK) return fs;
     if (ran) {
       if (launches) *launches = 1;
