@@ -225,44 +225,47 @@ __device__ __forceinline__ int32_t search_c(const int32_t *__restrict__ a, int32
 // Every arc (u, v) with label l enters the filter under two keys: the pair
 // (u, v) -- "is there an arc at all", for induced non-arcs and the opposite-arc
 // test -- and the triple (u, v, l) -- "is there an arc with this label", for
-// the pattern's arcs.  A key's two 64-bit hashes are sums A u + B v (+ C (l + 1))
-// with fixed odd constants (multilinear hashing: the upper halves of such sums
-// are pairwise independent over the choice of the constants; Dietzfelbinger,
-// "Universal hashing and k-wise independent random variables via integer
-// arithmetic without primes", STACS 1996).  The constants are the first six
-// splitmix64 outputs from seed 0x243F6A8885A308D3, made odd.  The first sum's
-// upper half chooses a 64-bit word, the second's four bits in it, two in each
-// half.  At 16 bits per key a key that was never inserted passes with
-// probability about 0.5 % (measured on R-MAT arcs); an inserted key always
-// passes.  The sums are linear, so the part of an endpoint that stays the same
-// over many probes is computed once; a probe is about 20 instructions and one
-// 8-byte load.  (A 256-bit block with one bit in each of eight words and a
-// 64-bit finalizer as the hash passed 0.1 % but took about 60 instructions and
-// two loads, and eight atomics per key to build: 286 us for 3.9M arcs, now 43.)
-constexpr uint64_t kHashU1 = 0x2cb0f69f4abea221ull, kHashV1 = 0x9417034723148989ull,
-                   kHashL1 = 0xdd555950609dfe03ull, kHashU2 = 0xdbafb150deb12801ull,
-                   kHashV2 = 0x7e789b2e6c442cb7ull, kHashL2 = 0xf41e5636c7e4f8c5ull;
+// the pattern's arcs.  A key's hash is the sum A u + B v (+ C (l + 1)) modulo
+// 2^64 with fixed odd constants (multilinear hashing: the upper halves of such
+// sums are pairwise independent over the choice of the constants;
+// Dietzfelbinger, "Universal hashing and k-wise independent random variables
+// via integer arithmetic without primes", STACS 1996).  The constants are the
+// first three splitmix64 outputs from seed 0x243F6A8885A308D3, made odd.  The
+// upper half chooses a 64-bit word, and both halves together four bits in it,
+// two in each half.  At 16 bits per key a key that was never inserted passes
+// with probability about 0.5 % (measured on R-MAT arcs; 0.8 % on a lattice);
+// an inserted key always passes.  The sum is linear, so the part of an endpoint
+// that stays the same over many probes is computed once; a probe is then about
+// 20 instructions and one 8-byte load.  (A 256-bit block with one bit in each
+// of eight words and a 64-bit finalizer as the hash passed 0.1 % but took about
+// 60 instructions and two loads, and eight atomics per key to build: 286 us for
+// 3.9M arcs, now 43.)
+constexpr uint64_t kHashU = 0x2cb0f69f4abea221ull, kHashV = 0x9417034723148989ull, kHashL = 0xdd555950609dfe03ull;
 
 struct ArcKey {
-  uint64_t a, b;
+  uint64_t h;
 };
 
 __host__ __device__ __forceinline__ ArcKey pair_key(int32_t u, int32_t v) {
-  return ArcKey{kHashU1 * (uint32_t)u + kHashV1 * (uint32_t)v, kHashU2 * (uint32_t)u + kHashV2 * (uint32_t)v};
+  return ArcKey{kHashU * (uint32_t)u + kHashV * (uint32_t)v};
 }
 
 __host__ __device__ __forceinline__ ArcKey labelled_key(ArcKey k, int32_t lab) {
-  const uint64_t l = (uint64_t)(uint32_t)lab + 1;
-  return ArcKey{k.a + kHashL1 * l, k.b + kHashL2 * l};
+  return ArcKey{k.h + kHashL * ((uint64_t)(uint32_t)lab + 1)};
 }
 
 __host__ __device__ __forceinline__ uint32_t filter_word(ArcKey k, uint32_t nword) {
-  return (uint32_t)(((k.a >> 32) * (uint64_t)nword) >> 32);
+  return (uint32_t)(((k.h >> 32) * (uint64_t)nword) >> 32);
+}
+
+// Both halves of the hash in one word: the bits in the filter word, the bucket of the table.
+__host__ __device__ __forceinline__ uint32_t key_fold(ArcKey k) {
+  return (uint32_t)(k.h >> 32) * 0x9e3779b1u ^ (uint32_t)k.h;
 }
 
 // The key's bits in its word: two in each 32-bit half.
 __host__ __device__ __forceinline__ uint2 filter_bits(ArcKey k) {
-  const uint32_t h = (uint32_t)(k.b >> 32);
+  const uint32_t h = key_fold(k);
   uint2 m;
   m.x = (1u << (h >> 27)) | (1u << ((h >> 22) & 31u));
   m.y = (1u << ((h >> 17) & 31u)) | (1u << ((h >> 12) & 31u));
@@ -328,7 +331,7 @@ __device__ __forceinline__ bool arc_maybe(const DevGraph &G, int32_t u, int32_t 
 // slot (u = -1) ends a probe sequence.  There are as many buckets as arcs
 // (half the slots used), so a lookup nearly always reads one sector.
 __host__ __device__ __forceinline__ uint32_t hash_bucket(ArcKey pair, uint32_t nbkt) {
-  return (uint32_t)(((pair.b >> 32) * (uint64_t)nbkt) >> 32);
+  return (uint32_t)((key_fold(pair) * (uint64_t)nbkt) >> 32);
 }
 
 // Is u -> v an arc?  If so, *lab is its label.

@@ -64,7 +64,7 @@ struct LvCons {
   int8_t q, kind;
   int16_t cls;
   int32_t lab;
-  uint64_t la, lb;  // the label's part of the two hashes of the arc filter
+  uint64_t la;  // the label's part of the arc filter's hash
 };
 
 // What a candidate for one position must satisfy.
@@ -139,7 +139,11 @@ struct LvArgs {
 };
 
 struct LvShared {
-  int4 rec[kLvWarps][32];          // the group's states
+  // the group's states: {first candidate - first position, flags, partial hash of the first probe},
+  // the first four images, and in a batch the pattern
+  int4 rec[kLvWarps][32];
+  int4 img[kLvWarps][32];
+  int32_t pid[kLvWarps][32];
   int2 buf[kLvWarps][kLvBuf];      // {state, candidate}
   int4 fresh[kLvWarps][kLvDrain];  // states of the next level: {first candidate, number, what, parent}
   // values all warps share, and each warp's matches, kept out of the registers of the expansion
@@ -272,11 +276,19 @@ __device__ __forceinline__ int4 lv_range(const LvArgs &A, int p, const int4 &m, 
   return make_int4(lo, best, what | pid << 7, 0);
 }
 
-// The cheap checks: candidate c of the state at mp for position p.
+// What the checks of a state's candidates have in common, in rec[].y: the list,
+// whether there is a positive condition besides the driving one (its probe comes
+// first), whether the candidate is the target of that arc, the driving
+// condition, and the first condition after the probed one.
+__device__ __forceinline__ int32_t lv_flags(int32_t list, bool probe, bool to, int32_t drive, int32_t next) {
+  return list | (probe ? 2 : 0) | (to ? 4 : 0) | drive << 3 | next << 9;
+}
+
+// The cheap checks: candidate c of a state for position p.  o and m are the
+// state's records, mp its images in memory (read beyond the fourth only).
 template <bool kSym>
-__device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan &L, const int32_t *mp, int p,
-                                                int drive, int32_t c, Bytes &none) {
-  const int4 m = lv_images(mp, p);
+__device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan &L, const int4 &o, const int4 &m,
+                                                const int32_t *mp, int p, int32_t c, Bytes &none) {
   if (m.x == c || m.y == c || m.z == c || m.w == c) return false;  // injective
   for (int i = 4; i < p; ++i)
     if (mp[i] == c) return false;
@@ -286,21 +298,23 @@ __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan
     while (g) {
       const int q = __ffs(g) - 1;
       g &= g - 1;
-      if (c <= mp[q]) return false;
+      if (c <= lv_image(m, mp, q)) return false;
     }
     while (l) {
       const int q = __ffs(l) - 1;
       l &= l - 1;
-      if (c >= mp[q]) return false;
+      if (c >= lv_image(m, mp, q)) return false;
     }
   }
-  for (int j = 0; j < L.npos; ++j) {
-    if (j == drive) continue;
+  if (!(o.y & 2)) return true;
+  const uint64_t part = (uint64_t)(uint32_t)o.w << 32 | (uint32_t)o.z;
+  if (!filter_has<false>(A.G, ArcKey{part + (o.y & 4 ? kHashV : kHashU) * (uint32_t)c}, none)) return false;
+  for (int j = o.y >> 9; j < L.npos; ++j) {
+    if (j == (o.y >> 3 & 63)) continue;
     const LvCons cs = L.cons[j];
     const int32_t f = lv_image(m, mp, cs.q);
     ArcKey k = pair_key(cs.kind == kOut ? f : c, cs.kind == kOut ? c : f);
-    k.a += cs.la;
-    k.b += cs.lb;
+    k.h += cs.la;
     if (!filter_has<false>(A.G, k, none)) return false;
   }
   return true;
@@ -663,7 +677,23 @@ __device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int
     }
     const uint32_t total = __shfl_sync(kFull, incl, 31);
     const uint32_t excl = r.y > 0 ? incl - (uint32_t)r.y : 0xffffffffu;
-    rec[lane] = make_int4((int32_t)((uint32_t)r.x - excl), r.z, 0, 0);
+    if (r.y > 0) {
+      const int32_t pid = lv_pid(r.z), drive = lv_drive(r.z), probe = drive == 0 ? 1 : 0;
+      const LevelPlan &L = kBatch ? A.levels[(int64_t)pid * A.kmax + p] : A.level1[p];
+      const int32_t *mp = A.base[p] + ((uint64_t)gi * 32 + lane) * (uint32_t)A.stride[p];
+      const int4 m = lv_images(mp, p);
+      uint64_t part = 0;
+      bool to = false;
+      if (probe < L.npos) {
+        const LvCons cs = L.cons[probe];
+        to = cs.kind == kOut;
+        part = (to ? kHashU : kHashV) * (uint32_t)lv_image(m, mp, cs.q) + cs.la;
+      }
+      rec[lane] = make_int4((int32_t)((uint32_t)r.x - excl), lv_flags(lv_list(r.z), probe < L.npos, to, drive, probe + 1),
+                            (int32_t)(uint32_t)part, (int32_t)(part >> 32));
+      sm.img[warp][lane] = m;
+      if (kBatch) sm.pid[warp][lane] = pid;
+    }
     __syncwarp();
     if (x < G.start || x - G.start >= ((unsigned long long)total + 31) >> 5) {
       // cannot happen (the group's chunks were counted from the same numbers); never spin
@@ -697,10 +727,10 @@ __device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int
       if (total - pos0 > (uint32_t)lane) {
         const int4 o = rec[ow];
         const uint32_t at = (uint32_t)o.x + pos0 + lane;
-        c = __ldg((lv_list(o.y) ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
-        const LevelPlan &L = kBatch ? A.levels[(int64_t)lv_pid(o.y) * A.kmax + p] : A.level1[p];
+        c = __ldg((o.y & 1 ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
+        const LevelPlan &L = kBatch ? A.levels[(int64_t)sm.pid[warp][ow] * A.kmax + p] : A.level1[p];
         const int32_t *mp = A.base[p] + ((uint64_t)gi * 32 + ow) * (uint32_t)A.stride[p];
-        ok = lv_first_checks<kSym>(A, L, mp, p, lv_drive(o.y), c, none);
+        ok = lv_first_checks<kSym>(A, L, o, sm.img[warp][ow], mp, p, c, none);
       }
       const uint32_t bal = __ballot_sync(kFull, ok);
       if (ok) buf[nbuf + __popc(bal & lt)] = make_int2((int32_t)(gi * 32 + ow), c);
@@ -948,9 +978,9 @@ void lv_level(const hm_graph *g, const Plan &P, bool deferred, int p, bool want_
   L.sym_gt = P.sym_gt[p];
   L.sym_lt = P.sym_lt[p];
   for (int j = 0; j < n; ++j) {
-    const ArcKey l = j < npos ? labelled_key(ArcKey{0, 0}, cons[j].lab) : ArcKey{0, 0};
+    const ArcKey l = j < npos ? labelled_key(ArcKey{0}, cons[j].lab) : ArcKey{0};
     L.cons[j] = LvCons{cons[j].q, cons[j].kind, j < npos ? lv_class(g, cons[j].lab, P.vlab[p]) : (int16_t)0,
-                       cons[j].lab, l.a, l.b};
+                       cons[j].lab, l.h};
   }
   // arcs to later positions: one is found missing by the next ranges phase anyway
   L.need_deg = !L.last && P.dout[p] + P.din[p] - npos >= 2;
