@@ -77,7 +77,7 @@ struct LevelPlan {
   int8_t final;           // level 1 of a plan with a deferred position 1: the level that matches it, else 0
   int32_t dout, din;
   uint32_t sym_gt, sym_lt;
-  LvCons cons[kMaxCons];
+  int32_t cons;           // its first condition in the table
 };
 
 // How a pattern's matches are written.
@@ -128,6 +128,7 @@ struct LvArgs {
   int32_t *rows;
   unsigned long long cap;
   const LevelPlan *levels;         // batch: [pattern][kmax]
+  const LvCons *cons;              // batch: the levels' conditions
   const EmitPlan *emit;
   const int8_t *aut;
   unsigned long long *counts;
@@ -136,7 +137,14 @@ struct LvArgs {
   int32_t kmax;                    // levels 1 .. kmax - 1
   EmitPlan emit1;
   LevelPlan level1[kMaxK];
+  LvCons cons1[kMaxK * (kMaxK - 1)];  // two for every pair of positions at most
 };
+
+// Condition j of the level whose plan is L.
+template <bool kBatch>
+__device__ __forceinline__ const LvCons &lv_cons(const LvArgs &A, const LevelPlan &L, int j) {
+  return kBatch ? A.cons[L.cons + j] : A.cons1[L.cons + j];
+}
 
 struct LvShared {
   // the group's states: {first candidate - first position, flags, partial hash of the first probe},
@@ -214,16 +222,18 @@ __device__ __forceinline__ int2 lv_group(const LvArgs &A, const LvCons &cs, int3
 // Has u a neighbour that the deferred position 1 (level plan Z) may take?  The
 // search over the other positions would be for nothing.  With arcs in both
 // directions, the filter is asked if the shorter list has at most 8 entries.
+template <bool kBatch>
 __device__ __forceinline__ bool lv_has_final(const LvArgs &A, const LevelPlan &Z, int32_t u) {
-  if (Z.cons[0].cls < 0) return false;
-  const int2 r = lv_group(A, Z.cons[0], u);
+  const LvCons &c0 = lv_cons<kBatch>(A, Z, 0), &c1 = lv_cons<kBatch>(A, Z, 1);
+  if (c0.cls < 0) return false;
+  const int2 r = lv_group(A, c0, u);
   if (Z.npos < 2 || r.y == 0) return r.y > 0;
-  if (Z.cons[1].cls < 0) return false;
-  const int2 r1 = lv_group(A, Z.cons[1], u);
+  if (c1.cls < 0) return false;
+  const int2 r1 = lv_group(A, c1, u);
   const bool second = r1.y < r.y;
   const int2 w = second ? r1 : r;
   if (w.y > 8) return true;
-  const LvCons &cs = Z.cons[second ? 1 : 0], &other = Z.cons[second ? 0 : 1];
+  const LvCons &cs = second ? c1 : c0, &other = second ? c0 : c1;
   const int32_t *list = cs.kind == kOut ? A.G.gout_adj : A.G.gin_adj;
   Bytes none;
 #pragma unroll 1
@@ -249,12 +259,13 @@ __device__ __forceinline__ int4 lv_range(const LvArgs &A, int p, const int4 &m, 
     const int2 need = kBatch ? A.deg0[pid] : make_int2(A.dout0, A.din0);
     const int4 vi = __ldg(&A.G.vi[HM_AT(A.G, c, A.G.n, kChkVertex)]);
     if (vi.y < need.x || vi.z < need.y) return dead;
-    if (L.final && !lv_has_final(A, kBatch ? A.levels[(int64_t)pid * A.kmax + L.final] : A.level1[L.final], c))
+    if (L.final && !lv_has_final<kBatch>(A, kBatch ? A.levels[(int64_t)pid * A.kmax + L.final] : A.level1[L.final],
+                                         c))
       return dead;
   }
   int32_t best = INT32_MAX, lo = 0, what = 0;
   for (int j = 0; j < L.npos; ++j) {
-    const LvCons cs = L.cons[j];
+    const LvCons cs = lv_cons<kBatch>(A, L, j);
     if (cs.cls < 0) return dead;
     const int2 r = lv_group(A, cs, cs.q == p - 1 ? c : lv_image(m, mp, cs.q));
     if (r.y < best) {
@@ -286,7 +297,7 @@ __device__ __forceinline__ int32_t lv_flags(int32_t list, bool probe, bool to, i
 
 // The cheap checks: candidate c of a state for position p.  o and m are the
 // state's records, mp its images in memory (read beyond the fourth only).
-template <bool kSym>
+template <bool kBatch, bool kSym>
 __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan &L, const int4 &o, const int4 &m,
                                                 const int32_t *mp, int p, int32_t c, Bytes &none) {
   if (m.x == c || m.y == c || m.z == c || m.w == c) return false;  // injective
@@ -311,7 +322,7 @@ __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan
   if (!filter_has<false>(A.G, ArcKey{part + (o.y & 4 ? kHashV : kHashU) * (uint32_t)c}, none)) return false;
   for (int j = o.y >> 9; j < L.npos; ++j) {
     if (j == (o.y >> 3 & 63)) continue;
-    const LvCons cs = L.cons[j];
+    const LvCons cs = lv_cons<kBatch>(A, L, j);
     const int32_t f = lv_image(m, mp, cs.q);
     ArcKey k = pair_key(cs.kind == kOut ? f : c, cs.kind == kOut ? c : f);
     k.h += cs.la;
@@ -321,6 +332,7 @@ __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan
 }
 
 // The exact checks of a candidate that passed the cheap ones.
+template <bool kBatch>
 __device__ __forceinline__ bool lv_exact_checks(const LvArgs &A, const LevelPlan &L, const int32_t *mp, int p, int drive,
                                                 int32_t c, Bytes &none) {
   const int4 m = lv_images(mp, p);
@@ -330,7 +342,7 @@ __device__ __forceinline__ bool lv_exact_checks(const LvArgs &A, const LevelPlan
   }
   for (int j = 0; j < L.ncons; ++j) {
     if (j == drive) continue;
-    const LvCons cs = L.cons[j];
+    const LvCons cs = lv_cons<kBatch>(A, L, j);
     const int32_t f = lv_image(m, mp, cs.q);
     const bool fwd = cs.kind == kOut || cs.kind == kNotOut;
     const int32_t x = fwd ? f : c, y = fwd ? c : f;
@@ -463,7 +475,7 @@ __device__ __forceinline__ int lv_drain(const LvArgs &A, LvShared &sm, int p, in
       pid = lv_pid(r.z);
       mp = A.base[p] + (uint64_t)(uint32_t)sc.x * (uint32_t)A.stride[p];
       ok = verified ||
-           lv_exact_checks(A, kBatch ? A.levels[(int64_t)pid * A.kmax + p] : A.level1[p], mp, p, lv_drive(r.z), sc.y,
+           lv_exact_checks<kBatch>(A, kBatch ? A.levels[(int64_t)pid * A.kmax + p] : A.level1[p], mp, p, lv_drive(r.z), sc.y,
                            none);
     }
     if (kBatch ? true : all_last) {
@@ -685,7 +697,7 @@ __device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int
       uint64_t part = 0;
       bool to = false;
       if (probe < L.npos) {
-        const LvCons cs = L.cons[probe];
+        const LvCons cs = lv_cons<kBatch>(A, L, probe);
         to = cs.kind == kOut;
         part = (to ? kHashU : kHashV) * (uint32_t)lv_image(m, mp, cs.q) + cs.la;
       }
@@ -730,7 +742,7 @@ __device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int
         c = __ldg((o.y & 1 ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
         const LevelPlan &L = kBatch ? A.levels[(int64_t)sm.pid[warp][ow] * A.kmax + p] : A.level1[p];
         const int32_t *mp = A.base[p] + ((uint64_t)gi * 32 + ow) * (uint32_t)A.stride[p];
-        ok = lv_first_checks<kSym>(A, L, o, sm.img[warp][ow], mp, p, c, none);
+        ok = lv_first_checks<kBatch, kSym>(A, L, o, sm.img[warp][ow], mp, p, c, none);
       }
       const uint32_t bal = __ballot_sync(kFull, ok);
       if (ok) buf[nbuf + __popc(bal & lt)] = make_int2((int32_t)(gi * 32 + ow), c);
@@ -957,7 +969,7 @@ void lv_defer(Plan &P) {
 }
 
 // `deferred`: lv_defer has been applied, position 1 is like any other.
-void lv_level(const hm_graph *g, const Plan &P, bool deferred, int p, bool want_rows, LevelPlan &L) {
+void lv_level(const hm_graph *g, const Plan &P, bool deferred, int p, bool want_rows, LevelPlan &L, LvCons *out) {
   std::memset(&L, 0, sizeof(L));
   if (p >= P.k) return;
   Cons cons[kMaxCons];
@@ -979,12 +991,32 @@ void lv_level(const hm_graph *g, const Plan &P, bool deferred, int p, bool want_
   L.sym_lt = P.sym_lt[p];
   for (int j = 0; j < n; ++j) {
     const ArcKey l = j < npos ? labelled_key(ArcKey{0}, cons[j].lab) : ArcKey{0};
-    L.cons[j] = LvCons{cons[j].q, cons[j].kind, j < npos ? lv_class(g, cons[j].lab, P.vlab[p]) : (int16_t)0,
+    out[j] = LvCons{cons[j].q, cons[j].kind, j < npos ? lv_class(g, cons[j].lab, P.vlab[p]) : (int16_t)0,
                        cons[j].lab, l.h};
   }
   // arcs to later positions: one is found missing by the next ranges phase anyway
   L.need_deg = !L.last && P.dout[p] + P.din[p] - npos >= 2;
   L.closed = L.last && !want_rows && npos == 1 && n == 1 && !L.root && !(L.sym_gt | L.sym_lt);
+}
+
+// The vertices the first level starts from: those with position 0's label and a
+// group for a condition of position 1, the shortest such list.
+const int32_t *lv_start(const hm_graph *g, const Plan &P, const LevelPlan &L, const LvCons *cons, int64_t *cnt) {
+  const int64_t lab = (int64_t)P.vlab[0] - g->vl0;
+  const int32_t *list = g->vby_out;
+  *cnt = 0;
+  if (lab < 0 || lab >= g->nvl) return list;
+  *cnt = INT64_MAX;
+  for (int j = 0; j < L.npos; ++j) {
+    const bool in = cons[j].kind == kIn;
+    const uint32_t *b = g->vstart + (in ? g->ncls * g->nvl + 1 : 0) + lab * g->ncls + std::max<int>(cons[j].cls, 0);
+    const int64_t here = cons[j].cls < 0 ? 0 : (int64_t)b[1] - b[0];
+    if (here < *cnt) {
+      *cnt = here;
+      list = (in ? g->vby_in : g->vby_out) + b[0];
+    }
+  }
+  return list;
 }
 
 void lv_emit(const Plan &P, EmitPlan &E, std::vector<int8_t> &aut) {
@@ -996,6 +1028,27 @@ void lv_emit(const Plan &P, EmitPlan &E, std::vector<int8_t> &aut) {
   if (P.naut > 1)
     for (int s = 0; s < P.naut; ++s) aut.insert(aut.end(), P.aut[s], P.aut[s] + kMaxK);
 }
+
+// A thread's page-locked block for what a call reads back: a copy into ordinary
+// memory is staged by the driver (1.5 to 2 us more per call).  Freed
+// when the thread ends.
+struct Landing {
+  static constexpr int32_t kCounts = 4096;
+  struct Block {
+    LvCtl ctl;
+    unsigned long long counts[kCounts];
+  } *p = nullptr;
+  Block *get() {
+    if (!p && cudaMallocHost((void **)&p, sizeof(Block)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      p = nullptr;
+    }
+    return p;
+  }
+  ~Landing() {
+    if (p) cudaFreeHost(p);
+  }
+};
 
 hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result, int *grid_out, int *threads_out,
                      float *ms) {
@@ -1019,6 +1072,7 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   LvArgs A{};
   std::vector<int8_t> aut;
   std::vector<LevelPlan> levels(batch ? (size_t)np * kmax : 0);
+  std::vector<LvCons> conds;
   std::vector<EmitPlan> emit(batch ? np : 0);
   std::vector<unsigned long long> vert_n(batch ? np + 1 : 0);
   std::vector<const int32_t *> vert_at(batch ? np : 0);
@@ -1034,26 +1088,17 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
     }
     const Plan &P = defer ? moved : P0;
     LevelPlan *lv = batch ? &levels[(size_t)i * kmax] : A.level1;
-    for (int p = 1; p < kmax; ++p) lv_level(g, P, defer, p, L.want_rows, lv[p]);
-    lv[1].final = defer ? (int8_t)(P.k - 1) : 0;
-    lv_emit(P, batch ? emit[i] : A.emit1, aut);
-    // the vertices with position 0's label and a group for one of position 1's conditions: the shortest list
-    const int64_t lab = (int64_t)P.vlab[0] - g->vl0;
     const int32_t *list = g->vby_out;
     int64_t cnt = 0;
-    if (lab >= 0 && lab < g->nvl) {
-      cnt = INT64_MAX;
-      for (int j = 0; j < lv[1].npos; ++j) {
-        const LvCons &cs = lv[1].cons[j];
-        const bool in = cs.kind == kIn;
-        const uint32_t *b = g->vstart + (in ? g->ncls * g->nvl + 1 : 0) + lab * g->ncls + std::max<int>(cs.cls, 0);
-        const int64_t here = cs.cls < 0 ? 0 : (int64_t)b[1] - b[0];
-        if (here < cnt) {
-          cnt = here;
-          list = (in ? g->vby_in : g->vby_out) + b[0];
-        }
-      }
+    for (int p = 1; p < std::min(kmax, (int)P.k); ++p) {
+      LvCons c[kMaxCons];
+      lv_level(g, P, defer, p, L.want_rows, lv[p], c);
+      lv[p].cons = (int32_t)conds.size();
+      conds.insert(conds.end(), c, c + lv[p].ncons);
+      if (p == 1) list = lv_start(g, P, lv[1], c, &cnt);
     }
+    lv[1].final = defer ? (int8_t)(P.k - 1) : 0;
+    lv_emit(P, batch ? emit[i] : A.emit1, aut);
     if (batch) {
       vert_n[i] = A.nvert;
       vert_at[i] = list - (int64_t)A.nvert;
@@ -1104,6 +1149,10 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
     at_st[p] = reserve(4 * (size_t)A.stride[p] * 32 * A.gcap[p]);
     if (p < top) at_ps[p] = reserve(sizeof(LvPause) * (size_t)warps);
   }
+  if (!batch) {
+    std::copy(conds.begin(), conds.end(), A.cons1);
+    conds.clear();
+  }
   // a batch's tables, and the automorphisms of symmetric patterns, in one host block and one copy
   size_t at_tab = bytes, tab = 0;
   auto place = [&](size_t n) {
@@ -1111,7 +1160,7 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
     tab += round(n);
     return a;
   };
-  const size_t t_levels = place(sizeof(LevelPlan) * levels.size()), t_emit = place(sizeof(EmitPlan) * emit.size()),
+  const size_t t_levels = place(sizeof(LevelPlan) * levels.size()), t_cons = place(sizeof(LvCons) * conds.size()), t_emit = place(sizeof(EmitPlan) * emit.size()),
                t_vn = place(8 * vert_n.size()), t_va = place(8 * vert_at.size()), t_deg = place(8 * deg0.size()),
                t_aut = place(aut.size());
   std::vector<unsigned char> host(tab);
@@ -1119,6 +1168,7 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
     if (n) std::memcpy(host.data() + a, src, n);
   };
   put(t_levels, levels.data(), sizeof(LevelPlan) * levels.size());
+  put(t_cons, conds.data(), sizeof(LvCons) * conds.size());
   put(t_emit, emit.data(), sizeof(EmitPlan) * emit.size());
   put(t_vn, vert_n.data(), 8 * vert_n.size());
   put(t_va, vert_at.data(), 8 * vert_at.size());
@@ -1144,6 +1194,7 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   A.ctl = reinterpret_cast<LvCtl *>(ws.p);
   unsigned char *t = ws.p + at_tab;
   A.levels = reinterpret_cast<const LevelPlan *>(t + t_levels);
+  A.cons = reinterpret_cast<const LvCons *>(t + t_cons);
   A.emit = reinterpret_cast<const EmitPlan *>(t + t_emit);
   A.vert_n = reinterpret_cast<const unsigned long long *>(t + t_vn);
   A.vert_at = reinterpret_cast<const int32_t *const *>(t + t_va);
@@ -1175,11 +1226,19 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   if (le == cudaSuccess) {
     *ran = true;
     if (ms) cudaEventRecord(ev[1], s);
-    if (cudaMemcpyAsync(result, A.ctl, sizeof(LvCtl), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        (L.counts_host && cudaMemcpyAsync(L.counts_host, L.counts, sizeof(unsigned long long) * L.npat,
-                                          cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
+    static thread_local Landing landing;
+    Landing::Block *l = L.npat <= Landing::kCounts ? landing.get() : nullptr;
+    LvCtl *to = l ? &l->ctl : result;
+    unsigned long long *counts = l ? l->counts : L.counts_host;
+    const size_t nc = L.counts_host ? sizeof(unsigned long long) * L.npat : 0;
+    if (cudaMemcpyAsync(to, A.ctl, sizeof(LvCtl), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        (nc && cudaMemcpyAsync(counts, L.counts, nc, cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
         cudaStreamSynchronize(s) != cudaSuccess)
       st = HM_ERR_CUDA;
+    if (l) {
+      *result = l->ctl;
+      if (nc) std::memcpy(L.counts_host, l->counts, nc);
+    }
     if (ms && st == HM_OK) cudaEventElapsedTime(ms, ev[0], ev[1]);
   }
   (void)cudaGetLastError();  // a launch that was refused: the caller searches depth first

@@ -109,24 +109,30 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   const bool timing = timing_enabled();
   const bool counters = counters_enabled();
   uint32_t launches = 0;
-  Plan plan = p->plan[mode];
+  const hm_tuning tu = tuning();
+  // a copy only where the call changes the plan (17 KB) or searches depth first
+  Plan changed;
+  const bool by_level = g->ncls > 0 && want != Want::kStates && nparts == 1 && default_search(tu) && !counters &&
+                        budget_chunks() == 0;
+  const bool change = root_mask || tu.symmetry < 0 || !by_level;
+  if (change) changed = p->plan[mode];
+  Plan &plan = changed;
   if (root_mask) {
     if (root < 0 || root >= p->k) return HM_ERR_ARG;
     for (int i = 0; i < p->k; ++i)
       if (plan.orig[i] == root) plan.root_pos = i;
     strip_symmetry(plan);  // the root restriction is on one map, not on its orbit
   }
-  if (tuning().symmetry < 0) strip_symmetry(plan);
+  if (tu.symmetry < 0) strip_symmetry(plan);
   const DevGraph G = g->dev();
   const int64_t m = g->m;
-  const hm_tuning tu = tuning();
   const bool rows = want == Want::kRows;
   Scratch sc(s);
   // Default knobs: the whole match level by level (hm_levels.cu).  The
   // depth-first search below keeps the other knobs, the instrumented kernels,
   // chunk budgets, arc-range parts, graphs with too many label classes, and
   // the injected states.
-  if (g->ncls > 0 && want != Want::kStates && nparts == 1 && default_search(tu) && !counters && budget_chunks() == 0) {
+  if (by_level) {
     NvtxRange r_lv("hm.extend");
     LvLaunch L{};
     L.g = g;
@@ -134,7 +140,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
     L.want_rows = rows;
     L.rows = out;
     L.workspace = level_workspace(g);
-    L.plan = &plan;
+    L.plan = change ? &plan : &p->plan[mode];
     L.cap = cap;
     L.defer = tu.share_seeds > 0;
     LvCtl h;
@@ -157,6 +163,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
       return h.count > cap ? HM_ERR_CAPACITY : sort_rows(g, p->k, out, h.count, sc, s, timing, st);
     }
   }
+  if (!change) changed = p->plan[mode];  // the levels could not run
   Ctl *ctl;
   int2 *seeds_a, *seeds_b = nullptr;
   HM_CUDA_TRY(sc.get((void **)&ctl, sizeof(Ctl)));
