@@ -484,6 +484,60 @@ __global__ void k_filter(const int32_t *__restrict__ src, const int32_t *__restr
   }
 }
 
+// The filter by endpoint, from rows sorted by that endpoint (column `key`): the
+// words of consecutive rows lie together, so a block collects those of its tile in
+// shared memory and writes the whole regions out; only the first and the last
+// vertex may go on in another tile and take atomics.  A tile over more words than
+// that (a hub, a run of isolated vertices) sets its bits in memory.  (All bits set
+// in memory added 120 us to the load of 3.9M arcs; this way 16M arcs load in 5.04
+// ms instead of 4.84 without the regions, 150M in 48.0 instead of 48.7.)
+constexpr int kRegionTile = 2048, kRegionWords = 4096;
+
+__global__ void __launch_bounds__(kThreads)
+k_regions(const int4 *__restrict__ rows, int64_t m, int key, const int64_t *__restrict__ off,
+          unsigned long long *__restrict__ words) {
+  __shared__ uint2 s_word[kRegionWords];
+  const int64_t ntile = (m + kRegionTile - 1) / kRegionTile;
+  for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x) {
+    const int64_t first = t * kRegionTile, last = min(m, first + kRegionTile) - 1;
+    const int32_t v0 = key ? rows[first].y : rows[first].x, v1 = key ? rows[last].y : rows[last].x;
+    const Region g0 = region_of(v0, (uint32_t)off[v0], (uint32_t)(off[v0 + 1] - off[v0]));
+    const Region g1 = region_of(v1, (uint32_t)off[v1], (uint32_t)(off[v1 + 1] - off[v1]));
+    const uint32_t span = g1.base + g1.nword - g0.base;
+    const bool local = span <= kRegionWords;
+    if (local)
+      for (uint32_t i = threadIdx.x; i < span; i += blockDim.x) s_word[i] = make_uint2(0, 0);
+    __syncthreads();
+    for (int64_t e = first + threadIdx.x; e <= last; e += blockDim.x) {
+      const int4 r = rows[e];
+      const int32_t v = key ? r.y : r.x;
+      const int64_t o = off[v];
+      const Region g = region_of(v, (uint32_t)o, (uint32_t)(off[v + 1] - o));
+      const ArcKey pair = pair_key(r.x, r.y), both[2] = {pair, labelled_key(pair, r.z)};
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if (local) {
+          const uint2 b = filter_bits(both[k]);
+          uint2 *w = &s_word[g.base - g0.base + filter_word(both[k], g.nword)];
+          atomicOr(&w->x, b.x);
+          atomicOr(&w->y, b.y);
+        } else {
+          filter_insert(both[k], g.nword, words + g.base);
+        }
+      }
+    }
+    __syncthreads();
+    if (local)
+      for (uint32_t i = threadIdx.x; i < span; i += blockDim.x) {
+        const unsigned long long w = s_word[i].x | (unsigned long long)s_word[i].y << 32;
+        unsigned long long *to = words + g0.base + i;
+        if (i >= g0.nword && i < g1.base - g0.base) *to = w;
+        else if (w) atomicOr(to, w);
+      }
+    __syncthreads();
+  }
+}
+
 __global__ void k_hash(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
                        const int32_t *__restrict__ elab, int64_t m, uint32_t nbkt,
                        int4 *__restrict__ table, uint32_t *__restrict__ err) {
@@ -701,6 +755,9 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   const Classes C{g->ncls, g->nvl, g->al0, g->vl0};
   g->afilt_nword = (uint32_t)(4 * std::max<int64_t>(1, (m + 7) / 8));
   g->ahash_nbkt = (uint32_t)std::max<int64_t>(1, m);
+  const int64_t region_words = (m >> 1) + n + 1;
+  g->regions = g->ncls && m >= kRegionArcs;
+  g->rf_nword = g->regions ? (uint32_t)region_words : g->afilt_nword;
   Arena A;
   A.add(&g->src, m);
   A.add(&g->out_adj, m);
@@ -717,8 +774,13 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   if (g->ncls) {
     A.add(&g->gofs_out, (int64_t)n * g->ncls + 1);
     A.add(&g->gofs_in, (int64_t)n * g->ncls + 1);
+    if (g->regions) {
+      A.add(&g->rfilt_out, region_words);
+      A.add(&g->rfilt_in, region_words);
+    }
   }
   HM_CUDA_TRY(A.allocate(g));
+  if (!g->regions) g->rfilt_out = g->rfilt_in = g->afilt;
   HM_CUDA_TRY(cudaMemsetAsync(g->afilt, 0, 8 * (size_t)g->afilt_nword, s));
   HM_CUDA_TRY(cudaMemsetAsync(g->ahash, 0xff, 32 * (size_t)g->ahash_nbkt, s));
 
@@ -755,6 +817,12 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
           k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 1, 0, nullptr, g->in_adj, g->in_elab, in_off, nullptr);
         }
         const int64_t *off = in ? in_off : out_off;
+        if (g->regions) {
+          uint2 *words = in ? g->rfilt_in : g->rfilt_out;
+          HM_CUDA_TRY(cudaMemsetAsync(words, 0, sizeof(uint2) * (size_t)region_words, s));
+          k_regions<<<grid_for(m), kThreads, 0, s>>>(reinterpret_cast<const int4 *>(rows), m, in, off,
+                                                     reinterpret_cast<unsigned long long *>(words));
+        }
         const int32_t *adj = in ? g->in_adj : g->out_adj, *elab = in ? g->in_elab : g->out_elab;
         int32_t *gadj = in ? g->gin_adj : g->gout_adj, *gofs = in ? g->gofs_in : g->gofs_out;
         int32_t *list = hubs + (size_t)in * (m / kHub + 1);
@@ -832,7 +900,9 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   if (h_err & kErrHash) return HM_ERR_CUDA;  // cannot happen (twice as many slots as arcs)
   g->bytes = sizeof(int32_t) * 7 * (size_t)m + (sizeof(int4) * 2 + sizeof(int2)) * (size_t)n +
              sizeof(int4) * (size_t)(g->ndir_out + g->ndir_in) + 8 * (size_t)g->afilt_nword +
-             32 * (size_t)g->ahash_nbkt + (g->ncls ? sizeof(int32_t) * (2 * ((size_t)n * g->ncls + 1) + (size_t)(g->ndir_out + g->ndir_in)) : 0);
+             32 * (size_t)g->ahash_nbkt + (g->ncls ? sizeof(int32_t) * (2 * ((size_t)n * g->ncls + 1) + (size_t)(g->ndir_out + g->ndir_in)) +
+                              (g->regions ? 2 * sizeof(uint2) * (size_t)region_words : 0)
+                        : 0);
   return HM_OK;
 }
 

@@ -148,8 +148,9 @@ __device__ __forceinline__ const LvCons &lv_cons(const LvArgs &A, const LevelPla
 
 struct LvShared {
   // the group's states: {first candidate - first position, flags, partial hash of the first probe},
-  // the first four images, and in a batch the pattern
+  // the first four images, the region of that probe, and in a batch the pattern
   int4 rec[kLvWarps][32];
+  Region reg[kLvWarps][32];
   int4 img[kLvWarps][32];
   int32_t pid[kLvWarps][32];
   int2 buf[kLvWarps][kLvBuf];      // {state, candidate}
@@ -299,7 +300,7 @@ __device__ __forceinline__ int32_t lv_flags(int32_t list, bool probe, bool to, i
 // state's records, mp its images in memory (read beyond the fourth only).
 template <bool kBatch, bool kSym>
 __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan &L, const int4 &o, const int4 &m,
-                                                const int32_t *mp, int p, int32_t c, Bytes &none) {
+                                                const Region &g, const int32_t *mp, int p, int32_t c, Bytes &none) {
   if (m.x == c || m.y == c || m.z == c || m.w == c) return false;  // injective
   for (int i = 4; i < p; ++i)
     if (mp[i] == c) return false;
@@ -319,7 +320,12 @@ __device__ __forceinline__ bool lv_first_checks(const LvArgs &A, const LevelPlan
   }
   if (!(o.y & 2)) return true;
   const uint64_t part = (uint64_t)(uint32_t)o.w << 32 | (uint32_t)o.z;
-  if (!filter_has<false>(A.G, ArcKey{part + (o.y & 4 ? kHashV : kHashU) * (uint32_t)c}, none)) return false;
+  // the fixed endpoint's own words of the filter
+  const ArcKey key{part + (o.y & 4 ? kHashV : kHashU) * (uint32_t)c};
+  const uint2 w = __ldg((o.y & 4 ? A.G.rfilt_out : A.G.rfilt_in) +
+                        HM_AT(A.G, (int64_t)g.base + filter_word(key, g.nword), A.G.rf_nword, kChkRegion));
+  const uint2 b = filter_bits(key);
+  if ((b.x & ~w.x) | (b.y & ~w.y)) return false;
   for (int j = o.y >> 9; j < L.npos; ++j) {
     if (j == (o.y >> 3 & 63)) continue;
     const LvCons cs = lv_cons<kBatch>(A, L, j);
@@ -699,7 +705,15 @@ __device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int
       if (probe < L.npos) {
         const LvCons cs = lv_cons<kBatch>(A, L, probe);
         to = cs.kind == kOut;
-        part = (to ? kHashU : kHashV) * (uint32_t)lv_image(m, mp, cs.q) + cs.la;
+        const int32_t f = lv_image(m, mp, cs.q);
+        part = (to ? kHashU : kHashV) * (uint32_t)f + cs.la;
+        Region g{0, A.G.rf_nword};
+        if (A.G.regions) {
+          const int4 vi = __ldg(&A.G.vi[HM_AT(A.G, f, A.G.n, kChkVertex)]);
+          const int2 off = __ldg(&A.G.off[HM_AT(A.G, f, A.G.n, kChkVertex)]);
+          g = region_of(f, (uint32_t)(to ? off.x : off.y), (uint32_t)(to ? vi.y : vi.z));
+        }
+        sm.reg[warp][lane] = g;
       }
       rec[lane] = make_int4((int32_t)((uint32_t)r.x - excl), lv_flags(lv_list(r.z), probe < L.npos, to, drive, probe + 1),
                             (int32_t)(uint32_t)part, (int32_t)(part >> 32));
@@ -742,7 +756,7 @@ __device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int
         c = __ldg((o.y & 1 ? A.G.gin_adj : A.G.gout_adj) + HM_AT(A.G, at, A.G.m, kChkList));
         const LevelPlan &L = kBatch ? A.levels[(int64_t)sm.pid[warp][ow] * A.kmax + p] : A.level1[p];
         const int32_t *mp = A.base[p] + ((uint64_t)gi * 32 + ow) * (uint32_t)A.stride[p];
-        ok = lv_first_checks<kBatch, kSym>(A, L, o, sm.img[warp][ow], mp, p, c, none);
+        ok = lv_first_checks<kBatch, kSym>(A, L, o, sm.img[warp][ow], sm.reg[warp][ow], mp, p, c, none);
       }
       const uint32_t bal = __ballot_sync(kFull, ok);
       if (ok) buf[nbuf + __popc(bal & lt)] = make_int2((int32_t)(gi * 32 + ow), c);

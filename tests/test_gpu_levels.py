@@ -104,3 +104,35 @@ def test_levels_that_do_not_fit_are_worked_off_in_parts():
     finally:
         srv.close()
     assert min(want) > 0
+
+
+def test_filter_by_endpoint_agrees_with_the_depth_first_search():
+    """From 2^23 arcs on the level search probes words of the fixed vertex's own: hubs, arcs
+    at both ends of the id range, long runs of isolated vertices between, two arc labels."""
+    import paper_2507_04130_gb300 as hm
+
+    rng = np.random.default_rng(12)
+    n, core, m = 400_000, 70_000, (1 << 23) + 999
+    u = rng.integers(0, core, m + 400_000)
+    v = rng.integers(0, core, m + 400_000)
+    u[:20_000], v[:20_000] = 5, np.arange(100, 20_100)
+    u[20_000:40_000], v[20_000:40_000] = np.arange(100, 20_100), 5
+    key = np.unique(np.where(u < core // 2, u, n - core + u) * n + np.where(v < core // 2, v, n - core + v))
+    key = key[key // n != key % n]
+    key = np.sort(rng.permutation(key)[:m])
+    assert key.size == m
+    G = hm.Graph(n, (key // n).astype(np.int32), (key % n).astype(np.int32), rng.integers(0, 2, n).astype(np.int32),
+                 rng.integers(3, 5, m).astype(np.int32))
+    pats = [hm.Pattern.from_synth(p) for p in (
+        _pattern(3, [(0, 1), (1, 2), (2, 0)], [0, 1, 0], [3, 4, 3]),
+        _pattern(3, [(0, 1), (1, 2), (0, 2)], [1, 1, 0], [4, 4, 3]),
+        _pattern(4, [(0, 1), (1, 2), (2, 3), (3, 0), (0, 2)], [0, 1, 1, 0], [3, 3, 4, 4, 3]))]
+    level = [[hm.count_matches(G, p, mode) for mode in (hm.MONO, hm.INDUCED)] for p in pats]
+    batch = [hm.count_batch(G, pats, mode) for mode in (hm.MONO, hm.INDUCED)]
+    hm.set_tuning(seeds_per_fetch=2)
+    try:
+        deep = [[hm.count_matches(G, p, mode) for mode in (hm.MONO, hm.INDUCED)] for p in pats]
+    finally:
+        hm.set_tuning()
+    assert level == deep and [list(c) for c in zip(*batch)] == deep
+    assert min(c for c, _ in deep) > 0
