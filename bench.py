@@ -96,11 +96,11 @@ def hbm_peak():
         return FALLBACK_HBM_GBS, "fallback (6.8 TB/s)"
 
 
-def kernel_source_hash():
-    """Hash of the sources that define k_extend's launches: its header, the shared device
+def kernel_source_hash(kernel="k_extend"):
+    """Hash of the sources that define the search kernel's launches: its file, the shared device
     helpers, and the single-pattern orchestration that picks the variant and its states."""
     h = hashlib.sha256()
-    for name in ("hm_kernels.cuh", "hm_internal.cuh", "hm_match.cu"):
+    for name in ("hm_levels.cu" if kernel == "k_levels" else "hm_kernels.cuh", "hm_internal.cuh", "hm_match.cu"):
         with open(os.path.join(ROOT, "paper_2507_04130_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -114,7 +114,7 @@ def committed_traffic(kernel, workload_key):
     text = open(path).read()
     src = re.search(r"kernel_source_sha256:\s*([0-9a-f]+)", text)
     per = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", text)
-    if not src or not per or src.group(1) != kernel_source_hash():
+    if not src or not per or src.group(1) != kernel_source_hash(kernel):
         return None
     return float(per.group(1))
 
@@ -338,9 +338,14 @@ def run_gpu(args):
     mean_ovl = [statistics.mean(x) for x in ovl_ms]
     mean_sort = [statistics.mean(x) for x in sort_ms]
     achieved_ext = sum(bytes_ext) / (sum(mean_ext) / 1e3) / 1e9
-    achieved_edge = sum(bytes_edge) / (sum(mean_edge) / 1e3) / 1e9
+    # the level-by-level search has no edge scan of its own; its bytes are the
+    # depth-first search's cost model (the instrumented pass runs that one), so
+    # what it requests itself is not counted
+    by_level = sum(mean_edge) == 0
+    search = "k_levels" if by_level else "k_extend"
+    achieved_edge = None if by_level else round(sum(bytes_edge) / (sum(mean_edge) / 1e3) / 1e9, 2)
     workload_key = f"rmat{args.scale}"
-    traffic = committed_traffic("k_extend", workload_key)
+    traffic = committed_traffic(search, workload_key)
     kbits = max(1, (g.n - 1).bit_length())
     # the row sort: a stable LSD radix sort of the k-word rows, 10 key bits per
     # pass; its inherent traffic is one read and one write of the rows per pass
@@ -354,24 +359,24 @@ def run_gpu(args):
     def frac_of(b, ms):
         return round(b / (ms / 1e3) / 1e9 / peak, 4) if ms > 0 else None
 
-    req_frac_ext = sum(req_ext) / (sum(mean_ext) / 1e3) / 1e9 / peak
+    req_frac_ext = None if by_level else round(sum(req_ext) / (sum(mean_ext) / 1e3) / 1e9 / peak, 4)
     roofline = {
-        "bound": "hbm", "kernel": "k_extend", "achieved": round(achieved_ext, 2), "peak": peak,
+        "bound": "hbm", "kernel": search, "achieved": round(achieved_ext, 2), "peak": peak,
         "unit": "GB/s", "frac": round(achieved_ext / peak, 4),
         "traffic": traffic, "peak_source": peak_src,
         "algorithmic_bytes_per_launch": [int(b) for b in bytes_ext],
         "algorithmic_bytes": ("the survey's cost model, counted by the instrumented launch: 8 B per candidate "
                               "read, ceil(log2(d+1)) x 4 B per membership or non-arc test over the shorter "
                               "list, 4 B per surviving candidate, 8 B per state, 4k B per row"),
-        "requested_bytes_per_launch": [int(b) for b in req_ext],
-        "requested_frac": round(req_frac_ext, 4),
+        "requested_bytes_per_launch": None if by_level else [int(b) for b in req_ext],
+        "requested_frac": req_frac_ext,
         "mean_launch_ms": [round(x, 4) for x in mean_ext],
         "kernels": {
-            "k_extend": {"ms_per_step": round(sum(mean_ext), 4), "GBps": round(achieved_ext, 2),
-                         "frac": round(achieved_ext / peak, 4), "requested_frac": round(req_frac_ext, 4),
-                         "dram_bytes_per_launch": traffic},
-            "k_edge_seed": {"ms_per_step": round(sum(mean_edge), 4), "GBps": round(achieved_edge, 2),
-                            "frac": round(achieved_edge / peak, 4),
+            search: {"ms_per_step": round(sum(mean_ext), 4), "GBps": round(achieved_ext, 2),
+                     "frac": round(achieved_ext / peak, 4), "requested_frac": req_frac_ext,
+                     "dram_bytes_per_launch": traffic},
+            "k_edge_seed": {"ms_per_step": round(sum(mean_edge), 4), "GBps": achieved_edge,
+                            "frac": frac_of(sum(bytes_edge), sum(mean_edge)),
                             "algorithmic_bytes_per_launch": bytes_edge,
                             "requested_bytes_per_launch": req_edge,
                             "requested_frac": frac_of(sum(req_edge), sum(mean_edge)),
@@ -577,7 +582,7 @@ def measure_batched(hm, G, torch, peak, reps=3):
                          "requested_bytes": int(cs["bytes_extend"]),
                          "GBps": rate(cs["model_bytes_extend"], ph["ms_extend"]),
                          "frac": frac(cs["model_bytes_extend"], ph["ms_extend"]),
-                         "requested_frac": frac(cs["bytes_extend"], ph["ms_extend"])},
+                         "requested_frac": frac(cs["bytes_extend"], ph["ms_extend"]) if ph["ms_edge_scan"] else None},
         "batch_sort": {"ms": round(ph["ms_sort"], 4), "algorithmic_bytes": sort_bytes,
                        "GBps": rate(sort_bytes, ph["ms_sort"]), "frac": frac(sort_bytes, ph["ms_sort"]),
                        "bytes": (f"{passes} passes of 10 key bits, one read + one write of the "
@@ -927,7 +932,8 @@ def _time_query(hm, G, P, mode, rows, reps, flush):
     return c, {
         "ms": _fig(tot[1:]), "ms_extend": _fig(ext), "ms_edge_scan": _fig(edge), "ms_sort": _fig(srt[1:]),
         "k_extend_GBps": round(st["model_bytes_extend"] / (statistics.mean(ext) / 1e3) / 1e9, 1) if statistics.mean(ext) else None,
-        "k_extend_requested_GBps": round(st["bytes_extend"] / (statistics.mean(ext) / 1e3) / 1e9, 1) if statistics.mean(ext) else None,
+        "k_extend_requested_GBps": (round(st["bytes_extend"] / (statistics.mean(ext) / 1e3) / 1e9, 1)
+                                    if statistics.mean(ext) and any(edge) else None),
         "k_edge_seed_GBps": round((st["model_bytes_edge_scan"] + st["model_bytes_overlap"]) / (statistics.mean(edge) / 1e3) / 1e9, 1)
         if statistics.mean(edge) else None,
     }
