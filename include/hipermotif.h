@@ -80,11 +80,17 @@ const char *hm_status_str(hm_status s);
  * by (dst, src), each with its arc labels, the CSR-order source array, and per
  * vertex {label, out-degree, in-degree} and {out-offset, in-offset}; copies
  * of both lists grouped by (arc label, neighbour label) with a directory; an
- * arc filter (split-block Bloom filter keyed by (u, v) and (u, v, label), 32
- * bits per arc) and an arc hash table (32 bytes per arc) that replace the
+ * arc filter (Bloom filter of 64-bit words keyed by (u, v) and (u, v, label),
+ * 32 bits per arc) and an arc hash table (32 bytes per arc) that replace the
  * paper's O(log d) edge-attribute lookup by one or two cache-sector reads.
+ * With at most 64 classes (arc labels x vertex labels, counted over the span
+ * of the label values) also the dense start of every group, the vertices that
+ * have each group, and from 2^23 arcs on the filter once by source and once by
+ * target.
  * Device memory: 64 bytes per arc, 16 per directory entry (at most 2 per arc)
- * and 40 per vertex (hm_graph_info reports the total).
+ * and 40 per vertex; with the dense starts 4 more per directory entry and 8 per
+ * vertex and class; with the filters by endpoint 8 more per arc and 16 per
+ * vertex (hm_graph_info reports the total).
  * The input arrays are copied; the caller keeps ownership.  m must be below
  * 2^31.  Errors: HM_ERR_ARG (id out of range, n or m negative, m >= 2^31,
  * NULL array),
@@ -372,7 +378,8 @@ hm_status hm_count_matches_static(const hm_graph *g, const hm_pattern *p, hm_mod
  * Work budget (watchdog).  Every extension kernel stops when either limit is
  * reached and the call returns HM_ERR_BUDGET:
  *   max_ms      wall-clock limit per kernel (0 = default, 120000 ms);
- *   max_chunks  limit on 32-candidate chunks examined per call (0 = none).
+ *   max_chunks  limit on 32-candidate chunks examined per call (0 = none; with
+ *               a limit, calls search depth first).
  * Process-wide setting; takes effect for calls that start afterwards.
  * ------------------------------------------------------------------------ */
 hm_status hm_set_budget(uint64_t max_ms, uint64_t max_chunks);
@@ -380,6 +387,11 @@ hm_status hm_set_budget(uint64_t max_ms, uint64_t max_chunks);
 /* ------------------------------------------------------------------------
  * Launch knobs of the extension kernel (process-wide; read by calls that
  * start afterwards).  None of them changes any result, only speed.
+ * With their defaults (symmetry and share_seeds may be set either way) a call
+ * on a graph with at most 64 classes is worked off level by level in one
+ * launch, where only those two have a meaning.  Any other setting, a chunk
+ * budget, the byte counters, an arc-range part, or more classes choose the
+ * depth-first search, which the rest is about.
  *   extend_min_blocks  resident 256-thread blocks per SM the kernel is
  *                      compiled for: 4 (default, 64 registers per thread),
  *                      5 or 6 (fewer registers, more warps to hide load
@@ -498,16 +510,21 @@ hm_status hm_autotune_cached(const hm_graph *g, const hm_pattern *const *pattern
  * by CUDA events on the call's stream and its duration is reported here.
  * ------------------------------------------------------------------------ */
 typedef struct {
-  uint64_t seeds_scanned;   /* target arcs scanned by the edge kernel       */
-  uint64_t states_injected; /* depth-2 states after both validators         */
+  uint64_t seeds_scanned;   /* target arcs scanned by the edge kernel (level
+                             * by level: the target's arcs, which the launch
+                             * covers without a scan)                       */
+  uint64_t states_injected; /* depth-2 states after both validators; level by
+                             * level the states with two mapped positions,
+                             * which no neighbour-overlap test has thinned  */
   uint64_t tasks_donated;   /* work items split off for idle warps          */
   uint64_t chunks;          /* 32-candidate chunks examined                 */
   uint64_t matches;         /* the count of the call                        */
-  float ms_edge_scan;       /* edge scan + validators                       */
+  float ms_edge_scan;       /* edge scan + validators (0 level by level)    */
   float ms_overlap;         /* neighbour-overlap part of the edge validator,
                              * plus the seed grouping of shared position-0
                              * states (share_seeds)                         */
-  float ms_extend;          /* persistent extension kernel                  */
+  float ms_extend;          /* persistent extension kernel; level by level
+                             * the whole search                             */
   float ms_sort;            /* row sort (enumerate only)                    */
   int32_t extend_grid;      /* blocks of the extension launch               */
   int32_t extend_block;     /* threads per block                            */

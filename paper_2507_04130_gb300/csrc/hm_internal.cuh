@@ -15,8 +15,9 @@
 //   ahash    int4[2*H] arc hash table: H = m buckets of two 16-byte slots
 //                      {u, v, label, 0} (32 bytes per arc, half the slots used)
 // A vertex's label and both degrees arrive in one 16-byte load, its list
-// offsets in a second one.  The label-grouped lists and their directory
-// (gout_adj, gin_adj, gdir_out, gdir_in, vdir) are described with DevGraph.
+// offsets in a second one.  The label-grouped lists, their directory and dense
+// offsets (gout_adj, gin_adj, gdir_out, gdir_in, vdir, gofs_out, gofs_in) and the
+// filter by endpoint (rfilt_out, rfilt_in) are described with DevGraph.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -50,7 +51,7 @@ struct DevGraph {
   const int4 *gdir_out;  // {arc label, neighbour label, first, end} (relative to the list start)
   const int4 *gdir_in;
   const int4 *vdir;      // {first out entry, out entries, first in entry, in entries}
-  // split-block Bloom filter over the arcs, keyed by (u, v) and by (u, v,
+  // Bloom filter over the arcs, one word per key, keyed by (u, v) and by (u, v,
   // label): a "no" is exact, a "maybe" needs the search.  Searches over more
   // than filt_min entries probe it first (filt_min < 0: never).
   const uint2 *afilt;
