@@ -4,7 +4,7 @@
 // arc-to-source array so that both endpoints of an arc are O(1) away, with
 // attributes in contiguous arrays and O(log d) edge-attribute lookup in
 // sorted adjacency (Sec. III-D).  Here the same storage is built on the GPU
-// from an arc list, plus one addition for the extension kernel:
+// from an arc list, plus what the search kernels look up:
 //   1. pack rows (src, dst, label, aux), check ids / self-loops, and find
 //      the label ranges                                         (k_pack, k_bounds)
 //   2. stable radix sort by (src, dst); split into src / out_adj / out_elab,
@@ -16,7 +16,8 @@
 //   5. a directory with one entry per (vertex, class) group, and the vertices
 //      of each (vertex label, class)            (k_group_dirs, k_class_place)
 //   6. per-vertex records {label, degrees}, {offsets}, {directory spans}
-//   7. the arc filter: every arc sets its bits under two keys       (k_filter)
+//   7. the arc filter: every arc sets its bits under two keys       (k_filter);
+//      with at least 2^23 arcs also by source and by target         (k_regions)
 //   8. the arc hash table: every arc claims a slot                  (k_hash)
 // With more than 64 classes steps 3-5 sort the rows by (key, arc label,
 // neighbour label) instead and read groups off the sorted rows (build_groups).
