@@ -56,6 +56,10 @@ constexpr int kLvDrain = 64;      // checked when this many wait (a chunk adds a
 constexpr int kLvChunkBits = 40;  // of a level's counter; the groups are above
 constexpr unsigned long long kLvChunkMask = (1ull << kLvChunkBits) - 1;
 constexpr int64_t kLvMaxGroups = 1 << 20;  // of a level (2^24 would fit the counter)
+// A group's candidates are numbered in 32 bits while it is expanded, and 32 states
+// on a hub of 2^27 arcs have 2^32: where the sum reaches this, every state
+// becomes a group of its own (a list has less than 2^31 entries).
+constexpr unsigned long long kLvGroupCands = 1ull << 31;
 constexpr uint64_t kLvBarrierNs = 10ull * 1000 * 1000 * 1000;
 
 // A condition of a level: Cons with the class (arc label, vertex label) whose
@@ -87,8 +91,9 @@ struct EmitPlan {
   int32_t orig[kMaxK];
 };
 
-// A group of states: its first chunk and its number of states.  Its states are
-// those numbered from 32 times the group's number on.
+// A group of states: its first chunk and its number of states (up to 32, with
+// fewer than kLvGroupCands candidates in all).  Its states are those numbered
+// from 32 times the group's number on.
 struct LvGroup {
   unsigned long long start;
   uint32_t n, pad;
@@ -407,9 +412,30 @@ __device__ __noinline__ bool lv_append(const LvArgs &A, LvShared &sm, int p, con
     t0 += __shfl_xor_sync(kFull, t0, o);
     t1 += __shfl_xor_sync(kFull, t1, o);
   }
-  t0 = (t0 + 31) >> 5;
-  t1 = (t1 + 31) >> 5;
-  const int ng = n > 32 ? 2 : 1;
+  const bool apart = t0 >= kLvGroupCands || t1 >= kLvGroupCands;  // the same in every lane
+  int ng = n > 32 ? 2 : 1;
+  unsigned long long c0 = 0, c1 = 0;  // apart: chunks before this lane's states
+  if (apart) {
+    const unsigned long long own0 = lane < n ? ((uint32_t)fresh[lane].y + 31u) >> 5 : 0u;
+    const unsigned long long own1 = lane + 32 < n ? ((uint32_t)fresh[lane + 32].y + 31u) >> 5 : 0u;
+    c0 = own0;
+    c1 = own1;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long a = __shfl_up_sync(kFull, c0, o), b = __shfl_up_sync(kFull, c1, o);
+      if (lane >= o) {
+        c0 += a;
+        c1 += b;
+      }
+    }
+    t0 = __shfl_sync(kFull, c0, 31);
+    t1 = __shfl_sync(kFull, c1, 31);
+    c0 -= own0;
+    c1 += t0 - own1;
+    ng = n;
+  } else {
+    t0 = (t0 + 31) >> 5;
+    t1 = (t1 + 31) >> 5;
+  }
   const unsigned long long add = ((unsigned long long)ng << kLvChunkBits) + t0 + t1;
   unsigned long long at = 0;
   int fits = 0;
@@ -424,7 +450,10 @@ __device__ __noinline__ bool lv_append(const LvArgs &A, LvShared &sm, int p, con
   at = __shfl_sync(kFull, at, 0);
   const uint32_t g0 = (uint32_t)(at >> kLvChunkBits);
   const unsigned long long chunk = at & kLvChunkMask;
-  if (lane < ng) {
+  if (apart) {
+    if (lane < n) A.grp[p][g0 + lane] = LvGroup{chunk + c0, 1u, 0u};
+    if (lane + 32 < n) A.grp[p][g0 + lane + 32] = LvGroup{chunk + c1, 1u, 0u};
+  } else if (lane < ng) {
     LvGroup g;
     g.start = lane ? chunk + t0 : chunk;
     g.n = lane ? n - 32 : min(n, 32);
@@ -432,7 +461,7 @@ __device__ __noinline__ bool lv_append(const LvArgs &A, LvShared &sm, int p, con
     A.grp[p][g0 + lane] = g;
   }
   for (int e = lane; e < n; e += 32) {
-    const uint64_t slot = (uint64_t)g0 * 32 + e;
+    const uint64_t slot = apart ? (uint64_t)(g0 + e) * 32 : (uint64_t)g0 * 32 + e;
     const int4 f = fresh[e];
     const int32_t c = buf[e].y;
     A.rng[p][slot] = make_int4(f.x, f.y, f.z, 0);
@@ -722,7 +751,7 @@ __device__ __forceinline__ uint32_t lv_expand(const LvArgs &A, LvShared &sm, int
     }
     __syncwarp();
     if (x < G.start || x - G.start >= ((unsigned long long)total + 31) >> 5) {
-      // cannot happen (the group's chunks were counted from the same numbers); never spin
+      // cannot happen (the group's chunks were counted from the same numbers, whose sum fits 32 bits); never spin
       if (lane == 0) atomicCAS(&A.ctl->status, 0, kStatQueue);
       return look;
     }
@@ -1147,7 +1176,8 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   for (int p = 2; p <= top; ++p)
     A.gcap[p] = (uint32_t)std::max<uint64_t>(std::min(most, L.workspace / 8 * 5 / per_group), 64);
   A.fill_warps = std::min((uint32_t)warps, A.gcap[1] / 2);  // each may leave a group that is not full
-  A.slice = (uint64_t)(A.gcap[1] - A.fill_warps) * 32;
+  // a slice's states fit whatever their candidates: one group each where 32 lists could exceed a group's sum
+  A.slice = (uint64_t)(A.gcap[1] - A.fill_warps) * (32ull * g->maxdeg >= kLvGroupCands ? 1 : 32);
   auto round = [](size_t b) { return (b + 255) / 256 * 256; };
   size_t bytes = round(sizeof(LvCtl));
   size_t at_rng[kMaxK + 1] = {}, at_grp[kMaxK + 1] = {}, at_ps[kMaxK + 1] = {}, at_st[kMaxK + 1] = {};
