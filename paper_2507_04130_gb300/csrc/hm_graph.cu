@@ -109,11 +109,20 @@ __device__ __forceinline__ void fill_gap(const int32_t *__restrict__ rows, int c
     for (int64_t v = (int64_t)cur + 1; v <= n; ++v) off[v] = m;
 }
 
+// The sorts of a load whose barriers may give up (radix_sort_rows_cols with `err`)
+// leave it to the host to ask once, behind all of them.  Until then the rows may be in
+// any order, or partly not written at all, and so may what was made of them: every
+// kernel that takes an index from either looks at the word first and does nothing
+// once it is set (one load per thread; reading it back on the host after each sort
+// would stop the launches twice).
+__device__ __forceinline__ bool sort_failed(const int *err) { return *(const volatile int *)err != 0; }
+
 // Split rows sorted by (key, other): adj = other column, lab = arc label, offsets on key.
 __global__ void k_split(const int32_t *__restrict__ rows, int64_t m, int32_t n, int key, int other,
                         int32_t *__restrict__ src_out, int32_t *__restrict__ adj,
                         int32_t *__restrict__ lab, int64_t *__restrict__ off,
-                        uint32_t *__restrict__ err) {
+                        uint32_t *__restrict__ err, const int *sort_err) {
+  if (sort_failed(sort_err)) return;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
     int32_t a = rows[kW * e + key], b = rows[kW * e + other];
@@ -251,7 +260,8 @@ __global__ void __launch_bounds__(kThreads)
 k_group_lists(const int64_t *__restrict__ off, const int32_t *__restrict__ adj, const int32_t *__restrict__ elab,
               const int32_t *__restrict__ vlab, int32_t n, int64_t m, Classes C, int32_t *__restrict__ gadj,
               int32_t *__restrict__ gofs, uint32_t *__restrict__ ngroup, int32_t *__restrict__ hubs,
-              uint32_t *__restrict__ nhub) {
+              uint32_t *__restrict__ nhub, const int *sort_err) {
+  if (sort_failed(sort_err)) return;
   __shared__ uint32_t s_cnt[kThreads / 32][64];
   const int lane = threadIdx.x & 31;
   uint32_t *cnt = s_cnt[threadIdx.x >> 5];
@@ -302,7 +312,9 @@ k_group_lists(const int64_t *__restrict__ off, const int32_t *__restrict__ adj, 
 __global__ void __launch_bounds__(1024)
 k_group_hubs(const int64_t *__restrict__ off, const int32_t *__restrict__ adj, const int32_t *__restrict__ elab,
              const int32_t *__restrict__ vlab, Classes C, int32_t *__restrict__ gadj, int32_t *__restrict__ gofs,
-             uint32_t *__restrict__ ngroup, const int32_t *__restrict__ hubs, const uint32_t *__restrict__ nhub) {
+             uint32_t *__restrict__ ngroup, const int32_t *__restrict__ hubs, const uint32_t *__restrict__ nhub,
+             const int *sort_err) {
+  if (sort_failed(sort_err)) return;
   __shared__ uint32_t s_cnt[32][64], s_all[64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t *cnt = s_cnt[warp];
@@ -476,7 +488,8 @@ __device__ __forceinline__ void filter_insert(ArcKey k, uint32_t nword, unsigned
 
 __global__ void k_filter(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
                          const int32_t *__restrict__ elab, int64_t m, uint32_t nword,
-                         unsigned long long *__restrict__ words) {
+                         unsigned long long *__restrict__ words, const int *sort_err) {
+  if (sort_failed(sort_err)) return;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
     const ArcKey h = pair_key(src[e], dst[e]);
@@ -496,7 +509,8 @@ constexpr int kRegionTile = 2048, kRegionWords = 4096;
 
 __global__ void __launch_bounds__(kThreads)
 k_regions(const int4 *__restrict__ rows, int64_t m, int key, const int64_t *__restrict__ off,
-          unsigned long long *__restrict__ words) {
+          unsigned long long *__restrict__ words, const int *sort_err) {
+  if (sort_failed(sort_err)) return;
   __shared__ uint2 s_word[kRegionWords];
   const int64_t ntile = (m + kRegionTile - 1) / kRegionTile;
   for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x) {
@@ -541,7 +555,8 @@ k_regions(const int4 *__restrict__ rows, int64_t m, int key, const int64_t *__re
 
 __global__ void k_hash(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
                        const int32_t *__restrict__ elab, int64_t m, uint32_t nbkt,
-                       int4 *__restrict__ table, uint32_t *__restrict__ err) {
+                       int4 *__restrict__ table, uint32_t *__restrict__ err, const int *sort_err) {
+  if (sort_failed(sort_err)) return;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int32_t u = src[e], v = dst[e];
@@ -793,18 +808,19 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   uint32_t *oidx = nullptr, *iidx = nullptr;
   std::vector<uint32_t> h_bins;
   const int nbin = g->ncls * g->nvl;
-  int *sort_err = reinterpret_cast<int *>(err + 1);  // looked at when the load is done
+  int *sort_err = reinterpret_cast<int *>(err + 1);  // looked at by the kernels behind the sorts, then by the host
   if (m) {
     const int by_src[2] = {0, 1}, by_dst[2] = {1, 0}, bits[2] = {nbits, nbits};
     const uint32_t xr[2] = {0u, 0u};
-    hm_status st = radix_sort_rows_cols(rows, tmp, m, kW, by_src, bits, xr, 2, s, nullptr, sort_err);
+    // (build_groups' kernels do not look at it: without dense offsets each sort is waited for)
+    hm_status st = radix_sort_rows_cols(rows, tmp, m, kW, by_src, bits, xr, 2, s, nullptr, g->ncls ? sort_err : nullptr);
     if (st != HM_OK) return st;
     k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 0, 1, g->src, g->out_adj, g->out_elab,
-                                             out_off, err);
+                                             out_off, err, sort_err);
     k_filter<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->afilt_nword,
-                                              reinterpret_cast<unsigned long long *>(g->afilt));
+                                              reinterpret_cast<unsigned long long *>(g->afilt), sort_err);
     k_hash<<<grid_for(m), kThreads, 0, s>>>(g->src, g->out_adj, g->out_elab, m, g->ahash_nbkt,
-                                            g->ahash, err);
+                                            g->ahash, err, sort_err);
     if (g->ncls) {
       // counts and cursors of both directions are zero; the starts follow them
       HM_CUDA_TRY(cudaMemsetAsync(err + 2, 0, sizeof(uint32_t) * (2 + 4 * (size_t)(nbin + 1)), s));
@@ -815,23 +831,24 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
           // the rows are in (src, dst) order: sorted by dst alone they are in (dst, src) order
           st = radix_sort_rows_cols(rows, tmp, m, kW, by_dst, bits, xr, 1, s, nullptr, sort_err);
           if (st != HM_OK) return st;
-          k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 1, 0, nullptr, g->in_adj, g->in_elab, in_off, nullptr);
+          k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 1, 0, nullptr, g->in_adj, g->in_elab, in_off, nullptr,
+                                                   sort_err);
         }
         const int64_t *off = in ? in_off : out_off;
         if (g->regions) {
           uint2 *words = in ? g->rfilt_in : g->rfilt_out;
           HM_CUDA_TRY(cudaMemsetAsync(words, 0, sizeof(uint2) * (size_t)region_words, s));
           k_regions<<<grid_for(m), kThreads, 0, s>>>(reinterpret_cast<const int4 *>(rows), m, in, off,
-                                                     reinterpret_cast<unsigned long long *>(words));
+                                                     reinterpret_cast<unsigned long long *>(words), sort_err);
         }
         const int32_t *adj = in ? g->in_adj : g->out_adj, *elab = in ? g->in_elab : g->out_elab;
         int32_t *gadj = in ? g->gin_adj : g->gout_adj, *gofs = in ? g->gofs_in : g->gofs_out;
         int32_t *list = hubs + (size_t)in * (m / kHub + 1);
         uint32_t *ng = ngroup + (size_t)in * (n + 1);
         k_group_lists<<<grid_for(32 * (int64_t)n), kThreads, 0, s>>>(off, adj, elab, d_vlab, n, m, C, gadj, gofs,
-                                                                     ng, list, nhub + in);
+                                                                     ng, list, nhub + in, sort_err);
         k_group_hubs<<<(unsigned)std::min<int64_t>(m / kHub + 1, num_sms()), 1024, 0, s>>>(
-            off, adj, elab, d_vlab, C, gadj, gofs, ng, list, nhub + in);
+            off, adj, elab, d_vlab, C, gadj, gofs, ng, list, nhub + in, sort_err);
       }
       st = exclusive_scan_u32(ngroup, didx, 2 * ((int64_t)n + 1), s);
       if (st != HM_OK) return st;
@@ -839,7 +856,10 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
       iidx = didx + (n + 1);
       HM_CUDA_TRY(cudaMemcpyAsync(&total[0], oidx + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
       HM_CUDA_TRY(cudaMemcpyAsync(&total[1], iidx + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+      int failed = 0;
+      HM_CUDA_TRY(cudaMemcpyAsync(&failed, sort_err, sizeof(int), cudaMemcpyDeviceToHost, s));
       HM_CUDA_TRY(cudaStreamSynchronize(s));
+      if (failed) return HM_ERR_CUDA;  // the totals mean nothing
       total[1] -= total[0];
       g->ndir_out = total[0];
       g->ndir_in = total[1];
@@ -856,7 +876,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
       st = radix_sort_rows(rows, tmp, m, kW, by_dst, 2, nbits, s);
       if (st != HM_OK) return st;
       k_split<<<grid_for(m), kThreads, 0, s>>>(rows, m, n, 1, 0, nullptr, g->in_adj, g->in_elab,
-                                               in_off, nullptr);
+                                               in_off, nullptr, sort_err);
       st = build_groups(rows, tmp, m, n, 1, 0, d_vlab, in_off, nbits, be, xe, bv, xv, s, T,
                         g->gin_adj, g, &g->gdir_in, &g->ndir_in, &iidx);
       if (st != HM_OK) return st;
@@ -884,13 +904,10 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     HM_CUDA_TRY(cudaMemcpyAsync(h_bins.data(), bins + 4 * (nbin + 1), sizeof(uint32_t) * h_bins.size(),
                                 cudaMemcpyDeviceToHost, s));
   }
-  uint32_t h_errs[2] = {0, 0};
-  HM_CUDA_TRY(cudaMemcpyAsync(h_errs, err, sizeof(h_errs), cudaMemcpyDeviceToHost, s));
+  HM_CUDA_TRY(cudaMemcpyAsync(&h_err, err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaMemcpyAsync(&hb, bnd, sizeof(Bounds), cudaMemcpyDeviceToHost, s));
   HM_CUDA_TRY(cudaStreamSynchronize(s));
   HM_CUDA_TRY(cudaGetLastError());
-  h_err = h_errs[0];
-  if (h_errs[1]) return HM_ERR_CUDA;
   g->maxdeg = hb.maxdeg;
   if (!h_bins.empty()) {
     g->vstart = (uint32_t *)malloc(sizeof(uint32_t) * h_bins.size());
