@@ -60,7 +60,6 @@ constexpr int64_t kLvMaxGroups = 1 << 20;  // of a level (2^24 would fit the cou
 // on a hub of 2^27 arcs have 2^32: where the sum reaches this, every state
 // becomes a group of its own (a list has less than 2^31 entries).
 constexpr unsigned long long kLvGroupCands = 1ull << 31;
-constexpr uint64_t kLvBarrierNs = 10ull * 1000 * 1000 * 1000;
 
 // A condition of a level: Cons with the class (arc label, vertex label) whose
 // group of f(q) holds the candidates, -1 if the graph has no such label.
@@ -170,6 +169,9 @@ struct LvShared {
   int ok;
 };
 
+// The time limit is looked at here too, so at least once per phase: a phase may
+// give each warp fewer chunks than lv_expand takes between two looks, and a search
+// have any number of such phases.  It also bounds the wait.
 __device__ __forceinline__ bool lv_barrier(const LvArgs &A, LvShared &sm, unsigned int target) {
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -177,12 +179,12 @@ __device__ __forceinline__ bool lv_barrier(const LvArgs &A, LvShared &sm, unsign
     atomicAdd(&A.ctl->bar, 1u);
     int ok = 1;
     for (;;) {
-      if (*(volatile unsigned int *)&A.ctl->bar >= target) break;
-      if (*(volatile int32_t *)&A.ctl->status != 0) break;
-      if (globaltimer_ns() > sm.deadline + kLvBarrierNs) {
-        atomicCAS(&A.ctl->status, 0, kStatQueue);
+      if (globaltimer_ns() > sm.deadline) {
+        atomicCAS(&A.ctl->status, 0, kStatBudget);
         break;
       }
+      if (*(volatile unsigned int *)&A.ctl->bar >= target) break;
+      if (*(volatile int32_t *)&A.ctl->status != 0) break;
       __nanosleep(32);
     }
     __threadfence();

@@ -1,5 +1,8 @@
-"""The level-by-level search at its limits: sums of list lengths that pass 32 bits."""
+"""The level-by-level search at its limits: sums of list lengths that pass 32 bits, the time
+limit when phases are short, levels that pause with rows waiting."""
 from __future__ import annotations
+
+import time
 
 import numpy as np
 import pytest
@@ -40,3 +43,70 @@ def test_a_group_of_states_with_more_than_32_bits_of_candidates():
         assert hm.count_matches_rooted(G, path, hm.MONO, 2, mask) == a * (d // 2)
     finally:
         hm.set_tuning()
+
+
+def _expect_timeout(hm, call, limit_ms):
+    """The call must end with HM_ERR_BUDGET, and within a second or two of its limit."""
+    hm.set_budget(limit_ms, 0)
+    try:
+        t0 = time.perf_counter()
+        with pytest.raises(hm.HMError) as ei:
+            call()
+        took = time.perf_counter() - t0
+    finally:
+        hm.set_budget(60_000, 0)
+    assert ei.value.status == hm.binding.HM_ERR_BUDGET
+    assert limit_ms / 1e3 <= took < limit_ms / 1e3 + 2
+
+
+@pytest.mark.parametrize("k,n,m", [(20, 1500, 6000), (12, 3000, 20000), (20, 100, 300)])
+def test_time_limit_of_searches_with_short_phases(k, n, m):
+    """Paths in sparse random graphs: far more than the limit allows, in phases of a few chunks per warp."""
+    import paper_2507_04130_gb300 as hm
+
+    G = hm.Graph.from_synth(synth.er_graph(n, m, 1, 1, seed=k + n))
+    P = hm.Pattern.from_synth(_pattern(k, [(i, i + 1) for i in range(k - 1)]))
+    triangle = hm.Pattern.from_synth(_pattern(3, [(0, 1), (1, 2), (2, 0)]))
+    want = hm.count_matches(G, triangle, hm.INDUCED)
+    _expect_timeout(hm, lambda: hm.count_matches(G, P, hm.MONO), 300)
+    _expect_timeout(hm, lambda: hm.count_batch(G, [triangle, P], hm.MONO), 300)
+    _expect_timeout(hm, lambda: hm.enumerate_matches(G, P, hm.MONO, capacity=1000), 300)
+    assert hm.count_matches(G, triangle, hm.INDUCED) == want
+    assert hm.count_batch(G, [triangle], hm.INDUCED) == [want]
+
+
+def test_time_limit_of_a_server_with_little_memory():
+    """A slot whose levels hold 8 MiB works a deep pattern off in many small parts."""
+    import paper_2507_04130_gb300 as hm
+
+    G = hm.Graph.from_synth(synth.er_graph(1500, 6000, 1, 1, seed=9))
+    P = _pattern(20, [(i, i + 1) for i in range(19)])
+    srv = hm.Server(G, slots=1, max_batch=2, mem_budget=(13 << 20))
+    try:
+        _expect_timeout(hm, lambda: srv.result(srv.submit(P, hm.MONO, want_rows=False)), 300)
+        assert srv.result(srv.submit(_pattern(2, [(0, 1)]), hm.MONO, want_rows=False))["count"] == 6000
+    finally:
+        srv.close()
+
+
+@pytest.mark.parametrize("k,arcs,n,m", [
+    (5, [(0, 1), (1, 2), (2, 3), (3, 4), (4, 0), (4, 1)], 64, 1300),  # no symmetry; 500,000 states of four positions
+    (5, [(0, 1), (0, 2), (0, 3), (4, 1), (4, 2), (4, 3)], 80, 2320),  # every match has six images; 290,000 such states
+])
+def test_levels_that_pause_keep_their_rows(k, arcs, n, m):
+    """Inner levels over what a graph of this size gives them, with rows: one call, and as a batch."""
+    import torch
+
+    import paper_2507_04130_gb300 as hm
+
+    G = hm.Graph.from_synth(synth.er_graph(n, m, 1, 1, seed=n))
+    P = hm.Pattern.from_synth(_pattern(k, arcs), order=list(range(k)))
+    got = hm.enumerate_matches(G, P, hm.MONO)
+    both = hm.enumerate_batch(G, [P, P], hm.MONO)
+    hm.set_tuning(seeds_per_fetch=2)
+    try:
+        want = hm.enumerate_matches(G, P, hm.MONO, capacity=len(got) + 1)
+    finally:
+        hm.set_tuning()
+    assert len(want) > 100_000
+    assert torch.equal(got, want) and torch.equal(both[0], want) and torch.equal(both[1], want)
