@@ -359,7 +359,7 @@ hm_status run_batch(const hm_graph *g, const hm_pattern *const *pats, const int3
     L.g = g;
     L.want_rows = want_rows;
     L.rows = rows;
-    L.workspace = workspace ? workspace : level_workspace(g);
+    L.workspace = workspace ? workspace : level_workspace(g, kmax);
     L.defer = tu.share_seeds > 0;
     L.npat = npat;
     L.plans = pp.data();

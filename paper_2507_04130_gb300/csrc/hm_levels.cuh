@@ -38,14 +38,25 @@ struct LvLaunch {
   unsigned long long *row_cursor;
 };
 
-// What a call's levels may take: as much as the graph's arrays do (about 80
-// bytes per arc) at most, and no more than 1 GiB.  A level that does not fit is
-// worked off in parts, at 20 to 40 us each.
+// What a call's levels may take.  A level that does not fit is worked off in
+// parts; each part costs a barrier per deeper level and begins and ends with
+// idle warps, so a part should hold some hundred states per warp.  With 64 bytes
+// per arc alone a 7-cycle on 564,000 arcs had 20 and took 37,000 phases (1,278 ms;
+// with 256 MB 386, with 1 GiB 278; depth first 375), an induced star of seven on
+// 166,000 arcs 933 ms (1 GiB 107; depth first 220), an induced path of five on
+// 18,600 arcs 23.4 ms (14.4 from 64 MB on; depth first 9.4, 4.7 with more blocks).
+// 128 MB for every level that keeps states, beside the first, is near the end of
+// that for all of them.  It stays in the device's pool: the first search of a
+// process takes about 0.1 ms longer for every 256 MB, the following ones nothing.
+// A level never gets more groups than the graph has arcs (or 8,192), so short
+// calls on small graphs take a few MB.
 constexpr uint64_t kLevelWorkspaceMax = 1ull << 30;
-constexpr uint64_t kLevelWorkspaceMin = 8ull << 20;
-inline uint64_t level_workspace(const hm_graph *g) {
-  const uint64_t w = 64 * (uint64_t)g->m;
-  return w < kLevelWorkspaceMin ? kLevelWorkspaceMin : w > kLevelWorkspaceMax ? kLevelWorkspaceMax : w;
+constexpr uint64_t kLevelWorkspacePer = 128ull << 20;
+constexpr uint64_t kLevelWorkspaceMin = 8ull << 20;  // on a device that is nearly full
+inline uint64_t level_workspace(const hm_graph *g, int k) {
+  const uint64_t arcs = 64 * (uint64_t)g->m, levels = kLevelWorkspacePer * (uint64_t)(k > 3 ? k - 2 : 1);
+  const uint64_t w = arcs > levels ? arcs : levels;
+  return w > kLevelWorkspaceMax ? kLevelWorkspaceMax : w;
 }
 
 // Runs a whole call, from the vertices that may be position 0's images to the

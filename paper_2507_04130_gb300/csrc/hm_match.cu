@@ -144,7 +144,7 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
     L.root_mask = root_mask;
     L.want_rows = rows;
     L.rows = out;
-    L.workspace = level_workspace(g);
+    L.workspace = level_workspace(g, p->k);
     L.plan = change ? &plan : &p->plan[mode];
     L.cap = cap;
     L.defer = tu.share_seeds > 0;

@@ -323,7 +323,7 @@ extern "C" hm_status hm_server_create(const hm_graph *g, int32_t nslots, int32_t
   }
   // what a slot's extension may take for its levels: what kBatchFixed leaves beside the control block, more
   // under a budget that hardly notices it (then taken off the budget)
-  S->workspace = std::min<uint64_t>(hm::level_workspace(g), std::max<uint64_t>(kSlotWorkspace, S->mem_budget / (64u * (uint64_t)nslots)));
+  S->workspace = std::min<uint64_t>(hm::level_workspace(g, HM_MAX_K), std::max<uint64_t>(kSlotWorkspace, S->mem_budget / (64u * (uint64_t)nslots)));
   S->mem_budget -= (S->workspace - kSlotWorkspace) * (uint64_t)nslots;
   for (int32_t i = 0; i < nslots; ++i) S->threads.emplace_back(serve_slot, S, i);
   *out = S;

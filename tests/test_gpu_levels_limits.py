@@ -110,3 +110,32 @@ def test_levels_that_pause_keep_their_rows(k, arcs, n, m):
         hm.set_tuning()
     assert len(want) > 100_000
     assert torch.equal(got, want) and torch.equal(both[0], want) and torch.equal(both[1], want)
+
+
+@pytest.mark.parametrize("k,arcs,mode,n,m", [
+    (7, [(0, j) for j in range(1, 7)], 1, 9542, 100_000),      # 107 of 220 ms at 166,000 arcs; 934 in parts of 8 MiB
+    (6, [(j, j + 1) for j in range(5)] + [(5, 0)], 0, 2000, 60_000),
+])
+def test_levels_hold_enough_states_to_match_the_depth_first_search(k, arcs, mode, n, m):
+    """Searches of many states on graphs of few arcs: about half the depth-first search's time, and several
+    times it where the levels hold too few states."""
+    import paper_2507_04130_gb300 as hm
+
+    G = hm.Graph.from_synth(synth.er_graph(n, m, 1, 1, seed=k))
+    P = hm.Pattern.from_synth(_pattern(k, arcs))
+
+    def best():
+        took = []
+        for _ in range(4):
+            t0 = time.perf_counter()
+            count = hm.count_matches(G, P, mode)
+            took.append(time.perf_counter() - t0)
+        return count, min(took)
+
+    level = best()
+    hm.set_tuning(poll_every=64)  # as fast as the default, and chooses the depth-first search
+    try:
+        deep = best()
+    finally:
+        hm.set_tuning()
+    assert level[0] == deep[0] and level[1] < 1.3 * deep[1], (level, deep)
