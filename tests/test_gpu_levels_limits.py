@@ -139,3 +139,20 @@ def test_levels_hold_enough_states_to_match_the_depth_first_search(k, arcs, mode
     finally:
         hm.set_tuning()
     assert level[0] == deep[0] and level[1] < 1.3 * deep[1], (level, deep)
+
+
+@pytest.mark.parametrize("k,n,m,at_least,at_most", [
+    (5, 60, 1800, 64, 1 << 20),   # few arcs, much work: more blocks than one per 256 arcs
+    (3, 1000, 5000, 1, 64),       # a short call: a small grid, whose barriers cost less
+    (2, 1000, 5000, 1, 64),
+])
+def test_blocks_follow_the_work_not_only_the_arcs(k, n, m, at_least, at_most):
+    import oracle
+    import paper_2507_04130_gb300 as hm
+
+    g = synth.er_graph(n, m, 1, 1, seed=k)
+    G, p = hm.Graph.from_synth(g), _pattern(k, [(i, j) for i in range(k) for j in range(i + 1, k)])
+    assert hm.count_matches(G, hm.Pattern.from_synth(p), hm.MONO) == oracle.OracleGraph.from_synth(g).match(p, hm.MONO)[0]
+    assert at_least <= hm.last_stats()["extend_grid"] <= at_most
+    hm.count_batch(G, [hm.Pattern.from_synth(p)] * 2, hm.MONO)
+    assert at_least <= hm.last_stats()["extend_grid"] <= at_most
