@@ -25,9 +25,10 @@
 // neighbouring words each), the shortest of which holds its candidates.  A
 // state whose anchor has an empty group is dropped, and so is one whose last
 // position has no other condition, if only its number is asked for: it is the
-// group's length.  Up to 64 states go to the next level with one addition,
-// which reserves their groups and numbers their chunks.  A grid barrier ends
-// the expansion.
+// group's length (where symmetry is broken, that of the part between two
+// images).  Up to 64 states go to the next level with one addition, which
+// reserves their groups and numbers their chunks.  A grid barrier ends the
+// expansion.
 // Memory is bounded: when the states of some warp do not fit the next level any
 // more, all remember where they stand; the deeper levels are worked off, and
 // then they go on (depth first over parts of levels).
@@ -76,7 +77,7 @@ struct LevelPlan {
   int8_t last;            // the position completes a match
   int8_t need_deg;        // test the degrees: at least two pattern arcs lead to positions after the next
   int8_t root;            // the root mask applies to this position
-  int8_t closed;          // the last position has one condition, and only the number of its images is wanted
+  int8_t closed;          // the last position has one condition (order constraints apart), and only the number of its images is wanted
   int8_t final;           // level 1 of a plan with a deferred position 1: the level that matches it, else 0
   int32_t dout, din;
   uint32_t sym_gt, sym_lt;
@@ -252,11 +253,25 @@ __device__ __forceinline__ bool lv_has_final(const LvArgs &A, const LevelPlan &Z
   return false;
 }
 
+// The first of the sorted entries [lo, lo + len) of a list that is at least x (lo + len: none).
+__device__ __forceinline__ int32_t lv_lower(const DevGraph &G, const int32_t *list, int32_t lo, int32_t len, int32_t x) {
+  while (len > 0) {
+    const int32_t half = len >> 1;
+    if (__ldg(list + HM_AT(G, (int64_t)lo + half, G.m, kChkList)) < x) {
+      lo += half + 1;
+      len -= half + 1;
+    } else {
+      len = half;
+    }
+  }
+  return lo;
+}
+
 // The candidates of a state of level p: of the parent at mp (images m) with
 // candidate c at position p - 1.  kClosed: this call only counts, and where the
 // level is closed the matches are added to `found` instead.  The fourth word is
 // not set.
-template <bool kBatch, bool kClosed>
+template <bool kBatch, bool kClosed, bool kSym>
 __device__ __forceinline__ int4 lv_range(const LvArgs &A, int p, const int4 &m, const int32_t *mp, int32_t c,
                                          int32_t pid, unsigned long long &found) {
   const LevelPlan &L = kBatch ? A.levels[(int64_t)pid * A.kmax + p] : A.level1[p];
@@ -287,6 +302,21 @@ __device__ __forceinline__ int4 lv_range(const LvArgs &A, int p, const int4 &m, 
     const int32_t *list = lv_list(what) ? A.G.gin_adj : A.G.gout_adj;
     Bytes none;
     int used = 0;
+    if (kSym && (L.sym_gt | L.sym_lt)) {
+      // between the images that the order constraints name; groups are sorted.  (Read entry by
+      // entry, six ordered leaves of a hub among 128 vertices took 15 ms in place of 42 depth first,
+      // but ordered pairs on a million arcs 449 us in place of 403.)
+      int32_t above = -1, below = INT32_MAX;
+      for (int i = 0; i < p; ++i) {
+        const int32_t x = i == p - 1 ? c : lv_image(m, mp, i);
+        if (L.sym_gt >> i & 1u) above = max(above, x);
+        if (L.sym_lt >> i & 1u) below = min(below, x);
+      }
+      const int32_t a = above < 0 ? lo : lv_lower(A.G, list, lo, best, above + 1);
+      const int32_t z = below == INT32_MAX ? lo + best : lv_lower(A.G, list, a, lo + best - a, below);
+      lo = a;
+      best = max(z - a, 0);
+    }
     for (int i = 0; i < p; ++i)
       if (search_g<false>(A.G, list, lo, best, i == p - 1 ? c : lv_image(m, mp, i), none) >= 0) ++used;
     found = (unsigned long long)(best - used);
@@ -557,7 +587,7 @@ __device__ __forceinline__ int lv_drain(const LvArgs &A, LvShared &sm, int p, in
     // the range of the new state
     int4 r = make_int4(0, 0, 0, 0);
     unsigned long long found = 0;
-    if (ok) r = lv_range<kBatch, !kRows>(A, p + 1, lv_images(mp, p), mp, sc.y, pid, found);
+    if (ok) r = lv_range<kBatch, !kRows, kSym>(A, p + 1, lv_images(mp, p), mp, sc.y, pid, found);
     if (p == 1 && !verified) {
       const uint32_t made = __popc(__ballot_sync(kFull, ok));
       if (lane == 0) sm.injected[warp] += made;
@@ -610,7 +640,7 @@ __device__ __forceinline__ void lv_fill(const LvArgs &A, LvShared &sm, unsigned 
       } else {
         u = __ldg(A.vert + s);
       }
-      r = lv_range<kBatch, !kRows>(A, 1, make_int4(0, 0, 0, 0), nullptr, u, pid, found);
+      r = lv_range<kBatch, !kRows, kSym>(A, 1, make_int4(0, 0, 0, 0), nullptr, u, pid, found);
     }
     if (!kRows) lv_add_found<kBatch, kSym>(A, sm, found, pid, lane);
     const uint32_t bal = __ballot_sync(kFull, r.y > 0);
@@ -1041,7 +1071,7 @@ void lv_level(const hm_graph *g, const Plan &P, bool deferred, int p, bool want_
   }
   // arcs to later positions: one is found missing by the next ranges phase anyway
   L.need_deg = !L.last && P.dout[p] + P.din[p] - npos >= 2;
-  L.closed = L.last && !want_rows && npos == 1 && n == 1 && !L.root && !(L.sym_gt | L.sym_lt);
+  L.closed = L.last && !want_rows && npos == 1 && n == 1 && !L.root;
 }
 
 // The vertices the first level starts from: those with position 0's label and a

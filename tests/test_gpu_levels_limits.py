@@ -156,3 +156,40 @@ def test_blocks_follow_the_work_not_only_the_arcs(k, n, m, at_least, at_most):
     assert at_least <= hm.last_stats()["extend_grid"] <= at_most
     hm.count_batch(G, [hm.Pattern.from_synth(p)] * 2, hm.MONO)
     assert at_least <= hm.last_stats()["extend_grid"] <= at_most
+
+
+@pytest.mark.parametrize("arcs", [
+    [(0, 1), (0, 2)], [(1, 0), (2, 0), (3, 0)], [(0, 1), (0, 2), (0, 3), (0, 4)],         # ordered leaves
+    [(0, 1), (0, 2), (3, 0), (4, 0)], [(0, 1), (1, 0), (0, 2), (0, 3)],                  # two kinds of leaves
+    [(0, 1), (1, 2), (3, 1), (1, 4)], [(0, 2), (1, 2), (2, 3)], [(0, 1), (2, 1), (2, 3), (4, 3)],  # leaves that earlier images may be
+])
+def test_ordered_last_positions_are_counted_by_length(arcs):
+    import oracle
+    import paper_2507_04130_gb300 as hm
+
+    k = max(max(a) for a in arcs) + 1
+    pats = [_pattern(k, arcs), _pattern(k, arcs, elab=[1] * len(arcs))]
+    for g in (synth.small_random_graph(40, 0.15, 1, 2, seed=k, recip=0.4, hub=True), synth.er_graph(25, 300, 1, 2, seed=k)):
+        G, og = hm.Graph.from_synth(g), oracle.OracleGraph.from_synth(g)
+        P = [hm.Pattern.from_synth(p) for p in pats]
+        want = [og.match(p, hm.MONO)[0] for p in pats]
+        assert [hm.count_matches(G, p, hm.MONO) for p in P] == want
+        assert hm.count_batch(G, P, hm.MONO) == want
+        hm.set_tuning(share_seeds=-1)
+        try:
+            assert [hm.count_matches(G, p, hm.MONO) for p in P] == want
+        finally:
+            hm.set_tuning()
+        assert min(want) > 0
+
+
+def test_ordered_leaves_of_a_hub_are_not_read_one_by_one():
+    import paper_2507_04130_gb300 as hm
+
+    d = 3000
+    z = np.zeros(d, np.int32)
+    G = hm.Graph(d + 1, z, np.arange(1, d + 1, dtype=np.int32), np.zeros(d + 1, np.int32), z)
+    fan = hm.Pattern.from_synth(_pattern(3, [(0, 1), (0, 2)]))
+    assert fan.automorphisms() == 2
+    assert hm.count_matches(G, fan, hm.MONO) == d * (d - 1)
+    assert hm.last_stats()["chunks"] < d  # d * d / 32 one by one
