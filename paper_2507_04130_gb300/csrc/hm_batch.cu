@@ -199,7 +199,9 @@ __global__ void k_unpack_rows(const int32_t *__restrict__ packed, const unsigned
   }
 }
 
-constexpr uint64_t kRankMaxCompares = 1ull << 29;  // run_batch: below, rows are sorted by counting
+// Up to both, a batch's rows are sorted by counting: compares of all lists, rows of the longest.
+constexpr uint64_t kRankMaxCompares = 1ull << 29;
+constexpr uint64_t kRankMaxList = 1 << 14;
 
 // Counts to the caller and, of the patterns whose rows fit their regions, the rows in order.
 hm_status finish_batch(const hm_graph *g, int32_t npat, const std::vector<int32_t> &ks, int32_t kmax, int32_t *rows,
@@ -230,15 +232,22 @@ hm_status finish_batch(const hm_graph *g, int32_t npat, const std::vector<int32_
   // few rows per pattern: every list ranked by counting, all lists in one
   // launch, in place of 12 or more radix passes over the padded rows of all
   // (33 us each; 64 patterns with 33,600 rows: 400 us).  kRankMaxCompares take
-  // about 290 us.
+  // about 290 us.  One long list is better off with the radix sort, which does
+  // not grow with its square (whole calls with one list of three columns: by
+  // counting 16,000 rows 231 us, 20,000 321, 23,000 386; by radix 20,000 rows
+  // 246 us, 23,000 264).
   std::vector<RankTile> tiles;
-  uint64_t compares = 0;
-  for (int32_t i = 0; i < npat; ++i) compares += (start[i + 1] - start[i]) * (start[i + 1] - start[i]);
-  if (compares <= kRankMaxCompares) {
-    int64_t dst = 0, longest = 0;
+  uint64_t compares = 0, most = 0;
+  for (int32_t i = 0; i < npat; ++i) {
+    const uint64_t n = start[i + 1] - start[i];
+    compares += n * n;
+    most = std::max(most, n);
+  }
+  if (compares <= kRankMaxCompares && most <= kRankMaxList) {
+    int64_t dst = 0;
+    const int64_t longest = (int64_t)most;
     for (int32_t i = 0; i < npat; ++i) {
       const int64_t n = (int64_t)(start[i + 1] - start[i]);
-      longest = std::max(longest, n);
       for (int64_t r = 0; n > 1 && r < n; r += kRankTileRows)
         tiles.push_back(RankTile{(int64_t)off[i], dst, (int32_t)start[i], (int32_t)n, ks[i], (int32_t)r});
       dst += n * ks[i];
