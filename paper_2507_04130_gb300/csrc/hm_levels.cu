@@ -41,6 +41,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "hm_levels.cuh"
@@ -1104,25 +1105,56 @@ void lv_emit(const Plan &P, EmitPlan &E, std::vector<int8_t> &aut) {
     for (int s = 0; s < P.naut; ++s) aut.insert(aut.end(), P.aut[s], P.aut[s] + kMaxK);
 }
 
-// A thread's page-locked block for what a call reads back: a copy into ordinary
-// memory is staged by the driver (1.5 to 2 us more per call).  Freed
-// when the thread ends.
+// A page-locked block for what a call reads back: a copy into ordinary memory is
+// staged by the driver (1.5 to 2 us more per call).  The process keeps the blocks
+// that were in use at one time, up to kMost (0.6 MB), for any thread's calls: a
+// thread that makes a single call neither locks a block (0.1 ms) nor frees one,
+// which would wait for the kernels of every stream.  A call that finds none left, or has more counts than
+// a block holds, reads into ordinary memory.
 struct Landing {
   static constexpr int32_t kCounts = 4096;
+  static constexpr int kMost = 16;
   struct Block {
     LvCtl ctl;
     unsigned long long counts[kCounts];
   } *p = nullptr;
-  Block *get() {
-    if (!p && cudaMallocHost((void **)&p, sizeof(Block)) != cudaSuccess) {
+  struct Pool {
+    std::mutex mu;
+    Block *idle[kMost];
+    int nidle = 0, made = 0;
+  };
+  // never destroyed: calls of other threads may outlast static objects
+  static Pool &pool() {
+    static Pool *q = new Pool;
+    return *q;
+  }
+  explicit Landing(bool wanted) {
+    if (!wanted) return;
+    Pool &q = pool();
+    {
+      std::lock_guard<std::mutex> lk(q.mu);
+      if (q.nidle) {
+        p = q.idle[--q.nidle];
+        return;
+      }
+      if (q.made == kMost) return;
+      ++q.made;
+    }
+    if (cudaMallocHost((void **)&p, sizeof(Block)) != cudaSuccess) {
       (void)cudaGetLastError();
       p = nullptr;
+      std::lock_guard<std::mutex> lk(q.mu);
+      --q.made;
     }
-    return p;
   }
   ~Landing() {
-    if (p) cudaFreeHost(p);
+    if (!p) return;
+    Pool &q = pool();
+    std::lock_guard<std::mutex> lk(q.mu);
+    q.idle[q.nidle++] = p;
   }
+  Landing(const Landing &) = delete;
+  Landing &operator=(const Landing &) = delete;
 };
 
 hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result, int *grid_out, int *threads_out,
@@ -1311,8 +1343,8 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   if (le == cudaSuccess) {
     *ran = true;
     if (ms) cudaEventRecord(ev[1], s);
-    static thread_local Landing landing;
-    Landing::Block *l = L.npat <= Landing::kCounts ? landing.get() : nullptr;
+    Landing landing(L.npat <= Landing::kCounts);
+    Landing::Block *l = landing.p;
     LvCtl *to = l ? &l->ctl : result;
     unsigned long long *counts = l ? l->counts : L.counts_host;
     const size_t nc = L.counts_host ? sizeof(unsigned long long) * L.npat : 0;
@@ -1320,7 +1352,9 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
         (nc && cudaMemcpyAsync(counts, L.counts, nc, cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
         cudaStreamSynchronize(s) != cudaSuccess)
       st = HM_ERR_CUDA;
-    if (l) {
+    if (l && st != HM_OK) {
+      landing.p = nullptr;  // a copy into it may be under way: it is not given to another call
+    } else if (l) {
       *result = l->ctl;
       if (nc) std::memcpy(L.counts_host, l->counts, nc);
     }

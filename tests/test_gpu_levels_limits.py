@@ -193,3 +193,59 @@ def test_ordered_leaves_of_a_hub_are_not_read_one_by_one():
     assert fan.automorphisms() == 2
     assert hm.count_matches(G, fan, hm.MONO) == d * (d - 1)
     assert hm.last_stats()["chunks"] < d  # d * d / 32 one by one
+
+
+def test_a_threads_end_does_not_wait_for_other_streams():
+    """A thread that made one call ends while another stream's kernel is still running."""
+    import threading
+
+    import torch
+
+    import paper_2507_04130_gb300 as hm
+
+    G = hm.Graph.from_synth(synth.er_graph(1000, 5000, 1, 1, seed=2))
+    P = hm.Pattern.from_synth(_pattern(3, [(0, 1), (1, 2), (2, 0)]))
+    want, got = hm.count_matches(G, P, hm.MONO), []
+    side, own = torch.cuda.Stream(), torch.cuda.Stream()
+    done = torch.cuda.Event()
+
+    def once():
+        got.append(hm.count_matches(G, P, hm.MONO, stream=own))
+
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(2_000_000_000)  # about a second on one SM
+        done.record()
+    for _ in range(20):
+        t = threading.Thread(target=once)
+        t.start()
+        t.join()
+    assert not done.query()
+    torch.cuda.synchronize()
+    assert got == [want] * 20
+
+
+def test_more_calls_at_once_than_page_locked_blocks():
+    import threading
+
+    import torch
+
+    import paper_2507_04130_gb300 as hm
+
+    G = hm.Graph.from_synth(synth.er_graph(1000, 5000, 1, 1, seed=2))
+    pats = [hm.Pattern.from_synth(_pattern(k, [(i, (i + 1) % k) for i in range(k)])) for k in (3, 4, 5)]
+    want = [hm.count_matches(G, p, hm.MONO) for p in pats]
+    many = [hm.Pattern.from_synth(_pattern(3, [(0, 1), (1, 2)]))] * 4097  # more counts than a block holds
+    lots, got = hm.count_batch(G, many[:1], hm.MONO)[0], []
+
+    def work(i):
+        s = torch.cuda.Stream()
+        for _ in range(20):
+            got.append((i % 3, hm.count_matches(G, pats[i % 3], hm.MONO, stream=s)))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(40)]
+    for t in threads:
+        t.start()
+    assert hm.count_batch(G, many, hm.MONO) == [lots] * 4097
+    for t in threads:
+        t.join()
+    assert len(got) == 800 and all(c == want[i] for i, c in got)
