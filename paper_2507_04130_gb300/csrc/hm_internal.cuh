@@ -24,6 +24,8 @@
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "hipermotif.h"
 
 namespace hm {
@@ -545,7 +547,26 @@ hm_status batch_run(const hm_graph *g, const hm_pattern *const *patterns, const 
                     uint64_t workspace, cudaStream_t stream);
 
 int bits_for(int64_t n);  // bits needed for values in [0, n)
-int num_sms();
+int num_sms();            // of the current device
+
+// kSlots values per device, each found once on the first kDevices devices and every
+// time on further ones (a process may hold graphs on several devices).  Zero-initialised,
+// so for static objects; `find` must not give 0.
+template <int kSlots>
+struct PerDevice {
+  static constexpr int kDevices = 64;
+  std::atomic<int> v[kDevices][kSlots];
+  template <typename F>
+  int get(int dev, int slot, F find) {
+    if (dev < 0 || dev >= kDevices) return find();
+    int x = v[dev][slot].load(std::memory_order_relaxed);
+    if (!x) {
+      x = find();
+      v[dev][slot].store(x, std::memory_order_relaxed);
+    }
+    return x;
+  }
+};
 
 }  // namespace hm
 

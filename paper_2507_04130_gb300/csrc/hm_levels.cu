@@ -39,7 +39,6 @@
 // Bound by the latency of its lookups in L2 and HBM (list entry, then filter
 // word, per candidate), which many independent warps hide.
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -953,20 +952,20 @@ LvKernel lv_kernel(bool rows, bool batch, bool sym) {
 }
 
 // Resident blocks of a variant (0: the device cannot run it).
+// Asked once per device: each needs the opt-in to more than 48 KB of shared memory.
 int lv_grid(LvKernel f, int slot) {
-  static std::atomic<int> cache[8];
-  int v = cache[slot].load(std::memory_order_relaxed);
-  if (!v) {
-    int per_sm = 0, coop = 0, dev = 0;
-    cudaGetDevice(&dev);
+  static PerDevice<8> cache;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const int v = cache.get(dev, slot, [&] {
+    int per_sm = 0, coop = 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
         cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LvShared)) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, kLvThreads, sizeof(LvShared)) != cudaSuccess)
       per_sm = 0;
     (void)cudaGetLastError();
-    v = per_sm > 0 ? per_sm * num_sms() : -1;
-    cache[slot].store(v, std::memory_order_relaxed);
-  }
+    return per_sm > 0 ? per_sm * num_sms() : -1;
+  });
   return std::max(v, 0);
 }
 

@@ -936,16 +936,14 @@ int bits_for(int64_t n) {
 }
 
 int num_sms() {
-  static std::atomic<int> cached{0};
-  int v = cached.load(std::memory_order_relaxed);
-  if (!v) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      v = 1;
-    cached.store(v, std::memory_order_relaxed);
-  }
-  return v;
+  static PerDevice<1> cached;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return cached.get(dev, 0, [dev] {
+    int v = 0;
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) v = 0;
+    return v > 0 ? v : 1;
+  });
 }
 
 hm_status radix_sort_rows(int32_t *rows, int32_t *tmp, int64_t nrows, int width,
