@@ -90,7 +90,9 @@ const char *hm_status_str(hm_status s);
  * Device memory: 64 bytes per arc, 16 per directory entry (at most 2 per arc)
  * and 40 per vertex; with the dense starts 4 more per directory entry and 8 per
  * vertex and class; with the filters by endpoint 8 more per arc and 16 per
- * vertex (hm_graph_info reports the total).
+ * vertex (hm_graph_info reports the total).  Where these do not fit, the graph is
+ * loaded without the filters by endpoint, then without the dense starts, and calls
+ * on it search depth first.
  * The input arrays are copied; the caller keeps ownership.  m must be below
  * 2^31.  Errors: HM_ERR_ARG (id out of range, n or m negative, m >= 2^31,
  * NULL array),

@@ -655,6 +655,15 @@ void ensure_pool() {
   done_for = dev;
 }
 
+// Gives back what the current device's pool holds unused.
+void trim_pool() {
+  int dev = 0;
+  cudaMemPool_t pool;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)
+    cudaMemPoolTrimTo(pool, 0);
+  (void)cudaGetLastError();
+}
+
 }  // namespace hm
 
 using namespace hm;
@@ -690,9 +699,12 @@ hm_status build_groups(int32_t *rows, int32_t *tmp, int64_t m, int32_t n, int ke
   return HM_OK;
 }
 
+// What a graph gets beside the storage itself, as memory allows.
+enum class Tables { kNone, kDense, kAll };  // kDense: without the filters by endpoint
+
 hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_t *dst,
                           const int32_t *vlab, const int32_t *elab, int device_ptrs,
-                          cudaStream_t s, hm_graph *g) {
+                          cudaStream_t s, hm_graph *g, Tables tables) {
   Temps T(s);
 #if HM_CHECK
   HM_CUDA_TRY(own(g, &g->check, 1));  // the bounds checks' violation word
@@ -714,23 +726,21 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     d_elab = t + 2 * m;
     d_vlab = t + 3 * m;
   }
-  // working memory: rows and their copy, offsets, groups per vertex and their
-  // prefix sums (both directions one after the other), long lists, class counts
-  int32_t *rows, *tmp, *hubs;
+  // working memory: rows and their copy, offsets, class counts
+  int32_t *rows, *tmp;
   int64_t *out_off, *in_off;
-  uint32_t *err, *ngroup, *didx, *bins;
+  uint32_t *err, *bins;
   Bounds *bnd;
+  size_t at = 0;
+  auto part = [&](size_t b) {
+    const size_t a = at;
+    at += (b + 255) / 256 * 256;
+    return a;
+  };
   {
-    size_t at = 0;
-    auto part = [&](size_t b) {
-      const size_t a = at;
-      at += (b + 255) / 256 * 256;
-      return a;
-    };
     const size_t bin_words = 6 * (size_t)(kMaxDense * kMaxDense + 1);
     const size_t a_rows = part(sizeof(int32_t) * (size_t)(kW * m + kW)), a_tmp = part(sizeof(int32_t) * (size_t)(kW * m + kW)),
-                 a_off = part(sizeof(int64_t) * 2 * (size_t)(n + 1)), a_grp = part(sizeof(uint32_t) * 4 * (size_t)(n + 1)),
-                 a_hub = part(sizeof(int32_t) * 2 * (size_t)(m / kHub + 1)),
+                 a_off = part(sizeof(int64_t) * 2 * (size_t)(n + 1)),
                  a_zero = part(sizeof(uint32_t) * (bin_words + 4)), a_bnd = part(sizeof(Bounds));
     unsigned char *w;
     HM_CUDA_TRY(T.get((void **)&w, at));
@@ -738,9 +748,6 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     tmp = reinterpret_cast<int32_t *>(w + a_tmp);
     out_off = reinterpret_cast<int64_t *>(w + a_off);
     in_off = out_off + (n + 1);
-    ngroup = reinterpret_cast<uint32_t *>(w + a_grp);
-    didx = ngroup + 2 * (size_t)(n + 1);
-    hubs = reinterpret_cast<int32_t *>(w + a_hub);
     err = reinterpret_cast<uint32_t *>(w + a_zero);  // {input errors, sort error}, then two list lengths, then the bins
     bins = err + 4;
     bnd = reinterpret_cast<Bounds *>(w + a_bnd);
@@ -760,7 +767,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
 
   // dense group offsets while there are few classes and the tables are no larger than the arcs' own data
   const int64_t nal = m ? (int64_t)hb.emax - hb.emin + 1 : 0, nvl = m ? (int64_t)hb.vmax - hb.vmin + 1 : 0;
-  if (m && nal <= kMaxDense && nvl <= kMaxDense && nal * nvl <= kMaxDense &&
+  if (tables != Tables::kNone && m && nal <= kMaxDense && nvl <= kMaxDense && nal * nvl <= kMaxDense &&
       (int64_t)n * nal * nvl <= 8 * std::max<int64_t>(m, 1 << 16)) {
     g->nal = (int32_t)nal;
     g->nvl = (int32_t)nvl;
@@ -772,7 +779,7 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
   g->afilt_nword = (uint32_t)(4 * std::max<int64_t>(1, (m + 7) / 8));
   g->ahash_nbkt = (uint32_t)std::max<int64_t>(1, m);
   const int64_t region_words = (m >> 1) + n + 1;
-  g->regions = g->ncls && m >= kRegionArcs;
+  g->regions = g->ncls && tables == Tables::kAll && m >= kRegionArcs;
   g->rf_nword = g->regions ? (uint32_t)region_words : g->afilt_nword;
   Arena A;
   A.add(&g->src, m);
@@ -796,6 +803,18 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     }
   }
   HM_CUDA_TRY(A.allocate(g));
+  // with dense offsets: groups per vertex and their prefix sums (both directions one after the other), long lists
+  uint32_t *ngroup = nullptr, *didx = nullptr;
+  int32_t *hubs = nullptr;
+  if (g->ncls) {
+    at = 0;
+    const size_t a_grp = part(sizeof(uint32_t) * 4 * (size_t)(n + 1)), a_hub = part(sizeof(int32_t) * 2 * (size_t)(m / kHub + 1));
+    unsigned char *w;
+    HM_CUDA_TRY(T.get((void **)&w, at));
+    ngroup = reinterpret_cast<uint32_t *>(w + a_grp);
+    didx = ngroup + 2 * (size_t)(n + 1);
+    hubs = reinterpret_cast<int32_t *>(w + a_hub);
+  }
   if (!g->regions) g->rfilt_out = g->rfilt_in = g->afilt;
   HM_CUDA_TRY(cudaMemsetAsync(g->afilt, 0, 8 * (size_t)g->afilt_nword, s));
   HM_CUDA_TRY(cudaMemsetAsync(g->ahash, 0xff, 32 * (size_t)g->ahash_nbkt, s));
@@ -945,19 +964,34 @@ extern "C" hm_status hm_load_graph(int32_t n, int64_t m, const int32_t *src, con
   ensure_pool();
   cudaStream_t s = (cudaStream_t)stream;
   hm_graph *g = new hm_graph();
-  std::memset(g, 0, sizeof(*g));
-  cudaGetDevice(&g->device);
-  g->n = n;
-  g->m = m;
-  hm_status st = load_graph_impl(n, m, src, dst, vlab, elab, device_ptrs, s, g);
-  if (st == HM_OK && cudaStreamSynchronize(s) != cudaSuccess) st = HM_ERR_CUDA;
-  if (st != HM_OK) {
+  Tables tables = Tables::kAll;
+  bool trimmed = false;
+  for (;;) {
+    std::memset(g, 0, sizeof(*g));
+    cudaGetDevice(&g->device);
+    g->n = n;
+    g->m = m;
+    hm_status st = load_graph_impl(n, m, src, dst, vlab, elab, device_ptrs, s, g, tables);
+    if (st == HM_OK && cudaStreamSynchronize(s) != cudaSuccess) st = HM_ERR_CUDA;
+    if (st == HM_OK) break;
     cudaStreamSynchronize(s);
     (void)cudaGetLastError();
     free_graph_arrays(g);
     free(g->vstart);
-    delete g;
-    return st;
+    // a device that is nearly full: once more with what the pool keeps given
+    // back, then without the tables that only make searches faster (the dense
+    // offsets and their vertex lists are up to 80 bytes per arc, the filters by
+    // endpoint 8; without them calls search depth first)
+    const bool dense = g->ncls > 0, regions = g->regions != 0;
+    if (st == HM_ERR_OOM && !trimmed) {
+      trimmed = true;
+      trim_pool();
+    } else if (st == HM_ERR_OOM && (dense || regions)) {
+      tables = regions ? Tables::kDense : Tables::kNone;
+    } else {
+      delete g;
+      return st;
+    }
   }
   *out = g;
   return HM_OK;

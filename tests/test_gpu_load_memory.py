@@ -1,0 +1,71 @@
+"""A graph that fits the device only without the tables that speed searches up loads without them.
+
+Runs in a child process that leaves the library 560 MB of device memory: a graph of 3.1M arcs and 64
+classes takes about 610 MB to load with its dense group offsets and 450 without.
+"""
+from __future__ import annotations
+
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+_CHILD = r"""
+import numpy as np
+import torch
+import paper_2507_04130_gb300 as hm
+
+n, m, dev = 390_000, 3_120_000, {"dtype": torch.int32, "device": "cuda"}
+gen = torch.Generator(device="cuda")
+gen.manual_seed(3)
+key = torch.unique(torch.randint(0, n * n, (m + 200_000,), generator=gen, device="cuda"))
+key = key[key // n != key % n]
+key = key[torch.randperm(key.numel(), generator=gen, device="cuda")[:m]]
+vlab = torch.randint(0, 8, (n,), generator=gen, device="cuda").int()
+arrays = [(key // n).int(), (key % n).int(), vlab, torch.randint(0, 8, (m,), generator=gen, device="cuda").int()]
+z = np.zeros(2, np.int32)
+pats = [hm.Pattern(3, z[:2] + [0, 1], z[:2] + [1, 2], [0, a, b], [a, b]) for a in range(8) for b in range(8)]
+del key
+small = hm.Graph(3, z[:2] + [0, 1], z[:2] + [1, 2], np.zeros(3, np.int32), z)  # the kernels' own memory
+hm.count_matches(small, hm.Pattern(2, z[:1], z[:1] + 1, z, z[:1]), hm.MONO)
+torch.cuda.synchronize()
+torch.cuda.empty_cache()
+rest = LEFT << 20
+fill = torch.empty(torch.cuda.mem_get_info()[0] - rest, dtype=torch.uint8, device="cuda")
+try:
+    tight = hm.Graph(n, *arrays)
+except hm.HMError as e:
+    print("status", e.status)
+    raise SystemExit
+del fill
+torch.cuda.empty_cache()
+full = hm.Graph(n, *arrays)
+print("bytes", tight.device_bytes(), full.device_bytes())
+a, b = [[hm.count_matches(g, p, hm.MONO) for p in pats] for g in (tight, full)]
+rows = [hm.enumerate_matches(g, pats[9], hm.INDUCED) for g in (tight, full)]
+print("same" if a == b and torch.equal(*rows) and len(rows[0]) > 0 else "different")
+"""
+
+
+def _load(left):
+    env = dict(os.environ, PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, "-c", _CHILD.replace("LEFT", str(left))], capture_output=True, text=True,
+                       timeout=300, cwd=ROOT, env=env)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout.split()
+
+
+def test_a_nearly_full_device_takes_the_graph_without_its_tables():
+    out = _load(560)
+    assert out[0] == "bytes" and int(out[1]) < int(out[2]) - (150 << 20) and out[3] == "same", out
+
+
+def test_a_device_without_room_refuses_the_graph():
+    from paper_2507_04130_gb300 import binding
+
+    assert _load(200) == ["status", str(binding.HM_ERR_OOM)]
