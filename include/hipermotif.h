@@ -496,8 +496,8 @@ hm_status hm_autotune(const hm_graph *g, const hm_pattern *const *patterns, cons
 
 /* hm_autotune_cached -- hm_autotune with a cache file (host path; NULL or ""
  * = none).  The key is a fingerprint of the graph (its sizes and a strided
- * sample of its sorted arc arrays) and of the workload (how many patterns of
- * each size and mode).  A setting stored under the key is installed without
+ * sample of its sorted arc arrays), whether calls on it may be worked off level
+ * by level, and the workload (how many patterns of each size and mode).  A setting stored under the key is installed without
  * timing (*from_cache = 1, *best_ms = the time stored with it); otherwise the
  * tuner runs and appends its choice to the file as one text line
  * "<key> name=value ... ms=<time>".  from_cache may be NULL. */

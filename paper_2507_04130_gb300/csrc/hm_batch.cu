@@ -643,7 +643,9 @@ constexpr int kNumTuneFields = 11;
 
 // A fingerprint of the graph (sizes, directory sizes and a strided sample of
 // its sorted arc arrays, FNV-1a) and of the workload (the multiset of pattern
-// sizes and modes): the cache key of a tuned setting.
+// sizes and modes), and whether the graph can be searched level by level: the
+// cache key of a tuned setting.  Nearly every knob chooses the depth-first search,
+// so a setting that was tuned without the other choice must not be taken over.
 std::string tune_key(const hm_graph *g, const hm_pattern *const *patterns, const int32_t *modes, int32_t npat,
                      cudaStream_t s) {
   uint64_t h = 1469598103934665603ull;
@@ -673,7 +675,7 @@ std::string tune_key(const hm_graph *g, const hm_pattern *const *patterns, const
   for (int32_t i = 0; i < npat; ++i) hist[modes[i] ? 1 : 0][patterns[i]->k]++;
   std::string key;
   char tmp[64];
-  std::snprintf(tmp, sizeof tmp, "g%016llx", (unsigned long long)h);
+  std::snprintf(tmp, sizeof tmp, "%sg%016llx", g->ncls > 0 ? "levels_" : "", (unsigned long long)h);
   key += tmp;
   for (int m = 0; m < 2; ++m)
     for (int k = 2; k <= HM_MAX_K; ++k)
