@@ -71,7 +71,6 @@ struct hm_server {
   int32_t nslots = 1;
   int32_t max_batch = 64;
   uint64_t mem_budget = 0;
-  uint64_t workspace = 0;         // bytes a slot's extension may take for its levels
   uint64_t row_guess = 1u << 18;  // rows a query's region holds on the first pass
   // arcs per (source label, arc label, target label)
   std::map<std::tuple<int32_t, int32_t, int32_t>, uint64_t> triples;
@@ -97,7 +96,30 @@ namespace {
 // states of the extension's levels (or the depth-first search's donation
 // queue) and the control block.
 constexpr uint64_t kBatchFixed = (12ull << 20);
-constexpr uint64_t kSlotWorkspace = (8ull << 20);
+constexpr uint64_t kSlotWorkspace = (8ull << 20);  // the part of kBatchFixed that the levels may take
+
+// One search of a batch.  Its levels take kSlotWorkspace and, while it runs, up to
+// half of the slot's share of what the budget has free: levels that hold few
+// states make deep patterns slow, but rows and admissions come first, so nothing
+// is set aside for good.
+hm_status search_batch(hm_server *S, const std::vector<const hm_pattern *> &pats, const std::vector<int32_t> &modes,
+                       int32_t *rows, const uint64_t *off, uint64_t *counts, uint8_t *fit, cudaStream_t stream) {
+  int kmax = 0;
+  for (const hm_pattern *p : pats) kmax = std::max(kmax, p->k);
+  uint64_t extra = 0;
+  {
+    std::lock_guard<std::mutex> lk(S->mu);
+    const uint64_t room = S->mem_budget > S->in_use ? S->mem_budget - S->in_use : 0;
+    const uint64_t most = hm::level_workspace(S->g, kmax) - kSlotWorkspace;
+    extra = std::min<uint64_t>(most, room / (2 * (uint64_t)S->nslots));
+    S->in_use += extra;
+  }
+  const hm_status st = hm::batch_run(S->g, pats.data(), modes.data(), (int32_t)pats.size(), rows, off, counts, fit,
+                                     kSlotWorkspace + extra, stream);
+  std::lock_guard<std::mutex> lk(S->mu);
+  S->in_use -= extra;
+  return st;
+}
 
 void serve_slot(hm_server *S, int slot) {
   cudaSetDevice(S->device);
@@ -144,8 +166,7 @@ void serve_slot(hm_server *S, int slot) {
     }
     hm_status st = HM_OK;
     if (!any_rows) {
-      st = hm::batch_run(S->g, pats.data(), modes.data(), nb, nullptr, nullptr, counts.data(), nullptr, S->workspace,
-                         stream);
+      st = search_batch(S, pats, modes, nullptr, nullptr, counts.data(), nullptr, stream);
       for (int32_t i = 0; i < nb && st == HM_OK; ++i) batch[i]->count = counts[i];
     } else {
       // one pass: rows into regions of row_guess rows (as many as the budget holds)
@@ -171,8 +192,7 @@ void serve_slot(hm_server *S, int slot) {
         (void)cudaGetLastError();
         st = HM_ERR_OOM;
       } else {
-        st = hm::batch_run(S->g, pats.data(), modes.data(), nb, d_rows, off.data(), counts.data(), fit.data(),
-                           S->workspace, stream);
+        st = search_batch(S, pats, modes, d_rows, off.data(), counts.data(), fit.data(), stream);
         if (st == HM_OK) {
           for (int32_t i = 0; i < nb; ++i) {
             auto &q = batch[i];
@@ -229,8 +249,7 @@ void serve_slot(hm_server *S, int slot) {
             (void)cudaGetLastError();
             st = HM_ERR_OOM;
           } else {
-            st = hm::batch_run(S->g, rp.data(), rm.data(), nr, d2, off2.data(), rc.data(), nullptr, S->workspace,
-                               stream);
+            st = search_batch(S, rp, rm, d2, off2.data(), rc.data(), nullptr, stream);
             if (st == HM_OK) {
               for (int32_t j = 0; j < nr; ++j) {
                 auto &q = batch[take[j]];
@@ -321,10 +340,6 @@ extern "C" hm_status hm_server_create(const hm_graph *g, int32_t nslots, int32_t
     delete S;
     return HM_ERR_ARG;  // the budget cannot admit even one batch
   }
-  // what a slot's extension may take for its levels: what kBatchFixed leaves beside the control block, more
-  // under a budget that hardly notices it (then taken off the budget)
-  S->workspace = std::min<uint64_t>(hm::level_workspace(g, HM_MAX_K), std::max<uint64_t>(kSlotWorkspace, S->mem_budget / (64u * (uint64_t)nslots)));
-  S->mem_budget -= (S->workspace - kSlotWorkspace) * (uint64_t)nslots;
   for (int32_t i = 0; i < nslots; ++i) S->threads.emplace_back(serve_slot, S, i);
   *out = S;
   return HM_OK;
