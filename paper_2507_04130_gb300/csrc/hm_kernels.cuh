@@ -353,8 +353,13 @@ __device__ __forceinline__ bool in_nbhd(const DevGraph &G, int32_t y, int4 iy, i
 
 // In batched launches (kB) each seed carries its pattern id; the threshold is
 // that pattern's, and seeds of patterns without an overlap test pass through.
+// Bound by the latency of the probes.  The blocks per SM are stated because the
+// compiler's own choice moves with the filter's code: for one pattern it settled
+// on 32 registers with spills inside the loop (16M arcs, a labelled triangle:
+// 428 us; 35 registers and six blocks 246), for a batch on 40 (32 of its
+// triangles 7.16 ms; 32 registers and eight blocks 6.05).
 template <bool kC, bool kB = false>
-__global__ void __launch_bounds__(kSeedThreads)
+__global__ void __launch_bounds__(kSeedThreads, kB ? 8 : 6)
 k_seed_overlap(const __grid_constant__ DevGraph G, int32_t need_all, const int2 *__restrict__ in,
                const unsigned long long *__restrict__ nin, int2 *__restrict__ out,
                unsigned long long cap, unsigned long long *__restrict__ nout,
