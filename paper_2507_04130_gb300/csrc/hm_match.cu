@@ -12,6 +12,8 @@ namespace {
 
 enum class Want { kCount, kRows, kStates };
 
+constexpr int64_t kScanArcs = 1 << 16;  // from here on pairs of an unlabelled graph are scanned (run_match)
+
 // The plan for shared position-0 states: the induced non-arcs between
 // position 1 and later positions leave the per-position condition lists and
 // become P.defer, read from the chosen image v of position 1.
@@ -112,8 +114,10 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   const hm_tuning tu = tuning();
   // a copy only where the call changes the plan (17 KB) or searches depth first
   Plan changed;
+  const Plan &own = p->plan[mode];
+  const bool scan = p->k == 2 && g->ncls == 1 && g->m >= kScanArcs && (want == Want::kRows || root_mask || own.back_req || own.back_forbid);
   const bool by_level = g->ncls > 0 && want != Want::kStates && nparts == 1 && default_search(tu) && !counters &&
-                        budget_chunks() == 0;
+                        budget_chunks() == 0 && !scan;
   const bool change = root_mask || tu.symmetry < 0 || !by_level;
   if (change) changed = p->plan[mode];
   Plan &plan = changed;
@@ -136,7 +140,12 @@ hm_status run_match(const hm_graph *g, const hm_pattern *p, hm_mode mode, int32_
   // motifs on 150M arcs 35 / 3.1 ms, 256 patterns in a batch 17.3 / 1.7 ms).  The
   // depth-first search below keeps the other knobs, the instrumented kernels,
   // chunk budgets, arc-range parts, graphs with too many label classes, and
-  // the injected states.
+  // the injected states; and pairs where every arc has the pattern's labels and
+  // must be read, which the edge scan streams (a million / 8 million arcs, scan
+  // against levels: rows 276 / 311 and 891 / 998 us, reciprocal pairs counted 55 /
+  // 66 and 114 / 140, induced pairs 66 / 79 and 153 / 177; even at 88,000 arcs,
+  // 53 / 44 at 5,000; with eight classes 87 / 53 on 8 million, and a pair with one
+  // condition is counted without reading arcs, 125 / 46).
   if (by_level) {
     NvtxRange r_lv("hm.extend");
     LvLaunch L{};
