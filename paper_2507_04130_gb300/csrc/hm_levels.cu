@@ -1239,7 +1239,10 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   auto group_bytes = [&](int p) { return sizeof(LvGroup) + 32 * (sizeof(int4) + 4 * (uint64_t)stride_of(p)); };
   uint64_t per_group = 0;
   for (int p = 2; p <= top; ++p) per_group += group_bytes(p);
-  const uint64_t most = std::min<uint64_t>({(uint64_t)kLvMaxGroups, std::max<uint64_t>((uint64_t)g->m, 8192),
+  // No more groups than the graph has arcs, or as the guess asks for: short calls on small graphs
+  // take a few MB, a batch of 64 six-vertex paths on 916 arcs (hundreds of millions of states) all.
+  const uint64_t room = std::max<uint64_t>({(uint64_t)g->m, 8192, (uint64_t)std::min(guess / 32, (double)kLvMaxGroups)});
+  const uint64_t most = std::min<uint64_t>({(uint64_t)kLvMaxGroups, room,
                                             (kLvChunkMask >> 1) / (uint64_t)std::max(g->maxdeg, 1)});
   // the first level holds all its vertices if they fit an eighth of the workspace
   const uint64_t first = std::min<uint64_t>({most, (A.nvert + 31) / 32 + (uint64_t)warps,

@@ -249,3 +249,27 @@ def test_more_calls_at_once_than_page_locked_blocks():
     for t in threads:
         t.join()
     assert len(got) == 800 and all(c == want[i] for i, c in got)
+
+
+def test_a_batch_on_few_arcs_matches_the_depth_first_search():
+    """64 six-vertex paths on 916 arcs: states by the million of every pattern, whose levels must not be sized by the arcs."""
+    import paper_2507_04130_gb300 as hm
+
+    G = hm.Graph.from_synth(synth.er_graph(70, 916, 1, 1, seed=92))
+    P = [hm.Pattern.from_synth(_pattern(6, [(i, i + 1) for i in range(5)]))] * 64
+
+    def best():
+        took = []
+        for _ in range(5):
+            t0 = time.perf_counter()
+            counts = hm.count_batch(G, P, hm.MONO)
+            took.append(time.perf_counter() - t0)
+        return counts, min(took)
+
+    level = best()
+    hm.set_tuning(poll_every=64)
+    try:
+        deep = best()
+    finally:
+        hm.set_tuning()
+    assert level[0] == deep[0] and level[1] < deep[1], (level[1], deep[1])
