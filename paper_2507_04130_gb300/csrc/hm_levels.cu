@@ -1181,8 +1181,10 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   std::vector<const int32_t *> vert_at(batch ? np : 0);
   std::vector<int2> deg0(batch ? np : 0);
   const int32_t *first_vertex = g->vby_out;
-  // a guess at the candidates: every position multiplies the states by a group's mean length
+  // a guess at the candidates: every position multiplies the states by a group's mean length, and
+  // every further condition keeps as many of them as a group holds of its label's vertices
   const double mean = (double)g->m / (double)std::max<int64_t>(1, std::min(g->ndir_out, g->ndir_in));
+  const double keeps = std::min(1.0, mean * g->nvl / (double)std::max(g->n, 1));
   double guess = 0;
   for (int32_t i = 0; i < np; ++i) {
     const Plan &P0 = batch ? *L.plans[i] : *L.plan;
@@ -1216,17 +1218,26 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
       A.root0 = L.root_mask && P.root_pos == 0;
     }
     A.nvert += (unsigned long long)cnt;
-    double states = (double)cnt;
-    for (int p = 1; p < P.k; ++p) guess += states *= mean;
+    double states = (double)cnt, last = defer ? mean : 1;  // (lv_has_final drops the vertices without a last image)
+    for (int j = 1; defer && j < lv[P.k - 1].npos; ++j) last *= keeps;
+    states *= std::min(last, 1.0);
+    for (int p = 1; p < P.k; ++p) {
+      guess += states *= mean;
+      for (int j = 1; j < lv[p].npos; ++j) states *= keeps;
+    }
   }
   if (batch) vert_n[np] = A.nvert;
   // Barriers cost less with fewer blocks: on 5,000 arcs with four labels a 4-cycle takes 56 us with 20
   // blocks and 65 with all 304.  But the arcs do not bound the work (a tournament of five on 60
-  // vertices: 3.06 ms with the 8 blocks that 1,800 arcs ask for, 1.50 depth first), so there is also
+  // vertices: 3.06 ms with the 8 blocks that 1,800 arcs ask for, 1.50 depth first), so there is
   // one block for every four chunks per warp of the guess (a 7-cycle on 5,000 unlabelled arcs: 20
-  // blocks 666 us, 304 blocks 241).
-  const double chunks_per_block = 32.0 * 4 * kLvWarps;
-  grid = (int)std::min<double>(grid, std::max((double)((g->m + 255) / 256), guess / chunks_per_block + 1));
+  // blocks 666 us, 304 blocks 241), and for every 512 arcs (pendant triangles on 73,000 R-MAT arcs: 60
+  // us, 68 with one for every 256); without hubs, where the mean says what a vertex has, 64 of
+  // these are enough (an 8-vertex pattern on 400,000 arcs: 106 us, 118 with 304).
+  const double by_guess = guess / (32.0 * 4 * kLvWarps) + 1;
+  int64_t by_arcs = (g->m + 511) / 512;
+  if ((int64_t)g->maxdeg * g->n <= 16 * g->m) by_arcs = std::min<int64_t>(by_arcs, 64);
+  grid = (int)std::min<double>(grid, std::max((double)by_arcs, by_guess));
 
   // The workspace: a quarter for the warps' resume points (fewer blocks if they
   // do not fit), the rest for the levels' states, equal numbers of groups each.
