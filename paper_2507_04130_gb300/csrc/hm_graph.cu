@@ -368,6 +368,13 @@ k_group_hubs(const int64_t *__restrict__ off, const int32_t *__restrict__ adj, c
   }
 }
 
+// Entries of both directories and the sorts' status, in one place for one copy.
+__global__ void k_dir_sizes(const uint32_t *oidx, const uint32_t *iidx, int32_t n, const int *sort_err, uint32_t *sizes) {
+  sizes[0] = oidx[n];
+  sizes[1] = iidx[n] - oidx[n];
+  sizes[2] = sort_failed(sort_err) ? 1u : 0u;
+}
+
 // Both directions of the steps below run in one launch (blockIdx.y).
 struct Direction {
   const int32_t *gofs;
@@ -726,31 +733,39 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     d_elab = t + 2 * m;
     d_vlab = t + 3 * m;
   }
-  // working memory: rows and their copy, offsets, class counts
-  int32_t *rows, *tmp;
+  // working memory: rows and their copy, offsets, class counts, and if there may be dense offsets
+  // groups per vertex and their prefix sums (both directions one after the other) and long lists
+  int32_t *rows, *tmp, *hubs;
   int64_t *out_off, *in_off;
-  uint32_t *err, *bins;
+  uint32_t *err, *ngroup, *didx, *bins, *sizes;
   Bounds *bnd;
-  size_t at = 0;
-  auto part = [&](size_t b) {
-    const size_t a = at;
-    at += (b + 255) / 256 * 256;
-    return a;
-  };
   {
+    size_t at = 0;
+    auto part = [&](size_t b) {
+      const size_t a = at;
+      at += (b + 255) / 256 * 256;
+      return a;
+    };
+    const bool dense = tables != Tables::kNone;
     const size_t bin_words = 6 * (size_t)(kMaxDense * kMaxDense + 1);
     const size_t a_rows = part(sizeof(int32_t) * (size_t)(kW * m + kW)), a_tmp = part(sizeof(int32_t) * (size_t)(kW * m + kW)),
                  a_off = part(sizeof(int64_t) * 2 * (size_t)(n + 1)),
-                 a_zero = part(sizeof(uint32_t) * (bin_words + 4)), a_bnd = part(sizeof(Bounds));
+                 a_grp = part(dense ? sizeof(uint32_t) * 4 * (size_t)(n + 1) : 0),
+                 a_hub = part(dense ? sizeof(int32_t) * 2 * (size_t)(m / kHub + 1) : 0),
+                 a_zero = part(sizeof(uint32_t) * (bin_words + 4)), a_bnd = part(sizeof(Bounds)), a_sizes = part(sizeof(uint32_t) * 3);
     unsigned char *w;
     HM_CUDA_TRY(T.get((void **)&w, at));
     rows = reinterpret_cast<int32_t *>(w + a_rows);
     tmp = reinterpret_cast<int32_t *>(w + a_tmp);
     out_off = reinterpret_cast<int64_t *>(w + a_off);
     in_off = out_off + (n + 1);
+    ngroup = reinterpret_cast<uint32_t *>(w + a_grp);
+    didx = ngroup + 2 * (size_t)(n + 1);
+    hubs = reinterpret_cast<int32_t *>(w + a_hub);
     err = reinterpret_cast<uint32_t *>(w + a_zero);  // {input errors, sort error}, then two list lengths, then the bins
     bins = err + 4;
     bnd = reinterpret_cast<Bounds *>(w + a_bnd);
+    sizes = reinterpret_cast<uint32_t *>(w + a_sizes);
   }
   k_begin<<<1, 1, 0, s>>>(err, bnd);
 
@@ -803,18 +818,6 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
     }
   }
   HM_CUDA_TRY(A.allocate(g));
-  // with dense offsets: groups per vertex and their prefix sums (both directions one after the other), long lists
-  uint32_t *ngroup = nullptr, *didx = nullptr;
-  int32_t *hubs = nullptr;
-  if (g->ncls) {
-    at = 0;
-    const size_t a_grp = part(sizeof(uint32_t) * 4 * (size_t)(n + 1)), a_hub = part(sizeof(int32_t) * 2 * (size_t)(m / kHub + 1));
-    unsigned char *w;
-    HM_CUDA_TRY(T.get((void **)&w, at));
-    ngroup = reinterpret_cast<uint32_t *>(w + a_grp);
-    didx = ngroup + 2 * (size_t)(n + 1);
-    hubs = reinterpret_cast<int32_t *>(w + a_hub);
-  }
   if (!g->regions) g->rfilt_out = g->rfilt_in = g->afilt;
   HM_CUDA_TRY(cudaMemsetAsync(g->afilt, 0, 8 * (size_t)g->afilt_nword, s));
   HM_CUDA_TRY(cudaMemsetAsync(g->ahash, 0xff, 32 * (size_t)g->ahash_nbkt, s));
@@ -844,7 +847,6 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
       // counts and cursors of both directions are zero; the starts follow them
       HM_CUDA_TRY(cudaMemsetAsync(err + 2, 0, sizeof(uint32_t) * (2 + 4 * (size_t)(nbin + 1)), s));
       uint32_t *nhub = err + 2;
-      uint32_t total[2] = {0, 0};
       for (int in = 0; in < 2; ++in) {
         if (in) {
           // the rows are in (src, dst) order: sorted by dst alone they are in (dst, src) order
@@ -873,15 +875,13 @@ hm_status load_graph_impl(int32_t n, int64_t m, const int32_t *src, const int32_
       if (st != HM_OK) return st;
       oidx = didx;
       iidx = didx + (n + 1);
-      HM_CUDA_TRY(cudaMemcpyAsync(&total[0], oidx + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-      HM_CUDA_TRY(cudaMemcpyAsync(&total[1], iidx + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-      int failed = 0;
-      HM_CUDA_TRY(cudaMemcpyAsync(&failed, sort_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+      k_dir_sizes<<<1, 1, 0, s>>>(oidx, iidx, n, sort_err, sizes);
+      uint32_t h_sizes[3] = {0, 0, 0};
+      HM_CUDA_TRY(cudaMemcpyAsync(h_sizes, sizes, sizeof(h_sizes), cudaMemcpyDeviceToHost, s));
       HM_CUDA_TRY(cudaStreamSynchronize(s));
-      if (failed) return HM_ERR_CUDA;  // the totals mean nothing
-      total[1] -= total[0];
-      g->ndir_out = total[0];
-      g->ndir_in = total[1];
+      if (h_sizes[2]) return HM_ERR_CUDA;  // a sort failed: the sizes mean nothing
+      g->ndir_out = h_sizes[0];
+      g->ndir_in = h_sizes[1];
       Arena D;
       D.add(&g->gdir_out, g->ndir_out);
       D.add(&g->gdir_in, g->ndir_in);
@@ -982,11 +982,11 @@ extern "C" hm_status hm_load_graph(int32_t n, int64_t m, const int32_t *src, con
     // back, then without the tables that only make searches faster (the dense
     // offsets and their vertex lists are up to 80 bytes per arc, the filters by
     // endpoint 8; without them calls search depth first)
-    const bool dense = g->ncls > 0, regions = g->regions != 0;
+    const bool regions = g->regions != 0;
     if (st == HM_ERR_OOM && !trimmed) {
       trimmed = true;
       trim_pool();
-    } else if (st == HM_ERR_OOM && (dense || regions)) {
+    } else if (st == HM_ERR_OOM && tables != Tables::kNone) {
       tables = regions ? Tables::kDense : Tables::kNone;
     } else {
       delete g;
