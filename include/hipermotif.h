@@ -291,12 +291,14 @@ hm_status hm_enumerate_batch(const hm_graph *g, const hm_pattern *const *pattern
  * with its own CUDA stream) serving queries against g, which must outlive the
  * server.  A free slot takes the waiting queries, in arrival order, that the
  * device-memory budget admits, up to max_batch, and runs them as one batch;
- * queries that arrive meanwhile join the next free slot's batch, and batches
- * of different slots overlap on the GPU.  Admission by what a query needs:
- * its seed queues, 24 B per target arc whose labels fit its seeding arc
- * (counted per (source label, arc label, target label) when the server is
- * created), plus 12 MiB per batch for the donation queue and control block;
- * the search stacks live in shared memory.  The head query always runs when
+ * queries that arrive meanwhile join the next free slot's batch, and one
+ * batch's search overlaps with the row sorts, copies and host work of other
+ * slots.  Admission by what a query may need: its seed queues, 24 B per target
+ * arc whose labels fit its seeding arc (counted per (source label, arc label,
+ * target label) when the server is created; the search by levels is charged
+ * the same), plus 12 MiB per batch for the control block and the levels' first
+ * 8 MiB or the donation queue.  While a search runs, its levels also take up
+ * to half of the slot's share of what the budget has free.  The head query always runs when
  * nothing else does, even if it alone exceeds the budget.  A batch makes one
  * pass: the rows of each query that wants them go to a region of up to 2^18
  * rows (fewer when the budget is short) and the batched enumeration keeps
@@ -393,7 +395,8 @@ hm_status hm_set_budget(uint64_t max_ms, uint64_t max_chunks);
  * on a graph with at most 64 classes is worked off level by level in one
  * launch, where only those two have a meaning.  Any other setting, a chunk
  * budget, the byte counters, an arc-range part, or more classes choose the
- * depth-first search, which the rest is about.
+ * depth-first search, which the rest is about (and so do two-vertex patterns on
+ * an unlabelled graph of 2^16 arcs or more, unless a single arc is counted).
  *   extend_min_blocks  resident 256-thread blocks per SM the kernel is
  *                      compiled for: 4 (default, 64 registers per thread),
  *                      5 or 6 (fewer registers, more warps to hide load
@@ -517,7 +520,9 @@ typedef struct {
                              * covers without a scan)                       */
   uint64_t states_injected; /* depth-2 states after both validators; level by
                              * level the states with two mapped positions,
-                             * which no neighbour-overlap test has thinned  */
+                             * which no neighbour-overlap test has thinned;
+                             * with the counters on (hm_set_counters) always
+                             * the former                                   */
   uint64_t tasks_donated;   /* work items split off for idle warps          */
   uint64_t chunks;          /* 32-candidate chunks examined                 */
   uint64_t matches;         /* the count of the call                        */

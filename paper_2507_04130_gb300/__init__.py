@@ -295,7 +295,7 @@ def _batch_args(patterns, modes):
 
 
 def count_batch(g: Graph, patterns, modes, stream=None) -> list[int]:
-    """Counts of many patterns from one edge scan and one persistent extension launch."""
+    """Counts of many patterns from one pass (with the default knobs, one launch)."""
     n, handles, m = _batch_args(patterns, modes)
     out = np.zeros(max(n, 1), np.uint64)
     check(lib.hm_count_batch(g.handle, ctypes.cast(handles, ctypes.c_void_p), _ptr(m), n,
@@ -342,8 +342,8 @@ class Server:
     """Query server over one resident graph (hm_server_*): submit from any thread, poll for results.
 
     `slots` dispatcher slots (each a host thread with its own stream) batch the
-    waiting queries that the device-memory budget admits; batches of different
-    slots overlap on the GPU.
+    waiting queries that the device-memory budget admits; one batch's search overlaps
+    with the row sorts, copies and host work of others.
     """
 
     def __init__(self, g: Graph, slots: int = 4, max_batch: int = 64, mem_budget: int = 0):

@@ -1,15 +1,19 @@
 // hm_batch.cu -- many patterns against one resident graph in one pass.
 //
-// The HiPerMotif algorithm (Sec. III-C) runs one edge loop per pattern.  A
-// batch shares that loop: one scan of the target's arcs tries every arc as
-// the seeding arc of every pattern whose signature (arc label, label of the
+// The HiPerMotif algorithm (Sec. III-C) runs one edge loop per pattern.  With the
+// default knobs a batch needs none: all patterns' first vertices stand in one list
+// and one launch works the levels of all of them off together (hm_levels.cu).
+// Otherwise (other knobs, byte counters, a chunk budget, graphs without dense group
+// offsets) the patterns share the loop: one scan of the target's arcs tries every
+// arc as the seeding arc of every pattern whose signature (arc label, label of the
 // arc's source, label of its target) it carries -- looked up in a small hash
 // table built on the host -- and applies that pattern's vertex and edge
 // validators (Alg. 2, Alg. 3).  Survivors carry their pattern id through the
-// overlap test and into ONE persistent extension launch, whose warps take
+// overlap test and into ONE persistent depth-first launch, whose warps take
 // depth-2 states of any pattern and read the pattern's plan from a device
-// table.  Rows of all patterns are sorted in one stable radix sort keyed on
-// (pattern id, row), then written back to each pattern's region.
+// table.  Either way the rows of all patterns are sorted together: short lists by
+// counting, others in one stable radix sort keyed on (pattern id, row) and written
+// back to each pattern's region.
 #include <algorithm>
 #include <cstring>
 #include <vector>

@@ -177,7 +177,7 @@ enum : int32_t { kStatOk = 0, kStatBudget = 1, kStatQueue = 2 };
 
 // Byte tallies of the instrumented kernel variants (hm_set_counters): `req`,
 // the bytes the kernel's accesses request at the granularity it reads them
-// (a 32-byte filter block per filter probe, a 16-byte vertex record, ...);
+// (an 8-byte word per filter probe, a 16-byte vertex record, ...);
 // `model`, the method's algorithmic bytes under the survey's cost model: 12 B
 // per arc scanned, 12 B per vertex record gathered (label and two degrees),
 // 8 B per candidate read from an adjacency list (neighbour and arc label),
@@ -289,9 +289,11 @@ __host__ __device__ __forceinline__ uint2 filter_bits(ArcKey k) {
 // 16M arcs, 600 MB for 150M, more than L2 holds).
 // kRegionArcs: from here on a graph gets them.  Measured with them against without:
 // 150M arcs, five connectome motifs 3.09 against 4.26 ms; 16M arcs, bi-fan 4.40
-// against 4.59, 4-cycles 2.67 against 2.76; but 3.9M arcs, a batch of 64 patterns
-// 428 against 420 us: a 16 MB filter is at home in L2 as it is, and what the
-// region of a vertex costs to look up is not won back.
+// against 4.59, 4-cycles 2.67 against 2.76.  The line lies where a batch of 64
+// cycles of three to five vertices crosses: 3.9M arcs 13.95 against 13.67 ms, 5.8M
+// 43.2 / 42.5, 8.0M 49.1 / 48.6, 10.8M 124 / 127, 14.1M 126 / 133, 16.1M 186 / 199.
+// Below, the filter is at home in L2 as it is, and what the region of a vertex
+// costs to look up is not won back; loading takes 4 to 5 % longer with them.
 constexpr int64_t kRegionArcs = (int64_t)1 << 23;
 
 struct Region {
@@ -506,9 +508,10 @@ hm_status radix_sort_rows(int32_t *rows, int32_t *tmp, int64_t nrows, int width,
                           const int *key_cols, int nkey, int bits, cudaStream_t stream,
                           int *launches = nullptr);
 
-// With `err` (device, zero) a failure sets *err instead of being waited for.
 // As radix_sort_rows, with a bit width (1..32) and an xor mask per key column
-// (the xor maps signed values to an unsigned order, e.g. 0x80000000).
+// (the xor maps signed values to an unsigned order, e.g. 0x80000000).  With
+// `err` (device, zero) the call does not wait: a barrier that gave up sets *err,
+// and what is launched behind must look at it before it uses the rows.
 hm_status radix_sort_rows_cols(int32_t *rows, int32_t *tmp, int64_t nrows, int width,
                                const int *key_cols, const int *key_bits, const uint32_t *key_xor,
                                int nkey, cudaStream_t stream, int *launches = nullptr, int *err = nullptr);

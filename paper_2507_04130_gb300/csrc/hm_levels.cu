@@ -110,8 +110,8 @@ struct LvPause {
 struct LvArgs {
   DevGraph G;
   LvCtl *ctl;
-  // each level: states (stride[p] words each, with the pattern's number after the images in a
-  // batch), their candidates {first, number, driving condition | list << 6 | pattern << 7, 0}, groups
+  // each level: states (their images, stride[p] words each), their candidates {first, number,
+  // driving condition | list << 6 | pattern << 7, 0}, groups
   int32_t *base[kMaxK + 1];
   int4 *rng[kMaxK + 1];
   LvGroup *grp[kMaxK + 1];
@@ -197,7 +197,7 @@ __device__ __forceinline__ bool lv_barrier(const LvArgs &A, LvShared &sm, unsign
 }
 
 // A state's first four images, in registers: most patterns' checks read no
-// more of it.  What is not a vertex (unmapped positions, a pattern number) is -1.
+// more of it.  Unmapped positions are -1.
 __device__ __forceinline__ int4 lv_images(const int32_t *mp, int p) {
   if (p == 1) return make_int4(mp[0], -1, -1, -1);
   if (p == 2) {
@@ -1069,7 +1069,7 @@ void lv_level(const hm_graph *g, const Plan &P, bool deferred, int p, bool want_
     out[j] = LvCons{cons[j].q, cons[j].kind, j < npos ? lv_class(g, cons[j].lab, P.vlab[p]) : (int16_t)0,
                        cons[j].lab, l.h};
   }
-  // arcs to later positions: one is found missing by the next ranges phase anyway
+  // arcs to later positions: a single one is found missing with the new state's range anyway
   L.need_deg = !L.last && P.dout[p] + P.din[p] - npos >= 2;
   L.closed = L.last && !want_rows && npos == 1 && n == 1 && !L.root;
 }
@@ -1229,7 +1229,7 @@ hm_status levels_try(const LvLaunch &L, cudaStream_t s, bool *ran, LvCtl *result
   if (batch) vert_n[np] = A.nvert;
   // Barriers cost less with fewer blocks: on 5,000 arcs with four labels a 4-cycle takes 56 us with 20
   // blocks and 65 with all 304.  But the arcs do not bound the work (a tournament of five on 60
-  // vertices: 3.06 ms with the 8 blocks that 1,800 arcs ask for, 1.50 depth first), so there is
+  // vertices: 3.06 ms with the 8 blocks that 1,800 arcs ask for, 1.50 depth first, 0.22 now), so there is
   // one block for every four chunks per warp of the guess (a 7-cycle on 5,000 unlabelled arcs: 20
   // blocks 666 us, 304 blocks 241), and for every 512 arcs (pendant triangles on 73,000 R-MAT arcs: 60
   // us, 68 with one for every 256); without hubs, where the mean says what a vertex has, 64 of

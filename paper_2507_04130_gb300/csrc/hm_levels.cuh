@@ -48,8 +48,8 @@ struct LvLaunch {
 // 128 MB for every level that keeps states, beside the first, is near the end of
 // that for all of them.  It stays in the device's pool: the first search of a
 // process takes about 0.1 ms longer for every 256 MB, the following ones nothing.
-// A level never gets more groups than the graph has arcs (or 8,192), so short
-// calls on small graphs take a few MB.
+// A level gets no more groups than the graph has arcs (at least 8,192), or than a
+// guess at the call's candidates asks for, so short calls on small graphs take a few MB.
 constexpr uint64_t kLevelWorkspaceMax = 1ull << 30;
 constexpr uint64_t kLevelWorkspacePer = 128ull << 20;
 constexpr uint64_t kLevelWorkspaceMin = 8ull << 20;  // on a device that is nearly full

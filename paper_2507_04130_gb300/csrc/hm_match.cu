@@ -1,6 +1,7 @@
 // hm_match.cu -- single-pattern entry points of the hot path (host orchestration)
-// and the count that allocates no device memory.  The kernels they launch are
-// in hm_kernels.cuh.
+// and the count that allocates no device memory.  Ordinary calls are worked off
+// level by level in one launch (hm_levels.cu); the kernels of the others (edge
+// scan, overlap test, depth-first extension) are in hm_kernels.cuh.
 #include <algorithm>
 #include <cstring>
 #include <mutex>

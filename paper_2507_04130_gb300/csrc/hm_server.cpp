@@ -6,16 +6,21 @@
 // slot is free it takes the waiting queries, in arrival order, that the
 // device-memory budget admits (up to max_batch) and runs them as ONE batch;
 // queries arriving while batches are on the GPU join the next free slot's
-// batch, and batches of different slots run concurrently on the device
-// (continuous batching at launch granularity).
+// batch (continuous batching at launch granularity).  The searches of two
+// batches run one after the other, since each is one launch whose blocks are all
+// resident and mostly fill the device; the slots overlap one batch's search with
+// the row sorts, copies and host work of others.
 //
-// Admission by the device memory a query needs: its depth-2 states can be no
+// Admission by the device memory a query may need: its depth-2 states can be no
 // more than the target arcs whose label and end labels fit its seeding arc
 // (counted once per (source label, arc label, target label) when the server
-// is created, from the graph's label-grouped directory), and each takes two
-// seed-queue entries (12 B each, with the pattern id); the donation queue and
-// control block (kBatchFixed) are charged once per batch.  The warps' DFS
-// stacks live in shared memory and cost no device memory.
+// is created, from the graph's label-grouped directory), and where the search is
+// depth first each takes two seed-queue entries (12 B each, with the pattern id).
+// The level-by-level search has no such queues; it is charged the same, which is
+// more than it takes.  kBatchFixed is charged once per batch: the control block
+// and the first 8 MiB of the levels, or the depth-first donation queue.  Levels
+// beyond that take part of what the budget has free while a search runs
+// (search_batch).
 //
 // One pass per batch: the rows of each query that wants them go to a region
 // sized by a guess (row_guess rows, within the budget); the batched

@@ -69,3 +69,31 @@ def test_a_device_without_room_refuses_the_graph():
     from paper_2507_04130_gb300 import binding
 
     assert _load(200) == ["status", str(binding.HM_ERR_OOM)]
+
+
+_SEARCH = r"""
+import numpy as np
+import torch
+import paper_2507_04130_gb300 as hm
+import synth
+
+g = synth.er_graph(9000, 100_000, 1, 1, seed=7)
+G = hm.Graph.from_synth(g, device=True)
+a = np.arange(7, dtype=np.int32)
+pats = [hm.Pattern(k, a[:k - 1], a[1:k], np.zeros(k, np.int32), np.zeros(k - 1, np.int32)) for k in (4, 6, 7)]
+torch.cuda.synchronize()
+torch.cuda.empty_cache()
+fill = torch.empty(torch.cuda.mem_get_info()[0] - (64 << 20), dtype=torch.uint8, device="cuda")
+tight = [hm.count_matches(G, p, hm.INDUCED) for p in pats] + hm.count_batch(G, pats, hm.INDUCED)
+del fill
+torch.cuda.empty_cache()
+full = [hm.count_matches(G, p, hm.INDUCED) for p in pats] + hm.count_batch(G, pats, hm.INDUCED)
+print("same" if tight == full and min(full) > 0 else (tight, full))
+"""
+
+
+def test_searches_on_a_nearly_full_device():
+    """64 MB are left, and the levels of these searches ask for 256 MB and more at first."""
+    r = subprocess.run([sys.executable, "-c", _SEARCH], capture_output=True, text=True, timeout=300, cwd=ROOT,
+                       env=dict(os.environ, PYTHONPATH=ROOT))
+    assert r.returncode == 0 and r.stdout.strip() == "same", r.stdout + r.stderr
